@@ -39,6 +39,7 @@
 
 #include "nb_internal.cuh"
 #include "ds.cuh"
+#include "pair.cuh"
 #include "tma.cuh"
 
 namespace nb {
@@ -216,6 +217,14 @@ __device__ __forceinline__ int member_index(const ISet &is, int k, unsigned *err
 // ...), so that a few hundred i-particles still fill an SM without cutting
 // the j-range into many grid-level pieces. Rows are added in shared memory at
 // the end, in fixed order.
+//
+// Bound by the FP32 pipe: 33 operations per interaction (27 for plain FP32), 1220 G/s at
+// 2070 MHz. The running totals live in shared memory (touched once per fold) and
+// not in 28 registers, so the packed loop, unrolled four pairs deep, runs without
+// spills at two CTAs per SM; with eps^2 >= FLT_MIN the SFU's reciprocal square root
+// is taken bare (rsqrtf adds a test and two FP32-pipe scalings per interaction).
+// N = 262144, F32-DS: 76.3 -> 67.8 ms = 1014 G/s, FMA pipe 84% of cycles (unroll 2:
+// 68.7 ms, 1: 68.5 ms); plain FP32 at N = 40961: 1.72 -> 1.56 ms.
 // ---------------------------------------------------------------------------
 
 template <int VAR, int IPT, int NWI, int NWJ, int JT, int NS>
@@ -245,10 +254,8 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     const int tile1 = (int)((long long)ntiles * (split + 1) / nsplit);
     const int my_tiles = tile1 - tile0;
 
-    // i-particles of this thread, negated and duplicated into both halves of a
-    // float2 (the packed pair arithmetic takes two j at a time)
-    float2 nxh[IPT], nyh[IPT], nzh[IPT], nxl[IPT], nyl[IPT], nzl[IPT], nvx[IPT], nvy[IPT],
-        nvz[IPT];
+    // i-particles of this thread
+    IPair ip[IPT];
     int iid[IPT];
 #pragma unroll
     for (int p = 0; p < IPT; ++p) {
@@ -258,36 +265,21 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
         const float4 a = __ldg(is.rec32 + (size_t)DS_REC * r);
         const float4 b = __ldg(is.rec32 + (size_t)DS_REC * r + 1);
         const float4 c = __ldg(is.rec32 + (size_t)DS_REC * r + 2);
-        nxh[p] = make_float2(-a.x, -a.x);
-        nyh[p] = make_float2(-a.y, -a.y);
-        nzh[p] = make_float2(-a.z, -a.z);
-        nxl[p] = make_float2(-b.x, -b.x);
-        nyl[p] = make_float2(-b.y, -b.y);
-        nzl[p] = make_float2(-b.z, -b.z);
-        nvx[p] = make_float2(-c.x, -c.x);
-        nvy[p] = make_float2(-c.y, -c.y);
-        nvz[p] = make_float2(-c.z, -c.z);
+        ip[p] = ipair_of(a, b, c);
         iid[p] = i_id(is, r, b.w);
     }
     const float2 e2 = make_float2(eps2f, eps2f);
+    const bool soft = soft_pairs(eps2f);
 
-    // running totals: double-single (DS) or plain FP32
-    float A_h[IPT][3], A_l[IPT][3], J_h[IPT][3], J_l[IPT][3], P_h[IPT], P_l[IPT];
+    // running totals (double-single, or plain FP32 in .x), this thread's own column
+    float2 *s_tot = reinterpret_cast<float2 *>(s_pair + (size_t)JT * DS_REC) + tid;
 #pragma unroll
-    for (int p = 0; p < IPT; ++p) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) A_h[p][c] = A_l[p][c] = J_h[p][c] = J_l[p][c] = 0.f;
-        P_h[p] = P_l[p] = 0.f;
-    }
+    for (int q = 0; q < 7 * IPT; ++q) s_tot[q * NT] = make_float2(0.f, 0.f);
     // FP32 partial sums between folds, two lanes each (even and odd j of a pair;
     // the masked scalar path adds into .x)
-    float2 ta[IPT][3], tja[IPT][3], tjb[IPT][3], tp[IPT];
+    PairSum ts[IPT];
 #pragma unroll
-    for (int p = 0; p < IPT; ++p) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) ta[p][c] = tja[p][c] = tjb[p][c] = make_float2(0.f, 0.f);
-        tp[p] = make_float2(0.f, 0.f);
-    }
+    for (int p = 0; p < IPT; ++p) pair_zero(ts[p]);
 
     if (tid == 0) {
         s_abort = 0;
@@ -335,15 +327,15 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
             for (int p = 0; p < IPT; ++p) {
                 float dx, dy, dz;
                 if (DS) {
-                    dx = (a.x + nxh[p].x) + (b.x + nxl[p].x);
-                    dy = (a.y + nyh[p].x) + (b.y + nyl[p].x);
-                    dz = (a.z + nzh[p].x) + (b.z + nzl[p].x);
+                    dx = (a.x + ip[p].xh.x) + (b.x + ip[p].xl.x);
+                    dy = (a.y + ip[p].yh.x) + (b.y + ip[p].yl.x);
+                    dz = (a.z + ip[p].zh.x) + (b.z + ip[p].zl.x);
                 } else {
-                    dx = a.x + nxh[p].x;
-                    dy = a.y + nyh[p].x;
-                    dz = a.z + nzh[p].x;
+                    dx = a.x + ip[p].xh.x;
+                    dy = a.y + ip[p].yh.x;
+                    dz = a.z + ip[p].zh.x;
                 }
-                const float dvx = c.x + nvx[p].x, dvy = c.y + nvy[p].x, dvz = c.z + nvz[p].x;
+                const float dvx = c.x + ip[p].vx.x, dvy = c.y + ip[p].vy.x, dvz = c.z + ip[p].vz.x;
                 float r2 = fmaf(dx, dx, eps2f);
                 r2 = fmaf(dy, dy, r2);
                 r2 = fmaf(dz, dz, r2);
@@ -356,16 +348,16 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
                 const float mrinv = a.w * rinv;
                 const float mr3 = mrinv * rinv2;
                 const float beta = (mr3 * rinv2) * rv;
-                tp[p].x += mrinv;
-                ta[p][0].x = fmaf(mr3, dx, ta[p][0].x);
-                ta[p][1].x = fmaf(mr3, dy, ta[p][1].x);
-                ta[p][2].x = fmaf(mr3, dz, ta[p][2].x);
-                tja[p][0].x = fmaf(mr3, dvx, tja[p][0].x);
-                tja[p][1].x = fmaf(mr3, dvy, tja[p][1].x);
-                tja[p][2].x = fmaf(mr3, dvz, tja[p][2].x);
-                tjb[p][0].x = fmaf(beta, dx, tjb[p][0].x);
-                tjb[p][1].x = fmaf(beta, dy, tjb[p][1].x);
-                tjb[p][2].x = fmaf(beta, dz, tjb[p][2].x);
+                ts[p].p.x += mrinv;
+                ts[p].a[0].x = fmaf(mr3, dx, ts[p].a[0].x);
+                ts[p].a[1].x = fmaf(mr3, dy, ts[p].a[1].x);
+                ts[p].a[2].x = fmaf(mr3, dz, ts[p].a[2].x);
+                ts[p].ja[0].x = fmaf(mr3, dvx, ts[p].ja[0].x);
+                ts[p].ja[1].x = fmaf(mr3, dvy, ts[p].ja[1].x);
+                ts[p].ja[2].x = fmaf(mr3, dvz, ts[p].ja[2].x);
+                ts[p].jb[0].x = fmaf(beta, dx, ts[p].jb[0].x);
+                ts[p].jb[1].x = fmaf(beta, dy, ts[p].jb[1].x);
+                ts[p].jb[2].x = fmaf(beta, dz, ts[p].jb[2].x);
             }
         };
         if (cnt == JT) {
@@ -382,60 +374,19 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
             __syncthreads();
             if (own) {
                 for (int jj = wj; jj < JT; jj += NWJ) body(jj, std::true_type{});
+            } else if (soft) {
+#pragma unroll 4
+                for (int q = wj; q < NPAIR; q += NWJ) {
+                    const JPair j = jpair_load<DS>(s_pair + 6 * q);
+#pragma unroll
+                    for (int p = 0; p < IPT; ++p) pair_add<DS, true>(j, ip[p], e2, ts[p], NoMask{});
+                }
             } else {
 #pragma unroll 2
                 for (int q = wj; q < NPAIR; q += NWJ) {
-                    const float4 *P = s_pair + 6 * q;
-                    const float4 q0 = P[0], q1 = P[1], q4 = P[4], q5 = P[5];
-                    float4 q2, q3;
-                    if (DS) {
-                        q2 = P[2];
-                        q3 = P[3];
-                    }
-                    const float2 XH = make_float2(q0.x, q0.y), YH = make_float2(q0.z, q0.w);
-                    const float2 ZH = make_float2(q1.x, q1.y), MJ = make_float2(q1.z, q1.w);
-                    const float2 VX = make_float2(q4.x, q4.y), VY = make_float2(q4.z, q4.w);
-                    const float2 VZ = make_float2(q5.x, q5.y);
+                    const JPair j = jpair_load<DS>(s_pair + 6 * q);
 #pragma unroll
-                    for (int p = 0; p < IPT; ++p) {
-                        float2 dx, dy, dz;
-                        if (DS) {
-                            dx = __fadd2_rn(__fadd2_rn(XH, nxh[p]),
-                                            __fadd2_rn(make_float2(q2.x, q2.y), nxl[p]));
-                            dy = __fadd2_rn(__fadd2_rn(YH, nyh[p]),
-                                            __fadd2_rn(make_float2(q2.z, q2.w), nyl[p]));
-                            dz = __fadd2_rn(__fadd2_rn(ZH, nzh[p]),
-                                            __fadd2_rn(make_float2(q3.x, q3.y), nzl[p]));
-                        } else {
-                            dx = __fadd2_rn(XH, nxh[p]);
-                            dy = __fadd2_rn(YH, nyh[p]);
-                            dz = __fadd2_rn(ZH, nzh[p]);
-                        }
-                        const float2 dvx = __fadd2_rn(VX, nvx[p]);
-                        const float2 dvy = __fadd2_rn(VY, nvy[p]);
-                        const float2 dvz = __fadd2_rn(VZ, nvz[p]);
-                        float2 r2 = __ffma2_rn(dx, dx, e2);
-                        r2 = __ffma2_rn(dy, dy, r2);
-                        r2 = __ffma2_rn(dz, dz, r2);
-                        float2 rv = __fmul2_rn(dx, dvx);
-                        rv = __ffma2_rn(dy, dvy, rv);
-                        rv = __ffma2_rn(dz, dvz, rv);
-                        const float2 rinv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-                        const float2 rinv2 = __fmul2_rn(rinv, rinv);
-                        const float2 mrinv = __fmul2_rn(MJ, rinv);
-                        const float2 mr3 = __fmul2_rn(mrinv, rinv2);
-                        const float2 beta = __fmul2_rn(__fmul2_rn(mr3, rinv2), rv);
-                        tp[p] = __fadd2_rn(tp[p], mrinv);
-                        ta[p][0] = __ffma2_rn(mr3, dx, ta[p][0]);
-                        ta[p][1] = __ffma2_rn(mr3, dy, ta[p][1]);
-                        ta[p][2] = __ffma2_rn(mr3, dz, ta[p][2]);
-                        tja[p][0] = __ffma2_rn(mr3, dvx, tja[p][0]);
-                        tja[p][1] = __ffma2_rn(mr3, dvy, tja[p][1]);
-                        tja[p][2] = __ffma2_rn(mr3, dvz, tja[p][2]);
-                        tjb[p][0] = __ffma2_rn(beta, dx, tjb[p][0]);
-                        tjb[p][1] = __ffma2_rn(beta, dy, tjb[p][1]);
-                        tjb[p][2] = __ffma2_rn(beta, dz, tjb[p][2]);
-                    }
+                    for (int p = 0; p < IPT; ++p) pair_add<DS, false>(j, ip[p], e2, ts[p], NoMask{});
                 }
             }
         } else if (own) {
@@ -450,27 +401,16 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
 #pragma unroll
             for (int p = 0; p < IPT; ++p) {
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const float sa = ta[p][c].x + ta[p][c].y;
-                    const float jt = fmaf(-3.f, tjb[p][c].x + tjb[p][c].y,
-                                          tja[p][c].x + tja[p][c].y);
-                    if (DS) {
-                        ds_add(A_h[p][c], A_l[p][c], sa);
-                        ds_add(J_h[p][c], J_l[p][c], jt);
-                    } else {
-                        A_h[p][c] += sa;
-                        J_h[p][c] += jt;
-                    }
+                for (int c = 0; c < 7; ++c) {
+                    float2 &h = s_tot[(p * 7 + c) * NT];
+                    float2 v = h;
+                    if (DS)
+                        ds_add(v.x, v.y, pair_total(ts[p], c));
+                    else
+                        v.x += pair_total(ts[p], c);
+                    h = v;
                 }
-                const float sp = tp[p].x + tp[p].y;
-                if (DS)
-                    ds_add(P_h[p], P_l[p], sp);
-                else
-                    P_h[p] += sp;
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    ta[p][c] = tja[p][c] = tjb[p][c] = make_float2(0.f, 0.f);
-                tp[p] = make_float2(0.f, 0.f);
+                pair_zero(ts[p]);
             }
         }
 
@@ -488,14 +428,12 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
 
     dsf v[IPT][7];
 #pragma unroll
-    for (int p = 0; p < IPT; ++p) {
+    for (int p = 0; p < IPT; ++p)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            v[p][c] = dsf{A_h[p][c], A_l[p][c]};
-            v[p][3 + c] = dsf{J_h[p][c], J_l[p][c]};
+        for (int c = 0; c < 7; ++c) {
+            const float2 h = s_tot[(p * 7 + c) * NT];
+            v[p][c] = dsf{h.x, h.y};
         }
-        v[p][6] = dsf{P_h[p], P_l[p]};
-    }
     if (NWJ > 1) {
         // add the warp rows in order 0..NWJ-1 (the tile ring is free: all tiles consumed)
         float2 *s_red = reinterpret_cast<float2 *>(s_tile);  // [NWJ][7][IB]
@@ -1734,6 +1672,15 @@ size_t plan_partial_doubles(const ForcePlan &p, int n_i)
     return (size_t)p.nsplit * 7 * (size_t)n_i;
 }
 
+// Shared memory of the tile kernel: the ring (36 KB; the warp-row sums, at most
+// 28 KB, reuse it), the transposed tile (12 KB) and the running totals of two
+// i-particles per thread.
+template <int NT>
+static constexpr size_t tile_smem()
+{
+    return (size_t)(NS32 + 1) * JT_TILE * DS_REC * sizeof(float4) + (size_t)NT * 14 * sizeof(float2);
+}
+
 template <int VAR, int IPT, int NWI, int NWJ>
 static cudaError_t go_tile32(const JSet &js, const ISet &is, float eps2f, int nsplit,
                              double *part, unsigned *cnt, Out3 out, unsigned *err,
@@ -1742,10 +1689,7 @@ static cudaError_t go_tile32(const JSet &js, const ISet &is, float eps2f, int ns
     auto kern = k_force_tile32<VAR, IPT, NWI, NWJ, JT_TILE, NS32>;
     constexpr int NT = 32 * NWI * NWJ;
     constexpr int IB = 32 * NWI * IPT;
-    // the ring (36 KB) and the transposed tile (12 KB); the warp-row sums reuse them
-    const size_t ring = (size_t)(NS32 + 1) * JT_TILE * DS_REC * sizeof(float4);
-    const size_t red = NWJ > 1 ? (size_t)NWJ * 7 * IB * sizeof(double) : 0;  // <= 28 KB
-    const size_t smem = ring > red ? ring : red;
+    const size_t smem = tile_smem<NT>();
     static const cudaError_t attr =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (attr != cudaSuccess) return attr;
@@ -1955,10 +1899,7 @@ template <int VAR, int NWI, int NWJ>
 static int tile_occ()
 {
     constexpr int NT = 32 * NWI * NWJ;
-    constexpr int IB = 32 * NWI * 2;
-    const size_t ring = (size_t)(NS32 + 1) * JT_TILE * DS_REC * sizeof(float4);
-    const size_t red = NWJ > 1 ? (size_t)NWJ * 7 * IB * sizeof(double) : 0;
-    const size_t smem = ring > red ? ring : red;
+    const size_t smem = tile_smem<NT>();
     auto kern = k_force_tile32<VAR, 2, NWI, NWJ, JT_TILE, NS32>;
     int nb = 0;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
