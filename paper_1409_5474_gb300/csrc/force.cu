@@ -29,13 +29,14 @@
 // Self pair: for i-particles that are members of the j-set the i == j pair is
 // masked by index (its potential term m_i/eps would otherwise swamp the FP32
 // sums, and with eps = 0 it is 0/0). The mask is applied only in the j-tiles
-// that contain one of the warp's own i-particles (a warp-uniform branch), so
-// the inner loop of every other tile carries no compare.
+// that contain one of the warp's own i-particles or are ragged (a warp-uniform
+// branch), so the inner loop of every other tile carries no compare. A warp holds
+// consecutive slots, so a sorted due set meets its own particles in few tiles.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
-#include <type_traits>
+#include <atomic>
 
 #include "nb_internal.cuh"
 #include "ds.cuh"
@@ -223,9 +224,13 @@ __device__ __forceinline__ int member_index(const ISet &is, int k, unsigned *err
 // not in 28 registers, so the packed loop, unrolled four pairs deep, runs without
 // spills at two CTAs per SM; with eps^2 >= FLT_MIN the SFU's reciprocal square root
 // is taken bare (rsqrtf adds a test and two FP32-pipe scalings per interaction).
-// N = 262144, F32-DS: 76.3 -> 67.8 ms = 1014 G/s, FMA pipe 84% of cycles (unroll 2:
-// 68.7 ms, 1: 68.5 ms); plain FP32 at N = 40961: 1.72 -> 1.56 ms.
+// N = 262144, F32-DS: 76.3 -> 67.8 ms, FMA pipe 84% of cycles (unroll 2: 68.7 ms, 1:
+// 68.5 ms). Tiles that are ragged or hold a warp's own particle stay on the packed path
+// with their halves masked, and warps without slots skip the arithmetic: 67.8 ->
+// 66.0 ms at N = 262144, 47.4 -> 43.3 us for N_i = 300 at N = 65536.
 // ---------------------------------------------------------------------------
+
+__host__ __device__ constexpr bool tile_ahead(int nwj) { return nwj == 8; }
 
 template <int VAR, int IPT, int NWI, int NWJ, int JT, int NS>
 __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
@@ -233,8 +238,8 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
                    double *__restrict__ part, long long pld, unsigned *counters, Out3 out,
                    unsigned *err)
 {
-    // NS ring stages of JT records (bulk-copy destinations), then the current
-    // tile transposed into j-pairs (JT / 2 pairs x 6 float4)
+    // NS ring stages of JT records (bulk-copy destinations), one or (AHEAD) two tiles as
+    // j-pairs (JT / 2 pairs x 6 float4 each), the running totals
     extern __shared__ __align__(128) float4 s_tile[];
     __shared__ __align__(8) uint64_t s_full[NS];
     __shared__ int s_abort;
@@ -242,10 +247,11 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     constexpr bool DS = (VAR == NB_F32DS);
     constexpr int NT = 32 * NWI * NWJ;
     constexpr int IB = 32 * NWI * IPT;
-    constexpr int NPAIR = JT / 2;
     // tiles per FP32 partial sum: about 128 terms in each half of a packed sum between folds
     constexpr int FOLD = (256 * NWJ / JT) > 1 ? (256 * NWJ / JT) : 1;
-    float4 *s_pair = s_tile + (size_t)NS * JT * DS_REC;
+    constexpr int PAIRS = JT * DS_REC;  // float4 of a pair buffer
+    constexpr bool AHEAD = tile_ahead(NWJ);
+    float4 *s_pair = s_tile + (size_t)NS * PAIRS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wi = warp % NWI, wj = warp / NWI;
     const int nsplit = gridDim.y;
@@ -259,7 +265,7 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     int iid[IPT];
 #pragma unroll
     for (int p = 0; p < IPT; ++p) {
-        int k = blockIdx.x * IB + p * (32 * NWI) + wi * 32 + lane;
+        int k = blockIdx.x * IB + (wi * IPT + p) * 32 + lane;
         if (k >= is.n) k = is.n - 1;  // idle slots compute a copy, never written
         const int r = i_row(is, k, err);
         const float4 a = __ldg(is.rec32 + (size_t)DS_REC * r);
@@ -270,13 +276,13 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     }
     const float2 e2 = make_float2(eps2f, eps2f);
     const bool soft = soft_pairs(eps2f);
+    const bool idle = blockIdx.x * IB + wi * IPT * 32 >= is.n;
 
     // running totals (double-single, or plain FP32 in .x), this thread's own column
-    float2 *s_tot = reinterpret_cast<float2 *>(s_pair + (size_t)JT * DS_REC) + tid;
+    float2 *s_tot = reinterpret_cast<float2 *>(s_pair + (AHEAD ? 2 : 1) * PAIRS) + tid;
 #pragma unroll
     for (int q = 0; q < 7 * IPT; ++q) s_tot[q * NT] = make_float2(0.f, 0.f);
-    // FP32 partial sums between folds, two lanes each (even and odd j of a pair;
-    // the masked scalar path adds into .x)
+    // FP32 partial sums between folds, two lanes each (even and odd j of a pair)
     PairSum ts[IPT];
 #pragma unroll
     for (int p = 0; p < IPT; ++p) pair_zero(ts[p]);
@@ -302,11 +308,38 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
         for (int kt = 0; kt < NS && kt < my_tiles; ++kt) issue(kt);
     }
 
-    for (int kt = 0; kt < my_tiles; ++kt) {
+    // AHEAD (eight warp rows): tile kt + 1 is rewritten as j-pairs into one buffer before
+    // the pair terms of tile kt are taken from the other, so there is one barrier per tile
+    // and the rewriting of some warps overlaps the arithmetic of others. A warp then has
+    // only 16 pairs of a tile: N_i = 300 and 1531 at N = 65536 take 41.3 and 133 us
+    // against 43.3 and 135.5 with one buffer and two barriers. With 128 or 32 pairs per
+    // warp and tile the second buffer's traffic costs more than the barrier (4.24 against
+    // 4.13 ms at N_i = 65536, 582 against 574 us at N_i = 8200).
+    auto fetch = [&](int kt) {
         const int stage = kt % NS;
-        const uint32_t parity = (uint32_t)((kt / NS) & 1);
-        if (!mbar_wait(&s_full[stage], parity)) s_abort = 1;
-        const float4 *T = s_tile + (size_t)stage * JT * DS_REC;
+        if (!mbar_wait(&s_full[stage], (uint32_t)((kt / NS) & 1))) s_abort = 1;
+        tile_to_pairs<JT, NT>(s_tile + (size_t)stage * JT * DS_REC,
+                              min(JT, nj - (tile0 + kt) * JT),
+                              s_pair + (AHEAD ? (kt & 1) * PAIRS : 0), tid);
+    };
+    if (AHEAD) {
+        if (my_tiles > 0) fetch(0);
+        __syncthreads();
+        if (s_abort) {
+            if (tid == 0) {
+                drain_ring<NS>(s_full, 0u, 0, my_tiles);
+                atomicOr(err, DERR_TIMEOUT);
+            }
+            return;
+        }
+        if (tid == 0 && NS < my_tiles) issue(NS);
+    }
+
+    for (int kt = 0; kt < my_tiles; ++kt) {
+        const int got = AHEAD ? kt + 1 : kt;  // the tile this iteration fetches
+        if (got < my_tiles) fetch(got);
+        if (!AHEAD) __syncthreads();
+        const float4 *pairs = s_pair + (AHEAD ? (kt & 1) * PAIRS : 0);
         const int jbase = (tile0 + kt) * JT;
         const int cnt = min(JT, nj - jbase);
 
@@ -316,85 +349,13 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
         for (int p = 0; p < IPT; ++p) own = own || (iid[p] >= jbase && iid[p] < jbase + cnt);
         own = __any_sync(0xffffffffu, own);
 
-        // scalar pair term of record jj (the self pair masked when MASKED)
-        auto body = [&](int jj, auto masked_tag) {
-            constexpr bool MASKED = decltype(masked_tag)::value;
-            const float4 a = T[DS_REC * jj];
-            const float4 c = T[DS_REC * jj + 2];
-            float4 b;
-            if (DS) b = T[DS_REC * jj + 1];
-#pragma unroll
-            for (int p = 0; p < IPT; ++p) {
-                float dx, dy, dz;
-                if (DS) {
-                    dx = (a.x + ip[p].xh.x) + (b.x + ip[p].xl.x);
-                    dy = (a.y + ip[p].yh.x) + (b.y + ip[p].yl.x);
-                    dz = (a.z + ip[p].zh.x) + (b.z + ip[p].zl.x);
-                } else {
-                    dx = a.x + ip[p].xh.x;
-                    dy = a.y + ip[p].yh.x;
-                    dz = a.z + ip[p].zh.x;
-                }
-                const float dvx = c.x + ip[p].vx.x, dvy = c.y + ip[p].vy.x, dvz = c.z + ip[p].vz.x;
-                float r2 = fmaf(dx, dx, eps2f);
-                r2 = fmaf(dy, dy, r2);
-                r2 = fmaf(dz, dz, r2);
-                float rv = dx * dvx;
-                rv = fmaf(dy, dvy, rv);
-                rv = fmaf(dz, dvz, rv);
-                float rinv = rsqrtf(r2);
-                if (MASKED) rinv = (jbase + jj == iid[p]) ? 0.f : rinv;
-                const float rinv2 = rinv * rinv;
-                const float mrinv = a.w * rinv;
-                const float mr3 = mrinv * rinv2;
-                const float beta = (mr3 * rinv2) * rv;
-                ts[p].p.x += mrinv;
-                ts[p].a[0].x = fmaf(mr3, dx, ts[p].a[0].x);
-                ts[p].a[1].x = fmaf(mr3, dy, ts[p].a[1].x);
-                ts[p].a[2].x = fmaf(mr3, dz, ts[p].a[2].x);
-                ts[p].ja[0].x = fmaf(mr3, dvx, ts[p].ja[0].x);
-                ts[p].ja[1].x = fmaf(mr3, dvy, ts[p].ja[1].x);
-                ts[p].ja[2].x = fmaf(mr3, dvz, ts[p].ja[2].x);
-                ts[p].jb[0].x = fmaf(beta, dx, ts[p].jb[0].x);
-                ts[p].jb[1].x = fmaf(beta, dy, ts[p].jb[1].x);
-                ts[p].jb[2].x = fmaf(beta, dz, ts[p].jb[2].x);
-            }
-        };
-        if (cnt == JT) {
-            // full tile: transpose it into j-pairs, {x_hi} {y_hi} {z_hi} {m} {x_lo}
-            // {y_lo} {z_lo} {index} {vx} {vy} {vz} of j = 2q, 2q + 1 side by side
-            for (int x = tid; x < 3 * NPAIR; x += NT) {
-                const int q = x % NPAIR, part = x / NPAIR;
-                const float4 u = T[DS_REC * (2 * q) + part];
-                const float4 v = T[DS_REC * (2 * q + 1) + part];
-                float4 *P = s_pair + 6 * q + 2 * part;
-                P[0] = make_float4(u.x, v.x, u.y, v.y);
-                P[1] = make_float4(u.z, v.z, u.w, v.w);
-            }
-            __syncthreads();
-            if (own) {
-                for (int jj = wj; jj < JT; jj += NWJ) body(jj, std::true_type{});
-            } else if (soft) {
-#pragma unroll 4
-                for (int q = wj; q < NPAIR; q += NWJ) {
-                    const JPair j = jpair_load<DS>(s_pair + 6 * q);
-#pragma unroll
-                    for (int p = 0; p < IPT; ++p) pair_add<DS, true>(j, ip[p], e2, ts[p], NoMask{});
-                }
-            } else {
-#pragma unroll 2
-                for (int q = wj; q < NPAIR; q += NWJ) {
-                    const JPair j = jpair_load<DS>(s_pair + 6 * q);
-#pragma unroll
-                    for (int p = 0; p < IPT; ++p) pair_add<DS, false>(j, ip[p], e2, ts[p], NoMask{});
-                }
-            }
-        } else if (own) {
-            for (int jj = wj; jj < cnt; jj += NWJ) body(jj, std::true_type{});
-        } else {
-#pragma unroll 2
-            for (int jj = wj; jj < cnt; jj += NWJ) body(jj, std::false_type{});
-        }
+        const bool masked = own || cnt < JT;
+        if (idle)
+            ;  // no slot of this warp is written
+        else if (soft)
+            tile_pairs<DS, IPT, JT, true>(pairs, wj, NWJ, jbase, cnt, masked, ip, iid, e2, ts);
+        else
+            tile_pairs<DS, IPT, JT, false>(pairs, wj, NWJ, jbase, cnt, masked, ip, iid, e2, ts);
 
         // fold the FP32 partial sums (both lanes) into the running totals
         if ((kt + 1) % FOLD == 0 || kt + 1 == my_tiles) {
@@ -414,65 +375,43 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
             }
         }
 
-        __syncthreads();  // every warp is done with this stage and the j-pairs
+        // every warp is done with the pairs of tile kt and the stage of tile got
+        __syncthreads();
         if (s_abort) {
-            if (tid == 0) drain_ring<NS>(s_full, 0u, kt, my_tiles);
-            break;
+            if (tid == 0) {
+                drain_ring<NS>(s_full, 0u, got, my_tiles);
+                atomicOr(err, DERR_TIMEOUT);
+            }
+            return;
         }
-        if (tid == 0 && kt + NS < my_tiles) issue(kt + NS);
-    }
-    if (s_abort) {
-        if (tid == 0) atomicOr(err, DERR_TIMEOUT);
-        return;
+        if (tid == 0 && got + NS < my_tiles) issue(got + NS);
     }
 
-    dsf v[IPT][7];
-#pragma unroll
-    for (int p = 0; p < IPT; ++p)
-#pragma unroll
-        for (int c = 0; c < 7; ++c) {
-            const float2 h = s_tot[(p * 7 + c) * NT];
-            v[p][c] = dsf{h.x, h.y};
-        }
-    if (NWJ > 1) {
-        // add the warp rows in order 0..NWJ-1 (the tile ring is free: all tiles consumed)
-        float2 *s_red = reinterpret_cast<float2 *>(s_tile);  // [NWJ][7][IB]
-#pragma unroll
-        for (int p = 0; p < IPT; ++p) {
-            const int slot = p * (32 * NWI) + wi * 32 + lane;
-#pragma unroll
-            for (int c = 0; c < 7; ++c)
-                s_red[(wj * 7 + c) * IB + slot] = make_float2(v[p][c].hi, v[p][c].lo);
-        }
-        __syncthreads();
-        if (wj == 0) {
-#pragma unroll
-            for (int p = 0; p < IPT; ++p) {
-                const int slot = p * (32 * NWI) + wi * 32 + lane;
-#pragma unroll
-                for (int c = 0; c < 7; ++c)
-                    for (int g = 1; g < NWJ; ++g) {
-                        const float2 w = s_red[(g * 7 + c) * IB + slot];
-                        ds_acc(v[p][c], dsf{w.x, w.y});
-                    }
-            }
-        }
-    }
     if (wj == 0) {
 #pragma unroll
         for (int p = 0; p < IPT; ++p) {
-            const int k = blockIdx.x * IB + p * (32 * NWI) + wi * 32 + lane;
+            const int k = blockIdx.x * IB + (wi * IPT + p) * 32 + lane;
             if (k >= is.n) continue;
+            // the warp rows' totals in order 0..NWJ-1 (columns 32 NWI threads apart)
+            dsf v[7];
+#pragma unroll
+            for (int c = 0; c < 7; ++c) {
+                const float2 *h = s_tot + (p * 7 + c) * NT;
+                v[c] = dsf{h[0].x, h[0].y};
+#pragma unroll
+                for (int g = 1; g < NWJ; ++g)
+                    ds_acc(v[c], dsf{h[32 * NWI * g].x, h[32 * NWI * g].y});
+            }
             if (nsplit == 1) {
                 double d[7];
 #pragma unroll
-                for (int c = 0; c < 7; ++c) d[c] = ds_to_double(v[p][c]);
+                for (int c = 0; c < 7; ++c) d[c] = ds_to_double(v[c]);
                 write_final(out, k, d, err);
             } else {
                 float2 *pp = reinterpret_cast<float2 *>(part);
 #pragma unroll
                 for (int c = 0; c < 7; ++c)
-                    pp[((size_t)split * 7 + c) * pld + k] = make_float2(v[p][c].hi, v[p][c].lo);
+                    pp[((size_t)split * 7 + c) * pld + k] = make_float2(v[c].hi, v[c].lo);
             }
         }
     }
@@ -1255,6 +1194,10 @@ __global__ void __launch_bounds__(256)
 }
 
 
+// As the tile kernel: bound by the FP32 pipe, totals in shared memory, ragged tiles and
+// tiles with a warp's own particles on the packed path (a 1000-particle system has a
+// quarter of its tiles of either kind), warps without rows skip the arithmetic. 512
+// clusters of 16-4096: a pass of eight steps 11.2 -> 10.3 ms.
 template <int VAR, int IPT, int NT, int JT, int NS>
 __global__ void __launch_bounds__(NT, 512 / NT)
     k_force_items32(const WorkItem *__restrict__ items, int nitems)
@@ -1264,9 +1207,10 @@ __global__ void __launch_bounds__(NT, 512 / NT)
     __shared__ __align__(8) uint64_t s_full[NS];
     __shared__ int s_abort;
     constexpr bool DS = (VAR == NB_F32DS);
-    constexpr int NPAIR = JT / 2;
     float4 *s_pair = s_tile + (size_t)NS * JT * DS_REC;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // the running totals (double-single, or plain FP32 in .x), this thread's own column
+    float2 *s_tot = reinterpret_cast<float2 *>(s_pair + (size_t)JT * DS_REC) + tid;
 
     if (tid == 0) {
         s_abort = 0;
@@ -1282,39 +1226,25 @@ __global__ void __launch_bounds__(NT, 512 / NT)
         unsigned *err = w.err;
         const float eps2f = w.eps2;
         const float2 e2 = make_float2(eps2f, eps2f);
+        const bool soft = soft_pairs(eps2f);
         const float4 *__restrict__ jrec = w.jrec;
         const int ntiles = (w.nj + JT - 1) / JT;
 
-        // the i-particles, negated and duplicated into both halves of a float2 (the
-        // packed pair terms take two j at a time; the scalar path uses .x)
-        float2 nxh[IPT], nyh[IPT], nzh[IPT], nxl[IPT], nyl[IPT], nzl[IPT], nvx[IPT], nvy[IPT],
-            nvz[IPT];
+        // the i-particles
+        IPair ip[IPT];
         int iid[IPT];
 #pragma unroll
         for (int p = 0; p < IPT; ++p) {
-            const int k = min(p * NT + tid, w.ni - 1);  // idle slots copy the last i
+            const int k = min((warp * IPT + p) * 32 + lane, w.ni - 1);  // idle slots copy the last i
             const int r = w.i0 + k;
             const float4 a = __ldg(w.irec + (size_t)DS_REC * r);
             const float4 b = __ldg(w.irec + (size_t)DS_REC * r + 1);
             const float4 c = __ldg(w.irec + (size_t)DS_REC * r + 2);
-            nxh[p] = make_float2(-a.x, -a.x);
-            nyh[p] = make_float2(-a.y, -a.y);
-            nzh[p] = make_float2(-a.z, -a.z);
-            nxl[p] = make_float2(-b.x, -b.x);
-            nyl[p] = make_float2(-b.y, -b.y);
-            nzl[p] = make_float2(-b.z, -b.z);
-            nvx[p] = make_float2(-c.x, -c.x);
-            nvy[p] = make_float2(-c.y, -c.y);
-            nvz[p] = make_float2(-c.z, -c.z);
+            ip[p] = ipair_of(a, b, c);
             iid[p] = w.gathered ? __float_as_int(b.w) : r;
         }
-        float A_h[IPT][3], A_l[IPT][3], J_h[IPT][3], J_l[IPT][3], P_h[IPT], P_l[IPT];
 #pragma unroll
-        for (int p = 0; p < IPT; ++p) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) A_h[p][c] = A_l[p][c] = J_h[p][c] = J_l[p][c] = 0.f;
-            P_h[p] = P_l[p] = 0.f;
-        }
+        for (int q = 0; q < 7 * IPT; ++q) s_tot[q * NT] = make_float2(0.f, 0.f);
 
         auto issue = [&](int kt) {
             const unsigned sq = seq + (unsigned)kt;
@@ -1339,154 +1269,31 @@ __global__ void __launch_bounds__(NT, 512 / NT)
 #pragma unroll
             for (int p = 0; p < IPT; ++p) own = own || (iid[p] >= jbase && iid[p] < jbase + cnt);
             own = __any_sync(0xffffffffu, own);
-            // FP32 sums of this tile, two lanes each (even and odd j of a pair; the
-            // scalar path adds into .x)
-            float2 ta[IPT][3], tja[IPT][3], tjb[IPT][3], tp[IPT];
+            // FP32 sums of this tile, two lanes each (even and odd j of a pair)
+            PairSum ts[IPT];
 #pragma unroll
-            for (int p = 0; p < IPT; ++p) {
+            for (int p = 0; p < IPT; ++p) pair_zero(ts[p]);
+            const bool masked = own || cnt < JT;
+            tile_to_pairs<JT, NT>(T, cnt, s_pair, tid);
+            __syncthreads();
+            if (warp * IPT * 32 >= w.ni)
+                ;  // no row of this warp is written
+            else if (soft)
+                tile_pairs<DS, IPT, JT, true>(s_pair, 0, 1, jbase, cnt, masked, ip, iid, e2, ts);
+            else
+                tile_pairs<DS, IPT, JT, false>(s_pair, 0, 1, jbase, cnt, masked, ip, iid, e2, ts);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) ta[p][c] = tja[p][c] = tjb[p][c] = make_float2(0.f, 0.f);
-                tp[p] = make_float2(0.f, 0.f);
-            }
-            auto body = [&](int jj, auto masked_tag) {
-                constexpr bool MASKED = decltype(masked_tag)::value;
-                const float4 a = T[DS_REC * jj];
-                const float4 c = T[DS_REC * jj + 2];
-                float4 b;
-                if (DS) b = T[DS_REC * jj + 1];
+            for (int p = 0; p < IPT; ++p)
 #pragma unroll
-                for (int p = 0; p < IPT; ++p) {
-                    float dx, dy, dz;
-                    if (DS) {
-                        dx = (a.x + nxh[p].x) + (b.x + nxl[p].x);
-                        dy = (a.y + nyh[p].x) + (b.y + nyl[p].x);
-                        dz = (a.z + nzh[p].x) + (b.z + nzl[p].x);
-                    } else {
-                        dx = a.x + nxh[p].x;
-                        dy = a.y + nyh[p].x;
-                        dz = a.z + nzh[p].x;
-                    }
-                    const float dvx = c.x + nvx[p].x, dvy = c.y + nvy[p].x, dvz = c.z + nvz[p].x;
-                    float r2 = fmaf(dx, dx, eps2f);
-                    r2 = fmaf(dy, dy, r2);
-                    r2 = fmaf(dz, dz, r2);
-                    float rv = dx * dvx;
-                    rv = fmaf(dy, dvy, rv);
-                    rv = fmaf(dz, dvz, rv);
-                    float rinv = rsqrtf(r2);
-                    if (MASKED) rinv = (jbase + jj == iid[p]) ? 0.f : rinv;
-                    const float rinv2 = rinv * rinv;
-                    const float mrinv = a.w * rinv;
-                    const float mr3 = mrinv * rinv2;
-                    const float beta = (mr3 * rinv2) * rv;
-                    tp[p].x += mrinv;
-                    ta[p][0].x = fmaf(mr3, dx, ta[p][0].x);
-                    ta[p][1].x = fmaf(mr3, dy, ta[p][1].x);
-                    ta[p][2].x = fmaf(mr3, dz, ta[p][2].x);
-                    tja[p][0].x = fmaf(mr3, dvx, tja[p][0].x);
-                    tja[p][1].x = fmaf(mr3, dvy, tja[p][1].x);
-                    tja[p][2].x = fmaf(mr3, dvz, tja[p][2].x);
-                    tjb[p][0].x = fmaf(beta, dx, tjb[p][0].x);
-                    tjb[p][1].x = fmaf(beta, dy, tjb[p][1].x);
-                    tjb[p][2].x = fmaf(beta, dz, tjb[p][2].x);
+                for (int c = 0; c < 7; ++c) {
+                    float2 &h = s_tot[(p * 7 + c) * NT];
+                    float2 v = h;
+                    if (DS)
+                        ds_add(v.x, v.y, pair_total(ts[p], c));
+                    else
+                        v.x += pair_total(ts[p], c);
+                    h = v;
                 }
-            };
-            if (cnt == JT) {
-                // full tile: transposed into j-pairs for the packed FP32x2 pair terms
-                for (int x = tid; x < 3 * NPAIR; x += NT) {
-                    const int q = x % NPAIR, part = x / NPAIR;
-                    const float4 u = T[DS_REC * (2 * q) + part];
-                    const float4 v = T[DS_REC * (2 * q + 1) + part];
-                    float4 *P = s_pair + 6 * q + 2 * part;
-                    P[0] = make_float4(u.x, v.x, u.y, v.y);
-                    P[1] = make_float4(u.z, v.z, u.w, v.w);
-                }
-                __syncthreads();
-                if (own) {
-                    for (int jj = 0; jj < JT; ++jj) body(jj, std::true_type{});
-                } else {
-#pragma unroll 2
-                    for (int q = 0; q < NPAIR; ++q) {
-                        const float4 *P = s_pair + 6 * q;
-                        const float4 q0 = P[0], q1 = P[1], q4 = P[4], q5 = P[5];
-                        float4 q2, q3;
-                        if (DS) {
-                            q2 = P[2];
-                            q3 = P[3];
-                        }
-                        const float2 XH = make_float2(q0.x, q0.y), YH = make_float2(q0.z, q0.w);
-                        const float2 ZH = make_float2(q1.x, q1.y), MJ = make_float2(q1.z, q1.w);
-                        const float2 VX = make_float2(q4.x, q4.y), VY = make_float2(q4.z, q4.w);
-                        const float2 VZ = make_float2(q5.x, q5.y);
-#pragma unroll
-                        for (int p = 0; p < IPT; ++p) {
-                            float2 dx, dy, dz;
-                            if (DS) {
-                                dx = __fadd2_rn(__fadd2_rn(XH, nxh[p]),
-                                                __fadd2_rn(make_float2(q2.x, q2.y), nxl[p]));
-                                dy = __fadd2_rn(__fadd2_rn(YH, nyh[p]),
-                                                __fadd2_rn(make_float2(q2.z, q2.w), nyl[p]));
-                                dz = __fadd2_rn(__fadd2_rn(ZH, nzh[p]),
-                                                __fadd2_rn(make_float2(q3.x, q3.y), nzl[p]));
-                            } else {
-                                dx = __fadd2_rn(XH, nxh[p]);
-                                dy = __fadd2_rn(YH, nyh[p]);
-                                dz = __fadd2_rn(ZH, nzh[p]);
-                            }
-                            const float2 dvx = __fadd2_rn(VX, nvx[p]);
-                            const float2 dvy = __fadd2_rn(VY, nvy[p]);
-                            const float2 dvz = __fadd2_rn(VZ, nvz[p]);
-                            float2 r2 = __ffma2_rn(dx, dx, e2);
-                            r2 = __ffma2_rn(dy, dy, r2);
-                            r2 = __ffma2_rn(dz, dz, r2);
-                            float2 rv = __fmul2_rn(dx, dvx);
-                            rv = __ffma2_rn(dy, dvy, rv);
-                            rv = __ffma2_rn(dz, dvz, rv);
-                            const float2 rinv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-                            const float2 rinv2 = __fmul2_rn(rinv, rinv);
-                            const float2 mrinv = __fmul2_rn(MJ, rinv);
-                            const float2 mr3 = __fmul2_rn(mrinv, rinv2);
-                            const float2 beta = __fmul2_rn(__fmul2_rn(mr3, rinv2), rv);
-                            tp[p] = __fadd2_rn(tp[p], mrinv);
-                            ta[p][0] = __ffma2_rn(mr3, dx, ta[p][0]);
-                            ta[p][1] = __ffma2_rn(mr3, dy, ta[p][1]);
-                            ta[p][2] = __ffma2_rn(mr3, dz, ta[p][2]);
-                            tja[p][0] = __ffma2_rn(mr3, dvx, tja[p][0]);
-                            tja[p][1] = __ffma2_rn(mr3, dvy, tja[p][1]);
-                            tja[p][2] = __ffma2_rn(mr3, dvz, tja[p][2]);
-                            tjb[p][0] = __ffma2_rn(beta, dx, tjb[p][0]);
-                            tjb[p][1] = __ffma2_rn(beta, dy, tjb[p][1]);
-                            tjb[p][2] = __ffma2_rn(beta, dz, tjb[p][2]);
-                        }
-                    }
-                }
-            } else if (own) {
-                for (int jj = 0; jj < cnt; ++jj) body(jj, std::true_type{});
-            } else {
-#pragma unroll 2
-                for (int jj = 0; jj < cnt; ++jj) body(jj, std::false_type{});
-            }
-#pragma unroll
-            for (int p = 0; p < IPT; ++p) {
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const float sa = ta[p][c].x + ta[p][c].y;
-                    const float jt = fmaf(-3.f, tjb[p][c].x + tjb[p][c].y,
-                                          tja[p][c].x + tja[p][c].y);
-                    if (DS) {
-                        ds_add(A_h[p][c], A_l[p][c], sa);
-                        ds_add(J_h[p][c], J_l[p][c], jt);
-                    } else {
-                        A_h[p][c] += sa;
-                        J_h[p][c] += jt;
-                    }
-                }
-                const float sp = tp[p].x + tp[p].y;
-                if (DS)
-                    ds_add(P_h[p], P_l[p], sp);
-                else
-                    P_h[p] += sp;
-            }
             __syncthreads();  // the stage and the pair buffer are free
             if (s_abort) {
                 if (tid == 0) {
@@ -1501,29 +1308,24 @@ __global__ void __launch_bounds__(NT, 512 / NT)
         if (w.nsplit <= 1) {
 #pragma unroll
             for (int p = 0; p < IPT; ++p) {
-                const int k = p * NT + tid;
+                const int k = (warp * IPT + p) * 32 + lane;
                 if (k >= w.ni) continue;
                 double d[7];
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    d[c] = ds_to_double(dsf{A_h[p][c], A_l[p][c]});
-                    d[3 + c] = ds_to_double(dsf{J_h[p][c], J_l[p][c]});
+                for (int c = 0; c < 7; ++c) {
+                    const float2 h = s_tot[(p * 7 + c) * NT];
+                    d[c] = ds_to_double(dsf{h.x, h.y});
                 }
-                d[6] = ds_to_double(dsf{P_h[p], P_l[p]});
                 write_final(Out3{w.acc, w.jerk, w.pot, w.ld}, w.i0 + k, d, err);
             }
         } else {
             float2 *pp = w.part + (size_t)w.split * 7 * w.ni;
 #pragma unroll
             for (int p = 0; p < IPT; ++p) {
-                const int k = p * NT + tid;
+                const int k = (warp * IPT + p) * 32 + lane;
                 if (k >= w.ni) continue;
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    pp[(size_t)c * w.ni + k] = make_float2(A_h[p][c], A_l[p][c]);
-                    pp[(size_t)(3 + c) * w.ni + k] = make_float2(J_h[p][c], J_l[p][c]);
-                }
-                pp[(size_t)6 * w.ni + k] = make_float2(P_h[p], P_l[p]);
+                for (int c = 0; c < 7; ++c) pp[(size_t)c * w.ni + k] = s_tot[(p * 7 + c) * NT];
             }
         }
     }
@@ -1672,13 +1474,29 @@ size_t plan_partial_doubles(const ForcePlan &p, int n_i)
     return (size_t)p.nsplit * 7 * (size_t)n_i;
 }
 
-// Shared memory of the tile kernel: the ring (36 KB; the warp-row sums, at most
-// 28 KB, reuse it), the transposed tile (12 KB) and the running totals of two
-// i-particles per thread.
-template <int NT>
+// Let kernel K take smem bytes of dynamic shared memory on the current device (the
+// attribute belongs to the device: set once on each).
+template <auto K>
+static cudaError_t allow_smem(size_t smem)
+{
+    static std::atomic<unsigned long long> done{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
+
+// Shared memory of the tile kernel: the ring (36 KB), one or two transposed tiles
+// (12 KB each) and the running totals of two i-particles per thread (28 KB).
+template <int NT, int NWJ>
 static constexpr size_t tile_smem()
 {
-    return (size_t)(NS32 + 1) * JT_TILE * DS_REC * sizeof(float4) + (size_t)NT * 14 * sizeof(float2);
+    return (size_t)(NS32 + (tile_ahead(NWJ) ? 2 : 1)) * JT_TILE * DS_REC * sizeof(float4) +
+           (size_t)NT * 14 * sizeof(float2);
 }
 
 template <int VAR, int IPT, int NWI, int NWJ>
@@ -1686,12 +1504,11 @@ static cudaError_t go_tile32(const JSet &js, const ISet &is, float eps2f, int ns
                              double *part, unsigned *cnt, Out3 out, unsigned *err,
                              cudaStream_t st)
 {
-    auto kern = k_force_tile32<VAR, IPT, NWI, NWJ, JT_TILE, NS32>;
+    constexpr auto kern = k_force_tile32<VAR, IPT, NWI, NWJ, JT_TILE, NS32>;
     constexpr int NT = 32 * NWI * NWJ;
     constexpr int IB = 32 * NWI * IPT;
-    const size_t smem = tile_smem<NT>();
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = tile_smem<NT, NWJ>();
+    const cudaError_t attr = allow_smem<kern>(smem);
     if (attr != cudaSuccess) return attr;
     const int ntiles = (js.n + JT_TILE - 1) / JT_TILE;
     dim3 grid((is.n + IB - 1) / IB, nsplit);
@@ -1815,11 +1632,22 @@ static cudaError_t dispatch64(const ForcePlan &p, const JSet &js, const ISet &is
     return go_tile64<1, 128>(js, is, eps2, p.nsplit, part, cnt, out, err, st);
 }
 
+// Shared memory of the batched kernel: the ring (18 KB), the transposed tile (6 KB)
+// and the running totals of two i-particles per thread.
+static size_t items_smem(int threads)
+{
+    return (size_t)(NS32 + 1) * JT32 * DS_REC * sizeof(float4) +
+           (size_t)threads * 14 * sizeof(float2);
+}
+
 template <int VAR, int NT>
 static cudaError_t go_items(const WorkItem *items, int nitems, int grid, cudaStream_t st)
 {
-    const size_t smem = (size_t)(NS32 + 1) * JT32 * DS_REC * sizeof(float4);
-    k_force_items32<VAR, 2, NT, JT32, NS32><<<grid, NT, smem, st>>>(items, nitems);
+    constexpr auto kern = k_force_items32<VAR, 2, NT, JT32, NS32>;
+    const size_t smem = items_smem(NT);
+    const cudaError_t attr = allow_smem<kern>(smem);
+    if (attr != cudaSuccess) return attr;
+    kern<<<grid, NT, smem, st>>>(items, nitems);
     return cudaGetLastError();
 }
 
@@ -1899,13 +1727,11 @@ template <int VAR, int NWI, int NWJ>
 static int tile_occ()
 {
     constexpr int NT = 32 * NWI * NWJ;
-    const size_t smem = tile_smem<NT>();
-    auto kern = k_force_tile32<VAR, 2, NWI, NWJ, JT_TILE, NS32>;
+    const size_t smem = tile_smem<NT, NWJ>();
+    constexpr auto kern = k_force_tile32<VAR, 2, NWI, NWJ, JT_TILE, NS32>;
     int nb = 0;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, NT, smem) !=
-        cudaSuccess) {
+    if (allow_smem<kern>(smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, NT, smem) != cudaSuccess) {
         cudaGetLastError();
         return 1;
     }
@@ -1921,31 +1747,29 @@ int tile_blocks_per_sm(int variant, int nwj)
                     : (nwj == 4 ? tile_occ<NB_F32, 2, 4>() : tile_occ<NB_F32, 1, 8>());
 }
 
-int batch_blocks_per_sm(int variant, int threads)
+template <int VAR, int NT>
+static int items_occ()
 {
+    constexpr auto kern = k_force_items32<VAR, 2, NT, JT32, NS32>;
+    const size_t smem = items_smem(NT);
     int nb = 0;
-    const size_t smem = (size_t)(NS32 + 1) * JT32 * DS_REC * sizeof(float4);
-    cudaError_t e;
-    if (variant == NB_F32DS) {
-        e = threads == 64    ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                &nb, k_force_items32<NB_F32DS, 2, 64, JT32, NS32>, 64, smem)
-            : threads == 128 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                   &nb, k_force_items32<NB_F32DS, 2, 128, JT32, NS32>, 128, smem)
-                             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                   &nb, k_force_items32<NB_F32DS, 2, 256, JT32, NS32>, 256, smem);
-    } else {
-        e = threads == 64    ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                &nb, k_force_items32<NB_F32, 2, 64, JT32, NS32>, 64, smem)
-            : threads == 128 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                   &nb, k_force_items32<NB_F32, 2, 128, JT32, NS32>, 128, smem)
-                             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                   &nb, k_force_items32<NB_F32, 2, 256, JT32, NS32>, 256, smem);
-    }
-    if (e != cudaSuccess) {
+    if (allow_smem<kern>(smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, NT, smem) != cudaSuccess) {
         cudaGetLastError();
         return 1;
     }
     return nb > 0 ? nb : 1;
+}
+
+int batch_blocks_per_sm(int variant, int threads)
+{
+    if (variant == NB_F32DS)
+        return threads == 64    ? items_occ<NB_F32DS, 64>()
+               : threads == 128 ? items_occ<NB_F32DS, 128>()
+                                : items_occ<NB_F32DS, 256>();
+    return threads == 64    ? items_occ<NB_F32, 64>()
+           : threads == 128 ? items_occ<NB_F32, 128>()
+                            : items_occ<NB_F32, 256>();
 }
 
 size_t plan_counters(const ForcePlan &p, int n_i)

@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 
 #include "ds.cuh"
+#include "nb_internal.cuh"
 
 namespace nb {
 
@@ -135,6 +136,67 @@ __device__ __forceinline__ void pair_add(const JPair &j, const IPair &i, float2 
 struct NoMask {
     __device__ __forceinline__ void operator()(float2 &) const {}
 };
+
+// The self pair and records past the end of a ragged tile contribute nothing: records
+// ja and ja + 1 of the j-set, the i-particle's own index, the end of the tile.
+struct PairMask {
+    int ja, own, end;
+    __device__ __forceinline__ void operator()(float2 &rinv) const
+    {
+        rinv.x = (ja == own || ja >= end) ? 0.f : rinv.x;
+        rinv.y = (ja + 1 == own || ja + 1 >= end) ? 0.f : rinv.y;
+    }
+};
+
+// Rewrite cnt records (of a tile of JT) at T as j-pairs at s_pair, by NT threads;
+// records past the end become zeros (their pairs are masked).
+template <int JT, int NT>
+__device__ __forceinline__ void tile_to_pairs(const float4 *T, int cnt, float4 *s_pair, int tid)
+{
+    constexpr int NPAIR = JT / 2;
+    auto put = [&](int x, bool full) {
+        const int q = x % NPAIR, part = x / NPAIR;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 u = full || 2 * q < cnt ? T[DS_REC * (2 * q) + part] : zero;
+        const float4 v = full || 2 * q + 1 < cnt ? T[DS_REC * (2 * q + 1) + part] : zero;
+        float4 *P = s_pair + 6 * q + 2 * part;
+        P[0] = make_float4(u.x, v.x, u.y, v.y);
+        P[1] = make_float4(u.z, v.z, u.w, v.w);
+    };
+    if (cnt == JT) {
+        for (int x = tid; x < DS_REC * NPAIR; x += NT) put(x, true);
+    } else {
+        for (int x = tid; x < DS_REC * NPAIR; x += NT) put(x, false);
+    }
+}
+
+// The pair terms of the j-pairs q0, q0 + step, ... of a tile (first record jbase, cnt
+// records) on IPT i-particles; own: their indices. masked: the tile is ragged or
+// holds one of the warp's own particles.
+template <bool DS, int IPT, int JT, bool SOFT>
+__device__ __forceinline__ void tile_pairs(const float4 *s_pair, int q0, int step, int jbase,
+                                           int cnt, bool masked, const IPair (&ip)[IPT],
+                                           const int (&own)[IPT], float2 e2, PairSum (&ts)[IPT])
+{
+    if (masked) {
+        const int npair = (cnt + 1) / 2;
+#pragma unroll 2
+        for (int q = q0; q < npair; q += step) {
+            const JPair j = jpair_load<DS>(s_pair + 6 * q);
+#pragma unroll
+            for (int p = 0; p < IPT; ++p)
+                pair_add<DS, SOFT>(j, ip[p], e2, ts[p],
+                                   PairMask{jbase + 2 * q, own[p], jbase + cnt});
+        }
+    } else {
+#pragma unroll 4
+        for (int q = q0; q < JT / 2; q += step) {
+            const JPair j = jpair_load<DS>(s_pair + 6 * q);
+#pragma unroll
+            for (int p = 0; p < IPT; ++p) pair_add<DS, SOFT>(j, ip[p], e2, ts[p], NoMask{});
+        }
+    }
+}
 
 // The sums of component c (0-2 acc, 3-5 jerk, 6 the positive potential) over both halves.
 __device__ __forceinline__ float pair_total(const PairSum &t, int c)
