@@ -30,6 +30,7 @@
 
 #include "ds.cuh"
 #include "nb_internal.cuh"
+#include "pair.cuh"
 #include "step_body.cuh"
 
 namespace nb {
@@ -128,37 +129,26 @@ __device__ __forceinline__ void tile_item(const FusedArgs &a, int na, int k0, in
     constexpr int NT = FUSED_THREADS, NW = NT / 32, PF = (DS_REC * FUSED_TILE + NT - 1) / NT;
     constexpr int NPAIR = FUSED_TILE / 2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // the lane's due particles (slots k0 + 32 p + lane), negated, in both halves
-    float2 nxh[IPT], nyh[IPT], nzh[IPT], nxl[IPT], nyl[IPT], nzl[IPT], nvx[IPT], nvy[IPT],
-        nvz[IPT];
+    // the lane's due particles (slots k0 + 32 p + lane)
+    IPair ip[IPT];
     int iid[IPT];
 #pragma unroll
     for (int p = 0; p < IPT; ++p) {
         const float4 *ir = a.irec + (size_t)DS_REC * min(k0 + 32 * p + lane, na - 1);
         const float4 I0 = __ldcg(ir), I1 = __ldcg(ir + 1), I2 = __ldcg(ir + 2);
-        nxh[p] = make_float2(-I0.x, -I0.x);
-        nyh[p] = make_float2(-I0.y, -I0.y);
-        nzh[p] = make_float2(-I0.z, -I0.z);
-        nxl[p] = make_float2(-I1.x, -I1.x);
-        nyl[p] = make_float2(-I1.y, -I1.y);
-        nzl[p] = make_float2(-I1.z, -I1.z);
-        nvx[p] = make_float2(-I2.x, -I2.x);
-        nvy[p] = make_float2(-I2.y, -I2.y);
-        nvz[p] = make_float2(-I2.z, -I2.z);
+        ip[p] = ipair_of(I0, I1, I2);
         iid[p] = __float_as_int(I1.w);
     }
     const float2 e2 = make_float2(a.eps2f, a.eps2f);
-    float A_h[IPT][3], A_l[IPT][3], J_h[IPT][3], J_l[IPT][3], P_h[IPT], P_l[IPT];
-    float2 ta[IPT][3], tja[IPT][3], tjb[IPT][3], tp[IPT];
+    const bool soft = soft_pairs(a.eps2f);
+    // running totals (double-single, or plain FP32 in .x) and the FP32 sums between folds
+    float2 tot[IPT][7];
+    PairSum ts[IPT];
 #pragma unroll
     for (int p = 0; p < IPT; ++p) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            A_h[p][c] = A_l[p][c] = J_h[p][c] = J_l[p][c] = 0.f;
-            ta[p][c] = tja[p][c] = tjb[p][c] = make_float2(0.f, 0.f);
-        }
-        P_h[p] = P_l[p] = 0.f;
-        tp[p] = make_float2(0.f, 0.f);
+        for (int c = 0; c < 7; ++c) tot[p][c] = make_float2(0.f, 0.f);
+        pair_zero(ts[p]);
     }
     const float4 *jr = a.s.rec;
     const int ntile = (j1 - j0 + FUSED_TILE - 1) / FUSED_TILE;
@@ -203,89 +193,21 @@ __device__ __forceinline__ void tile_item(const FusedArgs &a, int na, int k0, in
 #pragma unroll
         for (int p = 0; p < IPT; ++p) own = own || (iid[p] >= tb && iid[p] < tb + cnt);
         const bool masked = __any_sync(0xffffffffu, own) || cnt < FUSED_TILE;
-        auto body = [&](int q, bool msk) {
-            const float4 *P = T + 6 * q;
-            const float4 q0 = P[0], q1 = P[1], q4 = P[4], q5 = P[5];
-            float4 q2, q3;
-            if (DS) {
-                q2 = P[2];
-                q3 = P[3];
-            }
-#pragma unroll
-            for (int p = 0; p < IPT; ++p) {
-                float2 dx, dy, dz;
-                if (DS) {
-                    dx = __fadd2_rn(__fadd2_rn(make_float2(q0.x, q0.y), nxh[p]),
-                                    __fadd2_rn(make_float2(q2.x, q2.y), nxl[p]));
-                    dy = __fadd2_rn(__fadd2_rn(make_float2(q0.z, q0.w), nyh[p]),
-                                    __fadd2_rn(make_float2(q2.z, q2.w), nyl[p]));
-                    dz = __fadd2_rn(__fadd2_rn(make_float2(q1.x, q1.y), nzh[p]),
-                                    __fadd2_rn(make_float2(q3.x, q3.y), nzl[p]));
-                } else {
-                    dx = __fadd2_rn(make_float2(q0.x, q0.y), nxh[p]);
-                    dy = __fadd2_rn(make_float2(q0.z, q0.w), nyh[p]);
-                    dz = __fadd2_rn(make_float2(q1.x, q1.y), nzh[p]);
-                }
-                const float2 dvx = __fadd2_rn(make_float2(q4.x, q4.y), nvx[p]);
-                const float2 dvy = __fadd2_rn(make_float2(q4.z, q4.w), nvy[p]);
-                const float2 dvz = __fadd2_rn(make_float2(q5.x, q5.y), nvz[p]);
-                float2 r2 = __ffma2_rn(dx, dx, e2);
-                r2 = __ffma2_rn(dy, dy, r2);
-                r2 = __ffma2_rn(dz, dz, r2);
-                float2 rv = __fmul2_rn(dx, dvx);
-                rv = __ffma2_rn(dy, dvy, rv);
-                rv = __ffma2_rn(dz, dvz, rv);
-                float2 rinv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-                if (msk) {
-                    const int ja = tb + 2 * q;  // the self pair and records past the end: nothing
-                    rinv.x = (ja == iid[p] || 2 * q >= cnt) ? 0.f : rinv.x;
-                    rinv.y = (ja + 1 == iid[p] || 2 * q + 1 >= cnt) ? 0.f : rinv.y;
-                }
-                const float2 rinv2 = __fmul2_rn(rinv, rinv);
-                const float2 mrinv = __fmul2_rn(make_float2(q1.z, q1.w), rinv);
-                const float2 mr3 = __fmul2_rn(mrinv, rinv2);
-                const float2 beta = __fmul2_rn(__fmul2_rn(mr3, rinv2), rv);
-                tp[p] = __fadd2_rn(tp[p], mrinv);
-                ta[p][0] = __ffma2_rn(mr3, dx, ta[p][0]);
-                ta[p][1] = __ffma2_rn(mr3, dy, ta[p][1]);
-                ta[p][2] = __ffma2_rn(mr3, dz, ta[p][2]);
-                tja[p][0] = __ffma2_rn(mr3, dvx, tja[p][0]);
-                tja[p][1] = __ffma2_rn(mr3, dvy, tja[p][1]);
-                tja[p][2] = __ffma2_rn(mr3, dvz, tja[p][2]);
-                tjb[p][0] = __ffma2_rn(beta, dx, tjb[p][0]);
-                tjb[p][1] = __ffma2_rn(beta, dy, tjb[p][1]);
-                tjb[p][2] = __ffma2_rn(beta, dz, tjb[p][2]);
-            }
-        };
-        const int npair = (cnt + 1) / 2;
-        if (masked) {
-            for (int q = warp; q < npair; q += NW) body(q, true);
-        } else {
-#pragma unroll 2
-            for (int q = warp; q < NPAIR; q += NW) body(q, false);
-        }
+        if (soft)
+            tile_pairs<DS, IPT, FUSED_TILE, true>(T, warp, NW, tb, cnt, masked, ip, iid, e2, ts);
+        else
+            tile_pairs<DS, IPT, FUSED_TILE, false>(T, warp, NW, tb, cnt, masked, ip, iid, e2, ts);
         if ((t + 1) % FUSED_TILE_FOLD == 0 || t + 1 == ntile) {
 #pragma unroll
             for (int p = 0; p < IPT; ++p) {
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const float sa = ta[p][c].x + ta[p][c].y;
-                    const float jt = fmaf(-3.f, tjb[p][c].x + tjb[p][c].y, tja[p][c].x + tja[p][c].y);
-                    if (DS) {
-                        ds_add(A_h[p][c], A_l[p][c], sa);
-                        ds_add(J_h[p][c], J_l[p][c], jt);
-                    } else {
-                        A_h[p][c] += sa;
-                        J_h[p][c] += jt;
-                    }
-                    ta[p][c] = tja[p][c] = tjb[p][c] = make_float2(0.f, 0.f);
+                for (int c = 0; c < 7; ++c) {
+                    if (DS)
+                        ds_add(tot[p][c].x, tot[p][c].y, pair_total(ts[p], c));
+                    else
+                        tot[p][c].x += pair_total(ts[p], c);
                 }
-                const float sp = tp[p].x + tp[p].y;
-                if (DS)
-                    ds_add(P_h[p], P_l[p], sp);
-                else
-                    P_h[p] += sp;
-                tp[p] = make_float2(0.f, 0.f);
+                pair_zero(ts[p]);
             }
         }
         if (t + 1 < ntile) stash((t + 1) & 1);
@@ -296,18 +218,14 @@ __device__ __forceinline__ void tile_item(const FusedArgs &a, int na, int k0, in
     float2 *s_red = reinterpret_cast<float2 *>(&s_tile[0][0]);  // [NW][7][32]
 #pragma unroll
     for (int p = 0; p < IPT; ++p) {
-        const float2 mine[7] = {make_float2(A_h[p][0], A_l[p][0]), make_float2(A_h[p][1], A_l[p][1]),
-                                make_float2(A_h[p][2], A_l[p][2]), make_float2(J_h[p][0], J_l[p][0]),
-                                make_float2(J_h[p][1], J_l[p][1]), make_float2(J_h[p][2], J_l[p][2]),
-                                make_float2(P_h[p], P_l[p])};
 #pragma unroll
-        for (int c = 0; c < 7; ++c) s_red[(warp * 7 + c) * 32 + lane] = mine[c];
+        for (int c = 0; c < 7; ++c) s_red[(warp * 7 + c) * 32 + lane] = tot[p][c];
         __syncthreads();
         const int k = k0 + 32 * p + lane;
         if (warp == 0 && k < na) {
 #pragma unroll
             for (int c = 0; c < 7; ++c) {
-                dsf v{mine[c].x, mine[c].y};
+                dsf v{tot[p][c].x, tot[p][c].y};
 #pragma unroll
                 for (int w = 1; w < NW; ++w) {
                     const float2 x = s_red[(w * 7 + c) * 32 + lane];
@@ -466,11 +384,9 @@ __device__ __forceinline__ void small_item(const FusedArgs &a, int na, int n, in
     // fixed xor tree over the warp's 32 lanes (at most 256 terms per sum, fewer
     // than the 128-term sequential sums of the tile kernels' folds in error);
     // double-single from the sum over the warps on
-    float S[G][7];
+    float S[32];
 #pragma unroll
-    for (int p = 0; p < G; ++p)
-#pragma unroll
-        for (int q = 0; q < 7; ++q) S[p][q] = 0.f;
+    for (int q = 0; q < 32; ++q) S[q] = 0.f;
     const int j0 = c * jc, j1 = min(n, j0 + jc);
     const int per_w = (((j1 - j0) + NW - 1) / NW + 31) & ~31;
     const int wj0 = j0 + warp * per_w, wj1 = min(j1, wj0 + per_w);
@@ -527,27 +443,17 @@ __device__ __forceinline__ void small_item(const FusedArgs &a, int na, int n, in
                 tj1 = fmaf(beta, dy, fmaf(mr3, dvy, tj1));
                 tj2 = fmaf(beta, dz, fmaf(mr3, dvz, tj2));
             }
-            S[p][0] += ta0;
-            S[p][1] += ta1;
-            S[p][2] += ta2;
-            S[p][3] += tj0;
-            S[p][4] += tj1;
-            S[p][5] += tj2;
-            S[p][6] += tp;
+            S[7 * p + 0] += ta0;
+            S[7 * p + 1] += ta1;
+            S[7 * p + 2] += ta2;
+            S[7 * p + 3] += tj0;
+            S[7 * p + 4] += tj1;
+            S[7 * p + 5] += tj2;
+            S[7 * p + 6] += tp;
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int p = 0; p < G; ++p)
-#pragma unroll
-            for (int q = 0; q < 7; ++q) S[p][q] += __shfl_xor_sync(0xffffffffu, S[p][q], o);
-    if (lane == 0) {
-#pragma unroll
-        for (int p = 0; p < G; ++p)
-#pragma unroll
-            for (int q = 0; q < 7; ++q) s_red[warp][p * 7 + q] = make_float2(S[p][q], 0.f);
-    }
+    const float wsum = warp_scatter_sum<32>(S);  // lane 7 p + c: component c of slot p
+    if (lane < SMALL_Q) s_red[warp][lane] = make_float2(wsum, 0.f);
     __syncthreads();
     if (tid < SMALL_Q) {
         dsf v{s_red[0][tid].x, s_red[0][tid].y};
@@ -842,31 +748,19 @@ __global__ void __launch_bounds__(FUSED_THREADS)
                         x[u][q] = c < nchunk ? __ldcg(a.part + ((size_t)c * 7 + q) * na + k)
                                              : make_float2(0.f, 0.f);
                     }
-                dsf v[7];
+                dsf v[8];
 #pragma unroll
                 for (int q = 0; q < 7; ++q) {
                     v[q] = dsf{x[0][q].x, x[0][q].y};
 #pragma unroll
                     for (int u = 1; u < CPL; ++u) ds_acc(v[q], dsf{x[u][q].x, x[u][q].y});
                 }
-#pragma unroll
-                for (int q = 0; q < 7; ++q)
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) ds_acc(v[q], ds_shfl_xor(v[q], o));
-                // every lane holds the totals now; lane c takes component c
-                double a1 = 0.0, j1 = 0.0;
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    if (lane == c) {
-                        a1 = ds_to_double(v[c]);
-                        j1 = ds_to_double(v[3 + c]);
-                    }
-                if (lane == 0) {
-                    bool fin = true;
-#pragma unroll
-                    for (int q = 0; q < 7; ++q) fin = fin && isfinite(ds_to_double(v[q]));
-                    if (!fin) atomicOr(a.err, DERR_NONFINITE);
-                }
+                v[7] = dsf{0.f, 0.f};
+                // lane c < 7 holds component c; lane c < 3 takes acc and jerk component c
+                const double tot = ds_to_double(warp_scatter_sum<8>(v));
+                const double a1 = tot, j1 = __shfl_sync(0xffffffffu, tot, (lane + 3) & 31);
+                if (__any_sync(0xffffffffu, lane < 7 && !isfinite(tot)) && lane == 0)
+                    atomicOr(a.err, DERR_NONFINITE);
                 correct_lanes_pre(s, i, k, lane, 0, mine, tn, cs, a1, j1, a.prm, a.sd, a.err,
                                   a.dtmin_hits);
             }
@@ -1018,11 +912,11 @@ __device__ __forceinline__ void small6_item(const FusedArgs &a, int na, int n, i
 #pragma unroll
     for (int p = 0; p < G; ++p) iid[p] = __float_as_int(s_i[p][1].w);
     // FP32 sums per lane (at most F6_CHUNK_MAX_J / 256 = 32 terms each)
-    float t[G][10];
+    float t[G][16];
 #pragma unroll
     for (int p = 0; p < G; ++p)
 #pragma unroll
-        for (int q = 0; q < 10; ++q) t[p][q] = 0.f;
+        for (int q = 0; q < 16; ++q) t[p][q] = 0.f;
     const int j0 = c * jc, j1 = min(n, j0 + jc);
     const int per_w = (((j1 - j0) + NW - 1) / NW + 31) & ~31;
     const int wj0 = j0 + warp * per_w, wj1 = min(j1, wj0 + per_w);
@@ -1099,18 +993,12 @@ __device__ __forceinline__ void small6_item(const FusedArgs &a, int na, int n, i
             }
         }
     }
-    // the lanes' sums in a fixed FP32 xor tree (at most 1024 terms per sum per
-    // warp), one slot at a time; double-single from the sum over the warps on
+    // the lanes' sums in a fixed FP32 tree (at most 1024 terms per sum per warp),
+    // one slot at a time; double-single from the sum over the warps on
 #pragma unroll
     for (int p = 0; p < G; ++p) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int q = 0; q < 10; ++q) t[p][q] += __shfl_xor_sync(0xffffffffu, t[p][q], o);
-        if (lane == 0) {
-#pragma unroll
-            for (int q = 0; q < 10; ++q) s_red[warp][p * 10 + q] = make_float2(t[p][q], 0.f);
-        }
+        const float wsum = warp_scatter_sum<16>(t[p]);  // lane q: output q of slot p
+        if (lane < 10) s_red[warp][p * 10 + lane] = make_float2(wsum, 0.f);
     }
     __syncthreads();
     if (tid < F6_Q) {
