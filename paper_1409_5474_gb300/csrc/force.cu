@@ -127,15 +127,10 @@ __device__ __forceinline__ void finish_split_ds(int nsplit, int slot0, int nslot
                 }
             }
         }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            dsf v = acc[u];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) ds_acc(v, ds_shfl_xor(v, o));
-            const int q = q0 + u;
-            if (lane == 0 && q < total)
-                store_component(out, q / valid, slot0 + q % valid, ds_to_double(v), err);
-        }
+        const dsf v = warp_scatter_sum<U>(acc);
+        const int q = q0 + lane;
+        if (lane < U && q < total)
+            store_component(out, q / valid, slot0 + q % valid, ds_to_double(v), err);
     }
     if (threadIdx.x == 0) *counter = 0u;
 }
@@ -260,6 +255,18 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     const int tile1 = (int)((long long)ntiles * (split + 1) / nsplit);
     const int my_tiles = tile1 - tile0;
 
+    // running totals (double-single, or plain FP32 in .x), this thread's own column
+    float2 *s_tot = reinterpret_cast<float2 *>(s_pair + (AHEAD ? 2 : 1) * PAIRS) + tid;
+#pragma unroll
+    for (int q = 0; q < 7 * IPT; ++q) s_tot[q * NT] = make_float2(0.f, 0.f);
+    if (tid == 0) {
+        s_abort = 0;
+#pragma unroll
+        for (int s = 0; s < NS; ++s) mbar_init(&s_full[s], 1);
+        fence_mbar_init();
+    }
+    cudaGridDependencySynchronize();  // nothing above reads what another launch wrote
+
     // i-particles of this thread
     IPair ip[IPT];
     int iid[IPT];
@@ -278,21 +285,11 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     const bool soft = soft_pairs(eps2f);
     const bool idle = blockIdx.x * IB + wi * IPT * 32 >= is.n;
 
-    // running totals (double-single, or plain FP32 in .x), this thread's own column
-    float2 *s_tot = reinterpret_cast<float2 *>(s_pair + (AHEAD ? 2 : 1) * PAIRS) + tid;
-#pragma unroll
-    for (int q = 0; q < 7 * IPT; ++q) s_tot[q * NT] = make_float2(0.f, 0.f);
     // FP32 partial sums between folds, two lanes each (even and odd j of a pair)
     PairSum ts[IPT];
 #pragma unroll
     for (int p = 0; p < IPT; ++p) pair_zero(ts[p]);
 
-    if (tid == 0) {
-        s_abort = 0;
-#pragma unroll
-        for (int s = 0; s < NS; ++s) mbar_init(&s_full[s], 1);
-        fence_mbar_init();
-    }
     __syncthreads();
 
     auto issue = [&](int kt) {
@@ -419,33 +416,53 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     (void)counters;
 }
 
-// K3 of the tile kernel: one thread per output (component c of slot k) adds the
-// nsplit double-single partials in the order s = 0, 1, ... (the partials of
-// consecutive slots are adjacent, so the loads of a warp are coalesced), eight
-// loads in flight at a time.
+// K3 of the tile kernel: the nsplit double-single partials of every output (component c
+// of slot k) in a fixed order. A CTA is 256 / G consecutive outputs (their partials are
+// adjacent, so the loads of a warp are coalesced) times G groups of splits: group g adds the
+// splits g, g + G, ..., eight loads in flight at a time, and the groups are added in order
+// through shared memory. G = 1 where the outputs alone fill the GPU; with G = 8 a small due
+// set's many splits cost one or two round trips to L2 and not nsplit / 8 of them (64 slots,
+// 152 splits at N = 65536: force and reduction 27.0 -> 18.8 us, 14.3 as a dependent launch).
+template <int G>
 __global__ void __launch_bounds__(256)
     k_tile_split_reduce(const float2 *__restrict__ part, long long pld, int nsplit, int n_i,
                         Out3 out, unsigned *err)
 {
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= 7LL * n_i) return;
+    constexpr int NQ = 256 / G;
+    __shared__ float2 s_sum[G > 1 ? G - 1 : 1][NQ];
+    const int o = threadIdx.x % NQ, g = threadIdx.x / NQ;
+    const long long q = (long long)blockIdx.x * NQ + o;
+    const bool valid = q < 7LL * n_i;
     const int c = (int)(q / n_i), k = (int)(q % n_i);
-    const float2 *p = part + (size_t)c * pld + k;
-    const size_t stride = (size_t)7 * pld;
     dsf sum{0.f, 0.f};
-    int sp = 0;
-    for (; sp + 8 <= nsplit; sp += 8) {
+    cudaGridDependencySynchronize();
+    if (valid) {
+        const float2 *p = part + (size_t)c * pld + k;
+        const size_t stride = (size_t)7 * pld;
+        int sp = g;
+        for (; sp + 7 * G < nsplit; sp += 8 * G) {
+            float2 x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = __ldcg(p + (size_t)(sp + u * G) * stride);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) ds_acc(sum, dsf{x[u].x, x[u].y});
+        }
         float2 x[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) x[u] = __ldcg(p + (size_t)(sp + u) * stride);
+        for (int u = 0; u < 8; ++u)
+            x[u] = sp + u * G < nsplit ? __ldcg(p + (size_t)(sp + u * G) * stride)
+                                       : make_float2(0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < 8; ++u) ds_acc(sum, dsf{x[u].x, x[u].y});
     }
-    for (; sp < nsplit; ++sp) {
-        const float2 x = __ldcg(p + (size_t)sp * stride);
-        ds_acc(sum, dsf{x.x, x.y});
+    if (G > 1) {
+        if (g > 0) s_sum[g - 1][o] = make_float2(sum.hi, sum.lo);
+        __syncthreads();
+        if (g > 0) return;
+#pragma unroll
+        for (int u = 1; u < G; ++u) ds_acc(sum, dsf{s_sum[u - 1][o].x, s_sum[u - 1][o].y});
     }
-    store_component(out, c, k, ds_to_double(sum), err);
+    if (valid) store_component(out, c, k, ds_to_double(sum), err);
 }
 
 
@@ -793,6 +810,7 @@ __global__ void __launch_bounds__(256)
     __shared__ float2 s_red[NW][IPT * 7];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nsplit = gridDim.x, split = blockIdx.x;
+    cudaGridDependencySynchronize();
 
     // this thread's j-records: j = split * NT * JPT + r * NT + tid
     float4 ja[JPT], jb[JPT], jc[JPT];
@@ -828,7 +846,10 @@ __global__ void __launch_bounds__(256)
             vx[p] = c.x; vy[p] = c.y; vz[p] = c.z;
             iid[p] = i_id(is, r, b.w);
         }
-        dsf v[IPT][7];
+        constexpr int P = IPT == 1 ? 8 : (IPT == 2 ? 16 : 32);
+        dsf v[P];
+#pragma unroll
+        for (int q = 0; q < P; ++q) v[q] = dsf{0.f, 0.f};
 #pragma unroll
         for (int p = 0; p < IPT; ++p) {
             float ta0 = 0.f, ta1 = 0.f, ta2 = 0.f, tj0 = 0.f, tj1 = 0.f, tj2 = 0.f;
@@ -870,29 +891,17 @@ __global__ void __launch_bounds__(256)
                 tb1 = fmaf(beta, dy, tb1);
                 tb2 = fmaf(beta, dz, tb2);
             }
-            v[p][0] = dsf{ta0, 0.f};
-            v[p][1] = dsf{ta1, 0.f};
-            v[p][2] = dsf{ta2, 0.f};
-            v[p][3] = dsf{fmaf(-3.f, tb0, tj0), 0.f};
-            v[p][4] = dsf{fmaf(-3.f, tb1, tj1), 0.f};
-            v[p][5] = dsf{fmaf(-3.f, tb2, tj2), 0.f};
-            v[p][6] = dsf{tp, 0.f};
+            v[7 * p + 0] = dsf{ta0, 0.f};
+            v[7 * p + 1] = dsf{ta1, 0.f};
+            v[7 * p + 2] = dsf{ta2, 0.f};
+            v[7 * p + 3] = dsf{fmaf(-3.f, tb0, tj0), 0.f};
+            v[7 * p + 4] = dsf{fmaf(-3.f, tb1, tj1), 0.f};
+            v[7 * p + 5] = dsf{fmaf(-3.f, tb2, tj2), 0.f};
+            v[7 * p + 6] = dsf{tp, 0.f};
         }
-        // double-single xor tree across the lanes, all chains interleaved
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int p = 0; p < IPT; ++p)
-#pragma unroll
-                for (int c = 0; c < 7; ++c) ds_acc(v[p][c], ds_shfl_xor(v[p][c], o));
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int p = 0; p < IPT; ++p)
-#pragma unroll
-                for (int c = 0; c < 7; ++c)
-                    s_red[warp][p * 7 + c] = make_float2(v[p][c].hi, v[p][c].lo);
-        }
+        // double-single sums over the lanes: lane 7 p + c holds component c of slot p
+        const dsf wsum = warp_scatter_sum<P>(v);
+        if (lane < IPT * 7) s_red[warp][lane] = make_float2(wsum.hi, wsum.lo);
         __syncthreads();
         if (tid < IPT * 7) {
             const int p = tid / 7, c = tid % 7;
@@ -910,9 +919,8 @@ __global__ void __launch_bounds__(256)
         }
         __syncthreads();
     }
-    if (nsplit > 1)
-        finish_split_ds<NT>(nsplit, 0, is.n, is.n, reinterpret_cast<float2 *>(part), pld, counters,
-                            out, err);
+    // with nsplit > 1 the partials are summed by k_tile_split_reduce, launched next
+    (void)counters;
 }
 
 // FP64 j-parallel kernel: thread = j, all threads share IPT i's.
@@ -1121,16 +1129,17 @@ __device__ __forceinline__ void item_jpar(const WorkItem &w, float2 (*s_red)[28]
                     tjv[p][2] = fmaf(beta, dz, fmaf(mr3, dvz, tjv[p][2]));
                 }
             }
-            // lanes -> warp (fixed xor tree), warps -> CTA (fixed order) -> totals
+            // lanes -> warp (fixed tree), warps -> CTA (fixed order) -> totals
+            dsf v[32];
+#pragma unroll
+            for (int q = 0; q < 32; ++q) v[q] = dsf{0.f, 0.f};
 #pragma unroll
             for (int p = 0; p < G; ++p)
 #pragma unroll
-                for (int c = 0; c < 7; ++c) {
-                    dsf v{c < 3 ? ta[p][c] : (c < 6 ? tjv[p][c - 3] : tp[p]), 0.f};
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) ds_acc(v, ds_shfl_xor(v, o));
-                    if (lane == 0) s_red[warp][p * 7 + c] = make_float2(v.hi, v.lo);
-                }
+                for (int c = 0; c < 7; ++c)
+                    v[7 * p + c].hi = c < 3 ? ta[p][c] : (c < 6 ? tjv[p][c - 3] : tp[p]);
+            const dsf wsum = warp_scatter_sum<32>(v);
+            if (lane < G * 7) s_red[warp][lane] = make_float2(wsum.hi, wsum.lo);
             __syncthreads();
             if (tid < G * 7) {
                 dsf sum{s_tot[tid].x, s_tot[tid].y};
@@ -1366,6 +1375,10 @@ static void tiny_shape(int n_i, int n_j, ForcePlan &p)
     p.nsplit = (n_j + 256 * p.jt - 1) / (256 * p.jt);
 }
 
+// i-particles per thread of the tile kernel: two, but one for the sets that then fill one
+// warp column of eight warp rows (16 of 262144: 24.2 against 32.8 us).
+static int tile_ipt(int n_i, int nwj) { return nwj == 8 && n_i <= 32 ? 1 : 2; }
+
 ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms)
 {
     ForcePlan p{};
@@ -1388,48 +1401,52 @@ ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms)
                                 ntiles / 2 > 1 ? ntiles / 2 : 1);
         return p;
     }
-    if (n_i <= 4) {
+    // Tiny sets: the j-set in registers, a pass over them for every four i-particles. The
+    // tile kernel costs the same from one i-particle to 32: 4 of 65536 7.1 us against 9.4, 4 of
+    // 262144 11.0 against 18.9; a second pass pays on a large j-set only: 8 of 32768 9.4
+    // against 7.6, 8 of 65536 9.9 against 9.7, 8 of 262144 14.8 against 18.6.
+    if (n_i <= (n_j > 65536 ? 8 : 4)) {
         tiny_shape(n_i, n_j, p);
         return p;
     }
-    if (n_i < 4096) {
-        // warp groups: about 14 warps per SM in total, at least 1024 j per split
-        // (the best plans a sweep over N_i at N = 65536 found on GB300)
-        p.kind = 1;
-        wgrp_shape(n_i, p);
-        const long long groups = (n_i + p.ipt - 1) / p.ipt;
-        const long long cap = n_j / 1024 > 1 ? n_j / 1024 : 1;
-        p.nsplit = (int)clampll((14LL * num_sms + groups - 1) / groups, 1, cap);
-        return p;
-    }
-    // tiles: 256 threads, 2 i per thread; 8 or 4 warp rows share each j-tile
-    // below 65536 i; about 40 CTAs per SM, at least 16 tiles per split; then, up
-    // to twice that many splits, the fewest whose last wave of resident CTAs is at
-    // least 97% full, else the fullest (N = 2^20: 2048 i-blocks x 3 splits fill
-    // 21% of their 21st wave on 304 slots, x 4 splits 95% of their 27th)
+    // Tiles: the warp rows (8, 4 or 1: 64, 128 or 512 i-particles per CTA) and j-splits of
+    // least estimated time. An SM's CTAs share its pipes, so its time is its count of CTAs
+    // (at most ceil(CTAs / SMs)) times the tiles of a split times the SM's time for one
+    // tile of that shape, a little more where a CTA is left alone at the end (its eight
+    // warps do not fill the pipe); the splits' partials cost their traffic. Only split
+    // counts that fill a whole number of CTAs per SM are tried. Within 3% of the best of a
+    // sweep over shapes and splits at N = 2500 to 262144, almost everywhere. Against the rule
+    // before it (warp groups below 4096 i-particles, 16 tiles or more per split above),
+    // at N = 65536: N_i = 260 49.8 -> 39.4 us, 1531 184 -> 127 us, 3000 415 -> 234 us.
     p.kind = 0;
-    p.ipt = 2;
     p.threads = 256;
     p.jt = JT_TILE;
-    p.nwj = n_i >= 65536 ? 1 : (n_i >= 8192 ? 4 : 8);
-    const long long ib = (long long)(p.threads / p.nwj) * p.ipt;
-    const long long nblk = (n_i + ib - 1) / ib;
     const long long ntiles = (n_j + p.jt - 1) / p.jt;
-    const long long cap = ntiles / 16 > 1 ? ntiles / 16 : 1;
-    const long long ns0 = clampll((40LL * num_sms + nblk - 1) / nblk, 1, cap);
-    const long long slots = (long long)num_sms * tile_blocks_per_sm(variant, p.nwj);
-    long long best = ns0;
-    double best_eff = 0.0;
-    for (long long ns = ns0; ns <= std::min(cap, 2 * ns0); ++ns) {
-        const double waves = (double)(nblk * ns) / (double)slots;
-        const double eff = waves / std::ceil(waves);
-        if (eff > best_eff + 1e-9) {
-            best_eff = eff;
-            best = ns;
+    double best = 1e300;
+    for (const int nwj : {8, 4, 1}) {
+        const long long ib = 512 / nwj;
+        const long long nblk = (n_i + ib - 1) / ib;
+        // microseconds of an SM per 256-record tile (measured with whole waves at N = 65536)
+        const double t_tile = nwj == 8 ? 2.57 : (nwj == 4 ? 4.97 : 18.8);
+        long long last = 0;
+        for (const int per_sm : {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 14, 16, 20, 24, 32, 40, 48}) {
+            const long long ns =
+                clampll((long long)per_sm * num_sms / nblk, 1, ntiles < 512 ? ntiles : 512);
+            if (ns == last) continue;
+            last = ns;
+            const long long on_sm = (nblk * ns + num_sms - 1) / num_sms;
+            const long long tiles = (ntiles + ns - 1) / ns;
+            const double alone = on_sm % 2 ? 0.10 : 0.04;
+            const double t = ((double)on_sm + alone) * (double)tiles * t_tile + 0.5 * (double)on_sm +
+                             (ns > 1 ? 2.0 + 0.01 * (double)ns + 2e-5 * (double)(ns * n_i) : 0.0);
+            if (t < best) {
+                best = t;
+                p.nwj = nwj;
+                p.nsplit = (int)ns;
+            }
         }
-        if (eff >= 0.97) break;
     }
-    p.nsplit = (int)best;
+    p.ipt = tile_ipt(n_i, p.nwj);
     return p;
 }
 
@@ -1458,10 +1475,10 @@ ForcePlan plan_from_entry(const nb_plan &e, int variant, int n_i, int n_j)
         p.threads = 128;
         p.jt = JT64;
     } else {
-        p.ipt = 2;
         p.threads = 256;
         p.jt = JT_TILE;
         p.nwj = (e.nwj == 4 || e.nwj == 8) ? e.nwj : 1;
+        p.ipt = tile_ipt(n_i, p.nwj);
     }
     const int ntiles = (n_j + p.jt - 1) / p.jt;
     p.nsplit = (int)clampll(e.nsplit, 1, ntiles);
@@ -1472,6 +1489,22 @@ size_t plan_partial_doubles(const ForcePlan &p, int n_i)
 {
     if (p.nsplit <= 1) return 0;
     return (size_t)p.nsplit * 7 * (size_t)n_i;
+}
+
+// Outputs up to which the split reduction takes eight threads per output: above, one
+// thread per output gives every SM more than two CTAs.
+constexpr long long SPLIT_WIDE_OUTS = 1 << 17;
+
+static cudaError_t go_split_reduce(const double *part, int n_i, int nsplit, const Out3 &out,
+                                   unsigned *err, cudaStream_t st)
+{
+    const long long outs = 7LL * n_i;
+    const float2 *p = reinterpret_cast<const float2 *>(part);
+    if (nsplit > 8 && outs <= SPLIT_WIDE_OUTS)
+        return launch_dependent(k_tile_split_reduce<8>, dim3((unsigned)((outs + 31) / 32)), 256, 0,
+                                st, p, (long long)n_i, nsplit, n_i, out, err);
+    return launch_dependent(k_tile_split_reduce<1>, dim3((unsigned)((outs + 255) / 256)), 256, 0,
+                            st, p, (long long)n_i, nsplit, n_i, out, err);
 }
 
 // Let kernel K take smem bytes of dynamic shared memory on the current device (the
@@ -1512,13 +1545,10 @@ static cudaError_t go_tile32(const JSet &js, const ISet &is, float eps2f, int ns
     if (attr != cudaSuccess) return attr;
     const int ntiles = (js.n + JT_TILE - 1) / JT_TILE;
     dim3 grid((is.n + IB - 1) / IB, nsplit);
-    kern<<<grid, NT, smem, st>>>(js.rec32, js.n, is, eps2f, ntiles, part, is.n, cnt, out, err);
-    if (nsplit > 1) {
-        const long long outs = 7LL * is.n;
-        k_tile_split_reduce<<<(unsigned)((outs + 255) / 256), 256, 0, st>>>(
-            reinterpret_cast<const float2 *>(part), is.n, nsplit, is.n, out, err);
-    }
-    return cudaGetLastError();
+    const cudaError_t e = launch_dependent(kern, grid, NT, smem, st, js.rec32, js.n, is, eps2f,
+                                           ntiles, part, (long long)is.n, cnt, out, err);
+    if (e != cudaSuccess || nsplit <= 1) return e;
+    return go_split_reduce(part, is.n, nsplit, out, err, st);
 }
 
 template <int VAR, int IPT, int NWARP>
@@ -1538,9 +1568,11 @@ static cudaError_t go_tiny32(const JSet &js, const ISet &is, float eps2f, double
                              unsigned *cnt, Out3 out, unsigned *err, cudaStream_t st)
 {
     const int g = (js.n + 256 * JPT - 1) / (256 * JPT);
-    k_force_tiny32<VAR, IPT, JPT><<<g, 256, 0, st>>>(js.rec32, js.n, is, eps2f, part, is.n, cnt,
-                                                      out, err);
-    return cudaGetLastError();
+    const cudaError_t e =
+        launch_dependent(k_force_tiny32<VAR, IPT, JPT>, dim3(g), 256, 0, st, js.rec32, js.n, is,
+                         eps2f, part, (long long)is.n, cnt, out, err);
+    if (e != cudaSuccess || g <= 1) return e;
+    return go_split_reduce(part, is.n, g, out, err, st);
 }
 
 template <int VAR, int IPT>
@@ -1592,7 +1624,10 @@ static cudaError_t dispatch32(const ForcePlan &p, const JSet &js, const ISet &is
     switch (p.nwj) {
     case 1: return go_tile32<VAR, 2, 8, 1>(js, is, eps2f, p.nsplit, part, cnt, out, err, st);
     case 4: return go_tile32<VAR, 2, 2, 4>(js, is, eps2f, p.nsplit, part, cnt, out, err, st);
-    default: return go_tile32<VAR, 2, 1, 8>(js, is, eps2f, p.nsplit, part, cnt, out, err, st);
+    default:
+        if (p.ipt == 1)
+            return go_tile32<VAR, 1, 1, 8>(js, is, eps2f, p.nsplit, part, cnt, out, err, st);
+        return go_tile32<VAR, 2, 1, 8>(js, is, eps2f, p.nsplit, part, cnt, out, err, st);
     }
 }
 

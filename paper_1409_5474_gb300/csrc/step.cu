@@ -26,6 +26,7 @@ __global__ void k_predict(StateDev s, double t, unsigned *err, const double *t_d
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= s.n) return;
+    cudaGridDependencySynchronize();
     if (t_dev) t = *t_dev + t;
     const double d = t - s.t[i];
     const double d6 = d * (1.0 / 6.0), d2h = 0.5 * d;
@@ -56,25 +57,26 @@ cudaError_t launch_predict(const StateDev &s, double t, bool want_rec, unsigned 
     if (s.n <= 0) return cudaSuccess;
     const int bs = 256;
     const int g = (s.n + bs - 1) / bs;
-    if (want_rec)
-        k_predict<true><<<g, bs, 0, st>>>(s, t, err, t_dev);
-    else
-        k_predict<false><<<g, bs, 0, st>>>(s, t, err, t_dev);
-    return cudaGetLastError();
+    return launch_dependent(want_rec ? k_predict<true> : k_predict<false>, dim3(g), bs, 0, st, s, t,
+                            err, t_dev);
 }
 
-__global__ void k_advance(double *t_dev, double dt) { *t_dev = *t_dev + dt; }
+__global__ void k_advance(double *t_dev, double dt)
+{
+    cudaGridDependencySynchronize();
+    *t_dev = *t_dev + dt;
+}
 
 cudaError_t launch_advance(double *t_dev, double dt, cudaStream_t st)
 {
-    k_advance<<<1, 1, 0, st>>>(t_dev, dt);
-    return cudaGetLastError();
+    return launch_dependent(k_advance, dim3(1), 1, 0, st, t_dev, dt);
 }
 
 __global__ void k_correct(StateDev s, const int *__restrict__ act, int na, double t_new, Out3 f,
                           StepParams prm, SchedDev *sd, unsigned *err,
                           unsigned long long *dtmin_hits, const double *t_dev, bool xp_from_state)
 {
+    cudaGridDependencySynchronize();
     correct_body(s, act, na, t_new, f, prm, sd, err, dtmin_hits, t_dev,
                  blockIdx.x * blockDim.x + threadIdx.x, xp_from_state);
 }
@@ -152,9 +154,8 @@ cudaError_t launch_correct(const StateDev &s, const int *act, int n_a, double t_
 {
     if (n_a <= 0) return cudaSuccess;
     const int bs = CORRECT_THREADS;  // FP64-heavy: spread small active sets over many SMs
-    k_correct<<<(n_a + bs - 1) / bs, bs, 0, st>>>(s, act, n_a, t_new, f, p, sd, err, dtmin_hits,
-                                                   t_dev, xp_from_state);
-    return cudaGetLastError();
+    return launch_dependent(k_correct, dim3((n_a + bs - 1) / bs), bs, 0, st, s, act, n_a, t_new, f, p,
+                            sd, err, dtmin_hits, t_dev, xp_from_state);
 }
 
 cudaError_t launch_correct_trial(const StateDev &s, const int *act, int n_a, double t_new,
