@@ -46,7 +46,12 @@ __device__ __forceinline__ dsf ds_shfl_xor(dsf a, int o)
 
 __device__ __forceinline__ void sum_into(dsf &a, dsf b) { ds_acc(a, b); }
 __device__ __forceinline__ void sum_into(float &a, float b) { a += b; }
+__device__ __forceinline__ void sum_into(double &a, double b) { a += b; }
 __device__ __forceinline__ dsf lane_xor(dsf a, int o) { return ds_shfl_xor(a, o); }
+__device__ __forceinline__ double lane_xor(double a, int o)
+{
+    return __shfl_xor_sync(0xffffffffu, a, o);
+}
 __device__ __forceinline__ float lane_xor(float a, int o)
 {
     return __shfl_xor_sync(0xffffffffu, a, o);

@@ -339,6 +339,10 @@ int ensure_part(nb_handle h, const ForcePlan &p, int n_i)
     return NB_OK;
 }
 
+// The split counters of a force launch: the warp-group kernel's (FP64 plans and the tile and
+// tiny-set kernels sum their splits in a launch of their own).
+unsigned *counters_of(nb_handle h, int variant) { return variant == NB_F64 ? nullptr : h->split_cnt; }
+
 int bucket_of(int n_i)
 {
     int b = 0;
@@ -413,10 +417,10 @@ int run_force_plan(nb_handle h, int variant, const ForcePlan &p, const ISet &is,
         evp = ev;
     }
     const double eps2 = h->cfg.eps * h->cfg.eps;
-    CK(h, launch_force(variant, p, jset_of(h), is, eps2, h->part, h->split_cnt, out, h->d_err,
-                       h->stream, evp));
-    // the FP32 tile and tiny-set kernels' j-split partials are summed by a launch of their own
-    h->stats.kernel_launches += (p.kind != 1 && p.nsplit > 1 && variant != NB_F64) ? 2 : 1;
+    CK(h, launch_force(variant, p, jset_of(h), is, eps2, h->part, counters_of(h, variant), out,
+                       h->d_err, h->stream, evp));
+    // all but the warp groups' j-split partials are summed by a launch of their own
+    h->stats.kernel_launches += ((p.kind != 1 || variant == NB_F64) && p.nsplit > 1) ? 2 : 1;
     int lg = 0;
     while ((2LL << lg) <= is.n && lg < 31) ++lg;
     if (evp) {
@@ -998,8 +1002,8 @@ int handle_force(nb_handle h, int n_i, bool due, double eps2, unsigned *err, cud
     int rc = ensure_part(h, p, n_i);
     if (rc) return rc;
     const Out3 out{h->f_acc, h->f_jerk, h->f_pot, h->ld};
-    if (launch_force(variant, p, jset_of(h), is, eps2, h->part, h->split_cnt, out, err, st,
-                     nullptr) != cudaSuccess)
+    if (launch_force(variant, p, jset_of(h), is, eps2, h->part, counters_of(h, variant), out, err,
+                     st, nullptr) != cudaSuccess)
         return NB_ERR_CUDA;
     return NB_OK;
 }

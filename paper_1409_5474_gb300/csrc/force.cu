@@ -165,14 +165,9 @@ __device__ __forceinline__ void finish_split(int nsplit, int slot0, int nslots, 
                 }
             }
         }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            double v = acc[u];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            const int q = q0 + u;
-            if (lane == 0 && q < total) store_component(out, q / valid, slot0 + q % valid, v, err);
-        }
+        const double v = warp_scatter_sum<U>(acc);
+        const int q = q0 + lane;
+        if (lane < U && q < total) store_component(out, q / valid, slot0 + q % valid, v, err);
     }
     if (threadIdx.x == 0) *counter = 0u;
 }
@@ -412,104 +407,98 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
             }
         }
     }
-    // with nsplit > 1 the partials are summed by k_tile_split_reduce, launched next
+    // with nsplit > 1 the partials are summed by k_split_sums, launched next
     (void)counters;
 }
 
-// K3 of the tile kernel: the nsplit double-single partials of every output (component c
-// of slot k) in a fixed order. A CTA is 256 / G consecutive outputs (their partials are
-// adjacent, so the loads of a warp are coalesced) times G groups of splits: group g adds the
-// splits g, g + G, ..., eight loads in flight at a time, and the groups are added in order
-// through shared memory. G = 1 where the outputs alone fill the GPU; with G = 8 a small due
-// set's many splits cost one or two round trips to L2 and not nsplit / 8 of them (64 slots,
-// 152 splits at N = 65536: force and reduction 27.0 -> 18.8 us, 14.3 as a dependent launch).
-template <int G>
+// K3 of the tile, tiny-set and FP64 kernels: the nsplit partials (T: double-single float2, or
+// double) of every output (component c of slot k) in a fixed order. A CTA is 256 / G
+// consecutive outputs (their partials are adjacent, so the loads of a warp are coalesced)
+// times G groups of splits: group g adds the splits g, g + G, ..., eight at a time, all eight
+// loads in flight and added in pairs (FP64: 114 splits one after the other doubled the
+// rounding error of small i-sets), and the groups are added in order through shared memory.
+// G = 1 where the outputs alone fill the GPU; with G = 8 a small due set's many splits cost
+// one or two round trips to L2 and not nsplit / 8 of them (64 slots, 152 splits at N = 65536:
+// force and reduction 27.0 -> 18.8 us, 14.3 as a dependent launch).
+__device__ __forceinline__ dsf split_value(float2 x) { return dsf{x.x, x.y}; }
+__device__ __forceinline__ double split_value(double x) { return x; }
+__device__ __forceinline__ double split_total(dsf x) { return ds_to_double(x); }
+__device__ __forceinline__ double split_total(double x) { return x; }
+
+template <class T, int G>
 __global__ void __launch_bounds__(256)
-    k_tile_split_reduce(const float2 *__restrict__ part, long long pld, int nsplit, int n_i,
-                        Out3 out, unsigned *err)
+    k_split_sums(const T *__restrict__ part, long long pld, int nsplit, int n_i, Out3 out,
+                 unsigned *err)
 {
+    using V = decltype(split_value(T{}));
     constexpr int NQ = 256 / G;
-    __shared__ float2 s_sum[G > 1 ? G - 1 : 1][NQ];
+    __shared__ V s_sum[G > 1 ? G - 1 : 1][NQ];
     const int o = threadIdx.x % NQ, g = threadIdx.x / NQ;
     const long long q = (long long)blockIdx.x * NQ + o;
     const bool valid = q < 7LL * n_i;
     const int c = (int)(q / n_i), k = (int)(q % n_i);
-    dsf sum{0.f, 0.f};
+    V sum{};
     cudaGridDependencySynchronize();
     if (valid) {
-        const float2 *p = part + (size_t)c * pld + k;
+        const T *p = part + (size_t)c * pld + k;
         const size_t stride = (size_t)7 * pld;
-        int sp = g;
-        for (; sp + 7 * G < nsplit; sp += 8 * G) {
-            float2 x[8];
+        for (int sp = g; sp < nsplit; sp += 8 * G) {
+            V x[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) x[u] = __ldcg(p + (size_t)(sp + u * G) * stride);
+            for (int u = 0; u < 8; ++u)
+                x[u] = split_value(sp + u * G < nsplit ? __ldcg(p + (size_t)(sp + u * G) * stride)
+                                                       : T{});
 #pragma unroll
-            for (int u = 0; u < 8; ++u) ds_acc(sum, dsf{x[u].x, x[u].y});
+            for (int h = 1; h < 8; h <<= 1)
+#pragma unroll
+                for (int u = 0; u < 8; u += 2 * h) sum_into(x[u], x[u + h]);
+            sum_into(sum, x[0]);
         }
-        float2 x[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            x[u] = sp + u * G < nsplit ? __ldcg(p + (size_t)(sp + u * G) * stride)
-                                       : make_float2(0.f, 0.f);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) ds_acc(sum, dsf{x[u].x, x[u].y});
     }
     if (G > 1) {
-        if (g > 0) s_sum[g - 1][o] = make_float2(sum.hi, sum.lo);
+        if (g > 0) s_sum[g - 1][o] = sum;
         __syncthreads();
         if (g > 0) return;
 #pragma unroll
-        for (int u = 1; u < G; ++u) ds_acc(sum, dsf{s_sum[u - 1][o].x, s_sum[u - 1][o].y});
+        for (int u = 1; u < G; ++u) sum_into(sum, s_sum[u - 1][o]);
     }
-    if (valid) store_component(out, c, k, ds_to_double(sum), err);
+    if (valid) store_component(out, c, k, split_total(sum), err);
 }
-
 
 // ---------------------------------------------------------------------------
 // FP64 tile kernel.
+//
+// Bound by the FP64 pipe: a warp-wide FP64 instruction holds an SMSP's pipe for 64
+// cycles, and a pair takes about 32 of them, so one j costs a warp of 32 i-particles 1 us
+// and a GB300 does 19.7 G/s at most (17.3 measured at N = 20011; a reciprocal square root of
+// five FP64 instructions from the SFU's approximation gave the same time and bits as
+// rsqrt). What is left is to keep all
+// 608 pipes busy to the end: a CTA is 32 i-particles times four warp rows (one warp per
+// SMSP; row g takes j = g, g + 4, ... of every tile, the rows are added in order through
+// shared memory), so an SM's four pipes always carry the same load and the plan divides
+// the j-range in units of 16. The splits are summed by k_split_sums. N = 1024, all
+// i: 316 -> 75.7 us; 100 of 20011 688 -> 158 us; N = 6007, all i: 2380 -> 2123 us.
 // ---------------------------------------------------------------------------
 
-template <int IPT, int NT, int JT, int NS>
-__global__ void __launch_bounds__(NT)
-    k_force_tile64(JSet js, ISet is, double eps2, int ntiles, double *__restrict__ part,
-                   long long pld, unsigned *counters, Out3 out, unsigned *err)
+constexpr int T64_ROWS = 4;   // warp rows of a CTA
+constexpr int T64_UNIT = 16;  // j-ranges are whole units (16-byte aligned rows)
+
+template <int JT, int NS>
+__global__ void __launch_bounds__(32 * T64_ROWS)
+    k_force_tile64(JSet js, ISet is, double eps2, int nunits, double *__restrict__ part,
+                   long long pld, Out3 out, unsigned *err)
 {
     extern __shared__ __align__(128) double s_t64[];  // NS * 7 * JT
     __shared__ __align__(8) uint64_t s_full[NS];
     __shared__ int s_abort;
+    __shared__ double s_row[T64_ROWS - 1][7][32];
 
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, row = tid >> 5;
     const int nsplit = gridDim.y;
     const int split = blockIdx.y;
-    const int tile0 = (int)((long long)ntiles * split / nsplit);
-    const int tile1 = (int)((long long)ntiles * (split + 1) / nsplit);
-    const int my_tiles = tile1 - tile0;
-    const int nj = js.n;
-
-    double xi[IPT][3], vi[IPT][3], mi[IPT];
-    int iid[IPT];
-#pragma unroll
-    for (int p = 0; p < IPT; ++p) {
-        int k = blockIdx.x * (NT * IPT) + p * NT + tid;
-        if (k >= is.n) k = is.n - 1;
-        const int r = is.member ? member_index(is, k, err) : k;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            xi[p][c] = __ldg(is.pos64 + c * is.ld64 + r);
-            vi[p][c] = __ldg(is.vel64 + c * is.ld64 + r);
-        }
-        mi[p] = is.member ? __ldg(is.m64 + r) : 0.0;
-        iid[p] = is.member ? r : -1;
-    }
-
-    double A[IPT][3], J[IPT][3], P[IPT];
-#pragma unroll
-    for (int p = 0; p < IPT; ++p) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) A[p][c] = J[p][c] = 0.0;
-        P[p] = 0.0;
-    }
+    const int j0 = (int)((long long)nunits * split / nsplit) * T64_UNIT;
+    const int j1 = min(js.n, (int)((long long)nunits * (split + 1) / nsplit) * T64_UNIT);
+    const int my_tiles = (j1 - j0 + JT - 1) / JT;
 
     if (tid == 0) {
         s_abort = 0;
@@ -517,17 +506,31 @@ __global__ void __launch_bounds__(NT)
         for (int s = 0; s < NS; ++s) mbar_init(&s_full[s], 1);
         fence_mbar_init();
     }
+    cudaGridDependencySynchronize();  // nothing above reads what another launch wrote
+
+    const int k = blockIdx.x * 32 + lane;
+    const int kc = min(k, is.n - 1);  // idle lanes compute a copy, never written
+    const int r = is.member ? member_index(is, kc, err) : kc;
+    const int iid = is.member ? r : -1;
+    double xi[3], vi[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        xi[c] = __ldg(is.pos64 + c * is.ld64 + r);
+        vi[c] = __ldg(is.vel64 + c * is.ld64 + r);
+    }
+    double v[7];  // acc, jerk, positive potential
+#pragma unroll
+    for (int c = 0; c < 7; ++c) v[c] = 0.0;
     __syncthreads();
 
     // 7 rows per stage: x, y, z, vx, vy, vz, m
     auto issue = [&](int kt) {
         const int stage = kt % NS;
-        const int t = tile0 + kt;
-        const int cnt = min(JT, nj - t * JT);
+        const int cnt = min(JT, j1 - j0 - kt * JT);
         const uint32_t bytes = (uint32_t)(((cnt * 8) + 15) & ~15);  // rows are padded
         mbar_expect_tx(&s_full[stage], 7u * bytes);
         double *dst = s_t64 + (size_t)stage * 7 * JT;
-        const size_t off = (size_t)t * JT;
+        const size_t off = (size_t)j0 + (size_t)kt * JT;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             bulk_g2s(dst + c * JT, js.pos64 + c * js.ld + off, bytes, &s_full[stage]);
@@ -544,101 +547,75 @@ __global__ void __launch_bounds__(NT)
         const uint32_t parity = (uint32_t)((kt / NS) & 1);
         if (!mbar_wait(&s_full[stage], parity)) s_abort = 1;
         const double *T = s_t64 + (size_t)stage * 7 * JT;
-        const int jbase = (tile0 + kt) * JT;
-        const int cnt = min(JT, nj - jbase);
-        double ta[IPT][3], tja[IPT][3], tjb[IPT][3], tp[IPT];
+        const int jbase = j0 + kt * JT;
+        const int cnt = min(JT, j1 - jbase);
+        double ta[3], tja[3], tjb[3], tp = 0.0;
 #pragma unroll
-        for (int p = 0; p < IPT; ++p) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) ta[p][c] = tja[p][c] = tjb[p][c] = 0.0;
-            tp[p] = 0.0;
-        }
-        bool own = false;
-#pragma unroll
-        for (int p = 0; p < IPT; ++p) own = own || (iid[p] >= jbase && iid[p] < jbase + cnt);
-        own = __any_sync(0xffffffffu, own);
+        for (int c = 0; c < 3; ++c) ta[c] = tja[c] = tjb[c] = 0.0;
 #pragma unroll 2
-        for (int jj = 0; jj < cnt; ++jj) {
-            const double xj = T[jj], yj = T[JT + jj], zj = T[2 * JT + jj];
-            const double uj = T[3 * JT + jj], wj = T[4 * JT + jj], qj = T[5 * JT + jj];
-            const double mj = T[6 * JT + jj];
-#pragma unroll
-            for (int p = 0; p < IPT; ++p) {
-                const double dx = xj - xi[p][0], dy = yj - xi[p][1], dz = zj - xi[p][2];
-                const double dvx = uj - vi[p][0], dvy = wj - vi[p][1], dvz = qj - vi[p][2];
-                double r2 = fma(dx, dx, eps2);
-                r2 = fma(dy, dy, r2);
-                r2 = fma(dz, dz, r2);
-                double rv = dx * dvx;
-                rv = fma(dy, dvy, rv);
-                rv = fma(dz, dvz, rv);
-                double rinv = rsqrt(r2);
-                if (own) rinv = (jbase + jj == iid[p]) ? 0.0 : rinv;
-                const double rinv2 = rinv * rinv;
-                const double mrinv = mj * rinv;
-                const double mr3 = mrinv * rinv2;
-                const double beta = (mr3 * rinv2) * rv;
-                tp[p] += mrinv;
-                ta[p][0] = fma(mr3, dx, ta[p][0]);
-                ta[p][1] = fma(mr3, dy, ta[p][1]);
-                ta[p][2] = fma(mr3, dz, ta[p][2]);
-                tja[p][0] = fma(mr3, dvx, tja[p][0]);
-                tja[p][1] = fma(mr3, dvy, tja[p][1]);
-                tja[p][2] = fma(mr3, dvz, tja[p][2]);
-                tjb[p][0] = fma(beta, dx, tjb[p][0]);
-                tjb[p][1] = fma(beta, dy, tjb[p][1]);
-                tjb[p][2] = fma(beta, dz, tjb[p][2]);
-            }
+        for (int jj = row; jj < cnt; jj += T64_ROWS) {
+            const double dx = T[jj] - xi[0], dy = T[JT + jj] - xi[1], dz = T[2 * JT + jj] - xi[2];
+            const double dvx = T[3 * JT + jj] - vi[0], dvy = T[4 * JT + jj] - vi[1],
+                         dvz = T[5 * JT + jj] - vi[2];
+            double r2 = fma(dx, dx, eps2);
+            r2 = fma(dy, dy, r2);
+            r2 = fma(dz, dz, r2);
+            double rv = dx * dvx;
+            rv = fma(dy, dvy, rv);
+            rv = fma(dz, dvz, rv);
+            const double rinv = jbase + jj == iid ? 0.0 : rsqrt(r2);
+            const double rinv2 = rinv * rinv;
+            const double mrinv = T[6 * JT + jj] * rinv;
+            const double mr3 = mrinv * rinv2;
+            const double beta = (mr3 * rinv2) * rv;
+            tp += mrinv;
+            ta[0] = fma(mr3, dx, ta[0]);
+            ta[1] = fma(mr3, dy, ta[1]);
+            ta[2] = fma(mr3, dz, ta[2]);
+            tja[0] = fma(mr3, dvx, tja[0]);
+            tja[1] = fma(mr3, dvy, tja[1]);
+            tja[2] = fma(mr3, dvz, tja[2]);
+            tjb[0] = fma(beta, dx, tjb[0]);
+            tjb[1] = fma(beta, dy, tjb[1]);
+            tjb[2] = fma(beta, dz, tjb[2]);
         }
 #pragma unroll
-        for (int p = 0; p < IPT; ++p) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                A[p][c] += ta[p][c];
-                J[p][c] += fma(-3.0, tjb[p][c], tja[p][c]);
-            }
-            P[p] += tp[p];
+        for (int c = 0; c < 3; ++c) {
+            v[c] += ta[c];
+            v[3 + c] += fma(-3.0, tjb[c], tja[c]);
         }
+        v[6] += tp;
         __syncthreads();
         if (s_abort) {
-            if (tid == 0) drain_ring<NS>(s_full, 0u, kt, my_tiles);
-            break;
+            if (tid == 0) {
+                drain_ring<NS>(s_full, 0u, kt, my_tiles);
+                atomicOr(err, DERR_TIMEOUT);
+            }
+            return;
         }
         if (tid == 0 && kt + NS < my_tiles) issue(kt + NS);
     }
-    if (s_abort) {
-        if (tid == 0) atomicOr(err, DERR_TIMEOUT);
-        return;
-    }
 
+    if (row > 0) {
 #pragma unroll
-    for (int p = 0; p < IPT; ++p) {
-        const int k = blockIdx.x * (NT * IPT) + p * NT + tid;
-        if (k >= is.n) continue;
-        double v[7] = {A[p][0], A[p][1], A[p][2], J[p][0], J[p][1], J[p][2], P[p]};
-        if (nsplit == 1) {
-            write_final(out, k, v, err);
-        } else {
-#pragma unroll
-            for (int c = 0; c < 7; ++c) part[((size_t)split * 7 + c) * pld + k] = v[c];
-        }
+        for (int c = 0; c < 7; ++c) s_row[row - 1][c][lane] = v[c];
     }
-    if (nsplit > 1)
-        finish_split<NT>(nsplit, blockIdx.x * (NT * IPT), NT * IPT, is.n, part, pld,
-                         counters + blockIdx.x, out, err);
+    __syncthreads();
+    if (row > 0 || k >= is.n) return;
+#pragma unroll
+    for (int c = 0; c < 7; ++c)
+        v[c] = (v[c] + s_row[0][c][lane]) + (s_row[1][c][lane] + s_row[2][c][lane]);
+    if (nsplit == 1) {
+        write_final(out, k, v, err);
+    } else {
+#pragma unroll
+        for (int c = 0; c < 7; ++c) part[((size_t)split * 7 + c) * pld + k] = v[c];
+    }
 }
 
 // ---------------------------------------------------------------------------
 // j-parallel kernels for small i-sets (lanes over j).
 // ---------------------------------------------------------------------------
-
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 
 // FP32 / double-single warp-group kernel for small and mid-size i-sets: each
 // warp owns its own IPT i-particles (every lane holds the same ones) and its
@@ -919,7 +896,7 @@ __global__ void __launch_bounds__(256)
         }
         __syncthreads();
     }
-    // with nsplit > 1 the partials are summed by k_tile_split_reduce, launched next
+    // with nsplit > 1 the partials are summed by k_split_sums, launched next
     (void)counters;
 }
 
@@ -930,12 +907,13 @@ __global__ void __launch_bounds__(NT)
                     unsigned *counters, Out3 out, unsigned *err)
 {
     constexpr int NW = NT / 32;
-    __shared__ double s_red[NW][IPT][7];
+    __shared__ double s_red[NW][IPT * 7];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nsplit = gridDim.x, split = blockIdx.x;
     const int nj = js.n;
     const int j0 = (int)((long long)nj * split / nsplit);
     const int j1 = (int)((long long)nj * (split + 1) / nsplit);
+    cudaGridDependencySynchronize();
 
     for (int g0 = 0; g0 < is.n; g0 += IPT) {
         double xi[IPT][3], vi[IPT][3], mi[IPT];
@@ -975,8 +953,7 @@ __global__ void __launch_bounds__(NT)
                 double rv = dx * dvx;
                 rv = fma(dy, dvy, rv);
                 rv = fma(dz, dvz, rv);
-                double rinv = rsqrt(r2);
-                rinv = (j == iid[p]) ? 0.0 : rinv;
+                const double rinv = j == iid[p] ? 0.0 : rsqrt(r2);
                 const double rinv2 = rinv * rinv;
                 const double mrinv = mj * rinv;
                 const double mr3 = mrinv * rinv2;
@@ -993,21 +970,22 @@ __global__ void __launch_bounds__(NT)
                 tjb[p][2] = fma(beta, dz, tjb[p][2]);
             }
         }
+        // lane 7 p + c of a warp holds its sum of component c of slot p
+        constexpr int P = IPT == 1 ? 8 : (IPT == 2 ? 16 : 32);
+        double v[P];
+#pragma unroll
+        for (int q = 0; q < P; ++q) v[q] = 0.0;
 #pragma unroll
         for (int p = 0; p < IPT; ++p) {
-            double v[7];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                v[c] = ta[p][c];
-                v[3 + c] = fma(-3.0, tjb[p][c], tja[p][c]);
+                v[7 * p + c] = ta[p][c];
+                v[7 * p + 3 + c] = fma(-3.0, tjb[p][c], tja[p][c]);
             }
-            v[6] = tp[p];
-#pragma unroll
-            for (int c = 0; c < 7; ++c) {
-                const double w = warp_sum(v[c]);
-                if (lane == 0) s_red[warp][p][c] = w;
-            }
+            v[7 * p + 6] = tp[p];
         }
+        const double wsum = warp_scatter_sum<P>(v);
+        if (lane < IPT * 7) s_red[warp][lane] = wsum;
         __syncthreads();
         if (tid < IPT * 7) {
             const int p = tid / 7, c = tid % 7;
@@ -1015,7 +993,7 @@ __global__ void __launch_bounds__(NT)
             if (k < is.n) {
                 double s = 0.0;
 #pragma unroll
-                for (int w = 0; w < NW; ++w) s += s_red[w][p][c];
+                for (int w = 0; w < NW; ++w) s += s_red[w][tid];
                 if (nsplit == 1) {
                     if (c == 6) {
                         s = -s;
@@ -1033,7 +1011,9 @@ __global__ void __launch_bounds__(NT)
         }
         __syncthreads();
     }
-    if (nsplit > 1) finish_split<NT>(nsplit, 0, is.n, is.n, part, pld, counters, out, err);
+    // counters == null: the partials are summed by k_split_sums, launched next
+    if (nsplit > 1 && counters)
+        finish_split<NT>(nsplit, 0, is.n, is.n, part, pld, counters, out, err);
 }
 
 // ---------------------------------------------------------------------------
@@ -1384,21 +1364,50 @@ ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms)
     ForcePlan p{};
     p.nwj = 1;
     if (variant == NB_F64) {
-        if (n_i <= 32) {  // FP64 j-parallel kernel
-            p.kind = 1;
-            p.ipt = n_i <= 1 ? 1 : n_i <= 2 ? 2 : 4;
-            p.threads = 128;
-            p.nsplit = (int)clampll((n_j + 128LL * 4 - 1) / (128LL * 4), 1, 2LL * num_sms);
-            return p;
+        // j-parallel below 32 i-particles where it is faster: a pass over the j-set for
+        // every four (1 us for each pair of a lane, and the lanes' sums), one j per lane while
+        // that takes two CTAs per SM at most; the tile kernel takes as long for one
+        // i-particle as for 32 (a j on every SM's four warps is 1 us):
+        // 4 of 20011 39.5 -> 21.0 us, 32 of 20011 265 -> 52 us (tiles).
+        if (n_i <= 32) {
+            const long long ns = clampll((n_j + 127LL) / 128, 1, 2LL * num_sms);
+            const double passes = (double)((n_i + 3) / 4);
+            const double per_sm = (double)((n_j + 128LL * num_sms - 1) / (128LL * num_sms));
+            const double pass = per_sm * (double)(n_i < 4 ? n_i : 4) + 3.0;
+            if (passes * pass <= (double)n_j / (4.0 * num_sms) + 5.0) {
+                p.kind = 1;
+                p.ipt = n_i <= 1 ? 1 : n_i <= 2 ? 2 : 4;
+                p.threads = 128;
+                p.nsplit = (int)ns;
+                return p;
+            }
         }
+        // CTAs of 32 i-particles: the split count of least time, an SM's CTAs (at most
+        // ceil(CTAs / SMs)) times the units of a split (4 us each: four warps, four j each),
+        // with two CTAs per SM or more to cover the FP64 latencies where the j-range allows
         p.kind = 0;
         p.ipt = 1;
-        p.threads = 128;
-        p.jt = JT64;
-        const long long nblk = (n_i + 127) / 128;
-        const long long ntiles = (n_j + JT64 - 1) / JT64;
-        p.nsplit = (int)clampll((16LL * num_sms + nblk - 1) / nblk, 1,
-                                ntiles / 2 > 1 ? ntiles / 2 : 1);
+        p.threads = 32;
+        p.jt = T64_UNIT;
+        const long long nblk = (n_i + 31) / 32;
+        const long long nunits = (n_j + T64_UNIT - 1) / T64_UNIT;
+        double best = 1e300;
+        long long last = 0;
+        for (const int per_sm : {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 24, 32, 48}) {
+            const long long ns = clampll((long long)per_sm * num_sms / nblk, 1,
+                                         nunits < 512 ? nunits : 512);
+            if (ns == last) continue;
+            last = ns;
+            const long long on_sm = (nblk * ns + num_sms - 1) / num_sms;
+            const long long units = (nunits + ns - 1) / ns;
+            const double t = ((double)on_sm + (on_sm == 1 ? 0.15 : 0.0)) * (double)units * 4.0 +
+                             (double)on_sm +
+                             (ns > 1 ? 4.0 + 0.02 * (double)ns + 3e-5 * (double)(ns * n_i) : 0.0);
+            if (t < best) {
+                best = t;
+                p.nsplit = (int)ns;
+            }
+        }
         return p;
     }
     // Tiny sets: the j-set in registers, a pass over them for every four i-particles. The
@@ -1472,8 +1481,8 @@ ForcePlan plan_from_entry(const nb_plan &e, int variant, int n_i, int n_j)
     p.kind = 0;
     if (variant == NB_F64) {
         p.ipt = 1;
-        p.threads = 128;
-        p.jt = JT64;
+        p.threads = 32;  // i-particles of a CTA
+        p.jt = T64_UNIT;
     } else {
         p.threads = 256;
         p.jt = JT_TILE;
@@ -1495,16 +1504,17 @@ size_t plan_partial_doubles(const ForcePlan &p, int n_i)
 // thread per output gives every SM more than two CTAs.
 constexpr long long SPLIT_WIDE_OUTS = 1 << 17;
 
-static cudaError_t go_split_reduce(const double *part, int n_i, int nsplit, const Out3 &out,
-                                   unsigned *err, cudaStream_t st)
+template <class T>
+static cudaError_t go_split_sums(const double *part, int n_i, int nsplit, const Out3 &out,
+                                 unsigned *err, cudaStream_t st)
 {
     const long long outs = 7LL * n_i;
-    const float2 *p = reinterpret_cast<const float2 *>(part);
+    const T *p = reinterpret_cast<const T *>(part);
     if (nsplit > 8 && outs <= SPLIT_WIDE_OUTS)
-        return launch_dependent(k_tile_split_reduce<8>, dim3((unsigned)((outs + 31) / 32)), 256, 0,
-                                st, p, (long long)n_i, nsplit, n_i, out, err);
-    return launch_dependent(k_tile_split_reduce<1>, dim3((unsigned)((outs + 255) / 256)), 256, 0,
-                            st, p, (long long)n_i, nsplit, n_i, out, err);
+        return launch_dependent(k_split_sums<T, 8>, dim3((unsigned)((outs + 31) / 32)), 256, 0, st, p,
+                                (long long)n_i, nsplit, n_i, out, err);
+    return launch_dependent(k_split_sums<T, 1>, dim3((unsigned)((outs + 255) / 256)), 256, 0, st, p,
+                            (long long)n_i, nsplit, n_i, out, err);
 }
 
 // Let kernel K take smem bytes of dynamic shared memory on the current device (the
@@ -1548,7 +1558,7 @@ static cudaError_t go_tile32(const JSet &js, const ISet &is, float eps2f, int ns
     const cudaError_t e = launch_dependent(kern, grid, NT, smem, st, js.rec32, js.n, is, eps2f,
                                            ntiles, part, (long long)is.n, cnt, out, err);
     if (e != cudaSuccess || nsplit <= 1) return e;
-    return go_split_reduce(part, is.n, nsplit, out, err, st);
+    return go_split_sums<float2>(part, is.n, nsplit, out, err, st);
 }
 
 template <int VAR, int IPT, int NWARP>
@@ -1572,7 +1582,7 @@ static cudaError_t go_tiny32(const JSet &js, const ISet &is, float eps2f, double
         launch_dependent(k_force_tiny32<VAR, IPT, JPT>, dim3(g), 256, 0, st, js.rec32, js.n, is,
                          eps2f, part, (long long)is.n, cnt, out, err);
     if (e != cudaSuccess || g <= 1) return e;
-    return go_split_reduce(part, is.n, g, out, err, st);
+    return go_split_sums<float2>(part, is.n, g, out, err, st);
 }
 
 template <int VAR, int IPT>
@@ -1587,16 +1597,16 @@ static cudaError_t go_tiny32_j(int jpt, const JSet &js, const ISet &is, float ep
     }
 }
 
-template <int IPT, int NT>
 static cudaError_t go_tile64(const JSet &js, const ISet &is, double eps2, int nsplit, double *part,
-                             unsigned *cnt, Out3 out, unsigned *err, cudaStream_t st)
+                             Out3 out, unsigned *err, cudaStream_t st)
 {
-    auto kern = k_force_tile64<IPT, NT, JT64, NS64>;
     const size_t smem = (size_t)NS64 * 7 * JT64 * sizeof(double);  // 10.5 KB
-    const int ntiles = (js.n + JT64 - 1) / JT64;
-    dim3 grid((is.n + NT * IPT - 1) / (NT * IPT), nsplit);
-    kern<<<grid, NT, smem, st>>>(js, is, eps2, ntiles, part, is.n, cnt, out, err);
-    return cudaGetLastError();
+    const int nunits = (js.n + T64_UNIT - 1) / T64_UNIT;
+    const cudaError_t e =
+        launch_dependent(k_force_tile64<JT64, NS64>, dim3((is.n + 31) / 32, nsplit), 32 * T64_ROWS,
+                         smem, st, js, is, eps2, nunits, part, (long long)is.n, out, err);
+    if (e != cudaSuccess || nsplit <= 1) return e;
+    return go_split_sums<double>(part, is.n, nsplit, out, err, st);
 }
 
 template <int VAR>
@@ -1653,18 +1663,14 @@ static cudaError_t dispatch64(const ForcePlan &p, const JSet &js, const ISet &is
                               double *part, unsigned *cnt, Out3 out, unsigned *err,
                               cudaStream_t st)
 {
-    if (p.kind == 1) {
-        const int g = p.nsplit;
-#define JM(I) k_force_jmode64<I, 128><<<g, 128, 0, st>>>(js, is, eps2, part, is.n, cnt, out, err)
-        switch (p.ipt) {
-        case 1: JM(1); break;
-        case 2: JM(2); break;
-        default: JM(4); break;
-        }
-#undef JM
-        return cudaGetLastError();
-    }
-    return go_tile64<1, 128>(js, is, eps2, p.nsplit, part, cnt, out, err, st);
+    if (p.kind != 1) return go_tile64(js, is, eps2, p.nsplit, part, out, err, st);
+    const auto kern = p.ipt == 1   ? k_force_jmode64<1, 128>
+                      : p.ipt == 2 ? k_force_jmode64<2, 128>
+                                   : k_force_jmode64<4, 128>;
+    const cudaError_t e = launch_dependent(kern, dim3(p.nsplit), 128, 0, st, js, is, eps2, part,
+                                           (long long)is.n, cnt, out, err);
+    if (e != cudaSuccess || p.nsplit <= 1 || cnt) return e;
+    return go_split_sums<double>(part, is.n, p.nsplit, out, err, st);
 }
 
 // Shared memory of the batched kernel: the ring (18 KB), the transposed tile (6 KB)

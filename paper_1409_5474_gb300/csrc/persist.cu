@@ -127,7 +127,6 @@ __device__ __forceinline__ void tile_item(const FusedArgs &a, int na, int k0, in
                                           int chunk, float4 (*s_tile)[DS_REC * FUSED_TILE])
 {
     constexpr int NT = FUSED_THREADS, NW = NT / 32, PF = (DS_REC * FUSED_TILE + NT - 1) / NT;
-    constexpr int NPAIR = FUSED_TILE / 2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // the lane's due particles (slots k0 + 32 p + lane)
     IPair ip[IPT];

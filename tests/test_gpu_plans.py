@@ -32,6 +32,14 @@ def test_splits(nb, variant, n_i, nsplit):
     _one(nb, variant, p, 1e-3, idx, plan=(0, 8, nsplit))
 
 
+@pytest.mark.parametrize("n_i", [1, 4, 31, 33, 200])
+@pytest.mark.parametrize("plan", [(0, 1, 1), (0, 1, 7), (0, 1, 8), (0, 1, 63), (1, 1, 1), (1, 1, 9)])
+def test_splits_fp64(nb, plan, n_i):
+    p = ic.plummer(999, 5, masses="lognormal")  # 62 units of 16 j and one of 7
+    idx = np.random.default_rng(n_i).integers(0, 999, n_i).astype(np.int32)
+    _one(nb, "f64", p, 1e-3, idx, plan=plan)
+
+
 @pytest.mark.parametrize("n,n_i,kind", [(65536, 4, 2), (65536, 5, 0), (65537, 5, 2), (65537, 8, 2),
                                         (65537, 9, 0)])
 def test_tiny_sets(nb, n, n_i, kind):
