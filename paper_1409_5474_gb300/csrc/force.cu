@@ -36,11 +36,11 @@
 #include <math.h>
 #include <stdint.h>
 
-#include <atomic>
 
 #include "nb_internal.cuh"
 #include "ds.cuh"
 #include "pair.cuh"
+#include "split_sum.cuh"
 #include "tma.cuh"
 
 namespace nb {
@@ -411,58 +411,18 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     (void)counters;
 }
 
-// K3 of the tile, tiny-set and FP64 kernels: the nsplit partials (T: double-single float2, or
-// double) of every output (component c of slot k) in a fixed order. A CTA is 256 / G
-// consecutive outputs (their partials are adjacent, so the loads of a warp are coalesced)
-// times G groups of splits: group g adds the splits g, g + G, ..., eight at a time, all eight
-// loads in flight and added in pairs (FP64: 114 splits one after the other doubled the
-// rounding error of small i-sets), and the groups are added in order through shared memory.
-// G = 1 where the outputs alone fill the GPU; with G = 8 a small due set's many splits cost
-// one or two round trips to L2 and not nsplit / 8 of them (64 slots, 152 splits at N = 65536:
-// force and reduction 27.0 -> 18.8 us, 14.3 as a dependent launch).
-__device__ __forceinline__ dsf split_value(float2 x) { return dsf{x.x, x.y}; }
-__device__ __forceinline__ double split_value(double x) { return x; }
-__device__ __forceinline__ double split_total(dsf x) { return ds_to_double(x); }
-__device__ __forceinline__ double split_total(double x) { return x; }
-
+// K3 of the tile, tiny-set and FP64 kernels (split_sum): output q = component c of slot k.
 template <class T, int G>
 __global__ void __launch_bounds__(256)
     k_split_sums(const T *__restrict__ part, long long pld, int nsplit, int n_i, Out3 out,
                  unsigned *err)
 {
-    using V = decltype(split_value(T{}));
-    constexpr int NQ = 256 / G;
-    __shared__ V s_sum[G > 1 ? G - 1 : 1][NQ];
-    const int o = threadIdx.x % NQ, g = threadIdx.x / NQ;
-    const long long q = (long long)blockIdx.x * NQ + o;
-    const bool valid = q < 7LL * n_i;
+    const long long q = (long long)blockIdx.x * (256 / G) + threadIdx.x % (256 / G);
     const int c = (int)(q / n_i), k = (int)(q % n_i);
-    V sum{};
+    double v;
     cudaGridDependencySynchronize();
-    if (valid) {
-        const T *p = part + (size_t)c * pld + k;
-        const size_t stride = (size_t)7 * pld;
-        for (int sp = g; sp < nsplit; sp += 8 * G) {
-            V x[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                x[u] = split_value(sp + u * G < nsplit ? __ldcg(p + (size_t)(sp + u * G) * stride)
-                                                       : T{});
-#pragma unroll
-            for (int h = 1; h < 8; h <<= 1)
-#pragma unroll
-                for (int u = 0; u < 8; u += 2 * h) sum_into(x[u], x[u + h]);
-            sum_into(sum, x[0]);
-        }
-    }
-    if (G > 1) {
-        if (g > 0) s_sum[g - 1][o] = sum;
-        __syncthreads();
-        if (g > 0) return;
-#pragma unroll
-        for (int u = 1; u < G; ++u) sum_into(sum, s_sum[u - 1][o]);
-    }
-    if (valid) store_component(out, c, k, split_total(sum), err);
+    if (split_sum<T, G>(part + (size_t)c * pld + k, (size_t)7 * pld, nsplit, q < 7LL * n_i, v))
+        store_component(out, c, k, v, err);
 }
 
 // ---------------------------------------------------------------------------
@@ -1500,10 +1460,6 @@ size_t plan_partial_doubles(const ForcePlan &p, int n_i)
     return (size_t)p.nsplit * 7 * (size_t)n_i;
 }
 
-// Outputs up to which the split reduction takes eight threads per output: above, one
-// thread per output gives every SM more than two CTAs.
-constexpr long long SPLIT_WIDE_OUTS = 1 << 17;
-
 template <class T>
 static cudaError_t go_split_sums(const double *part, int n_i, int nsplit, const Out3 &out,
                                  unsigned *err, cudaStream_t st)
@@ -1515,22 +1471,6 @@ static cudaError_t go_split_sums(const double *part, int n_i, int nsplit, const 
                                 (long long)n_i, nsplit, n_i, out, err);
     return launch_dependent(k_split_sums<T, 1>, dim3((unsigned)((outs + 255) / 256)), 256, 0, st, p,
                             (long long)n_i, nsplit, n_i, out, err);
-}
-
-// Let kernel K take smem bytes of dynamic shared memory on the current device (the
-// attribute belongs to the device: set once on each).
-template <auto K>
-static cudaError_t allow_smem(size_t smem)
-{
-    static std::atomic<unsigned long long> done{0};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
-    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
-    e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
-    return e;
 }
 
 // Shared memory of the tile kernel: the ring (36 KB), one or two transposed tiles

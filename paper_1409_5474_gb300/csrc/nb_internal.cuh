@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/nbody.h"
 
 namespace nb {
@@ -28,6 +30,22 @@ static inline cudaError_t launch_dependent(void (*kern)(A...), dim3 grid, unsign
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<A>(args)...);
+}
+
+// Let kernel K take smem bytes of dynamic shared memory on the current device (the
+// attribute belongs to the device: set once on each).
+template <auto K>
+static inline cudaError_t allow_smem(size_t smem)
+{
+    static std::atomic<unsigned long long> done{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
 }
 
 // ---- device error word bits (OR-ed by kernels, read by the host) ----------
