@@ -41,6 +41,11 @@ struct nb_batch_s {
     float4 *rec = nullptr;
     WorkItem *d_items = nullptr;
     int nitems = 0;
+    SplitGroup *d_groups = nullptr;  // j-split groups of the large systems' i-blocks
+    int ngroups = 0;
+    float2 *d_part = nullptr;        // their partials
+    unsigned *d_ticket = nullptr;    // the item tickets of the force launches
+    size_t slab_bytes = 0;
     float *d_eps2 = nullptr;
     int *d_off = nullptr, *d_size = nullptr;
     double *d_time = nullptr;  // the shared time of every system
@@ -110,12 +115,45 @@ StepParams bparams(nb_batch b)
 
 Out3 bout(nb_batch b) { return Out3{b->f_acc, b->f_jerk, b->f_pot, b->ld}; }
 
+// Systems larger than this have their j-range split into equal parts of at most as many
+// (whole 128-record tiles), so that no work item holds the last CTAs long: a
+// 4096-particle system's items took a third of a 512-system step each, and ten times the
+// mean load of a 40-system step. The split depends on the system's size alone, so its
+// results are the same alone and in any batch.
+constexpr int BATCH_SPLIT_J = 1024;
+
+int batch_chunk(int n)
+{
+    if (n <= BATCH_SPLIT_J) return n;
+    const int parts = (n + BATCH_SPLIT_J - 1) / BATCH_SPLIT_J;
+    return ((n + parts - 1) / parts + 127) / 128 * 128;
+}
+
 // Work list for CTAs of `threads` threads (i-blocks of 2 * threads), sorted
-// by decreasing work (ni * nj), ties by position.
+// by decreasing work (ni * nj), ties by position. Without memory for the partials
+// (device, or the batch's budget) no system is split.
 int build_items(nb_batch b)
 {
     const int ib = 2 * b->threads;
     std::vector<WorkItem> items;
+    std::vector<SplitGroup> groups;
+    if (b->d_part) cudaFree(b->d_part);
+    if (b->d_groups) cudaFree(b->d_groups);
+    b->d_part = nullptr;
+    b->d_groups = nullptr;
+    size_t part = 0;  // float2 of partials: 7 per i-particle and split
+    for (int s = 0; s < b->n_sys; ++s) {
+        const int n = b->sizes[s], chunk = batch_chunk(n);
+        if (chunk < n) part += (size_t)((n + chunk - 1) / chunk) * 7 * (size_t)n;
+    }
+    bool split = part > 0 && (!b->cfg.budget_bytes ||
+                              b->slab_bytes + part * sizeof(float2) <= b->cfg.budget_bytes);
+    if (split && cudaMalloc(&b->d_part, part * sizeof(float2)) != cudaSuccess) {
+        cudaGetLastError();
+        b->d_part = nullptr;
+        split = false;
+    }
+    float2 *next_part = b->d_part;
     for (int s = 0; s < b->n_sys; ++s) {
         const int n = b->sizes[s], o = b->offs[s];
         const float4 *base = b->rec + (size_t)DS_REC * o;  // the system's records
@@ -130,11 +168,32 @@ int build_items(nb_batch b)
             w.ld = b->ld;
             w.i0 = i0;
             w.ni = std::min(ib, n - i0);
-            w.nj = n;
             w.gathered = 0;
             w.eps2 = e2;
             w.err = b->d_err;
-            items.push_back(w);
+            const int chunk = split ? batch_chunk(n) : n;
+            w.nsplit = (n + chunk - 1) / chunk;
+            w.part = w.nsplit > 1 ? next_part : nullptr;
+            for (int sp = 0; sp < w.nsplit; ++sp) {
+                w.split = sp;
+                w.j0 = sp * chunk;
+                w.nj = std::min(chunk, n - w.j0);
+                items.push_back(w);
+            }
+            if (w.nsplit > 1) {
+                SplitGroup g{};
+                g.part = w.part;
+                g.acc = w.acc;
+                g.jerk = w.jerk;
+                g.pot = w.pot;
+                g.ld = w.ld;
+                g.i0 = i0;
+                g.ni = w.ni;
+                g.nsplit = w.nsplit;
+                g.err = w.err;
+                groups.push_back(g);
+                next_part += (size_t)w.nsplit * 7 * w.ni;
+            }
         }
     }
     std::stable_sort(items.begin(), items.end(), [](const WorkItem &x, const WorkItem &y) {
@@ -146,6 +205,12 @@ int build_items(nb_batch b)
     BCK(b, cudaMemcpy(b->d_items, items.data(), sizeof(WorkItem) * items.size(),
                       cudaMemcpyHostToDevice));
     b->nitems = (int)items.size();
+    b->ngroups = (int)groups.size();
+    if (b->ngroups) {
+        BCK(b, cudaMalloc(&b->d_groups, sizeof(SplitGroup) * groups.size()));
+        BCK(b, cudaMemcpy(b->d_groups, groups.data(), sizeof(SplitGroup) * groups.size(),
+                          cudaMemcpyHostToDevice));
+    }
     b->grid = b->num_sms * batch_blocks_per_sm(b->cfg.variant, b->threads);
     return NB_OK;
 }
@@ -158,10 +223,19 @@ void drop_graph(nb_batch b)
     b->graph = nullptr;
 }
 
+// The batched force: the items, then the sums of the split systems.
+cudaError_t batch_force(nb_batch b)
+{
+    const cudaError_t e = launch_force_items(b->cfg.variant, b->threads, b->d_items, b->nitems,
+                                             b->grid, b->d_ticket, b->stream);
+    if (e != cudaSuccess || !b->ngroups) return e;
+    return launch_split_reduce(b->d_groups, b->ngroups, std::min(b->ngroups, 8 * b->num_sms),
+                               b->stream);
+}
+
 int launch_batch_force(nb_batch b)
 {
-    BCK(b, launch_force_items(b->cfg.variant, b->threads, b->d_items, b->nitems, b->grid,
-                              b->stream));
+    BCK(b, batch_force(b));
     return NB_OK;
 }
 
@@ -184,7 +258,7 @@ int binit(nb_batch b)
     int rc = launch_batch_force(b);
     if (rc) return rc;
     BCK(b, launch_init_steps(s, bout(b), bparams(b), b->sd, b->d_err, b->stream));
-    b->stats.kernel_launches += 3;
+    b->stats.kernel_launches += 3 + (b->ngroups ? 1 : 0);
     b->stats.force_launches += 1;
     b->stats.interactions += b->interactions_per_step;
     rc = check_berr(b);
@@ -202,9 +276,7 @@ int capture_step(nb_batch b)
     BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = launch_predict(s, b->dt, true, b->d_err, b->stream, b->d_time);
     if (e == cudaSuccess && (b->cfg.flags & NB_FLAG_TIMING)) e = cudaEventRecordWithFlags(b->ev[0], b->stream, cudaEventRecordExternal);
-    if (e == cudaSuccess)
-        e = launch_force_items(b->cfg.variant, b->threads, b->d_items, b->nitems, b->grid,
-                               b->stream);
+    if (e == cudaSuccess) e = batch_force(b);
     if (e == cudaSuccess && (b->cfg.flags & NB_FLAG_TIMING)) e = cudaEventRecordWithFlags(b->ev[1], b->stream, cudaEventRecordExternal);
     if (e == cudaSuccess)
         e = launch_correct(s, nullptr, (int)b->ntot, b->dt, bout(b), p, b->sd, b->d_err, nullptr,
@@ -283,6 +355,7 @@ int nb_batch_create(const nb_config *cfg, int n_sys, const int *sizes, const dou
         cudaGetLastError();
         return bail(NB_ERR_OOM);
     }
+    b->slab_bytes = bytes;
     char *p = static_cast<char *>(b->slab);
     auto take = [&](size_t n) {
         char *q = p;
@@ -313,6 +386,8 @@ int nb_batch_create(const nb_config *cfg, int n_sys, const int *sizes, const dou
         cudaMemcpy(b->d_eps2, e2.data(), sizeof(float) * n_sys, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(b->d_off, b->offs.data(), sizeof(int) * n_sys, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(b->d_size, sizes, sizeof(int) * n_sys, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMalloc(&b->d_ticket, 256) != cudaSuccess ||
+        cudaMemset(b->d_ticket, 0, 256) != cudaSuccess ||
         cudaMemset(b->d_err, 0, 256) != cudaSuccess || cudaMemset(b->sd, 0, sizeof(SchedDev)) != cudaSuccess ||
         cudaMemset(b->slab, 0, bytes) != cudaSuccess ||
         cudaEventCreate(&b->ev[0]) != cudaSuccess || cudaEventCreate(&b->ev[1]) != cudaSuccess) {
@@ -332,6 +407,9 @@ int nb_batch_destroy(nb_batch b)
     drop_graph(b);
     cudaFree(b->slab);
     cudaFree(b->d_items);
+    cudaFree(b->d_groups);
+    cudaFree(b->d_part);
+    cudaFree(b->d_ticket);
     cudaFree(b->d_eps2);
     cudaFree(b->d_off);
     cudaFree(b->d_size);
@@ -401,7 +479,7 @@ int nb_batch_step(nb_batch b, int n_steps, nb_stats *st)
         }
         b->stats.block_steps++;
         b->stats.force_launches++;
-        b->stats.kernel_launches += 4;
+        b->stats.kernel_launches += 4 + (b->ngroups ? 1 : 0);
         b->stats.interactions += b->interactions_per_step;
         b->t_host += b->dt;
     }

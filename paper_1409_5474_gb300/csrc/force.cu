@@ -980,8 +980,8 @@ __global__ void __launch_bounds__(NT)
 // Batched force kernel: many independent systems in one launch (the batched
 // clusters, and the requests of the serving loop). A work item is a block of
 // i-rows of one system against a range of the same system's j-records, with
-// its own pointers (WorkItem). The persistent CTAs walk the item list (sorted
-// by decreasing work on the host, so the round-robin assignment is balanced).
+// its own pointers (WorkItem). The persistent CTAs take the items of the list (sorted
+// by decreasing work on the host) by tickets, so that they finish together.
 // i-parallel items stage the j-tiles through the same bulk-copy ring as the
 // tile kernel (the mbarrier phases run on across items); j-parallel items read
 // the j-records straight from L1/L2. Items of a j-split group leave
@@ -1143,18 +1143,28 @@ __global__ void __launch_bounds__(256)
 }
 
 
+// The last CTA of a batched launch to finish (or to give up) puts the ticket back to zero for
+// the next launch on the stream. ticket: {items handed out, CTAs finished}.
+__device__ __forceinline__ void items_done(unsigned *ticket)
+{
+    if (atomicAdd(ticket + 1, 1u) == gridDim.x - 1u) {
+        ticket[0] = 0u;
+        ticket[1] = 0u;
+    }
+}
+
 // As the tile kernel: bound by the FP32 pipe, totals in shared memory, ragged tiles and
 // tiles with a warp's own particles on the packed path (a 1000-particle system has a
 // quarter of its tiles of either kind), warps without rows skip the arithmetic. 512
 // clusters of 16-4096: a pass of eight steps 11.2 -> 10.3 ms.
 template <int VAR, int IPT, int NT, int JT, int NS>
 __global__ void __launch_bounds__(NT, 512 / NT)
-    k_force_items32(const WorkItem *__restrict__ items, int nitems)
+    k_force_items32(const WorkItem *__restrict__ items, int nitems, unsigned *ticket)
 {
     // NS ring stages of JT records, then the current full tile as j-pairs
     extern __shared__ __align__(128) float4 s_tile[];
     __shared__ __align__(8) uint64_t s_full[NS];
-    __shared__ int s_abort;
+    __shared__ int s_abort, s_next;
     constexpr bool DS = (VAR == NB_F32DS);
     float4 *s_pair = s_tile + (size_t)NS * JT * DS_REC;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1170,7 +1180,9 @@ __global__ void __launch_bounds__(NT, 512 / NT)
     __syncthreads();
 
     unsigned seq = 0;  // tiles consumed so far by this CTA (ring position and phase)
-    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+    for (int it = blockIdx.x, next = 0; it < nitems; it = next) {
+        // the item after this one, taken now so that its number is there in time
+        if (tid == 0) s_next = (int)(gridDim.x + atomicAdd(ticket, 1u));
         const WorkItem w = items[it];
         unsigned *err = w.err;
         const float eps2f = w.eps2;
@@ -1225,6 +1237,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
             const bool masked = own || cnt < JT;
             tile_to_pairs<JT, NT>(T, cnt, s_pair, tid);
             __syncthreads();
+            next = s_next;  // thread 0 writes it again after the barrier below at the earliest
             if (warp * IPT * 32 >= w.ni)
                 ;  // no row of this warp is written
             else if (soft)
@@ -1248,6 +1261,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
                 if (tid == 0) {
                     drain_ring<NS>(s_full, seq, kt, ntiles);
                     atomicOr(err, DERR_TIMEOUT);
+                    items_done(ticket);
                 }
                 return;
             }
@@ -1278,6 +1292,7 @@ __global__ void __launch_bounds__(NT, 512 / NT)
             }
         }
     }
+    if (tid == 0) items_done(ticket);
 }
 
 // ---------------------------------------------------------------------------
@@ -1622,31 +1637,32 @@ static size_t items_smem(int threads)
 }
 
 template <int VAR, int NT>
-static cudaError_t go_items(const WorkItem *items, int nitems, int grid, cudaStream_t st)
+static cudaError_t go_items(const WorkItem *items, int nitems, int grid, unsigned *ticket,
+                            cudaStream_t st)
 {
     constexpr auto kern = k_force_items32<VAR, 2, NT, JT32, NS32>;
     const size_t smem = items_smem(NT);
     const cudaError_t attr = allow_smem<kern>(smem);
     if (attr != cudaSuccess) return attr;
-    kern<<<grid, NT, smem, st>>>(items, nitems);
+    kern<<<grid, NT, smem, st>>>(items, nitems, ticket);
     return cudaGetLastError();
 }
 
 cudaError_t launch_force_items(int variant, int threads, const WorkItem *items, int nitems,
-                               int grid, cudaStream_t st)
+                               int grid, unsigned *ticket, cudaStream_t st)
 {
     if (nitems <= 0) return cudaSuccess;
     if (variant == NB_F32DS) {
         switch (threads) {
-        case 64: return go_items<NB_F32DS, 64>(items, nitems, grid, st);
-        case 128: return go_items<NB_F32DS, 128>(items, nitems, grid, st);
-        default: return go_items<NB_F32DS, 256>(items, nitems, grid, st);
+        case 64: return go_items<NB_F32DS, 64>(items, nitems, grid, ticket, st);
+        case 128: return go_items<NB_F32DS, 128>(items, nitems, grid, ticket, st);
+        default: return go_items<NB_F32DS, 256>(items, nitems, grid, ticket, st);
         }
     }
     switch (threads) {
-    case 64: return go_items<NB_F32, 64>(items, nitems, grid, st);
-    case 128: return go_items<NB_F32, 128>(items, nitems, grid, st);
-    default: return go_items<NB_F32, 256>(items, nitems, grid, st);
+    case 64: return go_items<NB_F32, 64>(items, nitems, grid, ticket, st);
+    case 128: return go_items<NB_F32, 128>(items, nitems, grid, ticket, st);
+    default: return go_items<NB_F32, 256>(items, nitems, grid, ticket, st);
     }
 }
 

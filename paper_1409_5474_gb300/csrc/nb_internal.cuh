@@ -191,10 +191,11 @@ constexpr int ITEM_JPAR_MAX_NI = 64;
 constexpr int BATCH_THREADS[3] = {64, 128, 256};
 
 // Batched force (FP32 / double-single) over a list of i-parallel items (kind 0);
-// grid = number of persistent CTAs (items are taken round-robin, so sort them
-// by decreasing work).
+// grid = number of persistent CTAs (each takes the next item when it is done with one, so
+// sort them by decreasing work). ticket: two words, zero before the first launch and left
+// at zero by each; launches that share them run one after the other.
 cudaError_t launch_force_items(int variant, int threads, const WorkItem *items, int nitems,
-                               int grid, cudaStream_t st);
+                               int grid, unsigned *ticket, cudaStream_t st);
 
 // Resident CTAs per SM of the batched kernel with `threads` threads.
 int batch_blocks_per_sm(int variant, int threads);

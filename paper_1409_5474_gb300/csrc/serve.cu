@@ -114,6 +114,7 @@ struct nb_server_s {
     unsigned *d_errs = nullptr;                   // one error word per slot
     unsigned *h_errs = nullptr;                   // their pinned host copy
     unsigned long long *d_dtmin = nullptr;        // corrector dt_min clamps
+    unsigned *d_ticket = nullptr;                 // the batched force's item tickets
     char *d_stage = nullptr, *h_stage = nullptr;  // the tick's descriptors
     size_t stage_cap = 0;
     float2 *d_part = nullptr;          // j-split partials of the tick
@@ -544,7 +545,7 @@ int tick(nb_server s)
             if (ti.part_off[k] >= 0) items[k].part = s->d_part + ti.part_off[k];
         for (size_t g = 0; g < ti.groups.size(); ++g) ti.groups[g].part = s->d_part + ti.group_off[g];
         // i-parallel items, then j-parallel ones, each longest first (the
-        // persistent CTAs take them round-robin)
+        // persistent CTAs take them in order)
         const int nt = s->threads;
         std::stable_sort(items.begin(), items.end(), [nt](const WorkItem &x, const WorkItem &y) {
             if (x.kind != y.kind) return x.kind < y.kind;
@@ -588,7 +589,8 @@ int tick(nb_server s)
         CKS(cudaEventRecord(s->ev_join, s->stream2));
     }
     if (n0 > 0) {
-        CKS(launch_force_items(s->cfg.variant, s->threads, d_items, n0, std::min(n0, s->grid), st));
+        CKS(launch_force_items(s->cfg.variant, s->threads, d_items, n0, std::min(n0, s->grid),
+                               s->d_ticket, st));
         ++launches;
     }
     if (!ti.engine.empty()) {
@@ -809,7 +811,9 @@ int nb_server_create(const nb_server_cfg *cfg, nb_server *out)
         cudaMallocHost(&s->h_errs, c.max_inflight * sizeof(unsigned)) != cudaSuccess ||
         cudaMalloc(&s->d_dtmin, sizeof(unsigned long long)) != cudaSuccess ||
         cudaMemset(s->d_errs, 0, c.max_inflight * sizeof(unsigned)) != cudaSuccess ||
-        cudaMemset(s->d_dtmin, 0, sizeof(unsigned long long)) != cudaSuccess) {
+        cudaMemset(s->d_dtmin, 0, sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMalloc(&s->d_ticket, 2 * sizeof(unsigned)) != cudaSuccess ||
+        cudaMemset(s->d_ticket, 0, 2 * sizeof(unsigned)) != cudaSuccess) {
         cudaGetLastError();
         if (s->stream) cudaStreamDestroy(s->stream);
         if (s->stream2) cudaStreamDestroy(s->stream2);
@@ -819,6 +823,7 @@ int nb_server_create(const nb_server_cfg *cfg, nb_server *out)
         if (s->d_errs) cudaFree(s->d_errs);
         if (s->h_errs) cudaFreeHost(s->h_errs);
         if (s->d_dtmin) cudaFree(s->d_dtmin);
+        if (s->d_ticket) cudaFree(s->d_ticket);
         return NB_ERR_CUDA;
     }
     s->threads = 128;
@@ -851,6 +856,7 @@ int nb_server_destroy(nb_server s)
     cudaFree(s->d_errs);
     cudaFreeHost(s->h_errs);
     cudaFree(s->d_dtmin);
+    cudaFree(s->d_ticket);
     cudaStreamDestroy(s->stream);
     cudaStreamDestroy(s->stream2);
     cudaEventDestroy(s->ev_fork);

@@ -480,11 +480,12 @@ __device__ __forceinline__ void correct_step(const StateDev &s, int i, double t_
 }
 
 // The step of a particle whose time is t_i (block steps: a power of two, whose
-// reciprocal is exact by exponent arithmetic; a shared step may be any number).
+// reciprocal is exact by exponent arithmetic; shared steps do not use the reciprocals: no
+// step criterion).
 __device__ __forceinline__ void step_factors(double dt, const StepParams &prm, double &dt2,
                                              double &idt2, double &idt3)
 {
-    const double idt = prm.shared_dt > 0.0 ? 1.0 / dt : ldexp(1.0, -ilogb(dt));
+    const double idt = prm.shared_dt > 0.0 ? 0.0 : ldexp(1.0, -ilogb(dt));
     idt2 = idt * idt;
     idt3 = idt2 * idt;
     dt2 = dt * dt;
