@@ -419,8 +419,8 @@ int run_force_plan(nb_handle h, int variant, const ForcePlan &p, const ISet &is,
     const double eps2 = h->cfg.eps * h->cfg.eps;
     CK(h, launch_force(variant, p, jset_of(h), is, eps2, h->part, counters_of(h, variant), out,
                        h->d_err, h->stream, evp));
-    // all but the warp groups' j-split partials are summed by a launch of their own
-    h->stats.kernel_launches += ((p.kind != 1 || variant == NB_F64) && p.nsplit > 1) ? 2 : 1;
+    // the tile kernels' and the FP64 kernels' j-split partials are summed by a launch of their own
+    h->stats.kernel_launches += ((p.kind == 0 || variant == NB_F64) && p.nsplit > 1) ? 2 : 1;
     int lg = 0;
     while ((2LL << lg) <= is.n && lg < 31) ++lg;
     if (evp) {
