@@ -483,15 +483,15 @@ __device__ __forceinline__ void next_block_time(const FusedArgs &a, double t_cur
     const unsigned b0 = __ballot_sync(0xffffffffu, h0 > 0);
     const unsigned b1 = __ballot_sync(0xffffffffu, h1 > 0);
     const int kmax = b1 ? 63 - __clz(b1) : (b0 ? 31 - __clz(b0) : 0);
-    const double dm = ldexp(a.prm.dt_max, -kmax);
-    const double q = floor(t_cur * (1.0 / dm)) + 1.0;
+    double q;
+    const double tn = next_multiple(t_cur, a.prm.dt_max, kmax, &q);
     const unsigned long long qi = q < 9.0e18 ? (unsigned long long)q : 0ull;
     const int k0 = qi ? max(0, kmax - (__ffsll((long long)qi) - 1)) : NLEVEL;
     int c = (lane >= k0 ? h0 : 0) + (lane + 32 >= k0 ? h1 : 0);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if (lane == 0) {
-        s_tn = q * dm;
+        s_tn = tn;
         s_na = c;
     }
 }

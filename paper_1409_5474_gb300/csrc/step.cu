@@ -296,11 +296,8 @@ __device__ __forceinline__ void sched_body(const StateDev &s, SchedDev *sd,
         int kmax = 0;
         for (int w = 0; w < NLEVEL / 32; ++w)
             if (s_occ[w]) kmax = w * 32 + 31 - __clz(s_occ[w]);
-        const double dm = ldexp(dt_max, -kmax);
-        const double tc = s_tcur;
-        // next multiple of the power of two dm after tc: tc / dm is exact, so
-        // floor(tc / dm) + 1 times dm is too (no fmod, which is slow in FP64)
-        s_tnext = (floor(tc * (1.0 / dm)) + 1.0) * dm;
+        double steps;
+        s_tnext = next_multiple(s_tcur, dt_max, kmax, &steps);
     }
     __syncthreads();
     const int tile = s_tile;

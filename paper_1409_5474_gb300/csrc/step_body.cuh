@@ -54,6 +54,30 @@ __device__ __forceinline__ float f32_trunc(double x)
     return hi;
 }
 
+// Powers of two by their bits: an FP64 instruction holds its pipe for 64 cycles, and the
+// general ilogb and ldexp take several. pow2: 2^k for a normal 2^k; exponent_of: floor(log2 |x|)
+// of a normal x (-1023 for 0 and subnormal x).
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((k + 1023) << 20, 0); }
+
+__device__ __forceinline__ int exponent_of(double x)
+{
+    return ((__double2hiint(x) >> 20) & 0x7ff) - 1023;
+}
+
+// 2^-floor(log2 |x|).
+__device__ __forceinline__ double inv_pow2_of(double x)
+{
+    const int e = exponent_of(x);
+    return e > -1023 && e < 1023 ? pow2(-e) : ldexp(1.0, -ilogb(x));
+}
+
+// x halved (exactly, by its exponent; subnormal results by the multiplication).
+__device__ __forceinline__ double half_of(double x)
+{
+    const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+    return e > 1 && e < 0x7ff ? __hiloint2double(hi - (1 << 20), __double2loint(x)) : 0.5 * x;
+}
+
 // ---- K1 for one particle ------------------------------------------------------
 
 // The double-single j-record of particle i at position x, velocity v:
@@ -78,14 +102,14 @@ __device__ __forceinline__ bool predict_one(const StateDev &s, int i, double tn,
 {
     const double ti = s.t[i];
     const double d = tn - ti;
-    const double d6 = d * (1.0 / 6.0), d2h = 0.5 * d;
+    const double d6 = d * (1.0 / 6.0), d2h = half_of(d);
     const bool due = (ti + s.dt[i] == tn);
     double xp[3], vp[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const long long q = c * s.ld + i;
         const double x = s.pos[q], v = s.vel[q], a = s.acc[q], j = s.jerk[q];
-        xp[c] = fma(fma(fma(j, d6, 0.5 * a), d, v), d, x);
+        xp[c] = fma(fma(fma(j, d6, half_of(a)), d, v), d, x);
         vp[c] = fma(fma(j, d2h, a), d, v);
         if (STORE_P) {
             s.pos_p[q] = xp[c];
@@ -130,11 +154,11 @@ __device__ __forceinline__ bool predict_rec_from(const StateDev &s, const PState
                                                  double tn, float4 rec[3])
 {
     const double d = tn - q.t;
-    const double d6 = d * (1.0 / 6.0), d2h = 0.5 * d;
+    const double d6 = d * (1.0 / 6.0), d2h = half_of(d);
     double xp[3], vp[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        xp[c] = fma(fma(fma(q.j[c], d6, 0.5 * q.a[c]), d, q.v[c]), d, q.x[c]);
+        xp[c] = fma(fma(fma(q.j[c], d6, half_of(q.a[c])), d, q.v[c]), d, q.x[c]);
         vp[c] = fma(fma(q.j[c], d2h, q.a[c]), d, q.v[c]);
     }
     make_record(xp, vp, q.m, i, rec);
@@ -238,12 +262,33 @@ __device__ __forceinline__ double norm3(double x, double y, double z)
     return sqrt(x * x + y * y + z * z);
 }
 
-// t is a whole multiple of the power of two d: t / d is exact, so test it for an
-// integer (equivalent to fmod(t, d) == 0 for power-of-two d, and cheaper).
+// The next multiple after t of dt_max 2^-k, the smallest occupied step (a power of two: the
+// quotients are exact); *steps: how many of them it is.
+__device__ __forceinline__ double next_multiple(double t, double dt_max, int k, double *steps)
+{
+    const int e = exponent_of(dt_max) - k;
+    const bool normal = exponent_of(dt_max) > -1000 && e > -1000 && e < 1000;
+    const double d = normal ? pow2(e) : ldexp(dt_max, -k);
+    const double q = floor(t * (normal ? pow2(-e) : 1.0 / d)) + 1.0;
+    *steps = q;
+    return q * d;
+}
+
+// The exponent of the largest power of two that divides t (INT_MAX for 0).
+__device__ __forceinline__ int dyadic_exponent(double t)
+{
+    const unsigned long long u =
+        (unsigned long long)__double_as_longlong(t) & 0x7fffffffffffffffull;
+    if (u == 0ull) return 0x7fffffff;
+    const int e = (int)(u >> 52);
+    const unsigned long long m = (u & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+    return (e ? e : 1) - 1076 + __ffsll((long long)m);
+}
+
+// t is a whole multiple of the power of two d.
 __device__ __forceinline__ bool divides(double t, double d)
 {
-    const double q = t * ldexp(1.0, -ilogb(d));
-    return q == trunc(q);
+    return dyadic_exponent(t) >= exponent_of(d);
 }
 
 // Largest power of two <= raw (dt_max for raw >= dt_max or +inf), at most twice
@@ -273,7 +318,7 @@ static __device__ double quantize(double raw, double dt_old, double t_new, doubl
 // Level of a power-of-two step: dt = dt_max * 2^-k.
 __device__ __forceinline__ int step_level(double dt, double dt_max)
 {
-    int k = ilogb(dt_max) - ilogb(dt);
+    int k = exponent_of(dt_max) - exponent_of(dt);
     return k < 0 ? 0 : (k >= NLEVEL ? NLEVEL - 1 : k);
 }
 
@@ -327,7 +372,16 @@ static __device__ double quantize_log2(int e, double dt_old, double t_new, doubl
                                 bool *clamped)
 {
     const int half = e >= 0 ? e / 2 : -((1 - e) / 2);  // floor(e / 2)
-    double d = (half >= ilogb(dt_max)) ? dt_max : ldexp(1.0, half);
+    const int km = exponent_of(dt_min), kM = exponent_of(dt_max), ko = exponent_of(dt_old);
+    const long long frac = 0xfffffffffffffll;  // zero in a power of two
+    if (km > -1023 && ko > -1023 && dt_old > 0.0 && (__double_as_longlong(dt_old) & frac) == 0) {
+        // every bound is a power of two: the same rule in exponents
+        int k = min(min(half, kM), ko + 1);
+        *clamped = k < km;
+        k = max(km, min(k, dyadic_exponent(t_new)));
+        return pow2(k);
+    }
+    double d = (half >= kM) ? dt_max : ldexp(1.0, half);
     if (dt_old > 0.0 && d > 2.0 * dt_old) d = 2.0 * dt_old;
     if (d > dt_max) d = dt_max;
     *clamped = false;
@@ -368,8 +422,8 @@ __device__ __forceinline__ void hermite_correct(double xp, double vp, double a0,
 __device__ __forceinline__ void predict_xv(double x, double v, double a0, double j0, double dt,
                                            double &xp, double &vp)
 {
-    const double d = dt, d6 = d * (1.0 / 6.0), d2h = 0.5 * d;
-    xp = fma(fma(fma(j0, d6, 0.5 * a0), d, v), d, x);
+    const double d = dt, d6 = d * (1.0 / 6.0), d2h = half_of(d);
+    xp = fma(fma(fma(j0, d6, half_of(a0)), d, v), d, x);
     vp = fma(fma(j0, d2h, a0), d, v);
 }
 
@@ -485,7 +539,7 @@ __device__ __forceinline__ void correct_step(const StateDev &s, int i, double t_
 __device__ __forceinline__ void step_factors(double dt, const StepParams &prm, double &dt2,
                                              double &idt2, double &idt3)
 {
-    const double idt = prm.shared_dt > 0.0 ? 0.0 : ldexp(1.0, -ilogb(dt));
+    const double idt = prm.shared_dt > 0.0 ? 0.0 : inv_pow2_of(dt);
     idt2 = idt * idt;
     idt3 = idt2 * idt;
     dt2 = dt * dt;
@@ -667,7 +721,7 @@ __device__ __forceinline__ void correct6_lanes_pre(const StateDev &s, int i, int
         dt = t_new - q.t;
         dt_old = q.dt;
         T = 0.5 * dt;
-        const double iT = prm.shared_dt > 0.0 ? 1.0 / T : ldexp(1.0, -ilogb(T));
+        const double iT = prm.shared_dt > 0.0 ? 1.0 / T : inv_pow2_of(T);
         const double iT3 = iT * iT * iT, iT5 = iT3 * iT * iT;
         const double x0 = q.x, v0 = q.v, a0 = q.a0, j0 = q.j0, s0 = q.s0;
         // v1 = v0 + dt/2 (a0 + a1) - dt^2/10 (j1 - j0) + dt^3/120 (s0 + s1)
