@@ -64,11 +64,11 @@ extern "C" {
 /* ---- configuration ------------------------------------------------------ */
 #define NB_FLAG_TIMING 1 /* time every kernel launch with CUDA events (nb_stats) */
 /* Block steps of NB_F32 / NB_F32DS handles normally run in the fused
- * persistent kernel: one cooperative launch takes block steps (scheduler +
- * predictor, force, reduction, corrector, with grid-wide barriers between
- * the stages) until a due set larger than nb_config.fused_max_na (default
- * NB_FUSED_DEFAULT_NA) or t_end, so small
- * steps need no host round trip; larger due sets go to the planned force
+ * persistent kernel: one launch (cooperative, or one thread-block cluster up to
+ * 4096 particles at order 4) takes block steps (scheduler + predictor, force,
+ * reduction, corrector, with barriers between the stages) until a due set
+ * larger than nb_config.fused_max_na (default NB_FUSED_DEFAULT_NA) or t_end, so
+ * small steps need no host round trip; larger due sets go to the planned force
  * kernels. NB_FLAG_NO_FUSED takes every block step with separate launches. */
 #define NB_FLAG_NO_FUSED 2
 #define NB_FUSED_MAX_NA 4096      /* upper bound of nb_config.fused_max_na */

@@ -146,6 +146,7 @@ struct nb_handle_s {
 
     // fused persistent block steps (allocated at first use)
     int fused_grid = -1;                  // CTAs per launch; 0 = not available
+    int cluster_ok = -1;                  // one cluster can take the steps of a small system
     float2 *fused_part = nullptr;
     size_t fused_part_cap = 0;            // float2
     int *fused_cnt = nullptr;
@@ -864,6 +865,14 @@ bool fused_ready(nb_handle h)
         h->bytes += add;
     }
     return true;
+}
+
+// Whether one cluster takes the fused steps of this (4th-order) system.
+bool cluster_ready(nb_handle h)
+{
+    if (h->n > FUSED_CLUSTER_MAX_N) return false;
+    if (h->cluster_ok < 0) h->cluster_ok = cluster_steps_ready() ? 1 : 0;
+    return h->cluster_ok == 1;
 }
 
 // The arguments of the fused launches of nb_step to t_end (f: the order-4
@@ -1659,13 +1668,15 @@ int nb_step(nb_handle h, double t_end, nb_stats *st)
         // queued as soon as it is read
         const bool fused = fused_ready(h);
         const FusedArgs fa = fused ? fused_args(h, t_end, f) : FusedArgs{};
+        const bool cluster = fused && cluster_ready(h);
         auto launch_sched = [&]() -> int {
             const unsigned long long ep = h->seq_next++;
             int r;
             if (fused) {
                 r = timed(h, T_FUSED, [&] {
-                    return launch_fused_steps(fa, h->fused_grid, h->cfg.variant == NB_F32DS, 4,
-                                              h->stream);
+                    const bool ds = h->cfg.variant == NB_F32DS;
+                    return cluster ? launch_cluster_steps(fa, ds, h->stream)
+                                   : launch_fused_steps(fa, h->fused_grid, ds, 4, h->stream);
                 });
                 h->stats.fused_launches++;
             } else {

@@ -438,6 +438,11 @@ constexpr int FUSED_SMALL_NA = 16;
 // all on its small-set path; larger ones go to the planned kernels.
 constexpr int FUSED6_MAX_NA = NB_FUSED6_MAX_NA;
 
+// 4th-order systems of up to FUSED_CLUSTER_MAX_N particles are stepped by one cluster of
+// FUSED_CLUSTER CTAs (persist.cu).
+constexpr int FUSED_CLUSTER = 16;
+constexpr int FUSED_CLUSTER_MAX_N = 4096;
+
 // Ints of the fused kernel's counter array: grid per-CTA counts, 2 due-set
 // counters, the tickets of the small-set groups (at most FUSED6_MAX_NA / 4; padded).
 inline size_t fused_cnt_ints(int grid) { return (size_t)grid + 64; }
@@ -453,6 +458,10 @@ size_t fused_part_float2s(int grid, int na_max, int order);
 cudaError_t launch_selftest_mbar(unsigned *err, unsigned long long limit_ns, cudaStream_t st);
 cudaError_t launch_selftest_barrier(unsigned *bar, unsigned *err, unsigned long long limit_ns,
                                     cudaStream_t st);
+// The same steps (order 4) by one cluster: needs no cnt, bar or part. Ready: the current
+// device can run that cluster.
+bool cluster_steps_ready();
+cudaError_t launch_cluster_steps(const FusedArgs &a, bool ds, cudaStream_t st);
 cudaError_t launch_fused_steps(const FusedArgs &a, int grid, bool ds, int order,
                                cudaStream_t st);
 

@@ -19,6 +19,7 @@
 //   D  (larger due sets) one warp per due particle sums its chunk partials in
 //      chunk order (K3) and corrects it (K4: Hermite corrector, Aarseth step,
 //      histogram);                                          -- barrier
+// k_cluster_steps (order 4, small systems) runs the same steps in one thread-block cluster.
 // k_fused_steps6 runs the same loop for the 6th-order scheme with the small
 // path only (64-byte records, ten outputs per slot, the order-6 corrector).
 // Every inter-CTA wait is bounded; a CTA that gives up raises the abort flag
@@ -516,16 +517,17 @@ __device__ __forceinline__ void publish(const FusedArgs &a, double t_cur, double
 // every particle to tn (FP64 pos_p, vel_p (and acc_p at order 6) and records),
 // then gather the due set in ascending index (act, and at order 4 irec),
 // exactly as K5 + K1 would, for the planned kernels the caller runs next.
-// Returns false when a grid barrier gave up.
-template <int ORD>
+// barrier() synchronises the CTAs of the launch (of NT threads); returns false when
+// it gave up.
+template <int ORD, int NT, class Barrier>
 __device__ __forceinline__ bool handoff_predict_gather(const FusedArgs &a, double tn, int p0,
                                                        int p1, int nwords, unsigned *s_flags,
                                                        int *s_woff, int *s_wsum, int &s_total,
-                                                       int &s_base, unsigned &gen)
+                                                       int &s_base, Barrier barrier)
 {
-    constexpr int NT = FUSED_THREADS, NW = NT / 32;
+    constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int G = gridDim.x, bid = blockIdx.x;
+    const int bid = blockIdx.x;
     const StateDev &s = a.s;
     for (int w0 = 0; w0 < nwords; w0 += NW) {
         const int i = p0 + w0 * 32 + tid;
@@ -563,7 +565,7 @@ __device__ __forceinline__ bool handoff_predict_gather(const FusedArgs &a, doubl
         __syncthreads();
     }
     if (tid == 0) a.cnt[bid] = nwords > 0 ? s_base : 0;
-    if (!grid_barrier(a.bar, gen)) return false;
+    if (!barrier()) return false;
     // this CTA's offset; gather its due particles
     if (warp == 0) {
         int before = 0;
@@ -589,8 +591,7 @@ __device__ __forceinline__ bool handoff_predict_gather(const FusedArgs &a, doubl
             }
         }
     }
-    (void)G;
-    return grid_barrier(a.bar, gen);
+    return barrier();
 }
 
 // ---- the kernel ------------------------------------------------------------
@@ -647,8 +648,9 @@ __global__ void __launch_bounds__(FUSED_THREADS)
         if (!(tn <= a.t_end) || na < 1 || na > a.na_max) {
             // hand the step to the caller exactly as the scheduler kernel would
             if (tn <= a.t_end && na >= 1) {
-                ok = handoff_predict_gather<4>(a, tn, p0, p1, nwords, s_flags, s_woff, s_wsum,
-                                               s_total, s_base, gen);
+                ok = handoff_predict_gather<4, NT>(
+                    a, tn, p0, p1, nwords, s_flags, s_woff, s_wsum, s_total, s_base,
+                    [&] { return grid_barrier(a.bar, gen); });
                 mark(0);
                 if (!ok) break;
             }
@@ -797,6 +799,422 @@ __global__ void __launch_bounds__(FUSED_THREADS)
             a.stats->step_ns_hist[tid] += s_step_ns[tid];
         }
         if (tid < 4) a.stats->phase_ns[tid] += s_phase[tid];
+    }
+}
+
+// ---- small systems: one cluster ----------------------------------------------
+//
+// A step of a system of a few thousand particles is latency: at N = 2500 the grid kernel
+// takes 13 us for the smallest, mostly two grid barriers and the round trips to L2
+// between them. Here one cluster of CL_CTAS CTAs takes the steps: the stages are separated by
+// the hardware's cluster barrier, every CTA keeps the j-records of its own particles
+// in shared memory (as j-pairs) and sums every due particle's force over them, and the due
+// records and the partial sums travel through distributed shared memory. The state
+// stays in global memory (L2), so a launch may end after any step:
+//   A  t_next; the CTA's particles predicted, three threads each (a warp-wide FP64
+//      instruction holds its pipe for 64 cycles whatever its lanes do), their due bits
+//      sent to every CTA                                                  -- cluster barrier
+//   B  the due records of all CTAs (a window of CL_SLOTS) copied to shared memory; S
+//      lanes per one or two due particles split the CTA's pairs, their FP32 sums meet in a xor
+//      tree, and slot k's go to CTA k % CL_CTAS                   -- cluster barrier
+//   C  that CTA adds the CL_CTAS partials in double-single and corrects the particle,
+//      three lanes each                                           -- cluster barrier
+// The cluster barrier is a hardware barrier of co-scheduled CTAs (like __syncthreads):
+// no wait depends on another launch, and every exit is taken by all CTAs together.
+// Measured against the grid kernel, 1/16 time unit of block steps: N = 500 2.28 -> 1.57 ms,
+// 1000 5.27 -> 3.8, 2500 8.57 -> 7.2, 4000 11.7 -> 11.3. A step of 1 to 3 due at N = 2500 takes
+// 9.4 us for 13.2: the prediction and its barrier 3.5, the force 3, the corrector 2.2.
+// Sixteen SMs are a tenth of the GPU, so due sets of a hundred and more cost part
+// of that again (N = 2500, 512-1023 due: 41 against 20 us; N = 4000: 61 against 21), which at
+// 4096 particles leaves little: the line of the dispatch.
+constexpr int CL_CTAS = FUSED_CLUSTER;
+constexpr int CL_THREADS = 512;
+constexpr int CL_MAX_L = FUSED_CLUSTER_MAX_N / CL_CTAS;  // particles per CTA
+constexpr int CL_SLOTS = 1024;                           // due slots per window
+constexpr int CL_Q = 7;                                  // outputs of a slot
+// Two slots per lane from here on (half the shared-memory reads; below, one slot keeps more
+// lanes busy).
+constexpr int CL_IPT2_SLOTS = 64;
+
+struct ClusterSmem {
+    float4 pair[6][CL_MAX_L / 2];              // float4 u of pair q: pair[u][q]
+    float4 part[CL_CTAS][CL_SLOTS / CL_CTAS][2];  // sums by source CTA, slot / CL_CTAS
+    float4 own[CL_MAX_L][3];                   // own due records: {x_hi, x_lo, v, -} of component c
+    float i[9][CL_SLOTS];                      // due records: x_hi, x_lo, v of three components
+    int id[CL_SLOTS];
+    uint4 due[CL_CTAS][CL_MAX_L / 128];        // a bit for every particle of every CTA
+    double tn;
+    int na;
+    unsigned long long hist[32], step_ns[32], phase[4];
+    unsigned flags[CL_MAX_L / 32];
+    int woff[CL_MAX_L / 32], wsum[CL_THREADS / 32], total, base;
+};
+
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release;\n"
+                 "barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// The shared-memory address of p (in this CTA) in CTA rank of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, int rank)
+{
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;"
+        : "=r"(a)
+        : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+
+__device__ __forceinline__ float4 cluster_ld(uint32_t a)
+{
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(a)
+                 : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void cluster_st(uint32_t a, unsigned v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ void cluster_st(uint32_t a, float4 v)
+{
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y),
+                 "f"(v.z), "f"(v.w)
+                 : "memory");
+}
+
+// The float of record value u (0-2 x_hi, 3-5 x_lo, 6-8 v; 9 the mass) of own particle l.
+__device__ __forceinline__ float *cl_value(ClusterSmem &sm, int u, int l)
+{
+    const int c = u % 3;
+    const int quad = u == 9 ? 1 : 2 * (u / 3) + (c == 2 ? 1 : 0);  // {x y} {z m} of each triple
+    const int at = u == 9 ? 2 : (c == 1 ? 2 : 0);
+    return reinterpret_cast<float *>(&sm.pair[quad][l >> 1]) + at + (l & 1);
+}
+
+// Lanes per IPT due particles: the power of two with the least estimated time of a window's
+// pair terms (rounds of CL_THREADS / S lanes groups, the pairs of a lane and its share of
+// the xor tree).
+__device__ __forceinline__ int cluster_lanes_log2(int ngroups, int npair)
+{
+    const int lg = min((int)(threadIdx.x & 31), 5);
+    const int rounds = ((ngroups << lg) + CL_THREADS - 1) / CL_THREADS;
+    const int cost = rounds * (2 * ((npair + (1 << lg) - 1) >> lg) + 2 + lg);
+    return (int)(__reduce_min_sync(0xffffffffu, (unsigned)(cost << 3 | lg)) & 7u);
+}
+
+__device__ __forceinline__ JPair cluster_pair(const ClusterSmem &sm, int q)
+{
+    return JPair{sm.pair[0][q], sm.pair[1][q], sm.pair[2][q],
+                 sm.pair[3][q], sm.pair[4][q], sm.pair[5][q]};
+}
+
+// The pair terms of the CTA's particles [p0, p1) on IPT due ones (indices own): this lane's
+// share, pairs sub, sub + S, ... masked: one of the warp's due ones may be among them.
+template <bool DS, bool SOFT, int IPT>
+__device__ __forceinline__ void cluster_pairs(const ClusterSmem &sm, int sub, int S, int p0,
+                                              int p1, bool masked, const IPair (&ip)[IPT],
+                                              const int (&own)[IPT], float2 e2,
+                                              PairSum (&ts)[IPT])
+{
+    const int full = (p1 - p0) / 2;
+    if (!masked) {
+#pragma unroll 2
+        for (int q = sub; q < full; q += S) {
+            const JPair j = cluster_pair(sm, q);
+#pragma unroll
+            for (int p = 0; p < IPT; ++p) pair_add<DS, SOFT>(j, ip[p], e2, ts[p], NoMask{});
+        }
+    } else {
+#pragma unroll 1
+        for (int q = sub; q < full; q += S) {
+            const JPair j = cluster_pair(sm, q);
+#pragma unroll
+            for (int p = 0; p < IPT; ++p)
+                pair_add<DS, SOFT>(j, ip[p], e2, ts[p], PairMask{p0 + 2 * q, own[p], p1});
+        }
+    }
+    if (((p1 - p0) & 1) && (full & (S - 1)) == sub) {  // the last, half-empty pair
+        const JPair j = cluster_pair(sm, full);
+#pragma unroll
+        for (int p = 0; p < IPT; ++p)
+            pair_add<DS, SOFT>(j, ip[p], e2, ts[p], PairMask{p0 + 2 * full, own[p], p1});
+    }
+}
+
+// B for one window of nw due slots: the sums of every slot over the CTA's particles
+// [p0, p1), left in CTA slot % CL_CTAS. Groups of IPT slots (k, k + ngroups), S lanes each.
+template <bool DS, int IPT>
+__device__ __forceinline__ void cluster_force(ClusterSmem &sm, int nw, int p0, int p1, int npair,
+                                              int rank, float eps2f)
+{
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const int ng = (nw + IPT - 1) / IPT;
+    const int lgS = cluster_lanes_log2(ng, npair), S = 1 << lgS, sub = tid & (S - 1);
+    const float2 e2 = make_float2(eps2f, eps2f);
+    for (int g0 = 0; g0 < ng; g0 += CL_THREADS >> lgS) {
+        if (g0 + ((warp * 32) >> lgS) >= ng) break;  // a warp of idle groups
+        const int g = g0 + (tid >> lgS);
+        IPair ip[IPT];
+        PairSum ts[IPT];
+        int own[IPT];
+        bool mine = false;
+#pragma unroll
+        for (int p = 0; p < IPT; ++p) {
+            const int k = min(g + p * ng, nw - 1);  // idle slots copy the last one
+            ip[p] = ipair_of(make_float4(sm.i[0][k], sm.i[1][k], sm.i[2][k], 0.f),
+                             make_float4(sm.i[3][k], sm.i[4][k], sm.i[5][k], 0.f),
+                             make_float4(sm.i[6][k], sm.i[7][k], sm.i[8][k], 0.f));
+            own[p] = sm.id[k];
+            mine = mine || (own[p] >= p0 && own[p] < p1);
+            pair_zero(ts[p]);
+        }
+        const bool masked = __any_sync(0xffffffffu, mine);
+        if (soft_pairs(eps2f))
+            cluster_pairs<DS, true, IPT>(sm, sub, S, p0, p1, masked, ip, own, e2, ts);
+        else
+            cluster_pairs<DS, false, IPT>(sm, sub, S, p0, p1, true, ip, own, e2, ts);
+#pragma unroll
+        for (int p = 0; p < IPT; ++p) {
+            float v[CL_Q];
+#pragma unroll
+            for (int c = 0; c < CL_Q; ++c) v[c] = pair_total(ts[p], c);
+            for (int o = S >> 1; o > 0; o >>= 1)
+#pragma unroll
+                for (int c = 0; c < CL_Q; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+            const int k = g + p * ng;
+            if (sub == 0 && g < ng && k < nw) {
+                const uint32_t to = cluster_addr(sm.part[rank][k / CL_CTAS], k % CL_CTAS);
+                cluster_st(to, make_float4(v[0], v[1], v[2], v[3]));
+                cluster_st(to + 16u, make_float4(v[4], v[5], v[6], 0.f));
+            }
+        }
+    }
+}
+
+template <bool DS>
+__global__ void __launch_bounds__(CL_THREADS)
+    k_cluster_steps(FusedArgs a)
+{
+    extern __shared__ __align__(128) unsigned char s_cluster[];
+    ClusterSmem &sm = *reinterpret_cast<ClusterSmem *>(s_cluster);
+    constexpr int NT = CL_THREADS, NW = NT / 32;
+    static_assert(NW == CL_CTAS, "warp w copies the due records of CTA w");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = blockIdx.x;  // one cluster: the rank in it
+    const StateDev &s = a.s;
+    const int n = s.n;
+    const int per = (n + CL_CTAS - 1) / CL_CTAS;
+    const int p0 = min(n, rank * per), p1 = min(n, p0 + per);
+    const int L = p1 - p0, Lw = (L + 31) & ~31;
+    const int npair = (per + 1) / 2;
+    double t_cur = __ldcg(&a.sd->t_cur);
+    const unsigned long long epoch = __ldcg(&a.sd->seq);
+    unsigned long long steps = 0;
+    double inter = 0.0;
+    const bool scribe = rank == 0 && tid == 0;  // stage times
+    unsigned long long t_mark = globaltimer_ns(), t_step = t_mark;
+    auto mark = [&](int ph) {
+        if (scribe) {
+            const unsigned long long t = globaltimer_ns();
+            sm.phase[ph] += t - t_mark;
+            t_mark = t;
+        }
+    };
+    if (tid < 32) sm.hist[tid] = sm.step_ns[tid] = 0ull;
+    if (tid < 4) sm.phase[tid] = 0ull;
+    if (tid < CL_CTAS * (CL_MAX_L / 128)) (&sm.due[0][0])[tid] = make_uint4(0u, 0u, 0u, 0u);
+    for (int u = tid; u < 6 * (CL_MAX_L / 2); u += NT)
+        (&sm.pair[0][0])[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    cluster_barrier();  // every CTA runs before another writes to its shared memory
+    if (tid < L) *cl_value(sm, 9, tid) = f32_trunc(s.m[p0 + tid]);
+
+    for (;;) {
+        // the thread's first component, loaded while warp 0 finds the block time
+        struct Comp {
+            double x, v, a, j, t, dt;
+        } st[2];
+        auto load = [&](int it, Comp &q) {
+            const int c = it / Lw, l = it - c * Lw;
+            if (c < 3 && l < L) {
+                const long long k = c * s.ld + p0 + l;
+                q.x = s.pos[k];
+                q.v = s.vel[k];
+                q.a = s.acc[k];
+                q.j = s.jerk[k];
+                q.t = s.t[p0 + l];
+                q.dt = s.dt[p0 + l];
+            }
+        };
+        if (Lw > 0) {
+            load(tid, st[0]);
+            load(tid + NT, st[1]);
+        }
+        if (warp == 0) next_block_time(a, t_cur, sm.tn, sm.na);
+        __syncthreads();
+        const double tn = sm.tn;
+        const int na = sm.na;
+        if (!(tn <= a.t_end) || na < 1 || na > a.na_max) {
+            // hand the step to the caller exactly as the scheduler kernel would
+            if (tn <= a.t_end && na >= 1) {
+                handoff_predict_gather<4, NT>(
+                    a, tn, p0, p1, (L + 31) / 32, sm.flags, sm.woff, sm.wsum, sm.total, sm.base, [] {
+                        cluster_barrier();
+                        return true;
+                    });
+                mark(0);
+            }
+            if (scribe) publish(a, t_cur, tn, na, epoch);
+            break;
+        }
+
+        // A: predict, in the predictor's arithmetic; warps hold one component each
+        if (Lw > 0) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int it = tid + h * NT;
+                const int c = it / Lw, l = it - c * Lw;
+                bool due = false;
+                if (c < 3 && l < L) {
+                    const Comp &q = st[h];
+                    const double d = tn - q.t;
+                    double xp, vp;
+                    predict_xv(q.x, q.v, q.a, q.j, d, xp, vp);
+                    float hi, lo;
+                    split_ds(xp, hi, lo);
+                    *cl_value(sm, c, l) = hi;
+                    *cl_value(sm, 3 + c, l) = lo;
+                    const float v = f32_trunc(vp);
+                    *cl_value(sm, 6 + c, l) = v;
+                    // t, dt and tn are multiples of a power of two: t + dt == tn in their bits
+                    due = __double_as_longlong(d) == __double_as_longlong(q.dt);
+                    if (due) sm.own[l][c] = make_float4(hi, lo, v, 0.f);
+                }
+                if (c == 0) {  // (h = 0 only) particles 32 warp + lane: a word to every CTA
+                    const unsigned b = __ballot_sync(0xffffffffu, due);
+                    if (lane < CL_CTAS)
+                        cluster_st(cluster_addr(reinterpret_cast<unsigned *>(sm.due[rank]) + warp,
+                                                lane),
+                                   b);
+                }
+            }
+        }
+        cluster_barrier();
+        mark(0);
+        // lane l: the due counts of 128 particles of CTA l / 2
+        static_assert(CL_MAX_L == 256, "two 128-bit words of due bits per CTA");
+        const uint4 bits = sm.due[lane >> 1][lane & 1];
+        const int mycnt = __popc(bits.x) + __popc(bits.y) + __popc(bits.z) + __popc(bits.w);
+        if ((int)__reduce_add_sync(0xffffffffu, (unsigned)mycnt) != na) {
+            if (scribe) atomicOr(a.err, DERR_SCHED);  // the histogram and the states disagree
+            break;
+        }
+        // warp w copies the records of CTA w's due particles; their slots follow those of
+        // the CTAs before it
+        const int first = (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < 2 * warp ? mycnt : 0));
+
+        for (int w0 = 0; w0 < na; w0 += CL_SLOTS) {  // windows of due slots
+            const int nw = min(CL_SLOTS, na - w0);
+            int k = first - w0;
+            for (int u = 0; u < CL_MAX_L / 32; ++u) {
+                const unsigned word = reinterpret_cast<const unsigned *>(sm.due[warp])[u];
+                const int mk = k + __popc(word & ((1u << lane) - 1u)), l = 32 * u + lane;
+                k += __popc(word);
+                if ((word >> lane & 1u) && mk >= 0 && mk < nw) {
+                    const uint32_t from = cluster_addr(sm.own[l], warp);
+                    float4 v[3];
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) v[c] = cluster_ld(from + 16u * c);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        sm.i[c][mk] = v[c].x;
+                        sm.i[3 + c][mk] = v[c].y;
+                        sm.i[6 + c][mk] = v[c].z;
+                    }
+                    sm.id[mk] = warp * per + l;
+                }
+            }
+            __syncthreads();
+
+            // B: the pair terms
+            if (nw >= CL_IPT2_SLOTS)
+                cluster_force<DS, 2>(sm, nw, p0, p1, npair, rank, a.eps2f);
+            else
+                cluster_force<DS, 1>(sm, nw, p0, p1, npair, rank, a.eps2f);
+            // C's slots rank + CL_CTAS e: three lanes each, ten a warp, on four warps (one per
+            // FP64 pipe) or eight; their state is on its way during the barrier
+            static_assert(CL_SLOTS / CL_CTAS <= 80, "eight warps of ten");
+            const int ncor = (nw - rank + CL_CTAS - 1) / CL_CTAS;  // may be <= 0
+            const int ncw = ncor > 40 ? 8 : 4;
+            const int cc = lane % 3, ce = ncw * (lane / 3) + warp;
+            const bool mine = warp < ncw && lane < 30 && ce < ncor;
+            CState cs{};
+            int ci = 0;
+            if (mine) {
+                ci = sm.id[rank + CL_CTAS * ce];
+                cstate_load(s, ci, cc, cs);
+            }
+            cluster_barrier();
+            mark(1);
+
+            // C: the partials of the CTAs, then the corrector
+            if (warp < ncw) {
+                double a1 = 0.0, j1 = 0.0;
+                if (mine) {
+                    double tot[3];
+#pragma unroll
+                    for (int u = 0; u < 3; ++u) {  // acc and jerk component, potential
+                        const int c = u < 2 ? 3 * u + cc : 6;
+                        dsf x[CL_CTAS];
+#pragma unroll
+                        for (int r = 0; r < CL_CTAS; ++r)
+                            x[r] = dsf{reinterpret_cast<const float *>(sm.part[r][ce])[c], 0.f};
+#pragma unroll
+                        for (int h = 1; h < CL_CTAS; h <<= 1)
+#pragma unroll
+                            for (int r = 0; r < CL_CTAS; r += 2 * h) ds_acc(x[r], x[r + h]);
+                        tot[u] = ds_to_double(x[0]);
+                    }
+                    a1 = tot[0];
+                    j1 = tot[1];
+                    if (!isfinite(a1) || !isfinite(j1) || !isfinite(tot[2]))
+                        atomicOr(a.err, DERR_NONFINITE);
+                }
+                correct_lanes_pre(s, ci, w0 + rank + CL_CTAS * ce, cc, lane - cc, mine, tn, cs, a1,
+                                  j1, a.prm, a.sd, a.err, a.dtmin_hits);
+            }
+            mark(2);
+            cluster_barrier();
+        }
+        t_cur = tn;
+        if (scribe) {
+            ++steps;
+            inter += (double)na * (double)n;
+            const int lg = min(31, 31 - __clz(na));
+            sm.hist[lg] += 1ull;
+            const unsigned long long t = globaltimer_ns();
+            sm.phase[3] += t - t_mark;
+            t_mark = t;
+            sm.step_ns[lg] += t - t_step;
+            t_step = t;
+        }
+    }
+    cluster_barrier();  // no CTA leaves while another may still read its shared memory
+    if (rank == 0) {
+        if (tid == 0) {
+            a.stats->steps += steps;
+            a.stats->interactions += inter;
+        }
+        if (tid < 32) {
+            a.stats->active_hist[tid] += sm.hist[tid];
+            a.stats->step_ns_hist[tid] += sm.step_ns[tid];
+        }
+        if (tid < 4) a.stats->phase_ns[tid] += sm.phase[tid];
     }
 }
 
@@ -1065,8 +1483,9 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1)
         const int na = s_na;
         if (!(tn <= a.t_end) || na < 1 || na > a.na_max) {
             if (tn <= a.t_end && na >= 1) {
-                ok = handoff_predict_gather<6>(a, tn, p0, p1, nwords, s_flags, s_woff, s_wsum,
-                                               s_total, s_base, gen);
+                ok = handoff_predict_gather<6, NT>(
+                    a, tn, p0, p1, nwords, s_flags, s_woff, s_wsum, s_total, s_base,
+                    [&] { return grid_barrier(a.bar, gen); });
                 mark(0);
                 if (!ok) break;
             }
@@ -1166,6 +1585,30 @@ cudaError_t launch_selftest_barrier(unsigned *bar, unsigned *err, unsigned long 
     return cudaLaunchCooperativeKernel((const void *)k_selftest_barrier, 4, 64, args, 0, st);
 }
 
+static void cluster_steps_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at, cudaStream_t st)
+{
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = CL_CTAS;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(CL_CTAS);
+    cfg.blockDim = dim3(CL_THREADS);
+    cfg.dynamicSmemBytes = sizeof(ClusterSmem);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+}
+
+// Sixteen CTAs are more than a portable cluster.
+template <bool DS>
+static cudaError_t cluster_steps_attr()
+{
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_cluster_steps<DS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClusterSmem));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_cluster_steps<DS>, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                                1);
+}
+
 int fused_grid(int device, int order)
 {
     int coop = 0, sms = 0, per = 0;
@@ -1197,6 +1640,32 @@ size_t fused_part_float2s(int grid, int na_max, int order)
     if (small > need) need = small;
     (void)na_max;
     return need;
+}
+
+bool cluster_steps_ready()
+{
+    const cudaError_t e = [] {
+        cudaError_t r = cluster_steps_attr<true>();
+        return r != cudaSuccess ? r : cluster_steps_attr<false>();
+    }();
+    int clusters = 0;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    cluster_steps_config(cfg, at, nullptr);
+    if (e != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, k_cluster_steps<true>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return clusters >= 1;
+}
+
+cudaError_t launch_cluster_steps(const FusedArgs &a, bool ds, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    cluster_steps_config(cfg, at, st);
+    return cudaLaunchKernelEx(&cfg, ds ? k_cluster_steps<true> : k_cluster_steps<false>, a);
 }
 
 cudaError_t launch_fused_steps(const FusedArgs &a, int grid, bool ds, int order, cudaStream_t st)

@@ -138,3 +138,27 @@ def test_fused_single_steps_both_paths_vs_oracle_and_planned(nb):
             sizes.append(len(due))
     print("due-set sizes", sizes)
     assert sum(k > 16 for k in sizes) >= 3 and sum(k <= 16 for k in sizes) >= 3, sizes
+
+
+@pytest.mark.parametrize("variant", ["f32ds", "f32"])
+@pytest.mark.parametrize("n", [1, 3, 16, 17, 500, 2047, 4096])
+def test_small_system_cluster_matches_separate_launches(nb, n, variant):
+    """Systems of at most 4096 particles are stepped by one cluster of 16 CTAs: CTAs without
+    particles, with one, with an odd or a full range, and (due sets up to 4096) several
+    windows of 1024 due slots. The schedule and states of the separate launches: the
+    states differ by the pair sums' FP32 rounding (1e-6 of a force) over a span of 1/32."""
+    p = ic.plummer(n, 90 + n)
+    kw = dict(variant=variant, eps=0.25 / np.cbrt(n), eta=0.02, dt_max=1.0 / 32, device=0)
+    with nb.System(p.m, p.pos, p.vel, fused_max_na=4096, **kw) as a:
+        sa = a.step(1.0 / 32)
+        ga = a.state()
+    with nb.System(p.m, p.pos, p.vel, flags=nb.NB_FLAG_NO_FUSED, **kw) as b:
+        sb = b.step(1.0 / 32)
+        gb = b.state()
+    assert sb["fused_steps"] == 0 and sa["fused_steps"] == sa["block_steps"] >= 1
+    assert sa["fused_launches"] == 1
+    assert abs(sa["block_steps"] - sb["block_steps"]) <= 0.02 * sb["block_steps"]
+    np.testing.assert_array_equal(ga["t"], gb["t"])
+    assert (ga["dt"] == gb["dt"]).mean() > 0.99 - (1.0 / n if n < 100 else 0.0)
+    for q in ("pos", "vel"):
+        assert np.abs(ga[q] - gb[q]).max() < 1e-6 * max(np.abs(gb[q]).max(), 1e-30)
