@@ -252,6 +252,9 @@ struct Mailbox {
     volatile double t_next;
     volatile int n_active;
     volatile int pad;
+    // the cluster kernel's launch: block steps taken and their interactions
+    volatile long long steps;
+    volatile double interactions;
 };
 
 // Particles per scheduler CTA (256 threads x 8).
@@ -427,6 +430,9 @@ struct FusedArgs {
     unsigned *err;
     unsigned long long *dtmin_hits;
     FusedStats *stats;
+    // cluster kernel only: block steps of one launch (0: no limit); it then publishes the next
+    // block time without handing it off. stats may be null there.
+    int max_steps;
 };
 
 constexpr int FUSED_THREADS = 256;
@@ -442,6 +448,7 @@ constexpr int FUSED6_MAX_NA = NB_FUSED6_MAX_NA;
 // FUSED_CLUSTER CTAs (persist.cu).
 constexpr int FUSED_CLUSTER = 16;
 constexpr int FUSED_CLUSTER_MAX_N = 4096;
+constexpr int FUSED_CLUSTER_LIMIT_N = 8192;  // the most the kernel takes (request loop)
 
 // Ints of the fused kernel's counter array: grid per-CTA counts, 2 due-set
 // counters, the tickets of the small-set groups (at most FUSED6_MAX_NA / 4; padded).

@@ -29,6 +29,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <atomic>
+
 #include "ds.cuh"
 #include "nb_internal.cuh"
 #include "pair.cuh"
@@ -829,25 +831,26 @@ __global__ void __launch_bounds__(FUSED_THREADS)
 // 4096 particles leaves little: the line of the dispatch.
 constexpr int CL_CTAS = FUSED_CLUSTER;
 constexpr int CL_THREADS = 512;
-constexpr int CL_MAX_L = FUSED_CLUSTER_MAX_N / CL_CTAS;  // particles per CTA
 constexpr int CL_SLOTS = 1024;                           // due slots per window
 constexpr int CL_Q = 7;                                  // outputs of a slot
 // Two slots per lane from here on (half the shared-memory reads; below, one slot keeps more
 // lanes busy).
 constexpr int CL_IPT2_SLOTS = 64;
 
+// MAXL: the most particles of a CTA.
+template <int MAXL>
 struct ClusterSmem {
-    float4 pair[6][CL_MAX_L / 2];              // float4 u of pair q: pair[u][q]
+    float4 pair[6][MAXL / 2];              // float4 u of pair q: pair[u][q]
     float4 part[CL_CTAS][CL_SLOTS / CL_CTAS][2];  // sums by source CTA, slot / CL_CTAS
-    float4 own[CL_MAX_L][3];                   // own due records: {x_hi, x_lo, v, -} of component c
+    float4 own[MAXL][3];                   // own due records: {x_hi, x_lo, v, -} of component c
     float i[9][CL_SLOTS];                      // due records: x_hi, x_lo, v of three components
     int id[CL_SLOTS];
-    uint4 due[CL_CTAS][CL_MAX_L / 128];        // a bit for every particle of every CTA
+    uint4 due[CL_CTAS][MAXL / 128];        // a bit for every particle of every CTA
     double tn;
     int na;
     unsigned long long hist[32], step_ns[32], phase[4];
-    unsigned flags[CL_MAX_L / 32];
-    int woff[CL_MAX_L / 32], wsum[CL_THREADS / 32], total, base;
+    unsigned flags[MAXL / 32];
+    int woff[MAXL / 32], wsum[CL_THREADS / 32], total, base;
 };
 
 __device__ __forceinline__ void cluster_barrier()
@@ -889,7 +892,8 @@ __device__ __forceinline__ void cluster_st(uint32_t a, float4 v)
 }
 
 // The float of record value u (0-2 x_hi, 3-5 x_lo, 6-8 v; 9 the mass) of own particle l.
-__device__ __forceinline__ float *cl_value(ClusterSmem &sm, int u, int l)
+template <int MAXL>
+__device__ __forceinline__ float *cl_value(ClusterSmem<MAXL> &sm, int u, int l)
 {
     const int c = u % 3;
     const int quad = u == 9 ? 1 : 2 * (u / 3) + (c == 2 ? 1 : 0);  // {x y} {z m} of each triple
@@ -908,7 +912,8 @@ __device__ __forceinline__ int cluster_lanes_log2(int ngroups, int npair)
     return (int)(__reduce_min_sync(0xffffffffu, (unsigned)(cost << 3 | lg)) & 7u);
 }
 
-__device__ __forceinline__ JPair cluster_pair(const ClusterSmem &sm, int q)
+template <int MAXL>
+__device__ __forceinline__ JPair cluster_pair(const ClusterSmem<MAXL> &sm, int q)
 {
     return JPair{sm.pair[0][q], sm.pair[1][q], sm.pair[2][q],
                  sm.pair[3][q], sm.pair[4][q], sm.pair[5][q]};
@@ -916,8 +921,8 @@ __device__ __forceinline__ JPair cluster_pair(const ClusterSmem &sm, int q)
 
 // The pair terms of the CTA's particles [p0, p1) on IPT due ones (indices own): this lane's
 // share, pairs sub, sub + S, ... masked: one of the warp's due ones may be among them.
-template <bool DS, bool SOFT, int IPT>
-__device__ __forceinline__ void cluster_pairs(const ClusterSmem &sm, int sub, int S, int p0,
+template <bool DS, bool SOFT, int IPT, int MAXL>
+__device__ __forceinline__ void cluster_pairs(const ClusterSmem<MAXL> &sm, int sub, int S, int p0,
                                               int p1, bool masked, const IPair (&ip)[IPT],
                                               const int (&own)[IPT], float2 e2,
                                               PairSum (&ts)[IPT])
@@ -949,8 +954,8 @@ __device__ __forceinline__ void cluster_pairs(const ClusterSmem &sm, int sub, in
 
 // B for one window of nw due slots: the sums of every slot over the CTA's particles
 // [p0, p1), left in CTA slot % CL_CTAS. Groups of IPT slots (k, k + ngroups), S lanes each.
-template <bool DS, int IPT>
-__device__ __forceinline__ void cluster_force(ClusterSmem &sm, int nw, int p0, int p1, int npair,
+template <bool DS, int IPT, int MAXL>
+__device__ __forceinline__ void cluster_force(ClusterSmem<MAXL> &sm, int nw, int p0, int p1, int npair,
                                               int rank, float eps2f)
 {
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -997,13 +1002,15 @@ __device__ __forceinline__ void cluster_force(ClusterSmem &sm, int nw, int p0, i
     }
 }
 
-template <bool DS>
+template <bool DS, int MAXL>
 __global__ void __launch_bounds__(CL_THREADS)
     k_cluster_steps(FusedArgs a)
 {
     extern __shared__ __align__(128) unsigned char s_cluster[];
-    ClusterSmem &sm = *reinterpret_cast<ClusterSmem *>(s_cluster);
+    ClusterSmem<MAXL> &sm = *reinterpret_cast<ClusterSmem<MAXL> *>(s_cluster);
     constexpr int NT = CL_THREADS, NW = NT / 32;
+    constexpr int ROUNDS = (3 * MAXL + NT - 1) / NT;  // (component, particle) per thread
+    static_assert(MAXL <= NT && MAXL % 256 == 0, "the due bits of a CTA come in one round");
     static_assert(NW == CL_CTAS, "warp w copies the due records of CTA w");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = blockIdx.x;  // one cluster: the rank in it
@@ -1015,7 +1022,7 @@ __global__ void __launch_bounds__(CL_THREADS)
     const int npair = (per + 1) / 2;
     double t_cur = __ldcg(&a.sd->t_cur);
     const unsigned long long epoch = __ldcg(&a.sd->seq);
-    unsigned long long steps = 0;
+    int steps = 0;
     double inter = 0.0;
     const bool scribe = rank == 0 && tid == 0;  // stage times
     unsigned long long t_mark = globaltimer_ns(), t_step = t_mark;
@@ -1028,8 +1035,8 @@ __global__ void __launch_bounds__(CL_THREADS)
     };
     if (tid < 32) sm.hist[tid] = sm.step_ns[tid] = 0ull;
     if (tid < 4) sm.phase[tid] = 0ull;
-    if (tid < CL_CTAS * (CL_MAX_L / 128)) (&sm.due[0][0])[tid] = make_uint4(0u, 0u, 0u, 0u);
-    for (int u = tid; u < 6 * (CL_MAX_L / 2); u += NT)
+    if (tid < CL_CTAS * (MAXL / 128)) (&sm.due[0][0])[tid] = make_uint4(0u, 0u, 0u, 0u);
+    for (int u = tid; u < 6 * (MAXL / 2); u += NT)
         (&sm.pair[0][0])[u] = make_float4(0.f, 0.f, 0.f, 0.f);
     cluster_barrier();  // every CTA runs before another writes to its shared memory
     if (tid < L) *cl_value(sm, 9, tid) = f32_trunc(s.m[p0 + tid]);
@@ -1038,7 +1045,7 @@ __global__ void __launch_bounds__(CL_THREADS)
         // the thread's first component, loaded while warp 0 finds the block time
         struct Comp {
             double x, v, a, j, t, dt;
-        } st[2];
+        } st[ROUNDS];
         auto load = [&](int it, Comp &q) {
             const int c = it / Lw, l = it - c * Lw;
             if (c < 3 && l < L) {
@@ -1052,16 +1059,17 @@ __global__ void __launch_bounds__(CL_THREADS)
             }
         };
         if (Lw > 0) {
-            load(tid, st[0]);
-            load(tid + NT, st[1]);
+#pragma unroll
+            for (int h = 0; h < ROUNDS; ++h) load(tid + h * NT, st[h]);
         }
         if (warp == 0) next_block_time(a, t_cur, sm.tn, sm.na);
         __syncthreads();
         const double tn = sm.tn;
         const int na = sm.na;
-        if (!(tn <= a.t_end) || na < 1 || na > a.na_max) {
+        const bool limit = a.max_steps > 0 && steps >= a.max_steps;
+        if (!(tn <= a.t_end) || na < 1 || na > a.na_max || limit) {
             // hand the step to the caller exactly as the scheduler kernel would
-            if (tn <= a.t_end && na >= 1) {
+            if (tn <= a.t_end && na >= 1 && !limit) {
                 handoff_predict_gather<4, NT>(
                     a, tn, p0, p1, (L + 31) / 32, sm.flags, sm.woff, sm.wsum, sm.total, sm.base, [] {
                         cluster_barrier();
@@ -1069,14 +1077,18 @@ __global__ void __launch_bounds__(CL_THREADS)
                     });
                 mark(0);
             }
-            if (scribe) publish(a, t_cur, tn, na, epoch);
+            if (scribe) {
+                a.mail->steps = steps;
+                a.mail->interactions = inter;
+                publish(a, t_cur, tn, na, epoch);
+            }
             break;
         }
 
         // A: predict, in the predictor's arithmetic; warps hold one component each
         if (Lw > 0) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < ROUNDS; ++h) {
                 const int it = tid + h * NT;
                 const int c = it / Lw, l = it - c * Lw;
                 bool due = false;
@@ -1106,10 +1118,13 @@ __global__ void __launch_bounds__(CL_THREADS)
         }
         cluster_barrier();
         mark(0);
-        // lane l: the due counts of 128 particles of CTA l / 2
-        static_assert(CL_MAX_L == 256, "two 128-bit words of due bits per CTA");
-        const uint4 bits = sm.due[lane >> 1][lane & 1];
-        const int mycnt = __popc(bits.x) + __popc(bits.y) + __popc(bits.z) + __popc(bits.w);
+        // lane l: the due count of half the particles of CTA l / 2
+        int mycnt = 0;
+#pragma unroll
+        for (int u = 0; u < MAXL / 256; ++u) {
+            const uint4 bits = sm.due[lane >> 1][(lane & 1) * (MAXL / 256) + u];
+            mycnt += __popc(bits.x) + __popc(bits.y) + __popc(bits.z) + __popc(bits.w);
+        }
         if ((int)__reduce_add_sync(0xffffffffu, (unsigned)mycnt) != na) {
             if (scribe) atomicOr(a.err, DERR_SCHED);  // the histogram and the states disagree
             break;
@@ -1121,7 +1136,7 @@ __global__ void __launch_bounds__(CL_THREADS)
         for (int w0 = 0; w0 < na; w0 += CL_SLOTS) {  // windows of due slots
             const int nw = min(CL_SLOTS, na - w0);
             int k = first - w0;
-            for (int u = 0; u < CL_MAX_L / 32; ++u) {
+            for (int u = 0; u < MAXL / 32; ++u) {
                 const unsigned word = reinterpret_cast<const unsigned *>(sm.due[warp])[u];
                 const int mk = k + __popc(word & ((1u << lane) - 1u)), l = 32 * u + lane;
                 k += __popc(word);
@@ -1192,8 +1207,8 @@ __global__ void __launch_bounds__(CL_THREADS)
             cluster_barrier();
         }
         t_cur = tn;
+        ++steps;
         if (scribe) {
-            ++steps;
             inter += (double)na * (double)n;
             const int lg = min(31, 31 - __clz(na));
             sm.hist[lg] += 1ull;
@@ -1205,9 +1220,9 @@ __global__ void __launch_bounds__(CL_THREADS)
         }
     }
     cluster_barrier();  // no CTA leaves while another may still read its shared memory
-    if (rank == 0) {
+    if (rank == 0 && a.stats) {
         if (tid == 0) {
-            a.stats->steps += steps;
+            a.stats->steps += (unsigned long long)steps;
             a.stats->interactions += inter;
         }
         if (tid < 32) {
@@ -1585,6 +1600,7 @@ cudaError_t launch_selftest_barrier(unsigned *bar, unsigned *err, unsigned long 
     return cudaLaunchCooperativeKernel((const void *)k_selftest_barrier, 4, 64, args, 0, st);
 }
 
+template <int MAXL>
 static void cluster_steps_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at, cudaStream_t st)
 {
     at.id = cudaLaunchAttributeClusterDimension;
@@ -1592,21 +1608,39 @@ static void cluster_steps_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &a
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.gridDim = dim3(CL_CTAS);
     cfg.blockDim = dim3(CL_THREADS);
-    cfg.dynamicSmemBytes = sizeof(ClusterSmem);
+    cfg.dynamicSmemBytes = sizeof(ClusterSmem<MAXL>);
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
 }
 
 // Sixteen CTAs are more than a portable cluster.
-template <bool DS>
-static cudaError_t cluster_steps_attr()
+template <bool DS, int MAXL>
+static bool cluster_kernel_ready()
 {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_cluster_steps<DS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClusterSmem));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_cluster_steps<DS>, cudaFuncAttributeNonPortableClusterSizeAllowed,
-                                1);
+    constexpr auto kern = k_cluster_steps<DS, MAXL>;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    cluster_steps_config<MAXL>(cfg, at, nullptr);
+    int clusters = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)cfg.dynamicSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return clusters >= 1;
+}
+
+template <bool DS, int MAXL>
+static cudaError_t go_cluster_steps(const FusedArgs &a, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    cluster_steps_config<MAXL>(cfg, at, st);
+    return cudaLaunchKernelEx(&cfg, k_cluster_steps<DS, MAXL>, a);
 }
 
 int fused_grid(int device, int order)
@@ -1642,30 +1676,36 @@ size_t fused_part_float2s(int grid, int na_max, int order)
     return need;
 }
 
+constexpr int CL_SMALL_L = FUSED_CLUSTER_MAX_N / CL_CTAS;
+constexpr int CL_LARGE_L = FUSED_CLUSTER_LIMIT_N / CL_CTAS;
+
 bool cluster_steps_ready()
 {
-    const cudaError_t e = [] {
-        cudaError_t r = cluster_steps_attr<true>();
-        return r != cudaSuccess ? r : cluster_steps_attr<false>();
-    }();
-    int clusters = 0;
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    cluster_steps_config(cfg, at, nullptr);
-    if (e != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&clusters, k_cluster_steps<true>, &cfg) != cudaSuccess) {
+    // asked once on each device: what it is asked for does not change
+    static std::atomic<unsigned long long> known{0}, ready{0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return clusters >= 1;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (known.load() & bit) return (ready.load() & bit) != 0;
+    const bool ok =
+        cluster_kernel_ready<true, CL_SMALL_L>() && cluster_kernel_ready<false, CL_SMALL_L>() &&
+        cluster_kernel_ready<true, CL_LARGE_L>() && cluster_kernel_ready<false, CL_LARGE_L>();
+    if (ok) ready |= bit;
+    known |= bit;
+    return ok;
 }
 
 cudaError_t launch_cluster_steps(const FusedArgs &a, bool ds, cudaStream_t st)
 {
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    cluster_steps_config(cfg, at, st);
-    return cudaLaunchKernelEx(&cfg, ds ? k_cluster_steps<true> : k_cluster_steps<false>, a);
+    if (a.s.n > CL_CTAS * CL_LARGE_L) return cudaErrorInvalidValue;
+    if (a.s.n > CL_CTAS * CL_SMALL_L)
+        return ds ? go_cluster_steps<true, CL_LARGE_L>(a, st)
+                  : go_cluster_steps<false, CL_LARGE_L>(a, st);
+    return ds ? go_cluster_steps<true, CL_SMALL_L>(a, st)
+              : go_cluster_steps<false, CL_SMALL_L>(a, st);
 }
 
 cudaError_t launch_fused_steps(const FusedArgs &a, int grid, bool ds, int order, cudaStream_t st)

@@ -213,3 +213,30 @@ def test_sixty_four_stream_requests_alone_equal_mix(nb):
         for k in keys:
             np.testing.assert_array_equal(a[k], b[k])
         assert a["interactions"] == b["interactions"]
+
+
+@pytest.mark.parametrize("n", [5, 4097, 8192, 8193])
+def test_integrations_around_the_cluster_sizes_match_the_engine(nb, n):
+    """Integrations of up to 8192 particles run in cluster launches of at most 128 block steps
+    beside the ticks, larger ones in the ticks: the state nb_step gives (the pair sums differ
+    by their FP32 rounding, 1e-6 of a force, over a span of 1/32), and alone the same bits
+    as beside a force request and another integration."""
+    m, pos, vel = _req(n, 800 + n)
+    eps, span = 0.25 / np.cbrt(n), 1.0 / 32
+    with nb.Server(variant=nb.NB_F32DS, eta=0.01, dt_max=1.0 / 64, device=0) as srv:
+        alone = srv.wait(srv.evolve(m, pos, vel, eps=eps, t_span=span), timeout_s=60)
+        other = _req(900, 801)
+        tickets = [srv.evolve(m, pos, vel, eps=eps, t_span=span), srv.force(*other, eps=0.01),
+                   srv.evolve(*other, eps=0.01, t_span=span)]
+        mix = [srv.wait(t, timeout_s=60) for t in tickets][0]
+    assert alone["status"] == mix["status"] == nb.NB_STATUS_DONE
+    assert alone["block_steps"] == mix["block_steps"] > 0
+    assert alone["interactions"] == mix["interactions"]
+    with nb.System(m, pos.T, vel.T, variant="f32ds", eps=eps, eta=0.01, dt_max=1.0 / 64,
+                   device=0) as s:
+        st = s.step(span)
+        g = s.state()
+    assert abs(alone["block_steps"] - st["block_steps"]) <= 0.02 * st["block_steps"]
+    for q in ("pos", "vel"):
+        np.testing.assert_array_equal(alone[q], mix[q])
+        assert np.abs(alone[q] - g[q]).max() < 1e-6 * np.abs(g[q]).max()
