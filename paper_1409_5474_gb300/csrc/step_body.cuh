@@ -64,6 +64,14 @@ __device__ __forceinline__ int exponent_of(double x)
     return ((__double2hiint(x) >> 20) & 0x7ff) - 1023;
 }
 
+// Whether a particle whose own time is d before the block time is due there: d == dt. The
+// times of block steps are multiples of the steps, powers of two, so d is exact and the
+// comparison needs no FP64 instruction.
+__device__ __forceinline__ bool same_bits(double d, double dt)
+{
+    return __double_as_longlong(d) == __double_as_longlong(dt);
+}
+
 // 2^-floor(log2 |x|).
 __device__ __forceinline__ double inv_pow2_of(double x)
 {
@@ -166,7 +174,7 @@ __device__ __forceinline__ bool predict_rec_from(const StateDev &s, const PState
     rr[0] = rec[0];
     rr[1] = rec[1];
     rr[2] = rec[2];
-    return q.t + q.dt == tn;
+    return same_bits(d, q.dt);
 }
 
 // The 6th-order prediction of particle i to time tn (FP64 Taylor series through
@@ -252,7 +260,7 @@ __device__ __forceinline__ bool predict6_rec_from(const StateDev &s, const PStat
     rr[1] = r[1];
     rr[2] = r[2];
     rr[3] = make_float4(f32_trunc(ap[0]), f32_trunc(ap[1]), f32_trunc(ap[2]), 0.f);
-    return q.t + q.dt == tn;
+    return same_bits(d, q.dt);
 }
 
 // ---- step criterion and block quantization ---------------------------------
