@@ -430,8 +430,8 @@ struct FusedArgs {
     unsigned *err;
     unsigned long long *dtmin_hits;
     FusedStats *stats;
-    // cluster kernel only: block steps of one launch (0: no limit); it then publishes the next
-    // block time without handing it off. stats may be null there.
+    // cluster kernel only: block steps of one launch (0: no limit); at the limit it publishes the
+    // next block time with N_active = 0, nothing handed off. stats may be null there.
     int max_steps;
 };
 

@@ -1096,7 +1096,7 @@ __global__ void __launch_bounds__(CL_THREADS)
             if (scribe) {
                 a.mail->steps = steps;
                 a.mail->interactions = inter;
-                publish(a, t_cur, tn, na, epoch);
+                publish(a, t_cur, tn, limit ? 0 : na, epoch);
             }
             break;
         }

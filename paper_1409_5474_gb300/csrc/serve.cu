@@ -25,7 +25,7 @@
 // steps a launch, on a stream beside the ticks, and a tick only looks whether it has
 // ended. A block step in the ticks costs a round trip to the host and six launches, 25 us for a
 // few due particles, and every step of the longest integration waits for it; in a cluster
-// 9 to 14 us. 16 requests of 256-16384, half of them integrations: 24.8 -> 15.8 ms.
+// 9 to 14 us. 16 requests of 256-16384, half of them integrations: 24.8 -> 8.7 ms.
 // A request's items, splits and summation order depend only on the request
 // itself (and the SM count), so its results are the same whatever else is in
 // flight.
@@ -92,6 +92,11 @@ constexpr int NSIDE = 4;  // side streams of the engine-planned force launches
 // a cancelled request is dropped and a waiting one gets its turn.
 constexpr int NCLUSTER = 8;
 constexpr int CLUSTER_STEPS = 128;
+// Due sets of more interactions than this are handed to the ticks (one step; the cluster goes
+// on after it): sixteen SMs do about 60 interactions a nanosecond, all of them 700 and more,
+// and a step in the ticks costs some 50 us besides. The burst of 16 requests takes 12.3 ms with
+// the line at 1.2e6, 8.6 to 8.8 from 4e6 to 8e6, 10.6 at 12e6, 15.6 without one.
+constexpr double CLUSTER_MAX_INTERACTIONS = 6e6;
 
 int capacity_class(int n)
 {
@@ -114,6 +119,7 @@ struct nb_server_s {
     cudaStream_t cstream[NCLUSTER] = {};
     cudaEvent_t ev_init = nullptr;
     std::vector<cudaEvent_t> ev_cluster;       // end of the cluster launch, by slot
+    int *d_cnt = nullptr;                      // due counts of a hand-off, by slot
     std::chrono::steady_clock::time_point t0;
 
     std::mutex mu;
@@ -537,11 +543,12 @@ int tick(nb_server s)
                 r->final_copy = true;
                 continue;
             }
-            if (r->cluster) {
-                if (r->bits)
-                    r->pending = err_code(r->bits);
-                else
-                    cluster_go.push_back(r.get());
+            if (r->cluster && r->bits) {
+                r->pending = err_code(r->bits);
+                continue;
+            }
+            if (r->cluster && na == 0) {  // CLUSTER_STEPS taken
+                cluster_go.push_back(r.get());
                 continue;
             }
             if (na < 1 || na > r->n) {
@@ -564,7 +571,7 @@ int tick(nb_server s)
             c_blocks += (na + CORRECT_THREADS - 1) / CORRECT_THREADS;
             r->tick_steps++;
         }
-        if (r->phase == PH_INIT && r->cluster) {
+        if (r->cluster && (r->phase == PH_INIT || r->phase == PH_STEP)) {
             cluster_go.push_back(r.get());
         } else if (r->phase == PH_INIT || r->phase == PH_STEP) {
             // the integration goes on: its next scheduler launch
@@ -705,7 +712,8 @@ int tick(nb_server s)
         a.mail = v.mail_d;
         a.prm = prm;
         a.eps2f = (float)(r->eps * r->eps);
-        a.na_max = r->n;  // every due set: nothing is handed off
+        a.na_max = (int)std::min((double)r->n, CLUSTER_MAX_INTERACTIONS / r->n);
+        a.cnt = s->d_cnt + (size_t)r->slot * FUSED_CLUSTER;
         a.t_end = r->t_end;
         a.err = s->d_errs + r->slot;
         a.dtmin_hits = s->d_dtmin;
@@ -917,6 +925,8 @@ int nb_server_create(const nb_server_cfg *cfg, nb_server *out)
         cudaMalloc(&s->d_dtmin, sizeof(unsigned long long)) != cudaSuccess ||
         cudaMemset(s->d_errs, 0, c.max_inflight * sizeof(unsigned)) != cudaSuccess ||
         cudaMemset(s->d_dtmin, 0, sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMalloc(&s->d_cnt, (size_t)c.max_inflight * FUSED_CLUSTER * sizeof(int)) !=
+            cudaSuccess ||
         cudaMalloc(&s->d_ticket, 2 * sizeof(unsigned)) != cudaSuccess ||
         cudaMemset(s->d_ticket, 0, 2 * sizeof(unsigned)) != cudaSuccess) {
         cudaGetLastError();
@@ -929,6 +939,7 @@ int nb_server_create(const nb_server_cfg *cfg, nb_server *out)
         if (s->h_errs) cudaFreeHost(s->h_errs);
         if (s->d_dtmin) cudaFree(s->d_dtmin);
         if (s->d_ticket) cudaFree(s->d_ticket);
+        if (s->d_cnt) cudaFree(s->d_cnt);
         return NB_ERR_CUDA;
     }
     s->threads = 128;
@@ -962,6 +973,7 @@ int nb_server_destroy(nb_server s)
     cudaFreeHost(s->h_errs);
     cudaFree(s->d_dtmin);
     cudaFree(s->d_ticket);
+    cudaFree(s->d_cnt);
     cudaStreamDestroy(s->stream);
     cudaStreamDestroy(s->stream2);
     cudaEventDestroy(s->ev_fork);
