@@ -72,7 +72,6 @@ __device__ __forceinline__ void write_final(const Out3 &out, int k, double v[7],
     if (out.pot) out.pot[k] = v[6];
 }
 
-// Member index of slot k; an index outside the j-set is flagged and replaced by 0.
 // Store the reduced value s of component c of slot k (c == 6: the positive
 // potential sum, stored negated).
 __device__ __forceinline__ void store_component(const Out3 &out, int c, int k, double s,
@@ -89,8 +88,8 @@ __device__ __forceinline__ void store_component(const Out3 &out, int c, int k, d
     if (!isfinite(s)) atomicOr(err, DERR_NONFINITE);
 }
 
-// K3, folded into the force kernels: after a CTA has written its partial sums
-// for slots [slot0, slot0 + nslots), the last of the nsplit CTAs that share
+// K3, folded into the warp-group and the allocation-free FP64 kernels: after a CTA has
+// written its partial sums for slots [slot0, slot0 + nslots), the last of the nsplit CTAs that share
 // these slots (counted in *counter) reduces them and re-arms the counter. One
 // warp per (slot, component): lane l adds splits l, l + 32, ... in order, then a
 // fixed xor tree, so the result does not depend on which CTA finished last.
@@ -189,6 +188,7 @@ __device__ __forceinline__ int i_id(const ISet &is, int row, float id_bits)
     return is.member ? row : -1;
 }
 
+// Member index of slot k; an index outside the j-set is flagged and replaced by 0.
 __device__ __forceinline__ int member_index(const ISet &is, int k, unsigned *err)
 {
     const int r = is.idx ? __ldg(is.idx + k) : k;
@@ -225,8 +225,7 @@ __host__ __device__ constexpr bool tile_ahead(int nwj) { return nwj == 8; }
 template <int VAR, int IPT, int NWI, int NWJ, int JT, int NS>
 __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     k_force_tile32(const float4 *__restrict__ jrec, int nj, ISet is, float eps2f, int ntiles,
-                   double *__restrict__ part, long long pld, unsigned *counters, Out3 out,
-                   unsigned *err)
+                   double *__restrict__ part, long long pld, Out3 out, unsigned *err)
 {
     // NS ring stages of JT records (bulk-copy destinations), one or (AHEAD) two tiles as
     // j-pairs (JT / 2 pairs x 6 float4 each), the running totals
@@ -411,7 +410,6 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
         }
     }
     // with nsplit > 1 the partials are summed by k_split_sums, launched next
-    (void)counters;
 }
 
 // K3 of the tile, tiny-set and FP64 kernels (split_sum): output q = component c of slot k.
@@ -1522,7 +1520,7 @@ static constexpr size_t tile_smem()
 
 template <int VAR, int IPT, int NWI, int NWJ>
 static cudaError_t go_tile32(const JSet &js, const ISet &is, float eps2f, int nsplit,
-                             double *part, unsigned *cnt, Out3 out, unsigned *err,
+                             double *part, Out3 out, unsigned *err,
                              cudaStream_t st)
 {
     constexpr auto kern = k_force_tile32<VAR, IPT, NWI, NWJ, JT_TILE, NS32>;
@@ -1534,7 +1532,7 @@ static cudaError_t go_tile32(const JSet &js, const ISet &is, float eps2f, int ns
     const int ntiles = (js.n + JT_TILE - 1) / JT_TILE;
     dim3 grid((is.n + IB - 1) / IB, nsplit);
     const cudaError_t e = launch_dependent(kern, grid, NT, smem, st, js.rec32, js.n, is, eps2f,
-                                           ntiles, part, (long long)is.n, cnt, out, err);
+                                           ntiles, part, (long long)is.n, out, err);
     if (e != cudaSuccess || nsplit <= 1) return e;
     return go_split_sums<float2>(part, is.n, nsplit, out, err, st);
 }
@@ -1607,12 +1605,12 @@ static cudaError_t dispatch32(const ForcePlan &p, const JSet &js, const ISet &is
         }
     }
     switch (p.nwj) {
-    case 1: return go_tile32<VAR, 2, 8, 1>(js, is, eps2f, p.nsplit, part, cnt, out, err, st);
-    case 4: return go_tile32<VAR, 2, 2, 4>(js, is, eps2f, p.nsplit, part, cnt, out, err, st);
+    case 1: return go_tile32<VAR, 2, 8, 1>(js, is, eps2f, p.nsplit, part, out, err, st);
+    case 4: return go_tile32<VAR, 2, 2, 4>(js, is, eps2f, p.nsplit, part, out, err, st);
     default:
         if (p.ipt == 1)
-            return go_tile32<VAR, 1, 1, 8>(js, is, eps2f, p.nsplit, part, cnt, out, err, st);
-        return go_tile32<VAR, 2, 1, 8>(js, is, eps2f, p.nsplit, part, cnt, out, err, st);
+            return go_tile32<VAR, 1, 1, 8>(js, is, eps2f, p.nsplit, part, out, err, st);
+        return go_tile32<VAR, 2, 1, 8>(js, is, eps2f, p.nsplit, part, out, err, st);
     }
 }
 
