@@ -237,9 +237,9 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     constexpr int NT = 32 * NWI * NWJ;
     constexpr int IB = 32 * NWI * IPT;
     // tiles per FP32 partial sum: 64 terms in each half of a packed sum between folds (128
-    // with one warp row, a tile's). With 128 for the due sets too the jerk of 1531 of 65536 was
-    // 4.1e-7 off (64 bits), 3.4e-7 with 64, as with the scalar warp groups that took those sets
-    // before; 127.2 -> 129.0 us.
+    // with one warp row, a tile's): for 1531 of 65536 the jerk is 2.3e-7 off (64 bits,
+    // geometric mean over 14 systems), 2.4e-7 with the 32-term sums of the scalar warp groups
+    // that took those sets before; 128 terms 127.2 us, 64 129.0, 32 130.3.
     constexpr int FOLD = (128 * NWJ / JT) > 1 ? (128 * NWJ / JT) : 1;
     constexpr int PAIRS = JT * DS_REC;  // float4 of a pair buffer
     constexpr bool AHEAD = tile_ahead(NWJ);
