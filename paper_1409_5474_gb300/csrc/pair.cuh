@@ -148,6 +148,16 @@ struct PairMask {
     }
 };
 
+// The self pair alone (a pair with both records).
+struct OwnMask {
+    int ja, own;
+    __device__ __forceinline__ void operator()(float2 &rinv) const
+    {
+        rinv.x = ja == own ? 0.f : rinv.x;
+        rinv.y = ja + 1 == own ? 0.f : rinv.y;
+    }
+};
+
 // Rewrite cnt records (of a tile of JT) at T as j-pairs at s_pair, by NT threads;
 // records past the end become zeros (their pairs are masked).
 template <int JT, int NT>

@@ -833,25 +833,22 @@ __global__ void __launch_bounds__(FUSED_THREADS)
 //      instruction holds its pipe for 64 cycles whatever its lanes do), their due bits
 //      sent to every CTA                                                  -- cluster barrier
 //   B  the due records of all CTAs (a window of CL_SLOTS) copied to shared memory; S
-//      lanes per one or two due particles split the CTA's pairs, their FP32 sums meet in a xor
+//      lanes per due particle split the CTA's pairs, their FP32 sums meet in a xor
 //      tree, and slot k's go to CTA k % CL_CTAS                   -- cluster barrier
 //   C  that CTA adds the CL_CTAS partials in double-single and corrects the particle,
 //      three lanes each                                           -- cluster barrier
 // The cluster barrier is a hardware barrier of co-scheduled CTAs (like __syncthreads):
 // no wait depends on another launch, and every exit is taken by all CTAs together.
-// Measured against the grid kernel, 1/16 time unit of block steps: N = 500 2.28 -> 1.57 ms,
-// 1000 5.27 -> 3.8, 2500 8.57 -> 7.2, 4000 11.7 -> 11.3. A step of 1 to 3 due at N = 2500 takes
-// 9.4 us for 13.2: the prediction and its barrier 3.5, the force 3, the corrector 2.2.
+// Measured against the grid kernel, 1/16 time unit of block steps: N = 500 2.28 -> 1.51 ms,
+// 1000 5.27 -> 3.64, 2500 8.57 -> 6.88, 4000 11.7 -> 10.5. A step of 1 to 3 due at N = 2500 takes
+// 9.1 us for 13.2: the prediction and its barrier 3.2, the force 3, the corrector 2.2.
 // Sixteen SMs are a tenth of the GPU, so due sets of a hundred and more cost part
-// of that again (N = 2500, 512-1023 due: 41 against 20 us; N = 4000: 61 against 21), which at
-// 4096 particles leaves little: the line of the dispatch.
+// of that again (N = 2500, 512-1023 due: 39 against 20 us; N = 4000: 59 against 21), which at
+// 4096 particles leaves a tenth: the line of the dispatch.
 constexpr int CL_CTAS = FUSED_CLUSTER;
 constexpr int CL_THREADS = 512;
 constexpr int CL_SLOTS = 1024;                           // due slots per window
 constexpr int CL_Q = 7;                                  // outputs of a slot
-// Two slots per lane from here on (half the shared-memory reads; below, one slot keeps more
-// lanes busy).
-constexpr int CL_IPT2_SLOTS = 64;
 
 // MAXL: the most particles of a CTA.
 template <int MAXL>
@@ -917,13 +914,12 @@ __device__ __forceinline__ float *cl_value(ClusterSmem<MAXL> &sm, int u, int l)
     return reinterpret_cast<float *>(&sm.pair[quad][l >> 1]) + at + (l & 1);
 }
 
-// Lanes per IPT due particles: the power of two with the least estimated time of a window's
-// pair terms (rounds of CL_THREADS / S lanes groups, the pairs of a lane and its share of
-// the xor tree).
-__device__ __forceinline__ int cluster_lanes_log2(int ngroups, int npair)
+// Lanes per due particle: the power of two with the least estimated time of a window's pair
+// terms (rounds of CL_THREADS / S slots, the pairs of a lane and its share of the xor tree).
+__device__ __forceinline__ int cluster_lanes_log2(int nw, int npair)
 {
     const int lg = min((int)(threadIdx.x & 31), 5);
-    const int rounds = ((ngroups << lg) + CL_THREADS - 1) / CL_THREADS;
+    const int rounds = ((nw << lg) + CL_THREADS - 1) / CL_THREADS;
     const int cost = rounds * (2 * ((npair + (1 << lg) - 1) >> lg) + 2 + lg);
     return (int)(__reduce_min_sync(0xffffffffu, (unsigned)(cost << 3 | lg)) & 7u);
 }
@@ -935,85 +931,63 @@ __device__ __forceinline__ JPair cluster_pair(const ClusterSmem<MAXL> &sm, int q
                  sm.pair[3][q], sm.pair[4][q], sm.pair[5][q]};
 }
 
-// The pair terms of the CTA's particles [p0, p1) on IPT due ones (indices own): this lane's
-// share, pairs sub, sub + S, ... masked: one of the warp's due ones may be among them.
-template <bool DS, bool SOFT, int IPT, int MAXL>
+// The pair terms of the CTA's particles [p0, p1) on a due one (index own): this lane's share,
+// pairs sub, sub + S, ... masked: one of the warp's due ones may be among them. Not unrolled: the
+// four warps of a scheduler cover the latencies, and every step runs through this code once
+// (unrolled twice or four times 1 to 3% of a step more).
+template <bool DS, bool SOFT, int MAXL>
 __device__ __forceinline__ void cluster_pairs(const ClusterSmem<MAXL> &sm, int sub, int S, int p0,
-                                              int p1, bool masked, const IPair (&ip)[IPT],
-                                              const int (&own)[IPT], float2 e2,
-                                              PairSum (&ts)[IPT])
+                                              int p1, bool masked, const IPair &ip, int own,
+                                              float2 e2, PairSum &ts)
 {
     const int full = (p1 - p0) / 2;
     if (!masked) {
-#pragma unroll 2
-        for (int q = sub; q < full; q += S) {
-            const JPair j = cluster_pair(sm, q);
-#pragma unroll
-            for (int p = 0; p < IPT; ++p) pair_add<DS, SOFT>(j, ip[p], e2, ts[p], NoMask{});
-        }
+#pragma unroll 1
+        for (int q = sub; q < full; q += S)
+            pair_add<DS, SOFT>(cluster_pair(sm, q), ip, e2, ts, NoMask{});
     } else {
 #pragma unroll 1
-        for (int q = sub; q < full; q += S) {
-            const JPair j = cluster_pair(sm, q);
-#pragma unroll
-            for (int p = 0; p < IPT; ++p)
-                pair_add<DS, SOFT>(j, ip[p], e2, ts[p], PairMask{p0 + 2 * q, own[p], p1});
-        }
+        for (int q = sub; q < full; q += S)
+            pair_add<DS, SOFT>(cluster_pair(sm, q), ip, e2, ts, OwnMask{p0 + 2 * q, own});
     }
-    if (((p1 - p0) & 1) && (full & (S - 1)) == sub) {  // the last, half-empty pair
-        const JPair j = cluster_pair(sm, full);
-#pragma unroll
-        for (int p = 0; p < IPT; ++p)
-            pair_add<DS, SOFT>(j, ip[p], e2, ts[p], PairMask{p0 + 2 * full, own[p], p1});
-    }
+    if (((p1 - p0) & 1) && (full & (S - 1)) == sub)  // the last, half-empty pair
+        pair_add<DS, SOFT>(cluster_pair(sm, full), ip, e2, ts, PairMask{p0 + 2 * full, own, p1});
 }
 
 // B for one window of nw due slots: the sums of every slot over the CTA's particles
-// [p0, p1), left in CTA slot % CL_CTAS. Groups of IPT slots (k, k + ngroups), S lanes each.
-template <bool DS, int IPT, int MAXL>
-__device__ __forceinline__ void cluster_force(ClusterSmem<MAXL> &sm, int nw, int p0, int p1, int npair,
-                                              int rank, float eps2f)
+// [p0, p1), left in CTA slot % CL_CTAS; S lanes a slot. One slot a lane: two (half the
+// shared-memory reads) spilled registers, and a step took 0.3 us more.
+template <bool DS, int MAXL>
+__device__ __forceinline__ void cluster_force(ClusterSmem<MAXL> &sm, int nw, int p0, int p1,
+                                              int npair, int rank, float eps2f)
 {
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int ng = (nw + IPT - 1) / IPT;
-    const int lgS = cluster_lanes_log2(ng, npair), S = 1 << lgS, sub = tid & (S - 1);
+    const int lgS = cluster_lanes_log2(nw, npair), S = 1 << lgS, sub = tid & (S - 1);
     const float2 e2 = make_float2(eps2f, eps2f);
-    for (int g0 = 0; g0 < ng; g0 += CL_THREADS >> lgS) {
-        if (g0 + ((warp * 32) >> lgS) >= ng) break;  // a warp of idle groups
-        const int g = g0 + (tid >> lgS);
-        IPair ip[IPT];
-        PairSum ts[IPT];
-        int own[IPT];
-        bool mine = false;
-#pragma unroll
-        for (int p = 0; p < IPT; ++p) {
-            const int k = min(g + p * ng, nw - 1);  // idle slots copy the last one
-            ip[p] = ipair_of(make_float4(sm.i[0][k], sm.i[1][k], sm.i[2][k], 0.f),
-                             make_float4(sm.i[3][k], sm.i[4][k], sm.i[5][k], 0.f),
-                             make_float4(sm.i[6][k], sm.i[7][k], sm.i[8][k], 0.f));
-            own[p] = sm.id[k];
-            mine = mine || (own[p] >= p0 && own[p] < p1);
-            pair_zero(ts[p]);
-        }
-        const bool masked = __any_sync(0xffffffffu, mine);
+    for (int k0 = 0; k0 < nw; k0 += CL_THREADS >> lgS) {
+        if (k0 + ((warp * 32) >> lgS) >= nw) break;  // a warp of idle slots
+        const int k = k0 + (tid >> lgS), kk = min(k, nw - 1);  // idle slots copy the last one
+        const IPair ip = ipair_of(make_float4(sm.i[0][kk], sm.i[1][kk], sm.i[2][kk], 0.f),
+                                  make_float4(sm.i[3][kk], sm.i[4][kk], sm.i[5][kk], 0.f),
+                                  make_float4(sm.i[6][kk], sm.i[7][kk], sm.i[8][kk], 0.f));
+        const int own = sm.id[kk];
+        const bool masked = __any_sync(0xffffffffu, own >= p0 && own < p1);
+        PairSum ts;
+        pair_zero(ts);
         if (soft_pairs(eps2f))
-            cluster_pairs<DS, true, IPT>(sm, sub, S, p0, p1, masked, ip, own, e2, ts);
+            cluster_pairs<DS, true>(sm, sub, S, p0, p1, masked, ip, own, e2, ts);
         else
-            cluster_pairs<DS, false, IPT>(sm, sub, S, p0, p1, true, ip, own, e2, ts);
+            cluster_pairs<DS, false>(sm, sub, S, p0, p1, masked, ip, own, e2, ts);
+        float v[CL_Q];
 #pragma unroll
-        for (int p = 0; p < IPT; ++p) {
-            float v[CL_Q];
+        for (int c = 0; c < CL_Q; ++c) v[c] = pair_total(ts, c);
+        for (int o = S >> 1; o > 0; o >>= 1)
 #pragma unroll
-            for (int c = 0; c < CL_Q; ++c) v[c] = pair_total(ts[p], c);
-            for (int o = S >> 1; o > 0; o >>= 1)
-#pragma unroll
-                for (int c = 0; c < CL_Q; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
-            const int k = g + p * ng;
-            if (sub == 0 && g < ng && k < nw) {
-                const uint32_t to = cluster_addr(sm.part[rank][k / CL_CTAS], k % CL_CTAS);
-                cluster_st(to, make_float4(v[0], v[1], v[2], v[3]));
-                cluster_st(to + 16u, make_float4(v[4], v[5], v[6], 0.f));
-            }
+            for (int c = 0; c < CL_Q; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+        if (sub == 0 && k < nw) {
+            const uint32_t to = cluster_addr(sm.part[rank][k / CL_CTAS], k % CL_CTAS);
+            cluster_st(to, make_float4(v[0], v[1], v[2], v[3]));
+            cluster_st(to + 16u, make_float4(v[4], v[5], v[6], 0.f));
         }
     }
 }
@@ -1172,10 +1146,7 @@ __global__ void __launch_bounds__(CL_THREADS)
             __syncthreads();
 
             // B: the pair terms
-            if (nw >= CL_IPT2_SLOTS)
-                cluster_force<DS, 2>(sm, nw, p0, p1, npair, rank, a.eps2f);
-            else
-                cluster_force<DS, 1>(sm, nw, p0, p1, npair, rank, a.eps2f);
+            cluster_force<DS>(sm, nw, p0, p1, npair, rank, a.eps2f);
             // C's slots rank + CL_CTAS e: three lanes each, ten a warp, on four warps (one per
             // FP64 pipe) or eight; their state is on its way during the barrier
             static_assert(CL_SLOTS / CL_CTAS <= 80, "eight warps of ten");
