@@ -447,6 +447,15 @@ int grow_scratch(nb_server s, size_t part, size_t)
 
 namespace {
 
+// Whether r's cluster launch has ended (cudaErrorNotReady: not yet, which is no error and
+// is not left for the launches' checks to find).
+cudaError_t launch_ended(nb_server s, const Req &r)
+{
+    const cudaError_t e = cudaEventQuery(s->ev_cluster[r.slot]);
+    if (e == cudaErrorNotReady) cudaGetLastError();
+    return e;
+}
+
 // One tick (server thread): cancellations, admission, one batched force
 // launch, the per-request kernels and copies, one synchronisation, and the
 // bookkeeping of what finished. A CUDA failure returns NB_ERR_CUDA.
@@ -459,7 +468,7 @@ int tick(nb_server s)
         // running requests that were cancelled (none of their work is on the GPU)
         for (auto &r : s->inflight)
             if (r->running) {
-                const cudaError_t e = cudaEventQuery(s->ev_cluster[r->slot]);
+                const cudaError_t e = launch_ended(s, *r);
                 if (e == cudaErrorNotReady) continue;
                 if (e != cudaSuccess) return NB_ERR_CUDA;
                 r->running = false;
@@ -595,7 +604,7 @@ int tick(nb_server s)
         // only cluster launches are under way: wait a little for one to end
         do {
             for (auto &r : s->inflight)
-                if (cudaEventQuery(s->ev_cluster[r->slot]) != cudaErrorNotReady) return NB_OK;
+                if (launch_ended(s, *r) != cudaErrorNotReady) return NB_OK;
         } while (s->now() < t_begin + 20e-6);
         return NB_OK;
     }
