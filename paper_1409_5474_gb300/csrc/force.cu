@@ -191,7 +191,7 @@ __device__ __forceinline__ int i_id(const ISet &is, int row, float id_bits)
 // Member index of slot k; an index outside the j-set is flagged and replaced by 0.
 __device__ __forceinline__ int member_index(const ISet &is, int k, unsigned *err)
 {
-    const int r = is.idx ? __ldg(is.idx + k) : k;
+    const int r = is.idx ? is.idx[k] : k;
     if ((unsigned)r >= (unsigned)is.nj) {
         atomicOr(err, DERR_BADINDEX);
         return 0;
@@ -224,8 +224,8 @@ __host__ __device__ constexpr bool tile_ahead(int nwj) { return nwj == 8; }
 
 template <int VAR, int IPT, int NWI, int NWJ, int JT, int NS>
 __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
-    k_force_tile32(const float4 *__restrict__ jrec, int nj, ISet is, float eps2f, int ntiles,
-                   double *__restrict__ part, long long pld, Out3 out, unsigned *err)
+    k_force_tile32(const float4 *jrec, int nj, ISet is, float eps2f, int ntiles, double *part,
+                   long long pld, Out3 out, unsigned *err)
 {
     // NS ring stages of JT records (bulk-copy destinations), one or (AHEAD) two tiles as
     // j-pairs (JT / 2 pairs x 6 float4 each), the running totals
@@ -272,9 +272,9 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
         int k = blockIdx.x * IB + (wi * IPT + p) * 32 + lane;
         if (k >= is.n) k = is.n - 1;  // idle slots compute a copy, never written
         const int r = i_row(is, k, err);
-        const float4 a = __ldg(is.rec32 + (size_t)DS_REC * r);
-        const float4 b = __ldg(is.rec32 + (size_t)DS_REC * r + 1);
-        const float4 c = __ldg(is.rec32 + (size_t)DS_REC * r + 2);
+        const float4 a = is.rec32[(size_t)DS_REC * r];
+        const float4 b = is.rec32[(size_t)DS_REC * r + 1];
+        const float4 c = is.rec32[(size_t)DS_REC * r + 2];
         ip[p] = ipair_of(a, b, c);
         iid[p] = i_id(is, r, b.w);
     }
@@ -415,8 +415,7 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
 // K3 of the tile, tiny-set and FP64 kernels (split_sum): output q = component c of slot k.
 template <class T, int G>
 __global__ void __launch_bounds__(256)
-    k_split_sums(const T *__restrict__ part, long long pld, int nsplit, int n_i, Out3 out,
-                 unsigned *err)
+    k_split_sums(const T *part, long long pld, int nsplit, int n_i, Out3 out, unsigned *err)
 {
     const long long q = (long long)blockIdx.x * (256 / G) + threadIdx.x % (256 / G);
     const int c = (int)(q / n_i), k = (int)(q % n_i);
@@ -446,8 +445,8 @@ constexpr int T64_UNIT = 16;  // j-ranges are whole units (16-byte aligned rows)
 
 template <int JT, int NS>
 __global__ void __launch_bounds__(32 * T64_ROWS)
-    k_force_tile64(JSet js, ISet is, double eps2, int nunits, double *__restrict__ part,
-                   long long pld, Out3 out, unsigned *err)
+    k_force_tile64(JSet js, ISet is, double eps2, int nunits, double *part, long long pld,
+                   Out3 out, unsigned *err)
 {
     extern __shared__ __align__(128) double s_t64[];  // NS * 7 * JT
     __shared__ __align__(8) uint64_t s_full[NS];
@@ -476,8 +475,8 @@ __global__ void __launch_bounds__(32 * T64_ROWS)
     double xi[3], vi[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        xi[c] = __ldg(is.pos64 + c * is.ld64 + r);
-        vi[c] = __ldg(is.vel64 + c * is.ld64 + r);
+        xi[c] = is.pos64[c * is.ld64 + r];
+        vi[c] = is.vel64[c * is.ld64 + r];
     }
     double v[7];  // acc, jerk, positive potential
 #pragma unroll
@@ -739,9 +738,8 @@ __global__ void __launch_bounds__(32 * NWARP)
 // in registers).
 template <int VAR, int IPT, int JPT>
 __global__ void __launch_bounds__(256)
-    k_force_tiny32(const float4 *__restrict__ jrec, int nj, ISet is, float eps2f,
-                   double *__restrict__ part, long long pld, unsigned *counters, Out3 out,
-                   unsigned *err)
+    k_force_tiny32(const float4 *jrec, int nj, ISet is, float eps2f, double *part, long long pld,
+                   unsigned *counters, Out3 out, unsigned *err)
 {
     constexpr bool DS = (VAR == NB_F32DS);
     constexpr int NT = 256, NW = NT / 32;
@@ -758,9 +756,9 @@ __global__ void __launch_bounds__(256)
         const int j = split * NT * JPT + r * NT + tid;
         jidx[r] = j;
         if (j < nj) {
-            ja[r] = __ldg(jrec + (size_t)DS_REC * j);
-            jc[r] = __ldg(jrec + (size_t)DS_REC * j + 2);
-            if (DS) jb[r] = __ldg(jrec + (size_t)DS_REC * j + 1);
+            ja[r] = jrec[(size_t)DS_REC * j];
+            jc[r] = jrec[(size_t)DS_REC * j + 2];
+            if (DS) jb[r] = jrec[(size_t)DS_REC * j + 1];
         } else {
             ja[r] = make_float4(0.f, 0.f, 0.f, 0.f);  // massless: contributes nothing
             jc[r] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -776,9 +774,9 @@ __global__ void __launch_bounds__(256)
         for (int p = 0; p < IPT; ++p) {
             const int k = min(g0 + p, is.n - 1);
             const int r = i_row(is, k, err);
-            const float4 a = __ldg(is.rec32 + (size_t)DS_REC * r);
-            const float4 b = __ldg(is.rec32 + (size_t)DS_REC * r + 1);
-            const float4 c = __ldg(is.rec32 + (size_t)DS_REC * r + 2);
+            const float4 a = is.rec32[(size_t)DS_REC * r];
+            const float4 b = is.rec32[(size_t)DS_REC * r + 1];
+            const float4 c = is.rec32[(size_t)DS_REC * r + 2];
             xh[p] = a.x; yh[p] = a.y; zh[p] = a.z;
             xl[p] = b.x; yl[p] = b.y; zl[p] = b.z;
             vx[p] = c.x; vy[p] = c.y; vz[p] = c.z;
@@ -884,7 +882,7 @@ __global__ void __launch_bounds__(256)
 // FP64 j-parallel kernel: thread = j, all threads share IPT i's.
 template <int IPT, int NT>
 __global__ void __launch_bounds__(NT)
-    k_force_jmode64(JSet js, ISet is, double eps2, double *__restrict__ part, long long pld,
+    k_force_jmode64(JSet js, ISet is, double eps2, double *part, long long pld,
                     unsigned *counters, Out3 out, unsigned *err)
 {
     constexpr int NW = NT / 32;
@@ -905,10 +903,10 @@ __global__ void __launch_bounds__(NT)
             const int r = is.member ? member_index(is, k, err) : k;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                xi[p][c] = __ldg(is.pos64 + c * is.ld64 + r);
-                vi[p][c] = __ldg(is.vel64 + c * is.ld64 + r);
+                xi[p][c] = is.pos64[c * is.ld64 + r];
+                vi[p][c] = is.vel64[c * is.ld64 + r];
             }
-            mi[p] = is.member ? __ldg(is.m64 + r) : 0.0;
+            mi[p] = is.member ? is.m64[r] : 0.0;
             iid[p] = is.member ? r : -1;
         }
         double ta[IPT][3], tja[IPT][3], tjb[IPT][3], tp[IPT];
@@ -919,11 +917,9 @@ __global__ void __launch_bounds__(NT)
             tp[p] = 0.0;
         }
         for (int j = j0 + tid; j < j1; j += NT) {
-            const double xj = __ldg(js.pos64 + j), yj = __ldg(js.pos64 + js.ld + j),
-                         zj = __ldg(js.pos64 + 2 * js.ld + j);
-            const double uj = __ldg(js.vel64 + j), wj = __ldg(js.vel64 + js.ld + j),
-                         qj = __ldg(js.vel64 + 2 * js.ld + j);
-            const double mj = __ldg(js.m64 + j);
+            const double xj = js.pos64[j], yj = js.pos64[js.ld + j], zj = js.pos64[2 * js.ld + j];
+            const double uj = js.vel64[j], wj = js.vel64[js.ld + j], qj = js.vel64[2 * js.ld + j];
+            const double mj = js.m64[j];
 #pragma unroll
             for (int p = 0; p < IPT; ++p) {
                 const double dx = xj - xi[p][0], dy = yj - xi[p][1], dz = zj - xi[p][2];

@@ -80,7 +80,7 @@ __global__ void k_predict6(StateDev s, double t, unsigned *err)
 // Member index of slot k; an index outside [0, n) is flagged and replaced by 0.
 __device__ __forceinline__ int member6(const int *idx, int k, int n, unsigned *err)
 {
-    const int r = idx ? __ldg(idx + k) : k;
+    const int r = idx ? idx[k] : k;
     if ((unsigned)r >= (unsigned)n) {
         atomicOr(err, DERR_BADINDEX);
         return 0;
@@ -208,8 +208,8 @@ __device__ __forceinline__ void tile6_pairs(const float4 *pairs, int q0, int ste
 // 789 us with the splits' sums, N = 65536: 8.68 -> 7.76 ms.
 template <bool DS, int NWJ, int JT>
 __global__ void __launch_bounds__(32 * H6_NWARP, 2)
-    k_force6_tile32(const float4 *__restrict__ jrec, int nj, const int *__restrict__ idx,
-                    int n_i, float eps2f, int ntiles, float2 *__restrict__ part, long long pld,
+    k_force6_tile32(const float4 *jrec, int nj, const int *idx, int n_i, float eps2f, int ntiles,
+                    float2 *part, long long pld,
                     Out6 out, unsigned *err)
 {
     // H6_NS ring stages of JT records, the current tile as j-pairs, the running totals
@@ -248,8 +248,8 @@ __global__ void __launch_bounds__(32 * H6_NWARP, 2)
     IPair6 ip;
     {
         const float4 *r = jrec + (size_t)DS6_REC * ii;
-        const float4 d = __ldg(r + 3);
-        ip.p = ipair_of(__ldg(r), __ldg(r + 1), __ldg(r + 2));
+        const float4 d = r[3];
+        ip.p = ipair_of(r[0], r[1], r[2]);
         ip.ax = make_float2(-d.x, -d.x);
         ip.ay = make_float2(-d.y, -d.y);
         ip.az = make_float2(-d.z, -d.z);
@@ -428,8 +428,7 @@ __global__ void __launch_bounds__(H6_T64)
 // Output q = component c of slot k (split_sum).
 template <class T, int G>
 __global__ void __launch_bounds__(256)
-    k_force6_sums(const T *__restrict__ part, long long pld, int nsplit, int n_i, Out6 out,
-                  unsigned *err)
+    k_force6_sums(const T *part, long long pld, int nsplit, int n_i, Out6 out, unsigned *err)
 {
     const long long q = (long long)blockIdx.x * (256 / G) + threadIdx.x % (256 / G);
     const int c = (int)(q / n_i), k = (int)(q % n_i);
@@ -466,7 +465,7 @@ cudaError_t go_force6_sums(const double *part, int n_i, int nsplit, const Out6 &
 // Slot k: the order-6 corrector (correct6_lanes_pre) from the start-of-step state
 // and the new a1, j1, s1 (f, slot-indexed).
 __global__ void __launch_bounds__(CORRECT6_THREADS)
-    k_correct6(StateDev s, const int *__restrict__ act, int na, double t_new, Out6 f,
+    k_correct6(StateDev s, const int *act, int na, double t_new, Out6 f,
                StepParams prm, SchedDev *sd, unsigned *err, unsigned long long *dtmin_hits)
 {
     cudaGridDependencySynchronize();

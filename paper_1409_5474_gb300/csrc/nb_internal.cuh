@@ -11,10 +11,13 @@
 
 namespace nb {
 
-// Launch a kernel that begins with cudaGridDependencySynchronize(): its CTAs may be
-// scheduled while the last ones of the launch before it on the stream still run, so
-// their start-up is hidden; what the earlier launches wrote is visible after that call (a
-// force and its split reduction: 2.1 us less for the two).
+// Launch a kernel that calls cudaGridDependencySynchronize() before it reads anything an
+// earlier launch wrote: its launch and start-up overlap the end of the launch before it on
+// the stream (no kernel here triggers its dependents early, so that is the flush after its
+// last CTA), and what the earlier launches wrote is visible after that call (a force and
+// its split reduction: 2.1 us less for the two). Data of earlier launches are not constant
+// over such a kernel's whole run: it reads them by ordinary loads (or __ldcg), never as
+// read-only data (__ldg, const __restrict__), which may be moved above the call.
 template <class... A, class... B>
 static inline cudaError_t launch_dependent(void (*kern)(A...), dim3 grid, unsigned threads,
                                            size_t smem, cudaStream_t st, const B &...args)

@@ -72,7 +72,7 @@ cudaError_t launch_advance(double *t_dev, double dt, cudaStream_t st)
     return launch_dependent(k_advance, dim3(1), 1, 0, st, t_dev, dt);
 }
 
-__global__ void k_correct(StateDev s, const int *__restrict__ act, int na, double t_new, Out3 f,
+__global__ void k_correct(StateDev s, const int *act, int na, double t_new, Out3 f,
                           StepParams prm, SchedDev *sd, unsigned *err,
                           unsigned long long *dtmin_hits, const double *t_dev, bool xp_from_state)
 {
