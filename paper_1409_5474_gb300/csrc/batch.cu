@@ -43,6 +43,7 @@ struct nb_batch_s {
     int nitems = 0;
     SplitGroup *d_groups = nullptr;  // j-split groups of the large systems' i-blocks
     int ngroups = 0;
+    bool chunks = false;             // no partials: items take their j-ranges in turn
     float2 *d_part = nullptr;        // their partials
     unsigned *d_ticket = nullptr;    // the item tickets of the force launches
     size_t slab_bytes = 0;
@@ -118,8 +119,10 @@ Out3 bout(nb_batch b) { return Out3{b->f_acc, b->f_jerk, b->f_pot, b->ld}; }
 // Systems larger than this have their j-range split into equal parts of at most as many
 // (whole 128-record tiles), so that no work item holds the last CTAs long: a
 // 4096-particle system's items took a third of a 512-system step each, and ten times the
-// mean load of a 40-system step. The split depends on the system's size alone, so its
-// results are the same alone and in any batch.
+// mean load of a 40-system step. The parts depend on the system's size alone, and their
+// sums are added in the same order whether the parts are items of their own (with partials)
+// or one item takes them in turn (no memory for partials), so a system's results are the
+// same alone, in any batch, and at any budget.
 constexpr int BATCH_SPLIT_J = 1024;
 
 int batch_chunk(int n)
@@ -131,7 +134,7 @@ int batch_chunk(int n)
 
 // Work list for CTAs of `threads` threads (i-blocks of 2 * threads), sorted
 // by decreasing work (ni * nj), ties by position. Without memory for the partials
-// (device, or the batch's budget) no system is split.
+// (device, or the batch's budget) an item takes all parts of its system's j-range.
 int build_items(nb_batch b)
 {
     const int ib = 2 * b->threads;
@@ -153,6 +156,7 @@ int build_items(nb_batch b)
         b->d_part = nullptr;
         split = false;
     }
+    b->chunks = part > 0 && !split;
     float2 *next_part = b->d_part;
     for (int s = 0; s < b->n_sys; ++s) {
         const int n = b->sizes[s], o = b->offs[s];
@@ -172,6 +176,7 @@ int build_items(nb_batch b)
             w.eps2 = e2;
             w.err = b->d_err;
             const int chunk = split ? batch_chunk(n) : n;
+            w.chunk = split || batch_chunk(n) == n ? 0 : batch_chunk(n);
             w.nsplit = (n + chunk - 1) / chunk;
             w.part = w.nsplit > 1 ? next_part : nullptr;
             for (int sp = 0; sp < w.nsplit; ++sp) {
@@ -227,7 +232,7 @@ void drop_graph(nb_batch b)
 cudaError_t batch_force(nb_batch b)
 {
     const cudaError_t e = launch_force_items(b->cfg.variant, b->threads, b->d_items, b->nitems,
-                                             b->grid, b->d_ticket, b->stream);
+                                             b->grid, b->d_ticket, b->stream, b->chunks);
     if (e != cudaSuccess || !b->ngroups) return e;
     return launch_split_reduce(b->d_groups, b->ngroups, std::min(b->ngroups, 8 * b->num_sms),
                                b->stream);

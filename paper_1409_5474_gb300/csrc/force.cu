@@ -1174,7 +1174,10 @@ __device__ __forceinline__ void items_done(unsigned *ticket)
 // tiles with a warp's own particles on the packed path (a 1000-particle system has a
 // quarter of its tiles of either kind), warps without rows skip the arithmetic. 512
 // clusters of 16-4096: a pass of eight steps 11.2 -> 10.3 ms.
-template <int VAR, int IPT, int NT, int JT, int NS>
+// CHUNKS: items may take several j-ranges one after the other (WorkItem::chunk); the sums
+// between ranges wait as double-single pairs in the item's own output elements, which are as
+// wide, so that no other memory is needed.
+template <int VAR, int IPT, int NT, int JT, int NS, bool CHUNKS>
 __global__ void __launch_bounds__(NT, 512 / NT)
     k_force_items32(const WorkItem *__restrict__ items, int nitems, unsigned *ticket)
 {
@@ -1273,6 +1276,30 @@ __global__ void __launch_bounds__(NT, 512 / NT)
                         v.x += pair_total(ts[p], c);
                     h = v;
                 }
+            if (CHUNKS && w.chunk > 0 && (kt + 1 == ntiles || (kt + 1) * JT % w.chunk == 0)) {
+                // the end of a j-range: its sums join those of the ranges before it, as
+                // k_split_reduce adds them
+#pragma unroll 1
+                for (int p = 0; p < IPT; ++p) {
+                    const int k = (warp * IPT + p) * 32 + lane;
+                    if (k >= w.ni) continue;
+#pragma unroll 1
+                    for (int c = 0; c < 7; ++c) {
+                        double *slot = c < 3 ? w.acc + c * w.ld : c < 6 ? w.jerk + (c - 3) * w.ld : w.pot;
+                        float2 *kept = reinterpret_cast<float2 *>(slot + w.i0 + k);
+                        float2 &h = s_tot[(p * 7 + c) * NT];
+                        const float2 was = kt * JT < w.chunk ? make_float2(0.f, 0.f) : *kept;
+                        dsf sum{was.x, was.y};
+                        ds_acc(sum, dsf{h.x, h.y});
+                        if (kt + 1 == ntiles) {
+                            h = make_float2(sum.hi, sum.lo);
+                        } else {
+                            *kept = make_float2(sum.hi, sum.lo);
+                            h = make_float2(0.f, 0.f);
+                        }
+                    }
+                }
+            }
             __syncthreads();  // the stage and the pair buffer are free
             if (s_abort) {
                 if (tid == 0) {
@@ -1650,11 +1677,11 @@ static size_t items_smem(int threads)
            (size_t)threads * 14 * sizeof(float2);
 }
 
-template <int VAR, int NT>
+template <int VAR, int NT, bool CHUNKS>
 static cudaError_t go_items(const WorkItem *items, int nitems, int grid, unsigned *ticket,
                             cudaStream_t st)
 {
-    constexpr auto kern = k_force_items32<VAR, 2, NT, JT32, NS32>;
+    constexpr auto kern = k_force_items32<VAR, 2, NT, JT32, NS32, CHUNKS>;
     const size_t smem = items_smem(NT);
     const cudaError_t attr = allow_smem<kern>(smem);
     if (attr != cudaSuccess) return attr;
@@ -1662,22 +1689,25 @@ static cudaError_t go_items(const WorkItem *items, int nitems, int grid, unsigne
     return cudaGetLastError();
 }
 
+template <int VAR, bool CHUNKS>
+static cudaError_t go_items_of(int threads, const WorkItem *items, int nitems, int grid,
+                               unsigned *ticket, cudaStream_t st)
+{
+    switch (threads) {
+    case 64: return go_items<VAR, 64, CHUNKS>(items, nitems, grid, ticket, st);
+    case 128: return go_items<VAR, 128, CHUNKS>(items, nitems, grid, ticket, st);
+    default: return go_items<VAR, 256, CHUNKS>(items, nitems, grid, ticket, st);
+    }
+}
+
 cudaError_t launch_force_items(int variant, int threads, const WorkItem *items, int nitems,
-                               int grid, unsigned *ticket, cudaStream_t st)
+                               int grid, unsigned *ticket, cudaStream_t st, bool chunks)
 {
     if (nitems <= 0) return cudaSuccess;
-    if (variant == NB_F32DS) {
-        switch (threads) {
-        case 64: return go_items<NB_F32DS, 64>(items, nitems, grid, ticket, st);
-        case 128: return go_items<NB_F32DS, 128>(items, nitems, grid, ticket, st);
-        default: return go_items<NB_F32DS, 256>(items, nitems, grid, ticket, st);
-        }
-    }
-    switch (threads) {
-    case 64: return go_items<NB_F32, 64>(items, nitems, grid, ticket, st);
-    case 128: return go_items<NB_F32, 128>(items, nitems, grid, ticket, st);
-    default: return go_items<NB_F32, 256>(items, nitems, grid, ticket, st);
-    }
+    const auto go = variant == NB_F32DS
+                        ? (chunks ? go_items_of<NB_F32DS, true> : go_items_of<NB_F32DS, false>)
+                        : (chunks ? go_items_of<NB_F32, true> : go_items_of<NB_F32, false>);
+    return go(threads, items, nitems, grid, ticket, st);
 }
 
 cudaError_t launch_force_items_jpar(int variant, const WorkItem *items, int nitems, int grid,
@@ -1761,7 +1791,7 @@ int tile_blocks_per_sm(int variant, int nwj)
 template <int VAR, int NT>
 static int items_occ()
 {
-    constexpr auto kern = k_force_items32<VAR, 2, NT, JT32, NS32>;
+    constexpr auto kern = k_force_items32<VAR, 2, NT, JT32, NS32, false>;
     const size_t smem = items_smem(NT);
     int nb = 0;
     if (allow_smem<kern>(smem) != cudaSuccess ||

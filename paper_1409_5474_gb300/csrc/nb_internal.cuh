@@ -163,7 +163,9 @@ cudaError_t warm_force_jmode64(cudaStream_t st);
 // A j-split group (nsplit > 1 items with the same i-rows and consecutive
 // j-ranges) writes double-single partials to part ([nsplit][7][ni] float2);
 // launch_split_reduce, queued after the items, sums them in the order
-// split = 0..nsplit-1 (SplitGroup). nsplit <= 1: the item writes its outputs.
+// split = 0..nsplit-1 (SplitGroup). nsplit <= 1: the item writes its outputs; with chunk > 0
+// (a multiple of 128) it takes the j-ranges [j0, j0 + chunk), ... itself, one after the other,
+// and adds their sums as the split group's are added, to the same bits.
 struct WorkItem {
     const float4 *jrec;
     const float4 *irec;
@@ -173,7 +175,7 @@ struct WorkItem {
     int gathered, kind;
     int split, nsplit;
     float eps2;
-    int pad;
+    int chunk;
     float2 *part;
     unsigned *err;  // error word of the item's system
 };
@@ -196,9 +198,10 @@ constexpr int BATCH_THREADS[3] = {64, 128, 256};
 // Batched force (FP32 / double-single) over a list of i-parallel items (kind 0);
 // grid = number of persistent CTAs (each takes the next item when it is done with one, so
 // sort them by decreasing work). ticket: two words, zero before the first launch and left
-// at zero by each; launches that share them run one after the other.
+// at zero by each; launches that share them run one after the other. chunks: some items
+// have chunk > 0.
 cudaError_t launch_force_items(int variant, int threads, const WorkItem *items, int nitems,
-                               int grid, unsigned *ticket, cudaStream_t st);
+                               int grid, unsigned *ticket, cudaStream_t st, bool chunks = false);
 
 // Resident CTAs per SM of the batched kernel with `threads` threads.
 int batch_blocks_per_sm(int variant, int threads);

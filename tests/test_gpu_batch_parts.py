@@ -1,0 +1,49 @@
+"""Batched systems above 1024 particles: their j-range is taken in parts, whose sums are added
+in one order wherever the parts run, so a system's bits depend on the system alone."""
+import numpy as np
+import pytest
+
+from paper_1409_5474_gb300 import ic
+
+pytestmark = pytest.mark.gpu
+
+DT = 1.0 / 512
+
+
+def _smallest_budget(nb, sizes, variant):
+    """The least budget_bytes that nb_batch_create accepts: the state, no partials."""
+    lo, hi = 1, 1 << 30
+    while lo < hi:
+        mid = (lo + hi) // 2
+        cfg = nb.nb_config_default(variant=variant, device=0, budget_bytes=mid)
+        try:
+            nb.nb_batch_destroy(nb.nb_batch_create(cfg, sizes, [0.05] * len(sizes), DT))
+            hi = mid
+        except nb.NBodyError as e:
+            assert e.status == nb.NB_ERR_BUDGET
+            lo = mid + 1
+    return lo
+
+
+def _run(nb, systems, tune=False, **cfg):
+    eps = np.full(len(systems), 0.05)
+    with nb.Batch(systems, eps, DT, device=0, **cfg) as b:
+        if tune:
+            b.autotune()
+        b.step(3)
+        pos, vel, _ = b.get()
+        return [np.concatenate([b.system(s, pos), b.system(s, vel)]) for s in range(len(systems))]
+
+
+@pytest.mark.parametrize("variant", ["f32ds", "f32"])
+def test_bits_depend_on_the_system_alone(nb, variant):
+    sizes = [1024, 1025, 1500, 2049, 4096, 5000]
+    systems = [ic.plummer(n, 70 + k) for k, n in enumerate(sizes)]
+    mix = _run(nb, systems, variant=variant)
+    tight = _run(nb, systems, variant=variant, budget_bytes=_smallest_budget(nb, sizes, variant))
+    tuned = _run(nb, systems, tune=True, variant=variant)
+    for s, p in enumerate(systems):
+        alone = _run(nb, [p], variant=variant)[0]
+        np.testing.assert_array_equal(mix[s], alone)
+        np.testing.assert_array_equal(tight[s], alone)
+        np.testing.assert_array_equal(tuned[s], alone)
