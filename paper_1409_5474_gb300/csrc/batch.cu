@@ -116,19 +116,25 @@ StepParams bparams(nb_batch b)
 
 Out3 bout(nb_batch b) { return Out3{b->f_acc, b->f_jerk, b->f_pot, b->ld}; }
 
-// Systems larger than this have their j-range split into equal parts of at most as many
-// (whole 128-record tiles), so that no work item holds the last CTAs long: a
+// Systems larger than this have their j-range split into equal parts (whole 128-record
+// tiles), so that no work item holds the last CTAs long: a
 // 4096-particle system's items took a third of a 512-system step each, and ten times the
 // mean load of a 40-system step. The parts depend on the system's size alone, and their
 // sums are added in the same order whether the parts are items of their own (with partials)
 // or one item takes them in turn (no memory for partials), so a system's results are the
-// same alone, in any batch, and at any budget.
+// same alone, in any batch, and at any budget. The partials take
+// 56 bytes a particle and part (the state 272 in all): at most 16 parts up to 65536 particles
+// (59 MB; one such system 4.4 ms a step, 5.3 with 4 parts, 4.4 with the 64 of 1024 records
+// each), 4 above, where the i-blocks nearly fill the GPU (200000 particles 40.9 ms a step,
+// 40.1 with 196 parts and 2.2 GB of partials).
 constexpr int BATCH_SPLIT_J = 1024;
+
+int batch_max_parts(int n) { return n <= 65536 ? 16 : 4; }
 
 int batch_chunk(int n)
 {
     if (n <= BATCH_SPLIT_J) return n;
-    const int parts = (n + BATCH_SPLIT_J - 1) / BATCH_SPLIT_J;
+    const int parts = std::min((n + BATCH_SPLIT_J - 1) / BATCH_SPLIT_J, batch_max_parts(n));
     return ((n + parts - 1) / parts + 127) / 128 * 128;
 }
 

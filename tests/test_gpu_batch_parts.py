@@ -47,3 +47,25 @@ def test_bits_depend_on_the_system_alone(nb, variant):
         np.testing.assert_array_equal(mix[s], alone)
         np.testing.assert_array_equal(tight[s], alone)
         np.testing.assert_array_equal(tuned[s], alone)
+
+
+def test_partials_of_a_large_system_are_bounded(nb):
+    """262144 particles: 272 bytes of state and 4 x 56 of partials each, 130 MB; the allocator
+    hands out whole blocks of a few MB and the launches' own buffers come on top. Parts of
+    1024 would take 3.8 GB."""
+    import torch
+    rng = np.random.default_rng(2)
+    n = 262144
+    m, pos, vel = np.full(n, 1.0 / n), rng.standard_normal((3, n)), rng.standard_normal((3, n))
+    cfg = nb.nb_config_default(variant="f32ds", device=0)
+    b = nb.nb_batch_create(cfg, [64], [0.05], DT)
+    nb.nb_batch_set(b, m[:64], pos[:, :64].copy(), vel[:, :64].copy())
+    nb.nb_batch_step(b, 1)  # the module is loaded
+    nb.nb_batch_destroy(b)
+    free = torch.cuda.mem_get_info(0)[0]
+    b = nb.nb_batch_create(cfg, [n], [0.05], DT)
+    nb.nb_batch_set(b, m, pos, vel)
+    nb.nb_batch_step(b, 1)
+    used = free - torch.cuda.mem_get_info(0)[0]
+    nb.nb_batch_destroy(b)
+    assert used < 192 << 20
