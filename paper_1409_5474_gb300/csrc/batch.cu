@@ -138,6 +138,14 @@ int batch_chunk(int n)
     return ((n + parts - 1) / parts + 127) / 128 * 128;
 }
 
+void drop_graph(nb_batch b)
+{
+    if (b->gexec) cudaGraphExecDestroy(b->gexec);
+    if (b->graph) cudaGraphDestroy(b->graph);
+    b->gexec = nullptr;
+    b->graph = nullptr;
+}
+
 // Work list for CTAs of `threads` threads (i-blocks of 2 * threads), sorted
 // by decreasing work (ni * nj), ties by position. Without memory for the partials
 // (device, or the batch's budget) an item takes all parts of its system's j-range.
@@ -146,10 +154,16 @@ int build_items(nb_batch b)
     const int ib = 2 * b->threads;
     std::vector<WorkItem> items;
     std::vector<SplitGroup> groups;
-    if (b->d_part) cudaFree(b->d_part);
-    if (b->d_groups) cudaFree(b->d_groups);
+    // a captured step holds the addresses of the lists and partials: it goes first; until the
+    // new lists are uploaded there are none (ensure_items)
+    drop_graph(b);
+    b->nitems = b->ngroups = 0;
+    cudaFree(b->d_part);
+    cudaFree(b->d_groups);
+    cudaFree(b->d_items);
     b->d_part = nullptr;
     b->d_groups = nullptr;
+    b->d_items = nullptr;
     size_t part = 0;  // float2 of partials: 7 per i-particle and split
     for (int s = 0; s < b->n_sys; ++s) {
         const int n = b->sizes[s], chunk = batch_chunk(n);
@@ -210,29 +224,22 @@ int build_items(nb_batch b)
     std::stable_sort(items.begin(), items.end(), [](const WorkItem &x, const WorkItem &y) {
         return (long long)x.ni * x.nj > (long long)y.ni * y.nj;
     });
-    if (b->d_items) cudaFree(b->d_items);
-    b->d_items = nullptr;
     BCK(b, cudaMalloc(&b->d_items, sizeof(WorkItem) * std::max<size_t>(items.size(), 1)));
     BCK(b, cudaMemcpy(b->d_items, items.data(), sizeof(WorkItem) * items.size(),
                       cudaMemcpyHostToDevice));
-    b->nitems = (int)items.size();
-    b->ngroups = (int)groups.size();
-    if (b->ngroups) {
+    if (!groups.empty()) {
         BCK(b, cudaMalloc(&b->d_groups, sizeof(SplitGroup) * groups.size()));
         BCK(b, cudaMemcpy(b->d_groups, groups.data(), sizeof(SplitGroup) * groups.size(),
                           cudaMemcpyHostToDevice));
     }
+    b->nitems = (int)items.size();
+    b->ngroups = (int)groups.size();
     b->grid = b->num_sms * batch_blocks_per_sm(b->cfg.variant, b->threads);
     return NB_OK;
 }
 
-void drop_graph(nb_batch b)
-{
-    if (b->gexec) cudaGraphExecDestroy(b->gexec);
-    if (b->graph) cudaGraphDestroy(b->graph);
-    b->gexec = nullptr;
-    b->graph = nullptr;
-}
+// The work list is there: built again where an earlier attempt (the autotuner's) failed.
+int ensure_items(nb_batch b) { return b->nitems ? NB_OK : build_items(b); }
 
 // The batched force: the items, then the sums of the split systems.
 cudaError_t batch_force(nb_batch b)
@@ -246,6 +253,8 @@ cudaError_t batch_force(nb_batch b)
 
 int launch_batch_force(nb_batch b)
 {
+    const int rc = ensure_items(b);
+    if (rc) return rc;
     BCK(b, batch_force(b));
     return NB_OK;
 }
@@ -282,6 +291,8 @@ int binit(nb_batch b)
 int capture_step(nb_batch b)
 {
     drop_graph(b);
+    const int rc = ensure_items(b);
+    if (rc) return rc;
     StateDev s = bstate(b);
     const StepParams p = bparams(b);
     BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
@@ -582,7 +593,6 @@ int nb_batch_autotune(nb_batch b, int *threads)
     b->threads = best_t;
     int rc = build_items(b);
     if (rc) return rc;
-    drop_graph(b);
     if (threads) *threads = best_t;
     return check_berr(b);
 }

@@ -69,3 +69,18 @@ def test_partials_of_a_large_system_are_bounded(nb):
     used = free - torch.cuda.mem_get_info(0)[0]
     nb.nb_batch_destroy(b)
     assert used < 192 << 20
+
+
+def test_autotune_between_steps(nb):
+    """The autotuner rebuilds the lists after a step was captured: the next step is captured anew."""
+    systems = [ic.plummer(n, 80 + k) for k, n in enumerate((70, 900, 1100, 2500))]
+    eps = np.full(4, 0.05)
+    got = []
+    for tune in (False, True):
+        with nb.Batch(systems, eps, DT, variant="f32ds", device=0) as b:
+            b.step(2)
+            if tune:
+                b.autotune()
+            b.step(2)
+            got.append(b.get()[:2])
+    np.testing.assert_array_equal(got[0], got[1])
