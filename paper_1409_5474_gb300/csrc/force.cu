@@ -1508,8 +1508,9 @@ ForcePlan plan_from_entry(const nb_plan &e, int variant, int n_i, int n_j)
         p.nwj = (e.nwj == 4 || e.nwj == 8) ? e.nwj : 1;
         p.ipt = tile_ipt(n_i, p.nwj);
     }
+    // FP64 units are 16 records: above 2^20 of them there are more than a grid has rows (65535)
     const int ntiles = (n_j + p.jt - 1) / p.jt;
-    p.nsplit = (int)clampll(e.nsplit, 1, ntiles);
+    p.nsplit = (int)clampll(e.nsplit, 1, variant == NB_F64 && ntiles > 65535 ? 65535 : ntiles);
     return p;
 }
 
