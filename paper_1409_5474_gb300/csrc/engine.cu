@@ -272,12 +272,28 @@ ISet due_set(nb_handle h, int n_a)
 
 bool timing(nb_handle h) { return (h->cfg.flags & NB_FLAG_TIMING) != 0; }
 
+// Give back the split partials' scratch: the plans take what room there is at the next
+// evaluation, so nothing else is refused because of it.
+cudaError_t give_back_part(nb_handle h)
+{
+    const cudaError_t e = cudaStreamSynchronize(h->stream);
+    cudaFree(h->part);
+    h->part = nullptr;
+    h->bytes -= h->part_cap * sizeof(double);
+    h->part_cap = 0;
+    return e;
+}
+
 // Grow a device buffer (synchronising first so no kernel still uses it).
 template <typename T>
 int grow(nb_handle h, T **buf, size_t *cap, size_t need)
 {
     if (need <= *cap) return NB_OK;
     size_t want = std::max(need, *cap * 2);
+    const bool others = (void *)buf != (void *)&h->part && h->part_cap > 0;
+    if (others && h->cfg.budget_bytes &&
+        h->bytes + (need - *cap) * sizeof(T) > h->cfg.budget_bytes)
+        CK(h, give_back_part(h));
     const size_t add = want * sizeof(T) - *cap * sizeof(T);
     if (h->cfg.budget_bytes && h->bytes + add > h->cfg.budget_bytes) {
         want = need;
@@ -294,7 +310,13 @@ int grow(nb_handle h, T **buf, size_t *cap, size_t need)
         *cap = 0;
     }
     T *p = nullptr;
-    if (cudaMalloc(&p, want * sizeof(T)) != cudaSuccess) {
+    bool got = cudaMalloc(&p, want * sizeof(T)) == cudaSuccess;
+    if (!got && others && h->part_cap > 0) {
+        cudaGetLastError();
+        CK(h, give_back_part(h));
+        got = cudaMalloc(&p, want * sizeof(T)) == cudaSuccess;
+    }
+    if (!got) {
         cudaGetLastError();
         return fail(h, NB_ERR_OOM, "cudaMalloc of %zu bytes failed", want * sizeof(T));
     }
@@ -364,6 +386,22 @@ static long long blocks_of(const ForcePlan &p, int variant, int n_i)
     return (n_i + ib - 1) / ib;
 }
 
+// Whether the plan table has an entry of its own for n_i i-particles.
+bool table_plan(nb_handle h, int variant, int n_i)
+{
+    return h->plans[bucket_of(n_i)].kind >= 0 && variant == h->cfg.variant;
+}
+
+// Doubles that the partials of a built-in plan may take: what the handle's budget leaves
+// beside the split counters.
+size_t part_room(nb_handle h)
+{
+    if (!h->cfg.budget_bytes) return SIZE_MAX;
+    const size_t held = h->bytes + (h->split_cnt ? 0 : 64 * sizeof(unsigned));
+    const size_t left = h->cfg.budget_bytes > held ? h->cfg.budget_bytes - held : 0;
+    return h->part_cap + left / sizeof(double);
+}
+
 ForcePlan plan_for(nb_handle h, int variant, int n_i)
 {
     const int b = bucket_of(n_i);
@@ -384,7 +422,18 @@ ForcePlan plan_for(nb_handle h, int variant, int n_i)
         }
         return p;
     }
-    return plan_force(variant, n_i, h->n, h->num_sms);
+    return plan_force(variant, n_i, h->n, h->num_sms, part_room(h));
+}
+
+// The plan of an evaluation, with its scratch. A built-in plan makes do with one split where
+// the device has no memory for the partials (a table entry fails).
+int plan_with_scratch(nb_handle h, int variant, int n_i, ForcePlan *p)
+{
+    *p = plan_for(h, variant, n_i);
+    const int rc = ensure_part(h, *p, n_i);
+    if (rc != NB_ERR_OOM || table_plan(h, variant, n_i)) return rc;
+    *p = plan_force(variant, n_i, h->n, h->num_sms, 0);
+    return ensure_part(h, *p, n_i);
 }
 
 nb_plan entry_of(const ForcePlan &p)
@@ -403,7 +452,10 @@ int run_force_plan(nb_handle h, int variant, const ForcePlan &p, const ISet &is,
 int run_force(nb_handle h, int variant, const ISet &is, Out3 out)
 {
     if (is.n <= 0) return NB_OK;
-    return run_force_plan(h, variant, plan_for(h, variant, is.n), is, out);
+    ForcePlan p;
+    const int rc = plan_with_scratch(h, variant, is.n, &p);
+    if (rc) return rc;
+    return run_force_plan(h, variant, p, is, out);
 }
 
 int run_force_plan(nb_handle h, int variant, const ForcePlan &p, const ISet &is, Out3 out)
@@ -582,7 +634,12 @@ ForcePlan plan_for6(nb_handle h, int variant, int n_i)
         }
         return plan6_from_entry(variant, use.nwj, use.nsplit, n_i, h->n);
     }
-    return plan_force6(variant, n_i, h->n, h->num_sms);
+    return plan_force6(variant, n_i, h->n, h->num_sms, part_room(h));
+}
+
+int ensure_part6(nb_handle h, const ForcePlan &p, int n_i)
+{
+    return grow(h, &h->part, &h->part_cap, std::max<size_t>(plan6_partial_doubles(p, n_i), 1));
 }
 
 int run_force6_plan(nb_handle h, int variant, const ForcePlan &p, const int *idx_dev, int n_i,
@@ -593,14 +650,20 @@ int run_force6_plan(nb_handle h, int variant, const ForcePlan &p, const int *idx
 int run_force6(nb_handle h, int variant, const int *idx_dev, int n_i, const Out6 &out)
 {
     if (n_i <= 0) return NB_OK;
-    return run_force6_plan(h, variant, plan_for6(h, variant, n_i), idx_dev, n_i, out);
+    ForcePlan p = plan_for6(h, variant, n_i);
+    const int rc = ensure_part6(h, p, n_i);
+    if (rc == NB_ERR_OOM && !table_plan(h, variant, n_i))
+        p = plan_force6(variant, n_i, h->n, h->num_sms, 0);
+    else if (rc)
+        return rc;
+    return run_force6_plan(h, variant, p, idx_dev, n_i, out);
 }
 
 int run_force6_plan(nb_handle h, int variant, const ForcePlan &p, const int *idx_dev, int n_i,
                     const Out6 &out)
 {
     if (n_i <= 0) return NB_OK;
-    int rc = grow(h, &h->part, &h->part_cap, std::max<size_t>(plan6_partial_doubles(p, n_i), 1));
+    int rc = ensure_part6(h, p, n_i);
     if (rc) return rc;
     cudaEvent_t ev[4];
     cudaEvent_t *evp = nullptr;
@@ -843,7 +906,11 @@ bool fused_ready(nb_handle h)
         const size_t part = fused_part_float2s(g, NB_FUSED_MAX_NA, h->cfg.order);
         const size_t add =
             part * sizeof(float2) + fused_cnt_ints(g) * sizeof(int) + 256 + sizeof(FusedStats);
-        if (h->cfg.budget_bytes && h->bytes + add > h->cfg.budget_bytes) return false;
+        if (h->cfg.budget_bytes && h->bytes + add > h->cfg.budget_bytes) {
+            if (h->bytes - h->part_cap * sizeof(double) + add > h->cfg.budget_bytes ||
+                give_back_part(h) != cudaSuccess)
+                return false;
+        }
         if (cudaMalloc(&h->fused_part, part * sizeof(float2)) != cudaSuccess ||
             cudaMalloc(&h->fused_cnt, fused_cnt_ints(g) * sizeof(int)) != cudaSuccess ||
             cudaMalloc(&h->fused_bar, 256) != cudaSuccess ||
@@ -1007,8 +1074,8 @@ int handle_force(nb_handle h, int n_i, bool due, double eps2, unsigned *err, cud
     if (n_i <= 0) return NB_OK;
     const int variant = h->cfg.variant;
     const ISet is = due ? due_set(h, n_i) : members_of(h, nullptr, n_i);
-    const ForcePlan p = plan_for(h, variant, n_i);
-    int rc = ensure_part(h, p, n_i);
+    ForcePlan p;
+    const int rc = plan_with_scratch(h, variant, n_i, &p);
     if (rc) return rc;
     const Out3 out{h->f_acc, h->f_jerk, h->f_pot, h->ld};
     if (launch_force(variant, p, jset_of(h), is, eps2, h->part, counters_of(h, variant), out, err,

@@ -36,6 +36,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 
 #include "nb_internal.cuh"
 #include "ds.cuh"
@@ -1363,6 +1364,16 @@ static long long clampll(long long v, long long lo, long long hi)
     return v < lo ? lo : (v > hi ? hi : v);
 }
 
+// Whether the split count ns of a plan search is to be tried: not the one before it (last)
+// again, and none whose partials do not fit; where the first does not, the most that fit.
+bool splits_fit(long long fit, long long &last, long long &ns)
+{
+    if (ns > fit && last == 0) ns = fit > 1 ? fit : 1;
+    if (ns == last || (ns > fit && ns > 1)) return false;
+    last = ns;
+    return true;
+}
+
 // Tiny-set layout (FP32 kind 2): ipt i-particles per pass, jt = j per thread;
 // one j-split per CTA of 256 threads.
 static void tiny_shape(int n_i, int n_j, ForcePlan &p)
@@ -1378,10 +1389,12 @@ static void tiny_shape(int n_i, int n_j, ForcePlan &p)
 // warp column of eight warp rows (16 of 262144: 24.2 against 32.8 us).
 static int tile_ipt(int n_i, int nwj) { return nwj == 8 && n_i <= 32 ? 1 : 2; }
 
-ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms)
+ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms, size_t max_part)
 {
     ForcePlan p{};
     p.nwj = 1;
+    // the most splits whose partials (7 doubles an i-particle each) fit
+    const long long fit = (long long)std::min<size_t>(max_part / (7 * (size_t)n_i), 1 << 20);
     if (variant == NB_F64) {
         // j-parallel below 32 i-particles where it is faster: a pass over the j-set for
         // every four (1 us for each pair of a lane, and the lanes' sums), one j per lane while
@@ -1390,10 +1403,11 @@ ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms)
         // 4 of 20011 39.5 -> 21.0 us, 32 of 20011 265 -> 52 us (tiles).
         if (n_i <= 32) {
             const long long ns = clampll((n_j + 127LL) / 128, 1, 2LL * num_sms);
+            const bool room = ns == 1 || ns <= fit;
             const double passes = (double)((n_i + 3) / 4);
             const double per_sm = (double)((n_j + 128LL * num_sms - 1) / (128LL * num_sms));
             const double pass = per_sm * (double)(n_i < 4 ? n_i : 4) + 3.0;
-            if (passes * pass <= (double)n_j / (4.0 * num_sms) + 5.0) {
+            if (room && passes * pass <= (double)n_j / (4.0 * num_sms) + 5.0) {
                 p.kind = 1;
                 p.ipt = n_i <= 1 ? 1 : n_i <= 2 ? 2 : 4;
                 p.threads = 128;
@@ -1413,10 +1427,9 @@ ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms)
         double best = 1e300;
         long long last = 0;
         for (const int per_sm : {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 24, 32, 48}) {
-            const long long ns = clampll((long long)per_sm * num_sms / nblk, 1,
-                                         nunits < 512 ? nunits : 512);
-            if (ns == last) continue;
-            last = ns;
+            long long ns = clampll((long long)per_sm * num_sms / nblk, 1,
+                                   nunits < 512 ? nunits : 512);
+            if (!splits_fit(fit, last, ns)) continue;
             const long long on_sm = (nblk * ns + num_sms - 1) / num_sms;
             const long long units = (nunits + ns - 1) / ns;
             const double t = ((double)on_sm + (on_sm == 1 ? 0.15 : 0.0)) * (double)units * 4.0 +
@@ -1435,7 +1448,7 @@ ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms)
     // against 7.6, 8 of 65536 9.9 against 9.7, 8 of 262144 14.8 against 18.6.
     if (n_i <= (n_j > 65536 ? 8 : 4)) {
         tiny_shape(n_i, n_j, p);
-        return p;
+        if (p.nsplit == 1 || p.nsplit <= fit) return p;
     }
     // Tiles: the warp rows (8, 4 or 1: 64, 128 or 512 i-particles per CTA) and j-splits of
     // least estimated time. An SM's CTAs share its pipes, so its time is its count of CTAs
@@ -1458,10 +1471,9 @@ ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms)
         const double t_tile = nwj == 8 ? 2.57 : (nwj == 4 ? 4.97 : 18.8);
         long long last = 0;
         for (const int per_sm : {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 14, 16, 20, 24, 32, 40, 48}) {
-            const long long ns =
+            long long ns =
                 clampll((long long)per_sm * num_sms / nblk, 1, ntiles < 512 ? ntiles : 512);
-            if (ns == last) continue;
-            last = ns;
+            if (!splits_fit(fit, last, ns)) continue;
             const long long on_sm = (nblk * ns + num_sms - 1) / num_sms;
             const long long tiles = (ntiles + ns - 1) / ns;
             const double alone = on_sm % 2 ? 0.10 : 0.04;
@@ -1816,13 +1828,8 @@ int batch_blocks_per_sm(int variant, int threads)
 
 size_t plan_counters(const ForcePlan &p, int n_i)
 {
-    if (p.nsplit <= 1) return 1;
-    if (p.kind == 2) return 1;
-    long long ib;
-    if (p.kind == 1)
-        ib = (long long)(p.threads / 32) * p.ipt;  // FP32 warp groups (FP64 j-parallel: one)
-    else
-        ib = (long long)(p.threads / p.nwj) * p.ipt;
+    if (p.nsplit <= 1 || p.kind != 1) return 1;
+    const long long ib = (long long)(p.threads / 32) * p.ipt;  // FP32 warp groups (FP64: one)
     return (size_t)((n_i + ib - 1) / ib);
 }
 

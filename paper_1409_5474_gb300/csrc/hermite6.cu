@@ -575,9 +575,12 @@ cudaError_t launch_predict6(const StateDev &s, double t, bool want_rec, unsigned
 // -> 207; 300 of 2500 18.8 -> 8.1.
 // FP64: at least two waves of resident CTAs, then the fewest splits, up to eight times that
 // many, whose last wave is at least 97% full, else the fullest.
-ForcePlan plan_force6(int variant, int n_i, int n_j, int num_sms)
+ForcePlan plan_force6(int variant, int n_i, int n_j, int num_sms, size_t max_part)
 {
     ForcePlan p{};
+    // the most splits whose partials (H6_VALS doubles an i-particle each) fit
+    const long long fit = std::max<long long>(
+        1, (long long)std::min<size_t>(max_part / (H6_VALS * (size_t)n_i), 1 << 20));
     p.kind = 0;
     p.nwj = 1;
     p.ipt = 1;  // the packed pair terms already give each thread two j per step
@@ -592,10 +595,8 @@ ForcePlan plan_force6(int variant, int n_i, int n_j, int num_sms)
             const double t_tile = nwj == 8 ? 1.55 : (nwj == 4 ? 2.6 : (nwj == 2 ? 4.7 : 8.7));
             long long last = 0;
             for (const int per_sm : {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 14, 16, 20, 24, 32, 40, 48}) {
-                const long long ns =
-                    std::max(1LL, std::min({per_sm * sms / nblk, ntiles, 512LL}));
-                if (ns == last) continue;
-                last = ns;
+                long long ns = std::max(1LL, std::min({per_sm * sms / nblk, ntiles, 512LL}));
+                if (!splits_fit(fit, last, ns)) continue;
                 const long long on_sm = (nblk * ns + sms - 1) / sms;
                 const bool big = plan6_jt(nwj, (int)ns, n_j) == H6_JT_BIG;
                 const long long tiles =
@@ -620,7 +621,7 @@ ForcePlan plan_force6(int variant, int n_i, int n_j, int num_sms)
     p.jt = H6_JT64;
     const long long nblk = (n_i + p.threads - 1) / p.threads;
     const long long ntiles = (n_j + p.jt - 1) / p.jt;
-    const long long cap = std::max(1LL, ntiles / 4);
+    const long long cap = std::min(fit, std::max(1LL, ntiles / 4));
     const long long slots = 4 * sms;
     const long long ns0 = std::min(cap, std::max(1LL, (2 * slots + nblk - 1) / nblk));
     long long best = ns0;

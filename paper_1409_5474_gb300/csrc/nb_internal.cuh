@@ -117,8 +117,9 @@ struct ForcePlan {
     int nwj;      // warp rows sharing each j-tile (FP32 tile kind)
 };
 
-// Choose a plan for n_i i-particles against n_j j-particles.
-ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms);
+// Choose a plan for n_i i-particles against n_j j-particles whose partial sums take at most
+// max_part doubles (0: one split).
+ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms, size_t max_part = SIZE_MAX);
 
 // A plan from a plan-table entry (kind 0 or 1; sizes clamped to the sets).
 ForcePlan plan_from_entry(const nb_plan &e, int variant, int n_i, int n_j);
@@ -126,11 +127,15 @@ ForcePlan plan_from_entry(const nb_plan &e, int variant, int n_i, int n_j);
 // Resident CTAs per SM of the FP32 / double-single tile kernel with nwj warp rows.
 int tile_blocks_per_sm(int variant, int nwj);
 
+// Whether a plan search tries ns splits (fit: the most whose partials fit; last: the count
+// before, 0 at first).
+bool splits_fit(long long fit, long long &last, long long &ns);
+
 // Scratch doubles the plan needs for partial sums (0 when nsplit == 1).
 size_t plan_partial_doubles(const ForcePlan &p, int n_i);
 
-// Counters the split reduction needs: one per i-block (zero at allocation;
-// every launch leaves them at zero again).
+// Counters the split reduction needs: one per i-block of the warp groups, one in all for the
+// tiny sets, none for the tiles (zero at allocation; every launch leaves them at zero again).
 size_t plan_counters(const ForcePlan &p, int n_i);
 
 // Launch K2 and, when nsplit > 1, K3: the CTAs write their partial sums to part
@@ -370,8 +375,8 @@ struct Out6 {
 cudaError_t launch_predict6(const StateDev &s, double t, bool want_rec, unsigned *err,
                             cudaStream_t st);
 
-// Plan of a 6th-order evaluation: CTA shape and j-splits.
-ForcePlan plan_force6(int variant, int n_i, int n_j, int num_sms);
+// Plan of a 6th-order evaluation: CTA shape and j-splits (max_part as plan_force).
+ForcePlan plan_force6(int variant, int n_i, int n_j, int num_sms, size_t max_part = SIZE_MAX);
 // The 6th-order plan of a plan-table entry (kind 0: warp rows nwj, nsplit j-splits), and
 // the resident CTAs per SM of the F32 / double-single tile kernel with nwj warp rows.
 ForcePlan plan6_from_entry(int variant, int nwj, int nsplit, int n_i, int n_j);
