@@ -124,6 +124,7 @@ struct nb_handle_s {
     // growable scratch
     double *part = nullptr;
     size_t part_cap = 0;  // doubles
+    bool part_in_slab = false;  // the room nb_create set aside (part_reserve), not grown yet
     unsigned *split_cnt = nullptr;  // per-i-block counters of the folded split reduction
     size_t split_cnt_cap = 0;
     double *io = nullptr; // host-API staging: [7][n_i] outputs, ext inputs
@@ -290,7 +291,8 @@ int grow(nb_handle h, T **buf, size_t *cap, size_t need)
 {
     if (need <= *cap) return NB_OK;
     size_t want = std::max(need, *cap * 2);
-    const bool others = (void *)buf != (void *)&h->part && h->part_cap > 0;
+    const bool is_part = (void *)buf == (void *)&h->part;
+    const bool others = !is_part && h->part_cap > 0 && !h->part_in_slab;
     if (others && h->cfg.budget_bytes &&
         h->bytes + (need - *cap) * sizeof(T) > h->cfg.budget_bytes)
         CK(h, give_back_part(h));
@@ -303,6 +305,19 @@ int grow(nb_handle h, T **buf, size_t *cap, size_t need)
                         want * sizeof(T), h->cfg.budget_bytes);
     }
     CK(h, cudaStreamSynchronize(h->stream));
+    if (is_part && h->part_in_slab) {
+        // the room in the slab stays where it is, and in use if there is no more
+        T *more = nullptr;
+        if (cudaMalloc(&more, want * sizeof(T)) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(h, NB_ERR_OOM, "cudaMalloc of %zu bytes failed", want * sizeof(T));
+        }
+        *buf = more;
+        *cap = want;
+        h->bytes += want * sizeof(T);
+        h->part_in_slab = false;
+        return NB_OK;
+    }
     if (*buf) {
         cudaFree(*buf);
         h->bytes -= *cap * sizeof(T);
@@ -425,14 +440,14 @@ ForcePlan plan_for(nb_handle h, int variant, int n_i)
     return plan_force(variant, n_i, h->n, h->num_sms, part_room(h));
 }
 
-// The plan of an evaluation, with its scratch. A built-in plan makes do with one split where
-// the device has no memory for the partials (a table entry fails).
+// The plan of an evaluation, with its scratch. A built-in plan makes do with the splits there is
+// room for where the device has no memory for the partials (a table entry fails).
 int plan_with_scratch(nb_handle h, int variant, int n_i, ForcePlan *p)
 {
     *p = plan_for(h, variant, n_i);
     const int rc = ensure_part(h, *p, n_i);
     if (rc != NB_ERR_OOM || table_plan(h, variant, n_i)) return rc;
-    *p = plan_force(variant, n_i, h->n, h->num_sms, 0);
+    *p = plan_force(variant, n_i, h->n, h->num_sms, h->part_cap);
     return ensure_part(h, *p, n_i);
 }
 
@@ -653,7 +668,7 @@ int run_force6(nb_handle h, int variant, const int *idx_dev, int n_i, const Out6
     ForcePlan p = plan_for6(h, variant, n_i);
     const int rc = ensure_part6(h, p, n_i);
     if (rc == NB_ERR_OOM && !table_plan(h, variant, n_i))
-        p = plan_force6(variant, n_i, h->n, h->num_sms, 0);
+        p = plan_force6(variant, n_i, h->n, h->num_sms, h->part_cap);
     else if (rc)
         return rc;
     return run_force6_plan(h, variant, p, idx_dev, n_i, out);
@@ -1140,7 +1155,29 @@ const char *nb_last_error(nb_handle h)
 
 const char *nb_version(void) { return "nbody-gb300 0.1 (sm_103a)"; }
 
-int nb_create(const nb_config *cfg, nb_handle *out)
+int nb_create(const nb_config *cfg, nb_handle *out) { return create_handle(cfg, true, out); }
+
+}  // extern "C"
+
+namespace nb {
+
+// FP32 evaluations at order 4 take 7 float2 an i-particle and split, and a split has a tile of
+// 256 records or more. A buffer of 1 MB and more is allocated by a mapping of its own, some 95 us
+// with the wait for the stream, which is more than a fine split saves a short evaluation: the
+// first force of a handle on 1531 of 65536 took 236 us (217 with the coarse split that 0.3 MB
+// were enough for), on 8192 of 8192 201 (147). So those handles set room for the partials
+// aside in their slab, which costs no allocation: 149 and 111 us. Evaluations that need more
+// than 16 MB (three CTAs of 512 i-particles on every SM need 13) take longer than the
+// allocation.
+size_t part_reserve(const nb_config &c)
+{
+    if (c.variant == NB_F64 || c.order == 6 || c.budget_bytes) return 0;
+    const size_t n = (size_t)c.n_max, tiles = (n + 255) / 256;
+    const size_t need = 7 * sizeof(float2) * n * std::min<size_t>(tiles, 512);
+    return need < (1u << 20) ? 0 : align256(std::min<size_t>(need, 16u << 20));
+}
+
+int create_handle(const nb_config *cfg, bool reserve, nb_handle *out)
 {
     if (!cfg || !out) return fail(nullptr, NB_ERR_ARG, "cfg and out must not be NULL");
     *out = nullptr;
@@ -1218,13 +1255,25 @@ int nb_create(const nb_config *cfg, nb_handle *out)
         return fail(nullptr, NB_ERR_CUDA, "cudaStreamCreate failed");
     }
     h->stream = h->own_stream;
-    if (cudaMalloc(&h->slab, h->slab_bytes) != cudaSuccess) {
+    size_t room = reserve ? part_reserve(h->cfg) : 0;
+    bool got = cudaMalloc(&h->slab, h->slab_bytes + room) == cudaSuccess;
+    if (!got && room > 0) {
+        cudaGetLastError();
+        room = 0;
+        got = cudaMalloc(&h->slab, h->slab_bytes) == cudaSuccess;
+    }
+    if (!got) {
         cudaGetLastError();
         int code = fail(nullptr, NB_ERR_OOM, "cudaMalloc of %zu bytes failed", h->slab_bytes);
         bail(code);
         return code;
     }
-    h->bytes = h->slab_bytes;
+    h->bytes = h->slab_bytes + room;
+    if (room > 0) {
+        h->part = reinterpret_cast<double *>(static_cast<char *>(h->slab) + h->slab_bytes);
+        h->part_cap = room / sizeof(double);
+        h->part_in_slab = true;
+    }
     char *p = static_cast<char *>(h->slab);
     auto take = [&](size_t b) {
         char *q = p;
@@ -1291,6 +1340,10 @@ int nb_create(const nb_config *cfg, nb_handle *out)
     return NB_OK;
 }
 
+}  // namespace nb
+
+extern "C" {
+
 int nb_destroy(nb_handle h)
 {
     if (!h) return NB_OK;
@@ -1298,7 +1351,7 @@ int nb_destroy(nb_handle h)
     if (h->stream) cudaStreamSynchronize(h->stream);
     h->timer.harvest();
     cudaFree(h->slab);
-    cudaFree(h->part);
+    if (!h->part_in_slab) cudaFree(h->part);
     cudaFree(h->split_cnt);
     cudaFree(h->io);
     cudaFree(h->d_idx);

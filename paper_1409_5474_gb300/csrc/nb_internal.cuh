@@ -519,6 +519,10 @@ struct HandleView {
     int n, cap;
 };
 void handle_view(nb_handle h, HandleView *v);
+// nb_create; reserve: with the room for split partials that a handle of its own sets aside
+// (part_reserve bytes).
+int create_handle(const nb_config *cfg, bool reserve, nb_handle *out);
+size_t part_reserve(const nb_config &c);
 size_t handle_bytes(nb_handle h);
 // Epoch of the next scheduler launch on h (advances the handle's mirror).
 unsigned long long handle_take_epoch(nb_handle h);

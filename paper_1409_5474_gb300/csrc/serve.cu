@@ -194,7 +194,9 @@ nb_handle acquire_handle(nb_server s, int cap, size_t *bytes)
     c.dt_max = s->cfg.dt_max;
     c.device = s->dev;
     nb_handle h = nullptr;
-    if (nb_create(&c, &h) != NB_OK) return nullptr;
+    // the handles' room for partials comes after what requests are admitted by
+    const bool reserve = s->bytes_in_use + need + part_reserve(c) <= s->cfg.budget_bytes / 2;
+    if (create_handle(&c, reserve, &h) != NB_OK) return nullptr;
     nb_set_stream(h, s->stream);
     *bytes = handle_bytes(h);
     s->bytes_in_use += *bytes;
