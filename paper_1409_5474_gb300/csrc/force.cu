@@ -223,7 +223,7 @@ __device__ __forceinline__ int member_index(const ISet &is, int k, unsigned *err
 
 __host__ __device__ constexpr bool tile_ahead(int nwj) { return nwj == 8; }
 
-template <int VAR, int IPT, int NWI, int NWJ, int JT, int NS>
+template <int VAR, int IPT, int NWI, int NWJ, int JT, int NS, int RUN>
 __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     k_force_tile32(const float4 *jrec, int nj, ISet is, float eps2f, int ntiles, double *part,
                    long long pld, Out3 out, unsigned *err)
@@ -237,11 +237,12 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     constexpr bool DS = (VAR == NB_F32DS);
     constexpr int NT = 32 * NWI * NWJ;
     constexpr int IB = 32 * NWI * IPT;
-    // tiles per FP32 partial sum: 64 terms in each half of a packed sum between folds (128
-    // with one warp row, a tile's): for 1531 of 65536 the jerk is 2.3e-7 off (64 bits,
-    // geometric mean over 14 systems), 2.4e-7 with the 32-term sums of the scalar warp groups
-    // that took those sets before; 128 terms 127.2 us, 64 129.0, 32 130.3.
-    constexpr int FOLD = (128 * NWJ / JT) > 1 ? (128 * NWJ / JT) : 1;
+    // pairs that a warp row takes of a tile; a run ends with a tile, or several of them
+    // make up a tile (of RUNS each)
+    constexpr int ROW = JT / 2 / NWJ;
+    constexpr int FOLD = RUN > ROW ? RUN / ROW : 1;
+    constexpr int RUNS = RUN < ROW ? ROW / RUN : 1;
+    constexpr int JR = JT / RUNS;  // records of a run, of all warp rows
     constexpr int PAIRS = JT * DS_REC;  // float4 of a pair buffer
     constexpr bool AHEAD = tile_ahead(NWJ);
     float4 *s_pair = s_tile + (size_t)NS * PAIRS;
@@ -345,15 +346,17 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
         own = __any_sync(0xffffffffu, own);
 
         const bool masked = own || cnt < JT;
-        if (idle)
-            ;  // no slot of this warp is written
-        else if (soft)
-            tile_pairs<DS, IPT, JT, true>(pairs, wj, NWJ, jbase, cnt, masked, ip, iid, e2, ts);
-        else
-            tile_pairs<DS, IPT, JT, false>(pairs, wj, NWJ, jbase, cnt, masked, ip, iid, e2, ts);
+#pragma unroll 1
+        for (int f = 0; f < cnt && !idle; f += JR) {  // idle: no slot of this warp is written
+            const float4 *P = pairs + DS_REC * f;
+            const int fcnt = min(JR, cnt - f);
+            if (soft)
+                tile_pairs<DS, IPT, JR, true>(P, wj, NWJ, jbase + f, fcnt, masked, ip, iid, e2, ts);
+            else
+                tile_pairs<DS, IPT, JR, false>(P, wj, NWJ, jbase + f, fcnt, masked, ip, iid, e2, ts);
 
-        // fold the FP32 partial sums (both lanes) into the running totals
-        if ((kt + 1) % FOLD == 0 || kt + 1 == my_tiles) {
+            // fold the FP32 partial sums (both lanes) into the running totals
+            if (FOLD > 1 && (kt + 1) % FOLD != 0 && kt + 1 != my_tiles) continue;
 #pragma unroll
             for (int p = 0; p < IPT; ++p) {
 #pragma unroll
@@ -1347,6 +1350,19 @@ __global__ void __launch_bounds__(NT, 512 / NT)
 constexpr int JT32 = 128;    // j-tile of the batched items
 constexpr int JT_TILE = 256;  // j-tile of the tile kernel
 constexpr int NS32 = 3;
+
+// Runs of the tile kernel: the terms of each half of a packed FP32 sum before the two halves
+// are folded into the running totals. Sets of fewer than 4096 i-particles (every due set but the
+// largest) took the scalar warp groups once, whose lanes fold after 32 terms, and are to be as
+// accurate: the median jerk error for 2516 of 65536 is 1.79e-7 with runs of 16 (64 bits; Plummer
+// sphere with a mass spectrum), 1.89e-7 with 32, 2.4e-7 with 128, and 1.89e-7 by the warp
+// groups; for 1531 1.80e-7, 1.89e-7, 2.04e-7 (64) and 1.88e-7. The folds cost 132.6 us for 1531
+// (32: 125.8, 64: 123.4; the warp groups 184), 203 for 2516 (32: 195, 128: 189; 411). Larger sets
+// were taken by this kernel with runs of 128 (one warp row) and are not less accurate.
+constexpr int TILE_FINE_NI = 4096;
+constexpr int RUN_FINE = 16;
+constexpr int RUN_ROWS = 64;   // larger sets, several warp rows
+constexpr int RUN_WHOLE = 128;  // larger sets, one warp row: a tile
 constexpr int JT64 = 64;
 constexpr int NS64 = 3;
 
@@ -1554,12 +1570,12 @@ static constexpr size_t tile_smem()
            (size_t)NT * 14 * sizeof(float2);
 }
 
-template <int VAR, int IPT, int NWI, int NWJ>
+template <int VAR, int IPT, int NWI, int NWJ, int RUN>
 static cudaError_t go_tile32(const JSet &js, const ISet &is, float eps2f, int nsplit,
                              double *part, Out3 out, unsigned *err,
                              cudaStream_t st)
 {
-    constexpr auto kern = k_force_tile32<VAR, IPT, NWI, NWJ, JT_TILE, NS32>;
+    constexpr auto kern = k_force_tile32<VAR, IPT, NWI, NWJ, JT_TILE, NS32, RUN>;
     constexpr int NT = 32 * NWI * NWJ;
     constexpr int IB = 32 * NWI * IPT;
     const size_t smem = tile_smem<NT, NWJ>();
@@ -1640,14 +1656,12 @@ static cudaError_t dispatch32(const ForcePlan &p, const JSet &js, const ISet &is
         default: return go_wgrp32<VAR, 2, 8>(js, is, eps2f, p.nsplit, part, cnt, out, err, st);
         }
     }
-    switch (p.nwj) {
-    case 1: return go_tile32<VAR, 2, 8, 1>(js, is, eps2f, p.nsplit, part, out, err, st);
-    case 4: return go_tile32<VAR, 2, 2, 4>(js, is, eps2f, p.nsplit, part, out, err, st);
-    default:
-        if (p.ipt == 1)
-            return go_tile32<VAR, 1, 1, 8>(js, is, eps2f, p.nsplit, part, out, err, st);
-        return go_tile32<VAR, 2, 1, 8>(js, is, eps2f, p.nsplit, part, out, err, st);
-    }
+    const bool fine = is.n < TILE_FINE_NI;
+    const auto go = p.nwj == 1   ? (fine ? go_tile32<VAR, 2, 8, 1, RUN_FINE> : go_tile32<VAR, 2, 8, 1, RUN_WHOLE>)
+                    : p.nwj == 4 ? (fine ? go_tile32<VAR, 2, 2, 4, RUN_FINE> : go_tile32<VAR, 2, 2, 4, RUN_ROWS>)
+                    : p.ipt == 1 ? go_tile32<VAR, 1, 1, 8, RUN_FINE>
+                                 : (fine ? go_tile32<VAR, 2, 1, 8, RUN_FINE> : go_tile32<VAR, 2, 1, 8, RUN_ROWS>);
+    return go(js, is, eps2f, p.nsplit, part, out, err, st);
 }
 
 cudaError_t warm_force_jmode64(cudaStream_t st)
@@ -1782,7 +1796,7 @@ static int tile_occ()
 {
     constexpr int NT = 32 * NWI * NWJ;
     const size_t smem = tile_smem<NT, NWJ>();
-    constexpr auto kern = k_force_tile32<VAR, 2, NWI, NWJ, JT_TILE, NS32>;
+    constexpr auto kern = k_force_tile32<VAR, 2, NWI, NWJ, JT_TILE, NS32, NWJ == 1 ? RUN_WHOLE : RUN_ROWS>;
     int nb = 0;
     if (allow_smem<kern>(smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, NT, smem) != cudaSuccess) {
