@@ -565,6 +565,36 @@ cudaError_t launch_predict6(const StateDev &s, double t, bool want_rec, unsigned
 }
 
 
+// The warp rows of sets of 257 to 511 i-particles: of the shapes (and split counts just within
+// one to eight waves of two CTAs an SM, four j-tiles a split at least) the one of least waves x
+// (pairs of a CTA + 16384). A row of eight sums 8 FP32 terms a half between folds, one of four
+// 16, a single one 64, so the rows carry accuracy: this rule laid these sets out before the
+// cost model did, and with the model's rows the median jerk error for 498 of 65536 was 2.08e-7
+// and not 1.74e-7 (64 bits; Plummer sphere with a mass spectrum). The smaller and larger sets' rows
+// are as many as before, or more. 498 of 65536 74.8 -> 107 us (before the model 112), 300 of
+// 2500 7.6 -> 9.2 (18.8).
+int few_waves_rows(int n_i, int n_j, long long sms)
+{
+    const long long ntiles = (n_j + H6_JT - 1) / H6_JT;
+    const long long cap = std::max(1LL, std::min(ntiles / 4, 1024LL)), slots = 2 * sms;
+    int rows = 1;
+    long long best = -1;
+    for (int nwj = 1; nwj <= 8; nwj *= 2) {
+        const long long ib = 32LL * (H6_NWARP / nwj), nblk = (n_i + ib - 1) / ib;
+        for (int k = 0; k <= 9; ++k) {
+            const long long ns =
+                k == 0 ? 1 : (k == 9 ? cap : std::max(1LL, std::min(cap, k * slots / nblk)));
+            const long long jpc = (ntiles + ns - 1) / ns * H6_JT;
+            const long long t = (nblk * ns + slots - 1) / slots * (ib * jpc + 16384);
+            if (best < 0 || t < best) {
+                best = t;
+                rows = nwj;
+            }
+        }
+    }
+    return rows;
+}
+
 // FP32 kinds: the warp rows (8, 4, 2 or 1: 32, 64, 128 or 256 i-particles per CTA) and
 // j-splits of least estimated time, as the 4th-order plan: an SM's count of CTAs (at most
 // ceil(CTAs / SMs)) times the tiles of a split times the SM's time for a tile of that shape,
@@ -573,6 +603,7 @@ cudaError_t launch_predict6(const StateDev &s, double t, bool want_rec, unsigned
 // of a sweep at N = 2500 to 65536, mostly. Against the rule before it (shape by size, two
 // waves) and with the kernel as it was: 130 of 65536 51.5 -> 40 us, 520 127 -> 101, 1531 242
 // -> 207; 300 of 2500 18.8 -> 8.1.
+// Sets of 257 to 511 keep the rows of few_waves_rows.
 // FP64: at least two waves of resident CTAs, then the fewest splits, up to eight times that
 // many, whose last wave is at least 97% full, else the fullest.
 ForcePlan plan_force6(int variant, int n_i, int n_j, int num_sms, size_t max_part)
@@ -588,7 +619,8 @@ ForcePlan plan_force6(int variant, int n_i, int n_j, int num_sms, size_t max_par
     if (variant != NB_F64) {
         const long long ntiles = (n_j + H6_JT - 1) / H6_JT;
         double best = 1e300;
-        for (int nwj = 8; nwj >= 1; nwj /= 2) {
+        const int few = n_i > 256 && n_i < 512 ? few_waves_rows(n_i, n_j, sms) : 0;
+        for (int nwj = few ? few : 8; nwj >= (few ? few : 1); nwj /= 2) {
             const long long ib = 32LL * (H6_NWARP / nwj);
             const long long nblk = (n_i + ib - 1) / ib;
             // microseconds of an SM per 128-record tile

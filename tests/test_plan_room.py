@@ -38,3 +38,15 @@ def test_partials_fit(lib, order, variant, n_j):
             if room >= need:  # room enough: the plan is the free one
                 assert [getattr(p, k) for k, _ in Plan._fields_] == \
                     [getattr(free, k) for k, _ in Plan._fields_]
+
+
+# warp rows of the launch rule before the cost model, as a GB300 gave them
+ROWS = {(2500, 300): 8, (8192, 380): 8, (8192, 498): 8, (20011, 300): 8, (20011, 498): 8,
+        (65536, 300): 4, (65536, 498): 8, (131072, 498): 4}
+
+
+@pytest.mark.parametrize("n_j,n_i", sorted(ROWS))
+def test_order6_rows_of_257_to_511(lib, n_j, n_i):
+    """More rows mean shorter FP32 sums: these sets keep the rows they had."""
+    plan, _ = lib[6]
+    assert plan(1, n_i, n_j, 152, ctypes.c_size_t(-1).value).nwj == ROWS[n_j, n_i]
