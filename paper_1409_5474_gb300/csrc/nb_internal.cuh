@@ -476,10 +476,11 @@ size_t fused_part_float2s(int grid, int na_max, int order);
 cudaError_t launch_selftest_mbar(unsigned *err, unsigned long long limit_ns, cudaStream_t st);
 cudaError_t launch_selftest_barrier(unsigned *bar, unsigned *err, unsigned long long limit_ns,
                                     cudaStream_t st);
-// The same steps (order 4) by one cluster: needs no cnt, bar or part. Ready: the current
-// device can run that cluster.
+// The same steps (order 4) by one cluster: needs no cnt, bar or part. wide: sums beyond short FP32
+// runs in double-single (the request loop; up to FUSED_CLUSTER_LIMIT_N particles, else
+// FUSED_CLUSTER_MAX_N). Ready: the current device can run that cluster.
 bool cluster_steps_ready();
-cudaError_t launch_cluster_steps(const FusedArgs &a, bool ds, cudaStream_t st);
+cudaError_t launch_cluster_steps(const FusedArgs &a, bool ds, bool wide, cudaStream_t st);
 cudaError_t launch_fused_steps(const FusedArgs &a, int grid, bool ds, int order,
                                cudaStream_t st);
 

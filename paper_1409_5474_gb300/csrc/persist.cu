@@ -847,17 +847,27 @@ __global__ void __launch_bounds__(FUSED_THREADS)
 // 4096 particles leaves a tenth: the line of the dispatch.
 constexpr int CL_CTAS = FUSED_CLUSTER;
 constexpr int CL_THREADS = 512;
-constexpr int CL_SLOTS = 1024;                           // due slots per window
 constexpr int CL_Q = 7;                                  // outputs of a slot
 
-// MAXL: the most particles of a CTA.
-template <int MAXL>
+// WIDE: the sums of more than CL_RUN terms a half are double-single from there on, over the lanes
+// and over the CTAs. The request loop's integrations take it: their steps in the ticks add
+// FP32 terms in runs of 32 or 64, and without it a lane's run is all of its pairs (up to 256)
+// and a CTA's partial one FP32 sum of up to 512 terms. The handles' steps do without, as the grid
+// kernel does (FP32 sums of up to 256 terms). One integration of 2500 particles over 1/16
+// time unit 8.3 -> 9.1 ms, of 8000 18.5 -> 19.6 (in the ticks 48 and 70).
+constexpr int CL_RUN = 16;
+
+// MAXL: the most particles of a CTA. A window of the due set has SLOTS slots (the wide
+// partials take twice the room: half as many).
+template <int MAXL, bool WIDE>
 struct ClusterSmem {
+    static constexpr int SLOTS = WIDE ? 512 : 1024;
+    static constexpr int PQ = WIDE ? 4 : 2;  // float4 of a partial: 7 sums, or 7 {hi, lo}
     float4 pair[6][MAXL / 2];              // float4 u of pair q: pair[u][q]
-    float4 part[CL_CTAS][CL_SLOTS / CL_CTAS][2];  // sums by source CTA, slot / CL_CTAS
+    float4 part[CL_CTAS][SLOTS / CL_CTAS][PQ];  // sums by source CTA, slot / CL_CTAS
     float4 own[MAXL][3];                   // own due records: {x_hi, x_lo, v, -} of component c
-    float i[9][CL_SLOTS];                      // due records: x_hi, x_lo, v of three components
-    int id[CL_SLOTS];
+    float i[9][SLOTS];                         // due records: x_hi, x_lo, v of three components
+    int id[SLOTS];
     uint4 due[CL_CTAS][MAXL / 128];        // a bit for every particle of every CTA
     double tn;
     int na;
@@ -897,6 +907,11 @@ __device__ __forceinline__ void cluster_st(uint32_t a, unsigned v)
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
+__device__ __forceinline__ void cluster_st(uint32_t a, float2 v)
+{
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+
 __device__ __forceinline__ void cluster_st(uint32_t a, float4 v)
 {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y),
@@ -905,8 +920,8 @@ __device__ __forceinline__ void cluster_st(uint32_t a, float4 v)
 }
 
 // The float of record value u (0-2 x_hi, 3-5 x_lo, 6-8 v; 9 the mass) of own particle l.
-template <int MAXL>
-__device__ __forceinline__ float *cl_value(ClusterSmem<MAXL> &sm, int u, int l)
+template <int MAXL, bool WIDE>
+__device__ __forceinline__ float *cl_value(ClusterSmem<MAXL, WIDE> &sm, int u, int l)
 {
     const int c = u % 3;
     const int quad = u == 9 ? 1 : 2 * (u / 3) + (c == 2 ? 1 : 0);  // {x y} {z m} of each triple
@@ -924,8 +939,8 @@ __device__ __forceinline__ int cluster_lanes_log2(int nw, int npair)
     return (int)(__reduce_min_sync(0xffffffffu, (unsigned)(cost << 3 | lg)) & 7u);
 }
 
-template <int MAXL>
-__device__ __forceinline__ JPair cluster_pair(const ClusterSmem<MAXL> &sm, int q)
+template <int MAXL, bool WIDE>
+__device__ __forceinline__ JPair cluster_pair(const ClusterSmem<MAXL, WIDE> &sm, int q)
 {
     return JPair{sm.pair[0][q], sm.pair[1][q], sm.pair[2][q],
                  sm.pair[3][q], sm.pair[4][q], sm.pair[5][q]};
@@ -935,20 +950,30 @@ __device__ __forceinline__ JPair cluster_pair(const ClusterSmem<MAXL> &sm, int q
 // pairs sub, sub + S, ... masked: one of the warp's due ones may be among them. Not unrolled: the
 // four warps of a scheduler cover the latencies, and every step runs through this code once
 // (unrolled twice or four times 1 to 3% of a step more).
-template <bool DS, bool SOFT, int MAXL>
-__device__ __forceinline__ void cluster_pairs(const ClusterSmem<MAXL> &sm, int sub, int S, int p0,
-                                              int p1, bool masked, const IPair &ip, int own,
-                                              float2 e2, PairSum &ts)
+template <bool DS, bool SOFT, int MAXL, bool WIDE>
+__device__ __forceinline__ void cluster_pairs(const ClusterSmem<MAXL, WIDE> &sm, int sub, int S,
+                                              int p0, int p1, bool masked, const IPair &ip, int own,
+                                              float2 e2, PairSum &ts, dsf (&v)[CL_Q + 1])
 {
     const int full = (p1 - p0) / 2;
-    if (!masked) {
+    const int run = WIDE ? CL_RUN * S : full;
 #pragma unroll 1
-        for (int q = sub; q < full; q += S)
-            pair_add<DS, SOFT>(cluster_pair(sm, q), ip, e2, ts, NoMask{});
-    } else {
+    for (int f = 0; f < full; f += run) {
+        const int end = WIDE ? min(full, f + run) : full;
+        if (WIDE && f > 0) {
+#pragma unroll
+            for (int c = 0; c < CL_Q; ++c) ds_add(v[c].hi, v[c].lo, pair_total(ts, c));
+            pair_zero(ts);
+        }
+        if (!masked) {
 #pragma unroll 1
-        for (int q = sub; q < full; q += S)
-            pair_add<DS, SOFT>(cluster_pair(sm, q), ip, e2, ts, OwnMask{p0 + 2 * q, own});
+            for (int q = f + sub; q < end; q += S)
+                pair_add<DS, SOFT>(cluster_pair(sm, q), ip, e2, ts, NoMask{});
+        } else {
+#pragma unroll 1
+            for (int q = f + sub; q < end; q += S)
+                pair_add<DS, SOFT>(cluster_pair(sm, q), ip, e2, ts, OwnMask{p0 + 2 * q, own});
+        }
     }
     if (((p1 - p0) & 1) && (full & (S - 1)) == sub)  // the last, half-empty pair
         pair_add<DS, SOFT>(cluster_pair(sm, full), ip, e2, ts, PairMask{p0 + 2 * full, own, p1});
@@ -957,8 +982,8 @@ __device__ __forceinline__ void cluster_pairs(const ClusterSmem<MAXL> &sm, int s
 // B for one window of nw due slots: the sums of every slot over the CTA's particles
 // [p0, p1), left in CTA slot % CL_CTAS; S lanes a slot. One slot a lane: two (half the
 // shared-memory reads) spilled registers, and a step took 0.3 us more.
-template <bool DS, int MAXL>
-__device__ __forceinline__ void cluster_force(ClusterSmem<MAXL> &sm, int nw, int p0, int p1,
+template <bool DS, int MAXL, bool WIDE>
+__device__ __forceinline__ void cluster_force(ClusterSmem<MAXL, WIDE> &sm, int nw, int p0, int p1,
                                               int npair, int rank, float eps2f)
 {
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -974,30 +999,69 @@ __device__ __forceinline__ void cluster_force(ClusterSmem<MAXL> &sm, int nw, int
         const bool masked = __any_sync(0xffffffffu, own >= p0 && own < p1);
         PairSum ts;
         pair_zero(ts);
+        dsf w[CL_Q + 1];
+        if (WIDE) {
+#pragma unroll
+            for (int c = 0; c <= CL_Q; ++c) w[c] = dsf{0.f, 0.f};
+        }
         if (soft_pairs(eps2f))
-            cluster_pairs<DS, true>(sm, sub, S, p0, p1, masked, ip, own, e2, ts);
+            cluster_pairs<DS, true>(sm, sub, S, p0, p1, masked, ip, own, e2, ts, w);
         else
-            cluster_pairs<DS, false>(sm, sub, S, p0, p1, masked, ip, own, e2, ts);
-        float v[CL_Q];
+            cluster_pairs<DS, false>(sm, sub, S, p0, p1, masked, ip, own, e2, ts, w);
+        if (WIDE) {
 #pragma unroll
-        for (int c = 0; c < CL_Q; ++c) v[c] = pair_total(ts, c);
-        for (int o = S >> 1; o > 0; o >>= 1)
+            for (int c = 0; c < CL_Q; ++c) ds_add(w[c].hi, w[c].lo, pair_total(ts, c));
+            const uint32_t to = cluster_addr(sm.part[rank][min(k, nw - 1) / CL_CTAS], k % CL_CTAS);
+            if (S >= 8) {
+                // lane c of a slot's holds component c, as in warp_scatter_sum (9 sums of pairs
+                // for the 35 of a tree over every component)
 #pragma unroll
-            for (int c = 0; c < CL_Q; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
-        if (sub == 0 && k < nw) {
-            const uint32_t to = cluster_addr(sm.part[rank][k / CL_CTAS], k % CL_CTAS);
-            cluster_st(to, make_float4(v[0], v[1], v[2], v[3]));
-            cluster_st(to + 16u, make_float4(v[4], v[5], v[6], 0.f));
+                for (int h = 4; h >= 1; h >>= 1) {
+                    const bool up = (sub & h) != 0;
+#pragma unroll
+                    for (int c = 0; c < h; ++c) {
+                        dsf keep = up ? w[c + h] : w[c];
+                        const dsf send = up ? w[c] : w[c + h];
+                        ds_acc(keep, ds_shfl_xor(send, h));
+                        w[c] = keep;
+                    }
+                }
+                for (int o = 8; o < S; o <<= 1) ds_acc(w[0], ds_shfl_xor(w[0], o));
+                if (sub < CL_Q && k < nw) cluster_st(to + 8u * sub, make_float2(w[0].hi, w[0].lo));
+            } else {
+                for (int o = S >> 1; o > 0; o >>= 1)
+#pragma unroll
+                    for (int c = 0; c < CL_Q; ++c) ds_acc(w[c], ds_shfl_xor(w[c], o));
+                if (sub == 0 && k < nw) {
+#pragma unroll
+                    for (int c = 0; c < CL_Q; ++c)
+                        cluster_st(to + 8u * c, make_float2(w[c].hi, w[c].lo));
+                }
+            }
+        } else {
+            float v[CL_Q];
+#pragma unroll
+            for (int c = 0; c < CL_Q; ++c) v[c] = pair_total(ts, c);
+            for (int o = S >> 1; o > 0; o >>= 1)
+#pragma unroll
+                for (int c = 0; c < CL_Q; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+            if (sub == 0 && k < nw) {
+                const uint32_t to = cluster_addr(sm.part[rank][k / CL_CTAS], k % CL_CTAS);
+                cluster_st(to, make_float4(v[0], v[1], v[2], v[3]));
+                cluster_st(to + 16u, make_float4(v[4], v[5], v[6], 0.f));
+            }
         }
     }
 }
 
-template <bool DS, int MAXL>
+template <bool DS, int MAXL, bool WIDE>
 __global__ void __launch_bounds__(CL_THREADS)
     k_cluster_steps(FusedArgs a)
 {
     extern __shared__ __align__(128) unsigned char s_cluster[];
-    ClusterSmem<MAXL> &sm = *reinterpret_cast<ClusterSmem<MAXL> *>(s_cluster);
+    using Smem = ClusterSmem<MAXL, WIDE>;
+    Smem &sm = *reinterpret_cast<Smem *>(s_cluster);
+    constexpr int CL_SLOTS = Smem::SLOTS;
     constexpr int NT = CL_THREADS, NW = NT / 32;
     constexpr int ROUNDS = (3 * MAXL + NT - 1) / NT;  // (component, particle) per thread
     static_assert(MAXL <= NT && MAXL % 256 == 0, "the due bits of a CTA come in one round");
@@ -1174,7 +1238,12 @@ __global__ void __launch_bounds__(CL_THREADS)
                         dsf x[CL_CTAS];
 #pragma unroll
                         for (int r = 0; r < CL_CTAS; ++r)
-                            x[r] = dsf{reinterpret_cast<const float *>(sm.part[r][ce])[c], 0.f};
+                            if (WIDE) {
+                                const float2 h = reinterpret_cast<const float2 *>(sm.part[r][ce])[c];
+                                x[r] = dsf{h.x, h.y};
+                            } else {
+                                x[r] = dsf{reinterpret_cast<const float *>(sm.part[r][ce])[c], 0.f};
+                            }
 #pragma unroll
                         for (int h = 1; h < CL_CTAS; h <<= 1)
 #pragma unroll
@@ -1588,7 +1657,7 @@ cudaError_t launch_selftest_barrier(unsigned *bar, unsigned *err, unsigned long 
     return cudaLaunchCooperativeKernel((const void *)k_selftest_barrier, 4, 64, args, 0, st);
 }
 
-template <int MAXL>
+template <int MAXL, bool WIDE>
 static void cluster_steps_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at, cudaStream_t st)
 {
     at.id = cudaLaunchAttributeClusterDimension;
@@ -1596,20 +1665,20 @@ static void cluster_steps_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &a
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.gridDim = dim3(CL_CTAS);
     cfg.blockDim = dim3(CL_THREADS);
-    cfg.dynamicSmemBytes = sizeof(ClusterSmem<MAXL>);
+    cfg.dynamicSmemBytes = sizeof(ClusterSmem<MAXL, WIDE>);
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
 }
 
 // Sixteen CTAs are more than a portable cluster.
-template <bool DS, int MAXL>
+template <bool DS, int MAXL, bool WIDE>
 static bool cluster_kernel_ready()
 {
-    constexpr auto kern = k_cluster_steps<DS, MAXL>;
+    constexpr auto kern = k_cluster_steps<DS, MAXL, WIDE>;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at{};
-    cluster_steps_config<MAXL>(cfg, at, nullptr);
+    cluster_steps_config<MAXL, WIDE>(cfg, at, nullptr);
     int clusters = 0;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)cfg.dynamicSmemBytes) != cudaSuccess ||
@@ -1622,13 +1691,13 @@ static bool cluster_kernel_ready()
     return clusters >= 1;
 }
 
-template <bool DS, int MAXL>
+template <bool DS, int MAXL, bool WIDE>
 static cudaError_t go_cluster_steps(const FusedArgs &a, cudaStream_t st)
 {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at{};
-    cluster_steps_config<MAXL>(cfg, at, st);
-    return cudaLaunchKernelEx(&cfg, k_cluster_steps<DS, MAXL>, a);
+    cluster_steps_config<MAXL, WIDE>(cfg, at, st);
+    return cudaLaunchKernelEx(&cfg, k_cluster_steps<DS, MAXL, WIDE>, a);
 }
 
 int fused_grid(int device, int order)
@@ -1678,22 +1747,28 @@ bool cluster_steps_ready()
     }
     const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
     if (known.load() & bit) return (ready.load() & bit) != 0;
-    const bool ok =
-        cluster_kernel_ready<true, CL_SMALL_L>() && cluster_kernel_ready<false, CL_SMALL_L>() &&
-        cluster_kernel_ready<true, CL_LARGE_L>() && cluster_kernel_ready<false, CL_LARGE_L>();
+    const bool ok = cluster_kernel_ready<true, CL_SMALL_L, false>() &&
+                    cluster_kernel_ready<false, CL_SMALL_L, false>() &&
+                    cluster_kernel_ready<true, CL_SMALL_L, true>() &&
+                    cluster_kernel_ready<false, CL_SMALL_L, true>() &&
+                    cluster_kernel_ready<true, CL_LARGE_L, true>() &&
+                    cluster_kernel_ready<false, CL_LARGE_L, true>();
     if (ok) ready |= bit;
     known |= bit;
     return ok;
 }
 
-cudaError_t launch_cluster_steps(const FusedArgs &a, bool ds, cudaStream_t st)
+cudaError_t launch_cluster_steps(const FusedArgs &a, bool ds, bool wide, cudaStream_t st)
 {
-    if (a.s.n > CL_CTAS * CL_LARGE_L) return cudaErrorInvalidValue;
-    if (a.s.n > CL_CTAS * CL_SMALL_L)
-        return ds ? go_cluster_steps<true, CL_LARGE_L>(a, st)
-                  : go_cluster_steps<false, CL_LARGE_L>(a, st);
-    return ds ? go_cluster_steps<true, CL_SMALL_L>(a, st)
-              : go_cluster_steps<false, CL_SMALL_L>(a, st);
+    if (a.s.n > CL_CTAS * (wide ? CL_LARGE_L : CL_SMALL_L)) return cudaErrorInvalidValue;
+    const auto go = a.s.n > CL_CTAS * CL_SMALL_L
+                        ? (ds ? go_cluster_steps<true, CL_LARGE_L, true>
+                              : go_cluster_steps<false, CL_LARGE_L, true>)
+                    : wide ? (ds ? go_cluster_steps<true, CL_SMALL_L, true>
+                                 : go_cluster_steps<false, CL_SMALL_L, true>)
+                           : (ds ? go_cluster_steps<true, CL_SMALL_L, false>
+                                 : go_cluster_steps<false, CL_SMALL_L, false>);
+    return go(a, st);
 }
 
 cudaError_t launch_fused_steps(const FusedArgs &a, int grid, bool ds, int order, cudaStream_t st)

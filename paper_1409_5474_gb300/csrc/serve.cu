@@ -731,7 +731,7 @@ int tick(nb_server s)
         a.max_steps = CLUSTER_STEPS;
         r->epoch = handle_take_epoch(r->h);
         CKS(cudaStreamWaitEvent(cs, s->ev_init, 0));
-        CKS(launch_cluster_steps(a, s->cfg.variant == NB_F32DS, cs));
+        CKS(launch_cluster_steps(a, s->cfg.variant == NB_F32DS, true, cs));
         CKS(cudaEventRecord(s->ev_cluster[r->slot], cs));
         r->running = true;
         ++launches;
