@@ -263,9 +263,11 @@ struct Mailbox {
     volatile double t_next;
     volatile int n_active;
     volatile int pad;
-    // the cluster kernel's launch: block steps taken and their interactions
+    // the cluster kernel's launch: block steps taken and their interactions, and, where its steps
+    // are limited, the error bits that ended it
     volatile long long steps;
     volatile double interactions;
+    volatile unsigned err;
 };
 
 // Particles per scheduler CTA (256 threads x 8).
@@ -442,7 +444,8 @@ struct FusedArgs {
     unsigned long long *dtmin_hits;
     FusedStats *stats;
     // cluster kernel only: block steps of one launch (0: no limit); at the limit it publishes the
-    // next block time with N_active = 0, nothing handed off. stats may be null there.
+    // next block time with N_active = 0, nothing handed off, and it ends so at an error bit in *err
+    // too. stats may be null there.
     int max_steps;
 };
 

@@ -871,6 +871,7 @@ struct ClusterSmem {
     uint4 due[CL_CTAS][MAXL / 128];        // a bit for every particle of every CTA
     double tn;
     int na;
+    unsigned err;
     unsigned long long hist[32], step_ns[32], phase[4];
     unsigned flags[MAXL / 32];
     int woff[MAXL / 32], wsum[CL_THREADS / 32], total, base;
@@ -1116,11 +1117,14 @@ __global__ void __launch_bounds__(CL_THREADS)
 #pragma unroll
             for (int h = 0; h < ROUNDS; ++h) load(tid + h * NT, st[h]);
         }
+        // a limited launch also ends at the first step with an error (the word is the system's
+        // own, so every CTA reads the same)
+        if (tid == 32) sm.err = a.max_steps > 0 ? __ldcg(a.err) : 0u;
         if (warp == 0) next_block_time(a, t_cur, sm.tn, sm.na);
         __syncthreads();
         const double tn = sm.tn;
         const int na = sm.na;
-        const bool limit = a.max_steps > 0 && steps >= a.max_steps;
+        const bool limit = a.max_steps > 0 && (steps >= a.max_steps || sm.err != 0u);
         if (!(tn <= a.t_end) || na < 1 || na > a.na_max || limit) {
             // hand the step to the caller exactly as the scheduler kernel would
             if (tn <= a.t_end && na >= 1 && !limit) {
@@ -1134,6 +1138,7 @@ __global__ void __launch_bounds__(CL_THREADS)
             if (scribe) {
                 a.mail->steps = steps;
                 a.mail->interactions = inter;
+                a.mail->err = sm.err;
                 publish(a, t_cur, tn, limit ? 0 : na, epoch);
             }
             break;
@@ -1179,7 +1184,15 @@ __global__ void __launch_bounds__(CL_THREADS)
             mycnt += __popc(bits.x) + __popc(bits.y) + __popc(bits.z) + __popc(bits.w);
         }
         if ((int)__reduce_add_sync(0xffffffffu, (unsigned)mycnt) != na) {
-            if (scribe) atomicOr(a.err, DERR_SCHED);  // the histogram and the states disagree
+            if (scribe) {
+                atomicOr(a.err, DERR_SCHED);  // the histogram and the states disagree
+                if (a.max_steps > 0) {
+                    a.mail->steps = steps;
+                    a.mail->interactions = inter;
+                    a.mail->err = DERR_SCHED;
+                    publish(a, t_cur, tn, 0, epoch);
+                }
+            }
             break;
         }
         // warp w copies the records of CTA w's due particles; their slots follow those of

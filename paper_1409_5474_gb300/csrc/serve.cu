@@ -76,7 +76,7 @@ struct Req {
     bool final_copy = false;  // EVOLVE: t_end reached, results being copied out
     bool cluster = false;     // a small EVOLVE: one cluster takes its steps ...
     bool running = false;     // ... and its launch is on the GPU
-    unsigned bits = 0;        // its error word at the end of the last tick
+    unsigned bits = 0;        // the error bits its last launch ended with
     double tick_inter = 0.0;  // interactions / block steps of the running tick,
     long long tick_steps = 0; // published under the lock when it ends
     int pending = NB_OK;      // failure found on the host during the tick
@@ -467,7 +467,8 @@ int tick(nb_server s)
     std::vector<ReqP> admitted;
     {
         std::lock_guard<std::mutex> lk(s->mu);
-        // running requests that were cancelled (none of their work is on the GPU)
+        // cluster launches that have ended; then the cancelled requests that have no work on
+        // the GPU (a running launch's end is waited for)
         for (auto &r : s->inflight)
             if (r->running) {
                 const cudaError_t e = launch_ended(s, *r);
@@ -479,6 +480,7 @@ int tick(nb_server s)
                     r->pending = NB_ERR_STATE;
                     continue;
                 }
+                r->bits = v.mail_h->err;
                 r->block_steps += v.mail_h->steps;
                 r->interactions += v.mail_h->interactions;
                 s->st.interactions += v.mail_h->interactions;
@@ -550,12 +552,12 @@ int tick(nb_server s)
             }
             const double t_next = v.mail_h->t_next;
             const int na = v.mail_h->n_active;
-            if (!(t_next <= r->t_end)) {
-                r->final_copy = true;
-                continue;
-            }
             if (r->cluster && r->bits) {
                 r->pending = err_code(r->bits);
+                continue;
+            }
+            if (!(t_next <= r->t_end)) {
+                r->final_copy = true;
                 continue;
             }
             if (r->cluster && na == 0) {  // CLUSTER_STEPS taken
@@ -775,8 +777,7 @@ int tick(nb_server s)
             r->tick_steps = 0;
             const unsigned bits = r->slot >= 0 ? s->h_errs[r->slot] : 0u;
             if (r->running) {
-                r->phase = PH_STEP;
-                r->bits = bits;  // looked at when the launch has ended
+                r->phase = PH_STEP;  // its errors are looked at when the launch has ended
             } else if (r->pending || bits) {
                 finish_locked(s, *r, NB_STATUS_ERROR, r->pending ? r->pending : err_code(bits));
                 drop_handle(s, *r, false);
