@@ -32,6 +32,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <condition_variable>
@@ -122,6 +123,7 @@ struct nb_server_s {
     int *d_cnt = nullptr;                      // due counts of a hand-off, by slot
     std::chrono::steady_clock::time_point t0;
 
+    std::atomic<bool> poked{false};  // something was submitted or cancelled since the tick began
     std::mutex mu;
     std::condition_variable cv_work, cv_done;
     std::map<uint64_t, ReqP> table;
@@ -467,6 +469,7 @@ int tick(nb_server s)
     std::vector<ReqP> admitted;
     {
         std::lock_guard<std::mutex> lk(s->mu);
+        s->poked = false;
         // cluster launches that have ended; then the cancelled requests that have no work on
         // the GPU (a running launch's end is waited for)
         for (auto &r : s->inflight)
@@ -605,11 +608,13 @@ int tick(nb_server s)
     }
 
     if (!work) {
-        // only cluster launches are under way: wait a little for one to end
-        do {
-            for (auto &r : s->inflight)
-                if (launch_ended(s, *r) != cudaErrorNotReady) return NB_OK;
-        } while (s->now() < t_begin + 20e-6);
+        // only cluster launches are under way: wait for one to end (or for a request or a
+        // cancellation; the next tick sees to it)
+        bool ended = false;
+        while (!ended && !s->poked.load(std::memory_order_acquire) && s->now() < t_begin + 1e-3)
+            for (auto &r : s->inflight) ended = ended || launch_ended(s, *r) != cudaErrorNotReady;
+        std::lock_guard<std::mutex> lk(s->mu);
+        s->st.busy_s += s->now() - t_begin;
         return NB_OK;
     }
 
@@ -970,6 +975,7 @@ int nb_server_destroy(nb_server s)
     {
         std::lock_guard<std::mutex> lk(s->mu);
         s->stop = true;
+        s->poked = true;
     }
     s->cv_work.notify_all();
     if (s->thread.joinable()) s->thread.join();
@@ -1038,6 +1044,7 @@ int nb_submit(nb_server s, const nb_request *req, uint64_t *ticket)
         s->st.submitted++;
         s->st.queued = (int)s->queue.size();
         *ticket = r->id;
+        s->poked = true;
     }
     s->cv_work.notify_one();
     return NB_OK;
@@ -1115,6 +1122,7 @@ int nb_cancel(nb_server s, uint64_t ticket)
             s->st.queued = (int)s->queue.size();
         } else {
             r.cancel = true;  // the server thread retires it before its next tick
+            s->poked = true;
         }
     }
     s->cv_done.notify_all();
