@@ -262,9 +262,9 @@ struct Mailbox {
     volatile unsigned long long seq;
     volatile double t_next;
     volatile int n_active;
-    volatile int pad;
-    // the cluster kernel's launch: block steps taken and their interactions, and, where its steps
-    // are limited, the error bits that ended it
+    volatile int leave;  // order 4: the launch ended for the other kernel to take the next steps
+    // order 4: block steps the launch took; the cluster kernel's also their interactions and, where
+    // its steps are limited, the error bits that ended it
     volatile long long steps;
     volatile double interactions;
     volatile unsigned err;
@@ -447,6 +447,10 @@ struct FusedArgs {
     // next block time with N_active = 0, nothing handed off, and it ends so at an error bit in *err
     // too. stats may be null there.
     int max_steps;
+    // order 4: end the launch so (with Mailbox::leave) where the rule of small systems gives the steps
+    // to the other kernel, grid or cluster. It is asked at multiples of dt_max (the cluster: and a
+    // sixteenth of it later), and with ask_now at the launch's first step.
+    bool may_leave, ask_now;
 };
 
 constexpr int FUSED_THREADS = 256;

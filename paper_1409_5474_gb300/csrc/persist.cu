@@ -607,6 +607,90 @@ __device__ __forceinline__ bool handoff_predict_gather(const FusedArgs &a, doubl
     return barrier();
 }
 
+// ---- which kernel takes the steps of a small system --------------------------
+
+// Sixteenths of the power of two d beyond its last multiple at time t (0 to 15), -1 between them.
+// By the bits: asked at every step, and an FP64 instruction holds its pipe for 64 cycles.
+__device__ __forceinline__ int sixteenths(double t, double d)
+{
+    const unsigned long long u = (unsigned long long)__double_as_longlong(t) & ~(1ull << 63);
+    const int e = (int)(u >> 52);
+    const unsigned long long m = (u & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+    const int shift = exponent_of(d) - 4 - ((e ? e : 1) - 1075);  // t = m 2^-shift sixteenths
+    if (m == 0ull) return 0;
+    if (shift <= -4) return 0;
+    if (shift > 52 || (shift > 0 && (m & ((1ull << shift) - 1ull)))) return -1;
+    const int r = (int)(shift > 0 ? m >> shift : m << -shift) & 15;
+    return __double_as_longlong(t) < 0 ? (16 - r) & 15 : r;
+}
+
+// Either kernel asks where all particles are at one time, at the multiples of dt_max (and, with
+// ask_now, at its first step), so a run and its continuation from a checkpoint there ask the
+// same questions; it takes 2 us. The cluster asks again a sixteenth of dt_max later: the initial
+// steps are shorter and spread over more levels than the ones after them, and make it look up
+// to half as costly as it is. The answer: 32 times the ratio of the costs (cluster to grid)
+// from which on the grid kernel takes the steps, 0 for no question.
+__device__ __forceinline__ unsigned question(const FusedArgs &a, double t_cur, bool first,
+                                             bool cluster)
+{
+    if (!a.may_leave) return 0u;
+    const int r = first && a.ask_now ? 0 : sixteenths(t_cur, a.prm.dt_max);
+    return r == 0 ? 31u : (r == 1 && cluster ? 38u : 0u);
+}
+
+// Eighths of a microsecond of a step with na due of n (at most 4096 each): in the cluster, and in
+// the grid kernel (within 15% of Plummer spheres' and of the steps of systems with one occupied
+// small level, n = 300 to 4000).
+__device__ __forceinline__ unsigned cluster_step_cost(unsigned na, unsigned n)
+{
+    return 60u + n / 256u + (na * (20972u + 31u * n) >> 18);
+}
+
+__device__ __forceinline__ unsigned grid_step_cost(unsigned na, unsigned n)
+{
+    if (na <= (unsigned)FUSED_SMALL_NA) return 96u;
+    return na < (unsigned)FUSED_IPT2_NA ? 107u : 120u + (na * (3146u + 3u * n) >> 18);
+}
+
+// Whether a system of at most FUSED_CLUSTER_MAX_N particles is stepped by the grid kernel and not
+// by the cluster: by the mean cost of its steps, which the population of the levels tells. A block
+// time is a multiple of 2^z smallest steps and no more, with z = 0 half of the time, z = 1 a
+// quarter, ..., and its due set the particles of the levels whose steps divide it. Plummer spheres
+// stay in the cluster up to some 4000 particles (2500: 7.0 ms a 1/16 time unit, the grid
+// kernel 8.0; 4000: 9.9 and 10.1); with hundreds due in half of the steps it is the slower: 600 of
+// 4000 in a dense core, 500 steps, 14.3 ms and 8.0. One warp, whole numbers: both kernels find
+// the same.
+__device__ __forceinline__ bool grid_takes(const FusedArgs &a, unsigned ratio32)
+{
+    const int lane = threadIdx.x & 31;
+    int d0 = __ldcg(a.sd->hist + lane), d1 = __ldcg(a.sd->hist + 32 + lane);
+    const unsigned b0 = __ballot_sync(0xffffffffu, d0 > 0);
+    const unsigned b1 = __ballot_sync(0xffffffffu, d1 > 0);
+    const int kmax = b1 ? 63 - __clz(b1) : (b0 ? 31 - __clz(b0) : 0);
+    // the particles of level k and above (smaller steps)
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u0 = __shfl_down_sync(0xffffffffu, d0, o), u1 = __shfl_down_sync(0xffffffffu, d1, o);
+        if (lane + o < 32) {
+            d0 += u0;
+            d1 += u1;
+        }
+    }
+    d0 += __shfl_sync(0xffffffffu, d1, 0);
+    unsigned cl = 0u, gr = 0u;  // in 1/8192 of the steps
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int k = lane + 32 * h, na = h ? d1 : d0;
+        if (k > kmax || kmax - k > 12 || na < 1 || na > a.na_max) continue;  // larger: either hands on
+        const unsigned share = (4096u >> (kmax - k)) << (k == 0 ? 1 : 0);
+        cl += share * cluster_step_cost((unsigned)na, (unsigned)a.s.n);
+        gr += share * grid_step_cost((unsigned)na, (unsigned)a.s.n);
+    }
+    cl = __reduce_add_sync(0xffffffffu, cl);
+    gr = __reduce_add_sync(0xffffffffu, gr);
+    return 32u * cl > ratio32 * gr;
+}
+
 // ---- the kernel ------------------------------------------------------------
 
 template <bool DS>
@@ -619,6 +703,7 @@ __global__ void __launch_bounds__(FUSED_THREADS)
     __shared__ int s_wsum[NW];
     __shared__ int s_total, s_base, s_na, s_last;
     __shared__ double s_tn;
+    __shared__ bool s_leave;
     __shared__ unsigned long long s_hist[32], s_step_ns[32], s_phase[4];
     __shared__ __align__(16) float4 s_tile[2][DS_REC * FUSED_TILE];
     float2(*s_red)[SMALL_Q] = reinterpret_cast<float2(*)[SMALL_Q]>(&s_tile[0][0]);
@@ -637,7 +722,8 @@ __global__ void __launch_bounds__(FUSED_THREADS)
     bool ok = true;
     double t_cur = __ldcg(&a.sd->t_cur);
     const unsigned long long epoch = __ldcg(&a.sd->seq);
-    unsigned long long steps = 0;
+    unsigned long long steps = 0;  // counted by thread 0 of CTA 0
+    bool first = true;
     double inter = 0.0;
     if (tid < 32) s_hist[tid] = s_step_ns[tid] = 0ull;
     if (tid < 4) s_phase[tid] = 0ull;
@@ -658,20 +744,31 @@ __global__ void __launch_bounds__(FUSED_THREADS)
         PState q0, q1;
         if (p0 + tid < p1) pstate_load(s, p0 + tid, q0);
         if (p0 + tid + NT < p1) pstate_load(s, p0 + tid + NT, q1);
+        if (warp == 1) {
+            const unsigned r = question(a, t_cur, first, false);
+            const bool leave = r && !grid_takes(a, r);
+            if (lane == 0) s_leave = leave;
+        }
         if (warp == 0) next_block_time(a, t_cur, s_tn, s_na);
         __syncthreads();
         const double tn = s_tn;
         const int na = s_na;
-        if (!(tn <= a.t_end) || na < 1 || na > a.na_max) {
+        const bool leave = s_leave;
+        first = false;
+        if (!(tn <= a.t_end) || na < 1 || na > a.na_max || leave) {
             // hand the step to the caller exactly as the scheduler kernel would
-            if (tn <= a.t_end && na >= 1) {
+            if (tn <= a.t_end && na >= 1 && !leave) {
                 ok = handoff_predict_gather<4, NT>(
                     a, tn, p0, p1, nwords, s_flags, s_woff, s_wsum, s_total, s_base,
                     [&] { return grid_barrier(a.bar, gen); });
                 mark(0);
                 if (!ok) break;
             }
-            if (bid == 0 && tid == 0) publish(a, t_cur, tn, na, epoch);
+            if (bid == 0 && tid == 0) {
+                a.mail->steps = (long long)steps;
+                a.mail->leave = leave;
+                publish(a, t_cur, tn, leave ? 0 : na, epoch);
+            }
             break;
         }
 
@@ -872,6 +969,7 @@ struct ClusterSmem {
     double tn;
     int na;
     unsigned err;
+    bool leave;  // the grid kernel takes the next steps
     unsigned long long hist[32], step_ns[32], phase[4];
     unsigned flags[MAXL / 32];
     int woff[MAXL / 32], wsum[CL_THREADS / 32], total, base;
@@ -1120,11 +1218,17 @@ __global__ void __launch_bounds__(CL_THREADS)
         // a limited launch also ends at the first step with an error (the word is the system's
         // own, so every CTA reads the same)
         if (tid == 32) sm.err = a.max_steps > 0 ? __ldcg(a.err) : 0u;
+        if (warp == 1) {
+            const unsigned r = question(a, t_cur, steps == 0, true);
+            const bool leave = r && grid_takes(a, r);
+            if (lane == 0) sm.leave = leave;
+        }
         if (warp == 0) next_block_time(a, t_cur, sm.tn, sm.na);
         __syncthreads();
         const double tn = sm.tn;
         const int na = sm.na;
-        const bool limit = a.max_steps > 0 && (steps >= a.max_steps || sm.err != 0u);
+        const bool limit =
+            (a.max_steps > 0 && (steps >= a.max_steps || sm.err != 0u)) || sm.leave;
         if (!(tn <= a.t_end) || na < 1 || na > a.na_max || limit) {
             // hand the step to the caller exactly as the scheduler kernel would
             if (tn <= a.t_end && na >= 1 && !limit) {
@@ -1139,6 +1243,7 @@ __global__ void __launch_bounds__(CL_THREADS)
                 a.mail->steps = steps;
                 a.mail->interactions = inter;
                 a.mail->err = sm.err;
+                a.mail->leave = sm.leave;
                 publish(a, t_cur, tn, limit ? 0 : na, epoch);
             }
             break;

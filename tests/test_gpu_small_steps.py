@@ -1,0 +1,71 @@
+"""Block steps of small systems: the cluster and the grid kernel share them out by the levels'
+population."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _core(n, core, seed=3):
+    """A dense core of equal masses, whose particles share a small step, in a light halo."""
+    rng = np.random.default_rng(seed)
+
+    def ball(k, r):
+        d = rng.standard_normal((k, 3))
+        d /= np.linalg.norm(d, axis=1)[:, None]
+        return d * r * rng.uniform(0, 1, k)[:, None] ** (1 / 3)
+    x = np.concatenate([ball(core, 0.05), ball(n - core, 3.0)])
+    v = np.concatenate([rng.standard_normal((core, 3)), 0.01 * rng.standard_normal((n - core, 3))])
+    return np.concatenate([np.full(core, 0.5 / core), np.full(n - core, 1e-6)]), x, v
+
+
+def _system(nb, n, core, **cfg):
+    return nb.System(*_core(n, core), variant="f32ds", eps=0.02, eta=0.003, dt_max=1.0 / 64,
+                     device=0, **cfg)
+
+
+SIZES = [(300, 200), (1500, 1000), (2500, 300), (2500, 700), (4000, 150), (4000, 1000), (4096, 3000)]
+
+
+@pytest.mark.parametrize("n,core", SIZES)
+@pytest.mark.parametrize("fused_max_na", [0, 4096])
+def test_a_run_and_its_continuation_agree_bit_for_bit(nb, n, core, fused_max_na):
+    """In pieces, and from checkpoints (at times that are no multiple of dt_max too) in a handle that
+    has taken no step yet: which kernel takes a step follows from the state."""
+    t = 1.0 / 64
+    with _system(nb, n, core, fused_max_na=fused_max_na) as sy:
+        nb.nb_init(sy.h)
+        start = sy.state()
+        sy.step(t)
+        want = sy.state()
+        sy.set_state(start)
+        for k in range(1, 9):
+            sy.step(k * t / 8)
+            if k in (3, 6):
+                here = sy.state()
+                with _system(nb, n, core, fused_max_na=fused_max_na) as other:
+                    other.set_state(here)
+                    other.step(t)
+                    got = other.state()
+                for a, b in zip(want, got):
+                    np.testing.assert_array_equal(a, b)
+        for a, b in zip(want, sy.state()):
+            np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("n,core,grid", [(300, 200, False), (1000, 60, False), (2500, 700, True),
+                                         (4000, 1000, True), (4096, 3000, True)])
+def test_the_kernel_follows_the_levels(nb, n, core, grid):
+    """Hundreds due in half of the steps: the grid kernel takes them from the first multiple of dt_max
+    on; the cluster keeps small due sets. Told by the time of a step: at these sizes the kernels
+    differ by a third and more."""
+    with _system(nb, n, core, fused_max_na=4096) as sy:
+        sy.step(1.0 / 64)
+        st = sy.step(1.0 / 32)
+    steps, ms = np.array(st["active_hist"]), np.array(st["fused_step_ms_hist"])
+    k = int(np.argmax(steps[8:])) + 8 if grid else int(np.argmax(steps))
+    us = 1e3 * ms[k] / steps[k]
+    if grid:  # 256 and more due: the cluster takes 25 us and more
+        assert us < 16.5 + 2.0 ** k * n * 3e-6, (us, k)
+    else:     # the grid kernel takes 11 us and more
+        assert us < 14.0, (us, k)
