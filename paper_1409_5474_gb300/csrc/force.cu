@@ -213,8 +213,8 @@ __device__ __forceinline__ int member_index(const ISet &is, int k, unsigned *err
 // Bound by the FP32 pipe: 33 operations per interaction (27 for plain FP32), 1220 G/s at
 // 2070 MHz. The running totals live in shared memory (touched once per fold) and
 // not in 28 registers, so the packed loop, unrolled four pairs deep, runs without
-// spills at two CTAs per SM; with eps^2 >= FLT_MIN the SFU's reciprocal square root
-// is taken bare (rsqrtf adds a test and two FP32-pipe scalings per interaction).
+// spills at two CTAs per SM; with eps^2 >= FLT_MIN the reciprocal square root is the one
+// instruction rsqrt.approx.ftz.f32 (pair.cuh).
 // N = 262144, F32-DS: 76.3 -> 67.8 ms, FMA pipe 84% of cycles (unroll 2: 68.7 ms, 1:
 // 68.5 ms). Tiles that are ragged or hold a warp's own particle stay on the packed path
 // with their halves masked, and warps without slots skip the arithmetic: 67.8 ->
@@ -434,10 +434,8 @@ __global__ void __launch_bounds__(256)
 //
 // Bound by the FP64 pipe: a warp-wide FP64 instruction holds an SMSP's pipe for 64
 // cycles, and a pair takes about 32 of them, so one j costs a warp of 32 i-particles 1 us
-// and a GB300 does 19.7 G/s at most (17.3 measured at N = 20011; a reciprocal square root of
-// five FP64 instructions from the SFU's approximation gave the same time and bits as
-// rsqrt). What is left is to keep all
-// 608 pipes busy to the end: a CTA is 32 i-particles times four warp rows (one warp per
+// and a GB300 does 19.7 G/s at most (17.3 measured at N = 20011). What is
+// left is to keep all 608 pipes busy to the end: a CTA is 32 i-particles times four warp rows (one warp per
 // SMSP; row g takes j = g, g + 4, ... of every tile, the rows are added in order through
 // shared memory), so an SM's four pipes always carry the same load and the plan divides
 // the j-range in units of 16. The splits are summed by k_split_sums. N = 1024, all

