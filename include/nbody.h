@@ -152,7 +152,10 @@ const char *nb_version(void);
  * nb_create allocates the device state for cfg->n_max particles on
  * cfg->device. Rejects eps < 0, eta <= 0, dt_max or dt_min not a power of
  * two, dt_min > dt_max, shared_dt < 0, n_max < 1, an unknown variant
- * (NB_ERR_ARG), and a state larger than budget_bytes (NB_ERR_BUDGET).
+ * (NB_ERR_ARG), and a state larger than budget_bytes (NB_ERR_BUDGET). FP32
+ * handles of order 4 without a budget also hold up to 16 MB for the partial
+ * sums of split evaluations from the start; with a budget the built-in plans
+ * split as far as it leaves room.
  * nb_destroy frees everything; it is a no-op on NULL. */
 int nb_create(const nb_config *cfg, nb_handle *out);
 int nb_destroy(nb_handle h);
@@ -278,9 +281,11 @@ int nb_reset_stats(nb_handle h);
 /* ---- launch plans and the autotuner ---------------------------------------
  * How a force evaluation of n_i i-particles is laid out on the GPU (the
  * paper's i-parallel and j-parallel mappings, Sect. III.A):
- *   kind 0: tiles - a CTA of 256 threads holds 2 i-particles per thread in
- *           256/nwj/32 warp columns; nwj warp rows share each j-tile;
- *           nsplit CTAs split the j-range (FP32 kinds: nwj in {1, 4, 8});
+ *   kind 0: tiles - FP32 kinds: a CTA of 256 threads holds 2 i-particles per
+ *           thread (1 for up to 32 of them in eight rows) in 256/nwj/32 warp
+ *           columns; nwj warp rows (1, 4 or 8) share each j-tile; FP64: 32
+ *           i-particles times four warp rows (nwj is ignored); nsplit CTAs
+ *           split the j-range;
  *   kind 1: j-parallel warp groups - each warp holds up to 2 i-particles (FP64:
  *           all threads share up to 4) and its lanes stride over j; nsplit
  *           CTAs split the j-range;
@@ -295,7 +300,8 @@ int nb_reset_stats(nb_handle h);
 typedef struct nb_plan {
     int kind;   /* 0 tiles, 1 warp groups, 2 tiny sets, -1 = built-in heuristic */
     int nwj;    /* warp rows per CTA (kind 0) */
-    int nsplit; /* j-range splits (>= 1; clamped to the j-set) */
+    int nsplit; /* j-range splits (>= 1; clamped to the j-tiles: FP32 256 records,
+                 * FP64 16 and at most 65535) */
 } nb_plan;
 
 /* The plan used for an evaluation of n_i i-particles on the current j-set

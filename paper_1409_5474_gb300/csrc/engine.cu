@@ -379,8 +379,8 @@ int ensure_part(nb_handle h, const ForcePlan &p, int n_i)
     return NB_OK;
 }
 
-// The split counters of a force launch: the warp-group kernel's (FP64 plans and the tile and
-// tiny-set kernels sum their splits in a launch of their own).
+// The split counters of a force launch: the warp groups' and the tiny sets', whose last CTAs sum
+// the splits (FP64 plans and the tile kernels sum theirs in a launch of their own).
 unsigned *counters_of(nb_handle h, int variant) { return variant == NB_F64 ? nullptr : h->split_cnt; }
 
 int bucket_of(int n_i)

@@ -12,10 +12,10 @@
 //    cp.async.bulk) into an NS-deep ring of mbarrier-guarded buffers. The
 //    j-range is split across grid.y (the paper's j-parallel split for small
 //    N_i, after Makino's scheme), and the partial sums are reduced by K3.
-//  - j-parallel warp kernels for tiny i-sets (N_i <= 32, block-step tails):
-//    every thread holds the same few i-particles and a different j; partial
-//    sums are combined by warp shuffles, then across warps in FP64, then
-//    across CTAs by K3.
+//  - j-parallel warp kernels for tiny i-sets (FP32: N_i <= 4, or 8 above 65536 j; FP64:
+//    N_i <= 32 where that is faster; block-step tails): every thread holds the same few
+//    i-particles and a different j; partial sums are combined by warp shuffles, then
+//    across warps (double-single, FP64), then across CTAs by K3.
 //
 // Precision variants (Sect. III.A: emulated double precision for the
 // inter-particle distance, native FP64 for extreme mass ratios):
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
     // with nsplit > 1 the partials are summed by k_split_sums, launched next
 }
 
-// K3 of the tile, tiny-set and FP64 kernels (split_sum): output q = component c of slot k.
+// K3 of the tile and FP64 kernels (split_sum): output q = component c of slot k.
 template <class T, int G>
 __global__ void __launch_bounds__(256)
     k_split_sums(const T *part, long long pld, int nsplit, int n_i, Out3 out, unsigned *err)

@@ -140,8 +140,9 @@ size_t plan_counters(const ForcePlan &p, int n_i);
 
 // Launch K2 and, when nsplit > 1, K3: the CTAs write their partial sums to part
 // (plan_partial_doubles) and a dependent launch adds them in a fixed order. The FP32 warp
-// groups, and the FP64 j-parallel kernel when counters is given (a caller that makes one
-// launch), fold K3 in: the last CTA of every i-block (counted in counters) adds them.
+// groups and tiny sets, and the FP64 j-parallel kernel when counters is given (a caller that
+// makes one launch), fold K3 in: the last CTA of every i-block, or of the launch (counted in
+// counters), adds them.
 // eps2: softening squared. Results go to out (slot-indexed). Non-finite
 // results set DERR_NONFINITE in *err. ev (optional, 2 events) brackets the launch.
 cudaError_t launch_force(int variant, const ForcePlan &plan, const JSet &js, const ISet &is,

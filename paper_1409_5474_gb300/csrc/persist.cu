@@ -936,12 +936,12 @@ __global__ void __launch_bounds__(FUSED_THREADS)
 //      three lanes each                                           -- cluster barrier
 // The cluster barrier is a hardware barrier of co-scheduled CTAs (like __syncthreads):
 // no wait depends on another launch, and every exit is taken by all CTAs together.
-// Measured against the grid kernel, 1/16 time unit of block steps: N = 500 2.28 -> 1.51 ms,
-// 1000 5.27 -> 3.64, 2500 8.57 -> 6.88, 4000 11.7 -> 10.5. A step of 1 to 3 due at N = 2500 takes
-// 9.1 us for 13.2: the prediction and its barrier 3.2, the force 3, the corrector 2.2.
-// Sixteen SMs are a tenth of the GPU, so due sets of a hundred and more cost part
-// of that again (N = 2500, 512-1023 due: 39 against 20 us; N = 4000: 59 against 21), which at
-// 4096 particles leaves a tenth: the line of the dispatch.
+// Measured against the grid kernel, 1/16 time unit of block steps of Plummer spheres: N = 500
+// 5.3 -> 3.7 ms, 1000 5.3 -> 4.0, 2500 8.0 -> 7.0, 4000 10.1 -> 10.0. A step of 1 to 3 due at N = 2500
+// takes 9.1 us for 11.9: the prediction and its barrier 3.2, the force 3, the corrector 2.2.
+// Sixteen SMs are a tenth of the GPU, so due sets of a hundred and more cost that again
+// (N = 2500, 512-1023 due: 39 us against 17; N = 4000: 59 against 18): systems with many of them
+// stay with the grid kernel (grid_takes), and at 4096 particles nothing is gained any more.
 constexpr int CL_CTAS = FUSED_CLUSTER;
 constexpr int CL_THREADS = 512;
 constexpr int CL_Q = 7;                                  // outputs of a slot

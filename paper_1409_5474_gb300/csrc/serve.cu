@@ -94,9 +94,13 @@ constexpr int NSIDE = 4;  // side streams of the engine-planned force launches
 constexpr int NCLUSTER = 8;
 constexpr int CLUSTER_STEPS = 128;
 // Due sets of more interactions than this are handed to the ticks (one step; the cluster goes
-// on after it): sixteen SMs do about 60 interactions a nanosecond, all of them 700 and more,
-// and a step in the ticks costs some 50 us besides. The burst of 16 requests takes 12.3 ms with
-// the line at 1.2e6, 8.6 to 8.8 from 4e6 to 8e6, 10.6 at 12e6, 15.6 without one.
+// on after it): sixteen SMs do about 50 interactions a nanosecond, all of them 700 and more, and
+// a step in the ticks with the two launches around it costs some 70 us besides, so 50 and 700
+// break even at 70e3 / (1/50 - 1/700) = 3.8e6 interactions, and later where other integrations
+// wait for the tick. Swept on seven loads (a burst of 16 requests; one integration of 4000 or 8000
+// particles, spread or with a dense core; 8 of 8000; 16 of 6000) 4e6 to 8e6 are within 10% of each
+// load's best and 6e6 within 8%: the burst takes 12.3 ms at 1e6, 9.1 at 3e6, 8.7 at 6e6, 10.2 at
+// 12e6, one of 8000 22.8, 19.5, 19.5 and 21.6.
 constexpr double CLUSTER_MAX_INTERACTIONS = 6e6;
 
 int capacity_class(int n)
@@ -197,7 +201,7 @@ nb_handle acquire_handle(nb_server s, int cap, size_t *bytes)
     c.device = s->dev;
     nb_handle h = nullptr;
     // the handles' room for partials comes after what requests are admitted by
-    const bool reserve = s->bytes_in_use + need + part_reserve(c) <= s->cfg.budget_bytes / 2;
+    const bool reserve = s->bytes_in_use + need + part_reserve(c) <= s->cfg.budget_bytes / 4;
     if (create_handle(&c, reserve, &h) != NB_OK) return nullptr;
     nb_set_stream(h, s->stream);
     *bytes = handle_bytes(h);
