@@ -347,7 +347,9 @@ __global__ void __launch_bounds__(32 * NWI * NWJ, 2)
 
         const bool masked = own || cnt < JT;
 #pragma unroll 1
-        for (int f = 0; f < cnt && !idle; f += JR) {  // idle: no slot of this warp is written
+        for (int r = 0; r < (idle ? 0 : RUNS); ++r) {  // idle: no slot of this warp is written
+            const int f = r * JR;
+            if (RUNS > 1 && f >= cnt) break;
             const float4 *P = pairs + DS_REC * f;
             const int fcnt = min(JR, cnt - f);
             if (soft)
