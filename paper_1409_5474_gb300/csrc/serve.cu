@@ -23,9 +23,10 @@
 // Integrations of up to FUSED_CLUSTER_LIMIT_N particles leave the ticks after their initial
 // evaluation: one cluster (k_cluster_steps) takes up to CLUSTER_STEPS of their block
 // steps a launch, on a stream beside the ticks, and a tick only looks whether it has
-// ended. A block step in the ticks costs a round trip to the host and six launches, 25 us for a
-// few due particles, and every step of the longest integration waits for it; in a cluster
-// 9 to 14 us. 16 requests of 256-16384, half of them integrations: 24.8 -> 8.7 ms.
+// ended. A block step in the ticks costs a round trip to the host and six launches, 25 us and
+// more for a few due particles, and every step of the longest integration waits for it; in a cluster
+// 10 to 15 us. 16 requests of 256-16384, half of them integrations: 28.3 -> 9.5 ms; one
+// integration of 2500 particles over 1/16 time unit 48 -> 9.1, of 8000 70 -> 19.6.
 // A request's items, splits and summation order depend only on the request
 // itself (and the SM count), so its results are the same whatever else is in
 // flight.
