@@ -1804,7 +1804,7 @@ int nb_step(nb_handle h, double t_end, nb_stats *st)
                 r = timed(h, T_FUSED, [&] {
                     const bool ds = h->cfg.variant == NB_F32DS;
                     return cluster && !h->grid_last
-                               ? launch_cluster_steps(fa, ds, false, h->stream)
+                               ? launch_cluster_steps(fa, ds, h->n > FUSED_CLUSTER_NARROW_N, h->stream)
                                : launch_fused_steps(fa, h->fused_grid, ds, 4, h->stream);
                 });
                 h->stats.fused_launches++;

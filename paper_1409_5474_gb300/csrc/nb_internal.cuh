@@ -468,6 +468,8 @@ constexpr int FUSED6_MAX_NA = NB_FUSED6_MAX_NA;
 constexpr int FUSED_CLUSTER = 16;
 constexpr int FUSED_CLUSTER_MAX_N = 4096;
 constexpr int FUSED_CLUSTER_LIMIT_N = 8192;  // the most the kernel takes (request loop)
+// Up to here a handle's launch adds in FP32 alone within a CTA (32 particles).
+constexpr int FUSED_CLUSTER_NARROW_N = 512;
 
 // Ints of the fused kernel's counter array: grid per-CTA counts, 2 due-set
 // counters, the tickets of the small-set groups (at most FUSED6_MAX_NA / 4; padded).
@@ -485,8 +487,8 @@ cudaError_t launch_selftest_mbar(unsigned *err, unsigned long long limit_ns, cud
 cudaError_t launch_selftest_barrier(unsigned *bar, unsigned *err, unsigned long long limit_ns,
                                     cudaStream_t st);
 // The same steps (order 4) by one cluster: needs no cnt, bar or part. wide: sums beyond short FP32
-// runs in double-single (the request loop; up to FUSED_CLUSTER_LIMIT_N particles, else
-// FUSED_CLUSTER_MAX_N). Ready: the current device can run that cluster.
+// runs in double-single (the request loop and handles of more than FUSED_CLUSTER_NARROW_N
+// particles; up to FUSED_CLUSTER_LIMIT_N particles, else FUSED_CLUSTER_MAX_N). Ready: the current device can run that cluster.
 bool cluster_steps_ready();
 cudaError_t launch_cluster_steps(const FusedArgs &a, bool ds, bool wide, cudaStream_t st);
 cudaError_t launch_fused_steps(const FusedArgs &a, int grid, bool ds, int order,

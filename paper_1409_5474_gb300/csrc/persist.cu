@@ -947,11 +947,14 @@ constexpr int CL_THREADS = 512;
 constexpr int CL_Q = 7;                                  // outputs of a slot
 
 // WIDE: the sums of more than CL_RUN terms a half are double-single from there on, over the lanes
-// and over the CTAs. The request loop's integrations take it: their steps in the ticks add
-// FP32 terms in runs of 32 or 64, and without it a lane's run is all of its pairs (up to 256)
-// and a CTA's partial one FP32 sum of up to 512 terms. The handles' steps do without, as the grid
-// kernel does (FP32 sums of up to 256 terms). One integration of 2500 particles over 1/16
-// time unit 8.3 -> 9.1 ms, of 8000 18.5 -> 19.6 (in the ticks 48 and 70).
+// and over the CTAs. Without it a lane's run is all of its pairs (up to 256) and a CTA's partial
+// one FP32 sum of up to 512 terms. The request loop's integrations take it (their steps in the
+// ticks add FP32 terms in runs of 32 or 64), and the handles' steps above FUSED_CLUSTER_NARROW_N
+// particles: the median and 99% error of the jerk of Plummer spheres' due sets was 7 and 8% above the
+// grid kernel's at N = 1300, 8 and 9 at 1800, 12 and 16 at 2500, and is 0 to 4% below it; up to 512 a
+// CTA's 32 particles are one run, and the errors of either form no larger than the grid kernel's.
+// 1/16 time unit of Plummer spheres: N = 1000 4.0 -> 4.3 ms, 1800 4.9 -> 5.3, 2500 7.0 -> 7.6,
+// 8000 (request loop) 18.5 -> 19.6.
 constexpr int CL_RUN = 16;
 
 // MAXL: the most particles of a CTA. A window of the due set has SLOTS slots (the wide
