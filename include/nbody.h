@@ -65,11 +65,12 @@ extern "C" {
 #define NB_FLAG_TIMING 1 /* time every kernel launch with CUDA events (nb_stats) */
 /* Block steps of NB_F32 / NB_F32DS handles normally run in the fused
  * persistent kernel: one launch (cooperative, or one thread-block cluster for
- * systems of up to 4096 particles at order 4 whose due sets are small) takes block steps (scheduler + predictor, force,
- * reduction, corrector, with barriers between the stages) until a due set
- * larger than nb_config.fused_max_na (default NB_FUSED_DEFAULT_NA) or t_end, so
- * small steps need no host round trip; larger due sets go to the planned force
- * kernels. NB_FLAG_NO_FUSED takes every block step with separate launches. */
+ * systems of up to 2000 particles at order 4 whose due sets are small) takes block
+ * steps (scheduler + predictor, force, reduction, corrector, with barriers
+ * between the stages) until a due set larger than nb_config.fused_max_na
+ * (default NB_FUSED_DEFAULT_NA) or t_end, so small steps need no host round
+ * trip; larger due sets go to the planned force kernels. NB_FLAG_NO_FUSED takes
+ * every block step with separate launches. */
 #define NB_FLAG_NO_FUSED 2
 #define NB_FUSED_MAX_NA 4096      /* upper bound of nb_config.fused_max_na */
 #define NB_FUSED_DEFAULT_NA 1024  /* fused_max_na = 0 */
@@ -185,11 +186,7 @@ int nb_get_particles(nb_handle h, double *m, double *pos, double *vel);
 /* Full integrator state for checkpoint / resume: m[n], pos[3n], vel[3n],
  * acc[3n], jerk[3n], own time t[n], own step dt[n]. nb_set_state restores a
  * state taken by nb_get_state (same n <= n_max), after which nb_step resumes
- * bit-identically. (FP32 block steps of up to 4096 particles at order 4 choose
- * between two kernels where all particles are at one time, the multiples of
- * dt_max; a state taken between those may be continued by the other kernel,
- * whose pair sums run in another order.) Any output pointer of nb_get_state may
- * be NULL. */
+ * bit-identically. Any output pointer of nb_get_state may be NULL. */
 int nb_get_state(nb_handle h, int *n, double *m, double *pos, double *vel,
                  double *acc, double *jerk, double *t, double *dt);
 int nb_set_state(nb_handle h, int n, const double *m, const double *pos,

@@ -148,8 +148,7 @@ struct nb_handle_s {
     // fused persistent block steps (allocated at first use)
     int fused_grid = -1;                  // CTAs per launch; 0 = not available
     int cluster_ok = -1;                  // one cluster can take the steps of a small system
-    bool grid_last = false;               // the last of its steps was the grid kernel's
-    bool kernel_asked = false;            // and the rule was asked since its levels were set
+    bool grid_last = false;               // which of them is tried first: the last one's
     float2 *fused_part = nullptr;
     size_t fused_part_cap = 0;            // float2
     int *fused_cnt = nullptr;
@@ -573,7 +572,6 @@ int load_sched(nb_handle h, const double *t, const double *dt)
     CK(h, cudaStreamSynchronize(h->stream));
     h->t_cur = tc;
     h->sched_valid = true;
-    h->kernel_asked = false;
     return NB_OK;
 }
 
@@ -627,7 +625,6 @@ int do_init(nb_handle h)
     h->predicted = false;
     h->t_cur = t0;
     h->sched_valid = true;
-    h->kernel_asked = false;
     return NB_OK;
 }
 
@@ -1792,18 +1789,17 @@ int nb_step(nb_handle h, double t_end, nb_stats *st)
         // queued as soon as it is read
         const bool fused = fused_ready(h);
         FusedArgs fa = fused ? fused_args(h, t_end, f) : FusedArgs{};
-        // small systems: the cluster or the grid kernel, as the levels say at multiples of dt_max; a
-        // launch ends where the other is to go on
+        // small systems: the cluster, or above FUSED_CLUSTER_NARROW_N particles before every step the
+        // cluster or the grid kernel as the levels say; a launch ends where the other is to go on
         const bool cluster = fused && cluster_ready(h);
-        fa.may_leave = cluster;
+        fa.may_leave = cluster && h->n > FUSED_CLUSTER_NARROW_N;
         auto launch_sched = [&]() -> int {
             const unsigned long long ep = h->seq_next++;
             int r;
             if (fused) {
-                fa.ask_now = !h->kernel_asked;
                 r = timed(h, T_FUSED, [&] {
                     const bool ds = h->cfg.variant == NB_F32DS;
-                    return cluster && !h->grid_last
+                    return cluster && !(fa.may_leave && h->grid_last)
                                ? launch_cluster_steps(fa, ds, h->n > FUSED_CLUSTER_NARROW_N, h->stream)
                                : launch_fused_steps(fa, h->fused_grid, ds, 4, h->stream);
                 });
@@ -1827,13 +1823,9 @@ int nb_step(nb_handle h, double t_end, nb_stats *st)
             if (rc) return rc;
             const double t_next = h->mail_h->t_next;
             const int na = h->mail_h->n_active;
-            if (!(t_next <= t_end)) {
-                if (cluster && !h->mail_h->leave) h->kernel_asked = true;
-                break;
-            }
-            if (cluster && na == 0 && h->mail_h->leave && left < 2) {
+            if (!(t_next <= t_end)) break;
+            if (fa.may_leave && na == 0 && h->mail_h->leave && left < 2) {
                 left = h->mail_h->steps ? 0 : left + 1;
-                if (h->mail_h->steps) h->kernel_asked = true;
                 h->stats.fused_launches -= h->mail_h->steps ? 0 : 1;  // it only asked
                 h->grid_last = !h->grid_last;
                 rc = launch_sched();
@@ -1841,7 +1833,6 @@ int nb_step(nb_handle h, double t_end, nb_stats *st)
                 continue;
             }
             left = 0;
-            h->kernel_asked = true;
             if (na < 1 || na > h->n)
                 return fail(h, NB_ERR_STATE, "scheduler returned %d due particles", na);
             rc = run_force(h, h->cfg.variant, due_set(h, na), f);

@@ -448,10 +448,9 @@ struct FusedArgs {
     // next block time with N_active = 0, nothing handed off, and it ends so at an error bit in *err
     // too. stats may be null there.
     int max_steps;
-    // order 4: end the launch so (with Mailbox::leave) where the rule of small systems gives the steps
-    // to the other kernel, grid or cluster. It is asked at multiples of dt_max (the cluster: and a
-    // sixteenth of it later), and with ask_now at the launch's first step.
-    bool may_leave, ask_now;
+    // order 4: end the launch so (with Mailbox::leave) before a step that the rule of small systems
+    // (grid_takes) gives to the other kernel, grid or cluster.
+    bool may_leave;
 };
 
 constexpr int FUSED_THREADS = 256;
@@ -464,9 +463,11 @@ constexpr int FUSED_SMALL_NA = 16;
 constexpr int FUSED6_MAX_NA = NB_FUSED6_MAX_NA;
 
 // 4th-order systems of up to FUSED_CLUSTER_MAX_N particles are stepped by one cluster of
-// FUSED_CLUSTER CTAs (persist.cu).
+// FUSED_CLUSTER CTAs while their due sets are small (persist.cu, grid_takes). Above, the grid kernel
+// is as good: Plummer spheres of 1800 5.3 ms against 6.0, 2500 7.6 and 8.2, 3200 7.5 and 7.6, 4000 10.8
+// and 10.2.
 constexpr int FUSED_CLUSTER = 16;
-constexpr int FUSED_CLUSTER_MAX_N = 4096;
+constexpr int FUSED_CLUSTER_MAX_N = 2000;
 constexpr int FUSED_CLUSTER_LIMIT_N = 8192;  // the most the kernel takes (request loop)
 // Up to here a handle's launch adds in FP32 alone within a CTA (32 particles).
 constexpr int FUSED_CLUSTER_NARROW_N = 512;
@@ -488,7 +489,7 @@ cudaError_t launch_selftest_barrier(unsigned *bar, unsigned *err, unsigned long 
                                     cudaStream_t st);
 // The same steps (order 4) by one cluster: needs no cnt, bar or part. wide: sums beyond short FP32
 // runs in double-single (the request loop and handles of more than FUSED_CLUSTER_NARROW_N
-// particles; up to FUSED_CLUSTER_LIMIT_N particles, else FUSED_CLUSTER_MAX_N). Ready: the current device can run that cluster.
+// particles; at most FUSED_CLUSTER_LIMIT_N). Ready: the current device can run that cluster.
 bool cluster_steps_ready();
 cudaError_t launch_cluster_steps(const FusedArgs &a, bool ds, bool wide, cudaStream_t st);
 cudaError_t launch_fused_steps(const FusedArgs &a, int grid, bool ds, int order,

@@ -482,12 +482,36 @@ __device__ __forceinline__ void small_item(const FusedArgs &a, int na, int n, in
     __syncthreads();  // s_red, s_fin and s_last are free for the next item
 }
 
+// Whether a system of FUSED_CLUSTER_NARROW_N to FUSED_CLUSTER_MAX_N particles is stepped by the grid
+// kernel and not by the cluster: by the mean due set of the steps to come, which the population of
+// the levels tells (h0, h1: levels lane and 32 + lane; kmax the last occupied one). A block time is a
+// multiple of 2^z smallest steps and no more, with z = 0 half of the time, z = 1 a quarter, ...;
+// level k is due with z >= kmax - k, in 2^-(kmax - k) of the steps. A level of more than na_max is left
+// out: either kernel hands its steps on. Both ask before every step and of nothing but the levels
+// and the handle's sizes, so a run and its continuation from any state take every step in the
+// same kernel; the levels are in registers anyway. A warp, all lanes; whole numbers.
+// The line, 175 - n / 32 due: a step of the cluster costs 8 us at 700 particles to 9 at 2000 and
+// 0.03 to 0.05 for each due one, one of the grid kernel 12 to 14 and next to nothing for each. us a
+// step, cluster and grid kernel: 80 of 700 in a dense core (mean due set 42) 10.9 and 13.4, 400 of 700
+// (162) 13.7 and 14.0, 300 of 1000 (121) 13.8 and 14.0, 1000 of 1000 (395) 23.3 and 15.2, 120 of 1500
+// (68) 14.0 and 13.1, 300 of 1500 (131) 15.6 and 14.1, 1000 of 1500 (386) 26.0 and 15.4, Plummer
+// spheres of 1000 (46) 10.2 and 12.5, 1800 (85) 12.1 and 13.7.
+__device__ __forceinline__ bool grid_takes(int h0, int h1, int kmax, int n, int na_max)
+{
+    const int lane = threadIdx.x & 31;
+    const int s0 = kmax - lane, s1 = s0 - 32;
+    unsigned mean64 = 0u;  // 64 times the mean
+    if (s0 >= 0 && h0 <= na_max) mean64 = ((unsigned)h0 << 6) >> min(s0, 31);
+    if (s1 >= 0 && h1 <= na_max) mean64 += ((unsigned)h1 << 6) >> s1;
+    return __reduce_add_sync(0xffffffffu, mean64) + 2u * (unsigned)n > 11200u;
+}
+
 // t_next = next multiple after t_cur of the smallest occupied step; the due
 // particles are exactly those whose step divides t_next (every t_i is a
 // multiple of dt_i and t_i <= t_cur < t_i + dt_i), so the due count is the
 // level histogram's sum over the levels k >= k0. Warp 0 of the CTA; lane 0
-// writes s_tn and s_na.
-__device__ __forceinline__ void next_block_time(const FusedArgs &a, double t_cur, double &s_tn,
+// writes s_tn and s_na. Returns grid_takes for these levels.
+__device__ __forceinline__ bool next_block_time(const FusedArgs &a, double t_cur, double &s_tn,
                                                 int &s_na)
 {
     static_assert(NLEVEL == 64, "two ballot words of levels");
@@ -508,6 +532,7 @@ __device__ __forceinline__ void next_block_time(const FusedArgs &a, double t_cur
         s_tn = tn;
         s_na = c;
     }
+    return grid_takes(h0, h1, kmax, a.s.n, a.na_max);
 }
 
 // Publish the end of a launch: the block time reached and, for a step handed
@@ -607,90 +632,6 @@ __device__ __forceinline__ bool handoff_predict_gather(const FusedArgs &a, doubl
     return barrier();
 }
 
-// ---- which kernel takes the steps of a small system --------------------------
-
-// Sixteenths of the power of two d beyond its last multiple at time t (0 to 15), -1 between them.
-// By the bits: asked at every step, and an FP64 instruction holds its pipe for 64 cycles.
-__device__ __forceinline__ int sixteenths(double t, double d)
-{
-    const unsigned long long u = (unsigned long long)__double_as_longlong(t) & ~(1ull << 63);
-    const int e = (int)(u >> 52);
-    const unsigned long long m = (u & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
-    const int shift = exponent_of(d) - 4 - ((e ? e : 1) - 1075);  // t = m 2^-shift sixteenths
-    if (m == 0ull) return 0;
-    if (shift <= -4) return 0;
-    if (shift > 52 || (shift > 0 && (m & ((1ull << shift) - 1ull)))) return -1;
-    const int r = (int)(shift > 0 ? m >> shift : m << -shift) & 15;
-    return __double_as_longlong(t) < 0 ? (16 - r) & 15 : r;
-}
-
-// Either kernel asks where all particles are at one time, at the multiples of dt_max (and, with
-// ask_now, at its first step), so a run and its continuation from a checkpoint there ask the
-// same questions; it takes 2 us. The cluster asks again a sixteenth of dt_max later: the initial
-// steps are shorter and spread over more levels than the ones after them, and make it look up
-// to half as costly as it is. The answer: 32 times the ratio of the costs (cluster to grid)
-// from which on the grid kernel takes the steps, 0 for no question.
-__device__ __forceinline__ unsigned question(const FusedArgs &a, double t_cur, bool first,
-                                             bool cluster)
-{
-    if (!a.may_leave) return 0u;
-    const int r = first && a.ask_now ? 0 : sixteenths(t_cur, a.prm.dt_max);
-    return r == 0 ? 31u : (r == 1 && cluster ? 38u : 0u);
-}
-
-// Eighths of a microsecond of a step with na due of n (at most 4096 each): in the cluster, and in
-// the grid kernel (within 15% of Plummer spheres' and of the steps of systems with one occupied
-// small level, n = 300 to 4000).
-__device__ __forceinline__ unsigned cluster_step_cost(unsigned na, unsigned n)
-{
-    return 60u + n / 256u + (na * (20972u + 31u * n) >> 18);
-}
-
-__device__ __forceinline__ unsigned grid_step_cost(unsigned na, unsigned n)
-{
-    if (na <= (unsigned)FUSED_SMALL_NA) return 96u;
-    return na < (unsigned)FUSED_IPT2_NA ? 107u : 120u + (na * (3146u + 3u * n) >> 18);
-}
-
-// Whether a system of at most FUSED_CLUSTER_MAX_N particles is stepped by the grid kernel and not
-// by the cluster: by the mean cost of its steps, which the population of the levels tells. A block
-// time is a multiple of 2^z smallest steps and no more, with z = 0 half of the time, z = 1 a
-// quarter, ..., and its due set the particles of the levels whose steps divide it. Plummer spheres
-// stay in the cluster up to some 4000 particles (2500: 7.0 ms a 1/16 time unit, the grid
-// kernel 8.0; 4000: 9.9 and 10.1); with hundreds due in half of the steps it is the slower: 600 of
-// 4000 in a dense core, 500 steps, 14.3 ms and 8.0. One warp, whole numbers: both kernels find
-// the same.
-__device__ __forceinline__ bool grid_takes(const FusedArgs &a, unsigned ratio32)
-{
-    const int lane = threadIdx.x & 31;
-    int d0 = __ldcg(a.sd->hist + lane), d1 = __ldcg(a.sd->hist + 32 + lane);
-    const unsigned b0 = __ballot_sync(0xffffffffu, d0 > 0);
-    const unsigned b1 = __ballot_sync(0xffffffffu, d1 > 0);
-    const int kmax = b1 ? 63 - __clz(b1) : (b0 ? 31 - __clz(b0) : 0);
-    // the particles of level k and above (smaller steps)
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int u0 = __shfl_down_sync(0xffffffffu, d0, o), u1 = __shfl_down_sync(0xffffffffu, d1, o);
-        if (lane + o < 32) {
-            d0 += u0;
-            d1 += u1;
-        }
-    }
-    d0 += __shfl_sync(0xffffffffu, d1, 0);
-    unsigned cl = 0u, gr = 0u;  // in 1/8192 of the steps
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int k = lane + 32 * h, na = h ? d1 : d0;
-        if (k > kmax || kmax - k > 12 || na < 1 || na > a.na_max) continue;  // larger: either hands on
-        const unsigned share = (4096u >> (kmax - k)) << (k == 0 ? 1 : 0);
-        cl += share * cluster_step_cost((unsigned)na, (unsigned)a.s.n);
-        gr += share * grid_step_cost((unsigned)na, (unsigned)a.s.n);
-    }
-    cl = __reduce_add_sync(0xffffffffu, cl);
-    gr = __reduce_add_sync(0xffffffffu, gr);
-    return 32u * cl > ratio32 * gr;
-}
-
 // ---- the kernel ------------------------------------------------------------
 
 template <bool DS>
@@ -723,7 +664,6 @@ __global__ void __launch_bounds__(FUSED_THREADS)
     double t_cur = __ldcg(&a.sd->t_cur);
     const unsigned long long epoch = __ldcg(&a.sd->seq);
     unsigned long long steps = 0;  // counted by thread 0 of CTA 0
-    bool first = true;
     double inter = 0.0;
     if (tid < 32) s_hist[tid] = s_step_ns[tid] = 0ull;
     if (tid < 4) s_phase[tid] = 0ull;
@@ -744,17 +684,14 @@ __global__ void __launch_bounds__(FUSED_THREADS)
         PState q0, q1;
         if (p0 + tid < p1) pstate_load(s, p0 + tid, q0);
         if (p0 + tid + NT < p1) pstate_load(s, p0 + tid + NT, q1);
-        if (warp == 1) {
-            const unsigned r = question(a, t_cur, first, false);
-            const bool leave = r && !grid_takes(a, r);
-            if (lane == 0) s_leave = leave;
+        if (warp == 0) {
+            const bool grid = next_block_time(a, t_cur, s_tn, s_na);
+            if (lane == 0) s_leave = a.may_leave && !grid;
         }
-        if (warp == 0) next_block_time(a, t_cur, s_tn, s_na);
         __syncthreads();
         const double tn = s_tn;
         const int na = s_na;
-        const bool leave = s_leave;
-        first = false;
+        const bool leave = s_leave && tn <= a.t_end && na >= 1 && na <= a.na_max;
         if (!(tn <= a.t_end) || na < 1 || na > a.na_max || leave) {
             // hand the step to the caller exactly as the scheduler kernel would
             if (tn <= a.t_end && na >= 1 && !leave) {
@@ -937,24 +874,22 @@ __global__ void __launch_bounds__(FUSED_THREADS)
 // The cluster barrier is a hardware barrier of co-scheduled CTAs (like __syncthreads):
 // no wait depends on another launch, and every exit is taken by all CTAs together.
 // Measured against the grid kernel, 1/16 time unit of block steps of Plummer spheres: N = 500
-// 5.3 -> 3.7 ms, 1000 5.3 -> 4.0, 2500 8.0 -> 7.0, 4000 10.1 -> 10.0. A step of 1 to 3 due at N = 2500
-// takes 9.1 us for 11.9: the prediction and its barrier 3.2, the force 3, the corrector 2.2.
-// Sixteen SMs are a tenth of the GPU, so due sets of a hundred and more cost that again
-// (N = 2500, 512-1023 due: 39 us against 17; N = 4000: 59 against 18): systems with many of them
-// stay with the grid kernel (grid_takes), and at 4096 particles nothing is gained any more.
+// 5.3 -> 3.7 ms, 1000 5.3 -> 4.3, 1800 6.0 -> 5.3. A step of 1 to 3 due at N = 1800 takes 9.4 us for 12.
+// Sixteen SMs are a tenth of the GPU, so due sets of a hundred and more cost that again (N = 1800,
+// 256-511 due: 24 us against 16; 512-1023: 44 against 17): systems with many of them stay with the grid
+// kernel (grid_takes).
 constexpr int CL_CTAS = FUSED_CLUSTER;
 constexpr int CL_THREADS = 512;
 constexpr int CL_Q = 7;                                  // outputs of a slot
 
 // WIDE: the sums of more than CL_RUN terms a half are double-single from there on, over the lanes
-// and over the CTAs. Without it a lane's run is all of its pairs (up to 256) and a CTA's partial
-// one FP32 sum of up to 512 terms. The request loop's integrations take it (their steps in the
-// ticks add FP32 terms in runs of 32 or 64), and the handles' steps above FUSED_CLUSTER_NARROW_N
-// particles: the median and 99% error of the jerk of Plummer spheres' due sets was 7 and 8% above the
-// grid kernel's at N = 1300, 8 and 9 at 1800, 12 and 16 at 2500, and is 0 to 4% below it; up to 512 a
-// CTA's 32 particles are one run, and the errors of either form no larger than the grid kernel's.
-// 1/16 time unit of Plummer spheres: N = 1000 4.0 -> 4.3 ms, 1800 4.9 -> 5.3, 2500 7.0 -> 7.6,
-// 8000 (request loop) 18.5 -> 19.6.
+// and over the CTAs. Without it a lane's run is all of its pairs and a CTA's partial one FP32 sum: for
+// the handles' systems of up to FUSED_CLUSTER_NARROW_N particles, 32 a CTA, whose jerk errors are no
+// larger than the grid kernel's. Above, the median and 99% error of Plummer spheres' due sets were 7
+// and 8% larger at N = 1300, 8 and 9 at 1800, and are 0 to 4% smaller with it. The request loop's
+// integrations take it at any size (their steps in the ticks add FP32 terms in runs of 32 or 64).
+// 1/16 time unit of Plummer spheres: N = 1000 4.0 -> 4.3 ms, 1800 4.9 -> 5.3, 8000 (request loop)
+// 18.5 -> 19.6.
 constexpr int CL_RUN = 16;
 
 // MAXL: the most particles of a CTA. A window of the due set has SLOTS slots (the wide
@@ -1221,17 +1156,16 @@ __global__ void __launch_bounds__(CL_THREADS)
         // a limited launch also ends at the first step with an error (the word is the system's
         // own, so every CTA reads the same)
         if (tid == 32) sm.err = a.max_steps > 0 ? __ldcg(a.err) : 0u;
-        if (warp == 1) {
-            const unsigned r = question(a, t_cur, steps == 0, true);
-            const bool leave = r && grid_takes(a, r);
-            if (lane == 0) sm.leave = leave;
+        if (warp == 0) {
+            const bool grid = next_block_time(a, t_cur, sm.tn, sm.na);
+            if (lane == 0) sm.leave = a.may_leave && grid;
         }
-        if (warp == 0) next_block_time(a, t_cur, sm.tn, sm.na);
         __syncthreads();
         const double tn = sm.tn;
         const int na = sm.na;
+        const bool leave = sm.leave && tn <= a.t_end && na >= 1 && na <= a.na_max;
         const bool limit =
-            (a.max_steps > 0 && (steps >= a.max_steps || sm.err != 0u)) || sm.leave;
+            (a.max_steps > 0 && (steps >= a.max_steps || sm.err != 0u)) || leave;
         if (!(tn <= a.t_end) || na < 1 || na > a.na_max || limit) {
             // hand the step to the caller exactly as the scheduler kernel would
             if (tn <= a.t_end && na >= 1 && !limit) {
@@ -1246,7 +1180,7 @@ __global__ void __launch_bounds__(CL_THREADS)
                 a.mail->steps = steps;
                 a.mail->interactions = inter;
                 a.mail->err = sm.err;
-                a.mail->leave = sm.leave;
+                a.mail->leave = leave;
                 publish(a, t_cur, tn, limit ? 0 : na, epoch);
             }
             break;
@@ -1854,7 +1788,7 @@ size_t fused_part_float2s(int grid, int na_max, int order)
     return need;
 }
 
-constexpr int CL_SMALL_L = FUSED_CLUSTER_MAX_N / CL_CTAS;
+constexpr int CL_SMALL_L = 256;
 constexpr int CL_LARGE_L = FUSED_CLUSTER_LIMIT_N / CL_CTAS;
 
 bool cluster_steps_ready()
@@ -1881,7 +1815,7 @@ bool cluster_steps_ready()
 
 cudaError_t launch_cluster_steps(const FusedArgs &a, bool ds, bool wide, cudaStream_t st)
 {
-    if (a.s.n > CL_CTAS * (wide ? CL_LARGE_L : CL_SMALL_L)) return cudaErrorInvalidValue;
+    if (a.s.n > (wide ? FUSED_CLUSTER_LIMIT_N : FUSED_CLUSTER_NARROW_N)) return cudaErrorInvalidValue;
     const auto go = a.s.n > CL_CTAS * CL_SMALL_L
                         ? (ds ? go_cluster_steps<true, CL_LARGE_L, true>
                               : go_cluster_steps<false, CL_LARGE_L, true>)

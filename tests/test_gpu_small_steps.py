@@ -24,7 +24,13 @@ def _system(nb, n, core, **cfg):
                      device=0, **cfg)
 
 
-SIZES = [(300, 200), (1500, 1000), (2500, 300), (2500, 700), (4000, 150), (4000, 1000), (4096, 3000)]
+def _same(want, got):
+    for key in want:
+        np.testing.assert_array_equal(got[key], want[key], err_msg=key)
+
+
+SIZES = [(300, 200), (700, 400), (1500, 300), (1500, 1000), (1999, 150), (2500, 300), (2500, 700),
+         (4000, 150), (4000, 1000), (4096, 3000)]
 
 
 @pytest.mark.parametrize("n,core", SIZES)
@@ -47,16 +53,14 @@ def test_a_run_and_its_continuation_agree_bit_for_bit(nb, n, core, fused_max_na)
                     other.set_state(here)
                     other.step(t)
                     got = other.state()
-                for a, b in zip(want, got):
-                    np.testing.assert_array_equal(a, b)
-        for a, b in zip(want, sy.state()):
-            np.testing.assert_array_equal(a, b)
+                _same(want, got)
+        _same(want, sy.state())
 
 
-@pytest.mark.parametrize("n,core", [(2500, 700), (4000, 1000), (4096, 3000)])
+@pytest.mark.parametrize("n,core", [(1000, 1000), (1500, 1000), (2500, 700), (4000, 1000), (4096, 3000)])
 def test_large_due_sets_stay_with_the_grid_kernel(nb, n, core):
-    """Hundreds due in half of the steps: the grid kernel takes them from the first multiple of dt_max
-    on. Told by the time of a step, which is half and less of the cluster's at these sizes."""
+    """Hundreds due in half of the steps: the grid kernel takes them. Told by the time of a
+    step, which is half and less of the cluster's at these sizes."""
     with _system(nb, n, core, fused_max_na=4096) as sy:
         sy.step(1.0 / 64)
         st = sy.step(1.0 / 32)
@@ -64,3 +68,19 @@ def test_large_due_sets_stay_with_the_grid_kernel(nb, n, core):
     k = int(np.argmax(steps[8:])) + 8
     # measured: 17 to 38 us in the grid kernel, 41 to 202 in the cluster
     assert 1e3 * ms[k] / steps[k] < 25.0 + 2.0 ** k * n * 4e-6, k
+
+
+@pytest.mark.parametrize("n,core", [(300, 200), (512, 512), (513, 60), (1400, 300)])
+def test_steps_do_not_depend_on_the_system_before(nb, n, core):
+    """A handle whose last system was the grid kernel's steps the next one as a new handle does."""
+    t = 1.0 / 64
+    with _system(nb, n, core) as sy:
+        nb.nb_init(sy.h)
+        start = sy.state()
+        sy.step(t)
+        want = sy.state()
+    with _system(nb, 1500, 1000) as sy:
+        sy.step(t)
+        sy.set_state(start)
+        sy.step(t)
+        _same(want, sy.state())
