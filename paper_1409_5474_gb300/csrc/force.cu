@@ -1363,6 +1363,7 @@ constexpr int TILE_FINE_NI = 4096;
 constexpr int RUN_FINE = 16;
 constexpr int RUN_ROWS = 64;   // larger sets, several warp rows
 constexpr int RUN_WHOLE = 128;  // larger sets, one warp row: a tile
+constexpr int WGRP_NJ = 576;  // most j-particles of the warp groups' sets
 constexpr int JT64 = 64;
 constexpr int NS64 = 3;
 
@@ -1465,6 +1466,17 @@ ForcePlan plan_force(int variant, int n_i, int n_j, int num_sms, size_t max_part
     if (n_i <= (n_j > 65536 ? 8 : 4)) {
         tiny_shape(n_i, n_j, p);
         if (p.nsplit == 1 || p.nsplit <= fit) return p;
+    }
+    // A small j-set: the warp groups, whose lanes then add 18 terms at most. The tile kernel's runs, 32
+    // with both halves, are longer: its median jerk error for whole systems (60 Plummer spheres each) is 4%
+    // larger at 128, 5% at 200 and 256, 4% at 300, 1% at 500, 1% smaller at 600 and 3% at 800; and one
+    // launch without partials is as fast (a call for a whole system of 300 51.5 -> 49.9 us, of 512 52.6
+    // -> 51.2; for 2000 outside positions on 512 81 -> 86).
+    if (n_j <= WGRP_NJ && n_i < TILE_FINE_NI) {
+        p.kind = 1;
+        wgrp_shape(n_i, p);
+        p.nsplit = 1;
+        return p;
     }
     // Tiles: the warp rows (8, 4 or 1: 64, 128 or 512 i-particles per CTA) and j-splits of
     // least estimated time. An SM's CTAs share its pipes, so its time is its count of CTAs

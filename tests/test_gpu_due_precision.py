@@ -11,9 +11,9 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-def _field(nb, n, ni, entry=None):
+def _field(nb, n, ni, entry=None, grain=2.0 ** -18):
     rng = np.random.default_rng(n + ni)
-    m = 1.0 + 2.0 ** -18 * rng.integers(0, 2, n)
+    m = 1.0 + grain * rng.integers(0, 2, n)
     x = np.zeros((n, 3))
     x[:, 0] = 1.0
     with nb.System(m, x, np.zeros((n, 3)), variant="f32ds", eps=0.0, device=0) as sy:
@@ -29,6 +29,17 @@ def _field(nb, n, ni, entry=None):
 @pytest.mark.parametrize("entry", [None, (1, 1, 2)])
 def test_fp32_sums_of_due_sets_are_short(nb, n, ni, entry):
     total, acc, jerk, pot = _field(nb, n, ni, entry)
+    np.testing.assert_array_equal(pot, np.full(ni, -total))
+    np.testing.assert_array_equal(acc[0], np.full(ni, total))
+    assert not acc[1:].any() and not jerk.any()
+
+
+@pytest.mark.parametrize("n", [100, 200, 300, 400, 480])
+@pytest.mark.parametrize("ni", [5, 33, 300, 480, 1531])
+def test_fp32_sums_over_small_systems_are_shorter(nb, n, ni):
+    """Up to 480 particles a lane of the warp groups adds 15 terms at most: with masses of 1 or
+    1 + 2^-20 up to 15 are exact, and an odd sum of 16 and more is not."""
+    total, acc, jerk, pot = _field(nb, n, ni, grain=2.0 ** -20)
     np.testing.assert_array_equal(pot, np.full(ni, -total))
     np.testing.assert_array_equal(acc[0], np.full(ni, total))
     assert not acc[1:].any() and not jerk.any()
