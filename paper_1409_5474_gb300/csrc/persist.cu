@@ -874,9 +874,9 @@ __global__ void __launch_bounds__(FUSED_THREADS)
 // The cluster barrier is a hardware barrier of co-scheduled CTAs (like __syncthreads):
 // no wait depends on another launch, and every exit is taken by all CTAs together.
 // Measured against the grid kernel, 1/16 time unit of block steps of Plummer spheres: N = 500
-// 5.3 -> 3.7 ms, 1000 5.3 -> 4.3, 1800 6.0 -> 5.3. A step of 1 to 3 due at N = 1800 takes 9.4 us for 12.
+// 5.3 -> 3.8 ms, 1000 5.4 -> 4.3, 1800 6.0 -> 5.4. A step of 1 to 3 due at N = 1800 takes 9.7 us for 12.1.
 // Sixteen SMs are a tenth of the GPU, so due sets of a hundred and more cost that again (N = 1800,
-// 256-511 due: 24 us against 16; 512-1023: 44 against 17): systems with many of them stay with the grid
+// 256-511 due: 24 us against 17; 512-1023: 44 against 18): systems with many of them stay with the grid
 // kernel (grid_takes).
 constexpr int CL_CTAS = FUSED_CLUSTER;
 constexpr int CL_THREADS = 512;
